@@ -97,7 +97,7 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
   a.omega0 = omega_of(opts);
   a.mode = mode;
   ar->avg_mode = mode;
-  launch_reduce_S(A, M, lam, alpha, mode, false, st, true);
+  launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kPlain);
   // every sweep hands its path costs to the next one (the S reductions
   // between them leave lambda alone), except into the first sweep, whose
   // lambda comes from the caller, and across a re-projection
@@ -108,13 +108,13 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
     a.cost_out = A.nodecost;
     a.cost_in = handed ? A.nodecost : nullptr;
     launch_sweep(kFwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_reduce_S(A, M, lam, alpha, mode, false, st, true);
+    launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kPlain);
     if (lb_out && it == iters - 1) a.E = A.E;
     handed = it + 1 < iters && !rn;
     a.cost_out = handed ? A.nodecost : nullptr;
     a.cost_in = A.nodecost;
     launch_sweep(kBwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_reduce_S(A, M, lam, alpha, mode, rn, st, it + 1 < iters);
+    launch_reduce_S(A, M, lam, alpha, mode, rn, st, it + 1 < iters ? Scatter::kPlain : Scatter::kNone);
   }
   if (lb_out) {
     if (iters == 0) {
@@ -290,6 +290,8 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
     if (bytes) std::memcpy(h.data() + off, src, bytes);
   };
   cp(P.off.tiles, P.tiles.data(), P.tiles.size() * sizeof(Tile));
+  cp(P.off.unit_shapes, P.unit_shapes.data(), P.unit_shapes.size() * sizeof(UnitShape));
+  cp(P.off.unit_runs, P.unit_runs.data(), P.unit_runs.size() * 2);
   cp(P.off.desc, P.desc.data(), P.desc.size() * 2);
   cp(P.off.lohi8, P.lohi8.data(), P.lohi8.size() * 2);
   cp(P.off.slot_var, P.slot_var.data(), P.slot_var.size() * 4);
@@ -322,6 +324,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
     if (e != cudaSuccess) return cuda_fail(e, "dg_bind: device attribute");
     if ((size_t)optin < P.smem_sweep) return fail(DG_EINVAL, "dg_bind: tiles need more shared memory than a CTA has");
     e = set_sweep_smem_limit((size_t)optin);  // same limit for every arena of the process
+    if (e == cudaSuccess) e = set_unit_smem_limit((size_t)optin);
     if (e == cudaSuccess) e = set_adjoint_smem_limit((size_t)optin);
     set_cta_smem_cap((size_t)optin);
     if (e != cudaSuccess) return cuda_fail(e, "dg_bind: shared-memory limit");
@@ -348,6 +351,9 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   char* b = (char*)arena_dev;
   DevArena& A = ar->dev;
   A.tiles = (const Tile*)(b + P.off.tiles);
+  A.unit_shapes = (const UnitShape*)(b + P.off.unit_shapes);
+  A.unit_runs = (const uint16_t*)(b + P.off.unit_runs);
+  A.unit_slots = P.unit_slots;
   A.desc = (const uint16_t*)(b + P.off.desc);
   A.lohi8 = (const uint16_t*)(b + P.off.lohi8);
   A.slot_var = (const int32_t*)(b + P.off.slot_var);
@@ -504,7 +510,7 @@ dg_status dg_autotune(dg_arena* ar, void* stream, float* lam, float* M, int32_t 
     return ms / reps;
   };
   ar->avg_mode = 0;
-  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, true);
+  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, Scatter::kPlain);
   // timed as dg_iterate runs them after its first sweep: each sweep takes
   // its opposite-direction costs from the one before
   a.cost_out = A.nodecost;
@@ -517,8 +523,8 @@ dg_status dg_autotune(dg_arena* ar, void* stream, float* lam, float* M, int32_t 
   };
   // start from the occupancy choice, made explicit
   for (LaunchGroup& G : ar->groups) {
-    G.wpc_fwd = (int8_t)best_warps_per_cta((size_t)G.region_bytes0, 4, ar->cta_smem_cap);
-    G.wpc_bwd = (int8_t)best_warps_per_cta((size_t)G.region_bwd0, 4, ar->cta_smem_cap);
+    G.wpc_fwd = (int8_t)best_warps_per_cta((size_t)(G.unit_w ? G.unit_bytes0 : G.region_bytes0), 4, ar->cta_smem_cap);
+    G.wpc_bwd = (int8_t)best_warps_per_cta((size_t)(G.unit_w ? G.unit_bytes0 : G.region_bwd0), 4, ar->cta_smem_cap);
   }
   float best = 3.0e38f;
   int bestn = kStreams;
@@ -535,7 +541,7 @@ dg_status dg_autotune(dg_arena* ar, void* stream, float* lam, float* M, int32_t 
   for (LaunchGroup& G : ar->groups) {
     for (int dir = 0; dir < 2; ++dir) {
       int8_t& cur = dir == 0 ? G.wpc_fwd : G.wpc_bwd;
-      const size_t region = (size_t)(dir == 0 ? G.region_bytes0 : G.region_bwd0);
+      const size_t region = (size_t)(G.unit_w ? G.unit_bytes0 : dir == 0 ? G.region_bytes0 : G.region_bwd0);
       const int8_t keep = cur;
       for (int w = 1; w <= 4; w *= 2) {
         if (w == keep || region * w > ar->cta_smem_cap) continue;
@@ -583,7 +589,7 @@ dg_status dg_sum_M(dg_arena* ar, void* stream, const float* M, float* lam, const
   ar->avg_mode = mode;
   // a reduction without re-projection leaves lambda, so a hand-off survives it
   if (!renorm) keep_costs(ar);
-  launch_reduce_S(ar->dev, M, lam, alpha, mode, renorm != 0, (cudaStream_t)stream, true);
+  launch_reduce_S(ar->dev, M, lam, alpha, mode, renorm != 0, (cudaStream_t)stream, Scatter::kPlain);
   return check_launch("dg_sum_M");
 }
 
@@ -657,7 +663,7 @@ dg_status dg_lower_bound(dg_arena* ar, void* stream, const float* lam, const flo
   a.E = ar->dev.E;
   launch_sweep(kEnergy, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(),
                streams_for(ar, st));
-  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, st, false);
+  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, st, Scatter::kNone);
   launch_lower_bound(ar->dev, lb, st);
   if (E_per_row) {
     cudaError_t e = cudaMemcpyAsync(E_per_row, ar->dev.E, (size_t)ar->dev.m * 4, cudaMemcpyDeviceToDevice, st);
@@ -685,7 +691,7 @@ dg_status dg_lb_seed(dg_arena* ar, void* stream, const float* lam, const float* 
   a.M = g_lam;
   launch_sweep(kSeed, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(),
                streams_for(ar, st));
-  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, st, false);
+  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, st, Scatter::kNone);
   launch_seed_M(ar->dev, g_M, st);
   return check_launch("dg_lb_seed");
 }
@@ -858,7 +864,7 @@ dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, fl
   cudaError_t e = cudaSuccess;
   ar->avg_mode = mode;
   for (int sw = 0; sw < 2 * k; ++sw) {
-    launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, true);
+    launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, Scatter::kAll);
     if (e == cudaSuccess && n)
       e = cudaMemcpyAsync(w + L.seg_S + (size_t)sw * n * 4, A.S, n * 4, cudaMemcpyDeviceToDevice, st);
     SweepArgs ra = fa;
@@ -878,7 +884,7 @@ dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, fl
     launch_sweep(sw % 2 == 0 ? kFwdRec : kBwdRec, A, ra, threads_of(opts), ar->groups.data(), (int)ar->groups.size(),
                  streams_for(ar, st));
   }
-  launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, false);
+  launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, Scatter::kNone);
   if (lb_out) launch_lower_bound(A, lb_out, st);
   if (e != cudaSuccess) return cuda_fail(e, "recorded segment copies");
   return check_launch("recorded segment");
@@ -982,9 +988,9 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       f.cost_in = handed ? A.nodecost : nullptr;
       b.cost_in = A.nodecost;
       handed = true;
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, true);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kPlain);
       launch_sweep(kFwd, A, f, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, true);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kPlain);
       launch_sweep(kBwd, A, b, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
     }
   }
@@ -1017,7 +1023,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       cpy(w_M, ck_M + (size_t)c * NS, bNS);
     }
     for (int sw = 0; sw < (recorded ? 0 : nsw); ++sw) {
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, true);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kAll);
       cpy(seg_S + (size_t)sw * n, A.S, bn);
       SweepArgs ra = fa;
       ra.rec_meta = (uint16_t*)(rec_meta + (size_t)sw * L.meta_stride);

@@ -12,7 +12,9 @@
 #include <atomic>
 #include <cstring>
 #include <numeric>
+#include <string>
 #include <thread>
+#include <unordered_map>
 
 #include "dg_internal.h"
 
@@ -148,6 +150,125 @@ RowResult build_row(const int32_t* a, int k, int sense, int64_t rhs, RowScratch&
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Shape of a unit row as the unit kernels sweep it, before it has a place in
+// the arena.
+struct UnitRow {
+  UnitShape s{};
+  std::vector<uint8_t> type;  // per level
+};
+
+inline int unit_z(int t, int u) { return t == kSwap ? std::max(u - 1, 0) : u; }
+inline int unit_o(int t, int u) {
+  return t == kUp ? u + 1 : (t == kSwap ? u : (t == kDown ? std::max(u - 1, 0) : u - 1));
+}
+
+// Tries to read the row sum_h a_h x_h (<= or =) rhs, all a_h = +-1, as a unit
+// row (see UnitShape) whose states are the nodes of its canonical BDD
+// (level_keys, k levels).  Every arc of the BDD is compared with the shape.
+bool unit_candidate(const int8_t* a, int k, bool eq, int64_t rhs, const std::vector<std::vector<uint64_t>>& level_keys,
+                    UnitRow& out) {
+  // sums from which every completion is feasible act like clamp[g] ('<='),
+  // those outside the alive range like the bottom
+  std::vector<int64_t> pos(k + 1, 0), neg(k + 1, 0);
+  for (int h = k - 1; h >= 0; --h) {
+    pos[h] = pos[h + 1] + (a[h] > 0);
+    neg[h] = neg[h + 1] + (a[h] < 0);
+  }
+  auto clamp_at = [&](int g) { return eq ? INT64_MIN / 4 : rhs - pos[g]; };
+  std::vector<int64_t> l(k + 1), hi(k + 1);
+  l[0] = hi[0] = std::max<int64_t>(0, clamp_at(0));
+  for (int g = 0; g <= k; ++g) {
+    if (g > 0) {
+      l[g] = l[g - 1] - (a[g - 1] < 0);
+      hi[g] = hi[g - 1] + (a[g - 1] > 0);
+    }
+    hi[g] = std::max(std::min(hi[g], rhs + neg[g]), clamp_at(g));
+    l[g] = std::max(l[g], eq ? rhs - pos[g] : clamp_at(g));
+    if (l[g] > hi[g]) return false;
+  }
+  int64_t smin = l[0];
+  for (int g = 0; g < k; ++g) smin = std::min(smin, l[g]);
+  std::vector<int64_t> base(k + 1);
+  for (int g = 0; g < k; ++g) base[g] = std::max(smin, clamp_at(g));
+  base[k] = base[k - 1];
+  int64_t W = 1;
+  for (int g = 0; g < k; ++g) W = std::max(W, hi[g] - base[g] + 1);
+  W = std::max(W, hi[k] - base[k] + 1);
+  if (W > kUnitMaxW) return false;
+  UnitShape& s = out.s;
+  s.W = (int32_t)((W + 1) / 2 * 2);
+  s.k = k;
+  s.start = (int32_t)(l[0] - base[0]);
+  s.accept = 0;
+  for (int u = 0; u < s.W; ++u)
+    if (eq ? base[k] + u == rhs : base[k] + u <= rhs) s.accept |= 1 << u;
+  out.type.assign(k, 0);
+  for (int h = 0; h < k; ++h) {
+    const int64_t shift = base[h + 1] - base[h];
+    if (shift < 0 || shift > (a[h] > 0 ? 1 : 0)) return false;
+    out.type[h] = (uint8_t)(a[h] > 0 ? (shift == 0 ? kUp : kSwap) : (eq ? kDrop : kDown));
+  }
+  // the shape's own feasibility, then every node and arc of the BDD
+  std::vector<uint32_t> alive(k + 1);
+  alive[k] = (uint32_t)s.accept;
+  for (int h = k - 1; h >= 0; --h) {
+    alive[h] = 0;
+    for (int u = 0; u < s.W; ++u) {
+      const int z = unit_z(out.type[h], u), o = unit_o(out.type[h], u);
+      if (((alive[h + 1] >> z) & 1) || (o >= 0 && o < s.W && ((alive[h + 1] >> o) & 1))) alive[h] |= 1u << u;
+    }
+  }
+  std::vector<int> at(1, s.start), next;
+  if (level_keys[0].size() != 1 || !((alive[0] >> s.start) & 1)) return false;
+  for (int h = 0; h < k; ++h) {
+    const std::vector<uint64_t>& keys = level_keys[h];
+    next.assign(h + 1 < k ? level_keys[h + 1].size() : 0, -1);
+    for (size_t r = 0; r < keys.size(); ++r) {
+      if (at[r] < 0 || (r > 0 && at[r] >= at[r - 1])) return false;  // ranks descend in u
+      for (int beta = 0; beta < 2; ++beta) {
+        const int child = beta ? key_hi(keys[r]) : key_lo(keys[r]);
+        const int t = beta ? unit_o(out.type[h], at[r]) : unit_z(out.type[h], at[r]);
+        const bool live = t >= 0 && t < s.W && ((alive[h + 1] >> t) & 1);
+        if ((child != kCodeBot) != live) return false;
+        if (!live) continue;
+        if (h + 1 == k) {
+          if (child != kCodeTop) return false;
+        } else {
+          if (child < 0 || (next[child] >= 0 && next[child] != t)) return false;
+          next[child] = t;
+        }
+      }
+    }
+    at.swap(next);
+  }
+  return true;
+}
+
+bool unit_row(const int32_t* a, int k, int sense, int64_t rhs, const std::vector<std::vector<uint64_t>>& level_keys,
+              UnitRow& out) {
+  std::vector<int8_t> sign(k);
+  for (int h = 0; h < k; ++h) {
+    if (a[h] != 1 && a[h] != -1) return false;
+    sign[h] = (int8_t)(sense == 1 ? -a[h] : a[h]);
+  }
+  if (sense != 2) return unit_candidate(sign.data(), k, false, sense == 1 ? -rhs : rhs, level_keys, out);
+  if (unit_candidate(sign.data(), k, true, rhs, level_keys, out)) return true;
+  for (int h = 0; h < k; ++h) sign[h] = (int8_t)-sign[h];
+  return unit_candidate(sign.data(), k, true, -rhs, level_keys, out);
+}
+
+// A row's BDD as the builder keeps it for later rows with the same terms.
+struct RowBdd {
+  std::vector<std::vector<uint64_t>> level_keys;
+  int64_t nodes = 0;
+  int maxw = 0;
+  int unit = -1;  // index into the building thread's unit shapes
+};
+// ... up to kRowCache of them per building thread, none larger than this
+constexpr size_t kRowCache = 4096;
+constexpr int kRowCacheTerms = 512;
+constexpr int64_t kRowCacheNodes = 2048;
+
 }  // namespace
 
 dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
@@ -206,6 +327,8 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     std::vector<uint8_t> width;
     std::vector<int8_t> lo, hi;
     std::vector<int32_t> nodes_of_row;
+    std::vector<int32_t> unit_of_row;  // index into `units`, -1 for other rows
+    std::vector<UnitRow> units;        // distinct unit shapes, by first row
     // rows whose BDD exceeds the tile limits: row, level widths, child ranks
     std::vector<int64_t> long_rows;
     std::vector<int32_t> lwidth, llo, lhi;
@@ -219,31 +342,66 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     RowScratch sc;
     Part& pt = parts[t];
     pt.nodes_of_row.reserve(cut[t + 1] - cut[t]);
+    pt.unit_of_row.reserve(cut[t + 1] - cut[t]);
+    // most rows of an instance repeat a few (coefficients, sense, rhs): their
+    // BDD is built once per thread
+    std::unordered_map<std::string, RowBdd> cache;
+    std::unordered_map<std::string, int> unit_index;
+    std::string key;
+    RowBdd built;
     for (int64_t j = cut[t]; j < cut[t + 1]; ++j) {
       const int64_t b = R->row_ptr[j];
       const int k = (int)(R->row_ptr[j + 1] - b);
-      RowResult r = build_row(R->coef + b, k, R->sense[j], R->rhs[j], sc);
-      if (r.status != 0) {
-        pt.err = r;
-        pt.err_row = j;
-        return;
+      const RowBdd* bdd = nullptr;
+      if (k <= kRowCacheTerms) {
+        key.assign((const char*)(R->coef + b), (size_t)k * 4);
+        key.append((const char*)&R->rhs[j], 4);
+        key.push_back((char)R->sense[j]);
+        auto it = cache.find(key);
+        if (it != cache.end()) bdd = &it->second;
       }
-      if (sc.nodes <= kMaxNodesPerBdd && sc.maxw <= kMaxWidth) {
+      if (!bdd) {
+        RowResult r = build_row(R->coef + b, k, R->sense[j], R->rhs[j], sc);
+        if (r.status != 0) {
+          pt.err = r;
+          pt.err_row = j;
+          return;
+        }
+        built.level_keys.assign(sc.level_keys.begin(), sc.level_keys.begin() + k);
+        built.nodes = sc.nodes;
+        built.maxw = sc.maxw;
+        built.unit = -1;
+        UnitRow u;
+        if (sc.nodes <= kMaxNodesPerBdd && sc.maxw <= kUnitMaxW &&
+            unit_row(R->coef + b, k, R->sense[j], R->rhs[j], built.level_keys, u)) {
+          std::string uk((const char*)&u.s, sizeof(UnitShape));
+          uk.append((const char*)u.type.data(), u.type.size());
+          auto at = unit_index.emplace(uk, (int)pt.units.size());
+          if (at.second) pt.units.push_back(u);
+          built.unit = at.first->second;
+        }
+        if (k <= kRowCacheTerms && built.nodes <= kRowCacheNodes && cache.size() < kRowCache)
+          bdd = &cache.emplace(key, std::move(built)).first->second;
+        else
+          bdd = &built;
+      }
+      pt.unit_of_row.push_back(bdd->unit);
+      if (bdd->nodes <= kMaxNodesPerBdd && bdd->maxw <= kMaxWidth) {
         for (int h = 0; h < k; ++h) {
-          pt.width.push_back((uint8_t)sc.level_keys[h].size());
-          for (uint64_t key : sc.level_keys[h]) {
+          pt.width.push_back((uint8_t)bdd->level_keys[h].size());
+          for (uint64_t key : bdd->level_keys[h]) {
             pt.lo.push_back((int8_t)key_lo(key));
             pt.hi.push_back((int8_t)key_hi(key));
           }
         }
-        pt.nodes_of_row.push_back((int32_t)sc.nodes);
+        pt.nodes_of_row.push_back((int32_t)bdd->nodes);
       } else {
         pt.width.insert(pt.width.end(), (size_t)k, (uint8_t)0);
         pt.nodes_of_row.push_back(0);
         pt.long_rows.push_back(j);
         for (int h = 0; h < k; ++h) {
-          pt.lwidth.push_back((int32_t)sc.level_keys[h].size());
-          for (uint64_t key : sc.level_keys[h]) {
+          pt.lwidth.push_back((int32_t)bdd->level_keys[h].size());
+          for (uint64_t key : bdd->level_keys[h]) {
             pt.llo.push_back(key_lo(key));
             pt.lhi.push_back(key_hi(key));
           }
@@ -267,14 +425,27 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
   P.node_ptr.assign(m + 1, 0);
   std::vector<int64_t> long_rows;
   std::vector<int32_t> long_width;  // level widths of the long BDDs, in row order
+  std::vector<UnitRow> units;       // distinct unit shapes, by first row
+  std::vector<int32_t> unit_of_row(m, -1);
   {
+    std::unordered_map<std::string, int> unit_index;
     int64_t j = 0;
     for (int t = 0; t < nthreads; ++t) {
       width.insert(width.end(), parts[t].width.begin(), parts[t].width.end());
       P.lo8.insert(P.lo8.end(), parts[t].lo.begin(), parts[t].lo.end());
       P.hi8.insert(P.hi8.end(), parts[t].hi.begin(), parts[t].hi.end());
-      for (int32_t c : parts[t].nodes_of_row) {
-        P.node_ptr[j + 1] = P.node_ptr[j] + c;
+      std::vector<int> global;
+      for (const UnitRow& u : parts[t].units) {
+        std::string uk((const char*)&u.s, sizeof(UnitShape));
+        uk.append((const char*)u.type.data(), u.type.size());
+        auto at = unit_index.emplace(uk, (int)units.size());
+        if (at.second) units.push_back(u);
+        global.push_back(at.first->second);
+      }
+      for (size_t x = 0; x < parts[t].nodes_of_row.size(); ++x) {
+        const int u = parts[t].unit_of_row[x];
+        if (u >= 0) unit_of_row[j] = global[u];
+        P.node_ptr[j + 1] = P.node_ptr[j] + parts[t].nodes_of_row[x];
         ++j;
       }
       long_rows.insert(long_rows.end(), parts[t].long_rows.begin(), parts[t].long_rows.end());
@@ -296,27 +467,79 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
 
   // ---- 2. tiles: 32 BDDs per tile, one per lane ---------------------------
   // Rows are cut into chunks of consecutive rows (so that a tile's variables,
-  // and the S values its lanes gather, stay close together); inside a chunk
-  // BDDs are sorted by hop count and node count, longest first, and every 32
-  // consecutive BDDs form a tile.  Inside a tile everything is interleaved by
+  // and the S values its lanes gather, stay close together).  Inside a chunk
+  // the unit rows of one shape fill tiles of their own (row order), the other
+  // rows are sorted by hop count and node count, longest first, and every 32
+  // consecutive ones form a tile.  Inside a tile everything is interleaved by
   // lane: slot (h, b) is slot_base + 32 h + b and node number n of lane b is
   // element 32 n + b of the per-tile arrays.  Node numbers 0 and 1 stand for
   // the top and bottom terminals, the BDD's own nodes are numbered 2, 3, ...
   // level by level; child codes are node numbers (8 bits).
   // Rows of the long BDDs take no tile (they are laid out after the tiles).
   const int64_t kChunkRows = opts && opts->chunk_rows > 0 ? opts->chunk_rows : 16384;
+  struct TileSrc {
+    int64_t first;  // its rows: order[first .. first + count)
+    int count, unit;
+  };
   std::vector<int64_t> order;
+  std::vector<TileSrc> src;
   order.reserve(m - (int64_t)long_rows.size());
-  for (int64_t j = 0; j < m; ++j)
-    if (P.long_of_row[j] < 0) order.push_back(j);
-  const int64_t m_tiles = (int64_t)order.size();
-  std::stable_sort(order.begin(), order.end(), [&](int64_t x, int64_t y) {
-    const int64_t cx = x / kChunkRows, cy = y / kChunkRows;
-    if (cx != cy) return cx < cy;
-    int64_t kx = R->row_ptr[x + 1] - R->row_ptr[x], ky = R->row_ptr[y + 1] - R->row_ptr[y];
-    if (kx != ky) return kx > ky;
-    return (P.node_ptr[x + 1] - P.node_ptr[x]) > (P.node_ptr[y + 1] - P.node_ptr[y]);
-  });
+  {
+    // a shape's last tile is rarely full.  It becomes a unit tile of its own
+    // when at least half its lanes are in use, or while a chunk has few such
+    // tiles (an empty lane costs memory, a mixed tile several times a unit
+    // tile's time); the rows of the others join the mixed tiles
+    constexpr int kHalf = kWarp / 2, kFewPartial = 64;
+    std::vector<std::pair<int32_t, int64_t>> by_shape;
+    std::vector<int64_t> mixed;
+    std::vector<TileSrc> part;
+    for (int64_t c0 = 0; c0 < m; c0 += kChunkRows) {
+      const int64_t c1 = std::min(m, c0 + kChunkRows);
+      by_shape.clear();
+      mixed.clear();
+      part.clear();
+      for (int64_t j = c0; j < c1; ++j) {
+        if (P.long_of_row[j] >= 0) continue;
+        if (unit_of_row[j] >= 0)
+          by_shape.emplace_back(unit_of_row[j], j);
+        else
+          mixed.push_back(j);
+      }
+      std::sort(by_shape.begin(), by_shape.end());
+      size_t full = 0;
+      for (size_t x = 0; x < by_shape.size();) {
+        size_t e = x;
+        while (e < by_shape.size() && e - x < (size_t)kWarp && by_shape[e].first == by_shape[x].first) ++e;
+        if (e - x == (size_t)kWarp) {
+          src.push_back({(int64_t)order.size(), kWarp, by_shape[x].first});
+          for (size_t y = x; y < e; ++y) order.push_back(by_shape[y].second);
+          ++full;
+        } else {
+          part.push_back({(int64_t)x, (int)(e - x), by_shape[x].first});
+        }
+        x = e;
+      }
+      std::stable_sort(part.begin(), part.end(), [](const TileSrc& x, const TileSrc& y) { return x.count > y.count; });
+      for (size_t i = 0; i < part.size(); ++i) {
+        const TileSrc& t = part[i];
+        const bool own = t.count >= kHalf || i < std::max<size_t>(kFewPartial, full / 8);
+        if (own) src.push_back({(int64_t)order.size(), t.count, t.unit});
+        for (int64_t y = t.first; y < t.first + t.count; ++y)
+          (own ? order : mixed).push_back(by_shape[y].second);
+      }
+      std::stable_sort(mixed.begin(), mixed.end(), [&](int64_t x, int64_t y) {
+        const int64_t kx = R->row_ptr[x + 1] - R->row_ptr[x], ky = R->row_ptr[y + 1] - R->row_ptr[y];
+        if (kx != ky) return kx > ky;
+        const int64_t nx = P.node_ptr[x + 1] - P.node_ptr[x], ny = P.node_ptr[y + 1] - P.node_ptr[y];
+        return nx != ny ? nx > ny : x < y;
+      });
+      for (size_t x = 0; x < mixed.size(); x += kWarp) {
+        const size_t e = std::min(mixed.size(), x + kWarp);
+        src.push_back({(int64_t)order.size(), (int)(e - x), -1});
+        order.insert(order.end(), mixed.begin() + x, mixed.begin() + e);
+      }
+    }
+  }
   int max_hops = 0, max_width = 0;
   for (int64_t j = 0; j < m; ++j) {
     int k = (int)(R->row_ptr[j + 1] - R->row_ptr[j]);
@@ -326,7 +549,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
   for (uint8_t w : width) max_width = std::max<int>(max_width, w);
   for (int32_t w : long_width) max_width = std::max<int>(max_width, w);
 
-  const int T = (int)((m_tiles + kWarp - 1) / kWarp);
+  const int T = (int)src.size();
   if (opts && opts->host_mb_limit > 0) {
     // host bytes of the arena image about to be built: child codes, slot
     // arrays (descriptor, variable, row, CSR position), variable CSR and ELL
@@ -336,12 +559,12 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       return fail(DG_ENOMEM, "dg_plan: the arena image needs about " + std::to_string((long long)(est / 1048576.0)) +
                                  " MiB of host memory, more than host_mb_limit");
   }
-  // tile t takes BDDs order[32 t .. 32 t + 31]; tiles are then laid out by
-  // shared-memory footprint, largest first, so that tiles of one launch group
-  // are contiguous (and the longest tiles start first)
+  // tiles are laid out by shared-memory footprint, largest first (the unit
+  // tiles, then the others), so that tiles of one launch group are contiguous
+  // and the longest tiles start first
   std::vector<int> tile_nh(T, 0), tile_nmax(T, 2), tile_maxw(T, 1), tile_order(T);
   for (int t = 0; t < T; ++t) {
-    for (int64_t q = (int64_t)t * kWarp; q < std::min<int64_t>(m_tiles, (int64_t)(t + 1) * kWarp); ++q) {
+    for (int64_t q = src[t].first; q < src[t].first + src[t].count; ++q) {
       const int64_t j = order[q];
       tile_nh[t] = std::max<int>(tile_nh[t], (int)(R->row_ptr[j + 1] - R->row_ptr[j]));
       tile_nmax[t] = std::max<int>(tile_nmax[t], 2 + (int)(P.node_ptr[j + 1] - P.node_ptr[j]));
@@ -349,20 +572,43 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     }
     tile_order[t] = t;
   }
-  auto tile_smem = [&](int t) { return sweep_smem_bytes(tile_nmax[t], tile_nh[t], 1, ring_size(tile_maxw[t])); };
-  std::stable_sort(tile_order.begin(), tile_order.end(), [&](int x, int y) { return tile_smem(x) > tile_smem(y); });
+  auto tile_smem = [&](int t) {
+    return src[t].unit >= 0 ? unit_smem_bytes(units[src[t].unit].s.W, tile_nh[t], 1)
+                            : sweep_smem_bytes(tile_nmax[t], tile_nh[t], 1, ring_size(tile_maxw[t]));
+  };
+  std::stable_sort(tile_order.begin(), tile_order.end(), [&](int x, int y) {
+    const bool ux = src[x].unit >= 0, uy = src[y].unit >= 0;
+    return ux != uy ? ux : tile_smem(x) > tile_smem(y);
+  });
+  // the shapes in use, in tile order
+  std::vector<int> shape_slot(units.size(), -1);
+  P.unit_shapes.clear();
+  P.unit_runs.clear();
+  for (int t : tile_order) {
+    const int u = src[t].unit;
+    if (u < 0 || shape_slot[u] >= 0) continue;
+    shape_slot[u] = (int)P.unit_shapes.size();
+    UnitShape s = units[u].s;
+    s.run_base = (int32_t)P.unit_runs.size();
+    for (int h = 0; h < s.k; ++h)
+      if (h + 1 == s.k || units[u].type[h + 1] != units[u].type[h])
+        P.unit_runs.push_back((uint16_t)((h + 1) << 2 | units[u].type[h]));
+    s.nruns = (int32_t)P.unit_runs.size() - s.run_base;
+    P.unit_shapes.push_back(s);
+  }
   P.tiles.resize(T);
   P.slot_to_csr.clear();
   std::vector<int64_t> slot_of_csr(nnz, -1);
   int64_t node_base = 0, slot_base = 0;
   size_t smem_max = 0, smem_adj_max = 0;
   for (int t = 0; t < T; ++t) {
-    const int src = tile_order[t];
-    const int64_t q0 = (int64_t)src * kWarp, q1 = std::min<int64_t>(m_tiles, q0 + kWarp);
-    const int nb = (int)(q1 - q0);
-    const int nh = tile_nh[src], nmax = tile_nmax[src];
+    const int ts = tile_order[t];
+    const int64_t q0 = src[ts].first;
+    const int nb = src[ts].count;
+    const int nh = tile_nh[ts], nmax = tile_nmax[ts];
     const int64_t tslots = (int64_t)nh * kWarp;
     Tile& tile = P.tiles[t];
+    tile.unit = src[ts].unit >= 0 ? 1 + shape_slot[src[ts].unit] : 0;
     tile.node_base = (int32_t)node_base;
     tile.slot_base = (int32_t)slot_base;
     tile.nmax = nmax;
@@ -410,37 +656,63 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     P.max_tile_hops = std::max(P.max_tile_hops, nh);
     node_base += (int64_t)(nmax - 2) * kWarp;
     slot_base += tslots;
+    if (tile.unit) P.unit_slots = (int32_t)slot_base;
   }
   // launch groups: consecutive tiles whose footprints stay within 1/kGroupRatio
   // of the group's largest one
   {
     const double kGroupRatio =
         opts && opts->group_ratio_pct > 0 && opts->group_ratio_pct <= 100 ? opts->group_ratio_pct / 100.0 : 0.85;
+    // ... or any smaller one while the group's tiles do not fill the chip (its
+    // smaller tiles then cost it no occupancy and save a launch)
+    constexpr size_t kSms = 152, kSmSmem = 224 * 1024;
     int32_t t0 = 0;
-    size_t gmax = 0, gmax0 = 0;
-    for (int t = 0; t < T; ++t) {
-      const size_t r = sweep_smem_bytes(P.tiles[t].nmax, P.tiles[t].nhops, 1, P.tiles[t].ring);
-      if (t > t0 && (double)r < kGroupRatio * (double)gmax) {
-        P.groups.push_back({t0, t, (int32_t)gmax, (int32_t)gmax0, 0, 0, 0, 0, 0, 0, {0, 0}});
+    size_t gmax = 0;
+    auto group_smem = [&](int t) {
+      const Tile& tl = P.tiles[t];
+      return tl.unit ? unit_smem_bytes(P.unit_shapes[tl.unit - 1].W, tl.nhops, 1)
+                     : sweep_smem_bytes(tl.nmax, tl.nhops, 1, tl.ring);
+    };
+    for (int t = 0; t <= T; ++t) {
+      const size_t r = t < T ? group_smem(t) : 0;
+      const bool kind = t < T && t > t0 && (P.tiles[t].unit != 0) != (P.tiles[t0].unit != 0);
+      const bool full = gmax > 0 && (size_t)(t - t0) >= kSms * std::min<size_t>(64, kSmSmem / gmax);
+      if (t == T || kind || (t > t0 && full && (double)r < kGroupRatio * (double)gmax)) {
+        if (t > t0) {
+          LaunchGroup g{};
+          g.tile0 = t0;
+          g.tile1 = t;
+          P.groups.push_back(g);
+        }
         t0 = t;
         gmax = 0;
-        gmax0 = 0;
       }
       gmax = std::max(gmax, r);
-      gmax0 = std::max(gmax0, sweep_smem_bytes(P.tiles[t].nmax, P.tiles[t].nhops, 0, P.tiles[t].ring));
     }
-    if (T > 0) P.groups.push_back({t0, T, (int32_t)gmax, (int32_t)gmax0, 0, 0, 0, 0, 0, 0, {0, 0}});
     for (LaunchGroup& g : P.groups)
       for (int t = g.tile0; t < g.tile1; ++t) {
+        const Tile& tl = P.tiles[t];
+        g.region_bytes = std::max<int32_t>(g.region_bytes, (int32_t)sweep_smem_bytes(tl.nmax, tl.nhops, 1, tl.ring));
+        g.region_bytes0 = std::max<int32_t>(g.region_bytes0, (int32_t)sweep_smem_bytes(tl.nmax, tl.nhops, 0, tl.ring));
+        if (tl.unit) {
+          const UnitShape& s = P.unit_shapes[tl.unit - 1];
+          g.unit_w = std::max(g.unit_w, s.W);
+          g.unit_bytes0 = std::max<int32_t>(g.unit_bytes0, (int32_t)unit_smem_bytes(s.W, s.k, 0));
+          g.unit_bytes1 = std::max<int32_t>(g.unit_bytes1, (int32_t)unit_smem_bytes(s.W, s.k, 1));
+        }
         g.region_bwd1 = std::max<int32_t>(g.region_bwd1, (int32_t)sweep_smem_bytes_bwd(P.tiles[t].nmax, P.tiles[t].nhops, 1));
         g.region_bwd0 = std::max<int32_t>(g.region_bwd0, (int32_t)sweep_smem_bytes_bwd(P.tiles[t].nmax, P.tiles[t].nhops, 0));
         g.meta_bytes = std::max<int32_t>(g.meta_bytes, (P.tiles[t].nmax - 2) * kWarp * 2);
-        smem_max = std::max<size_t>(smem_max, (size_t)g.region_bwd1);
+        smem_max = std::max<size_t>(smem_max, (size_t)std::max(g.region_bwd1, g.unit_bytes1));
       }
     // work estimate per group, then longest-processing-time assignment of the
     // groups to the kStreams streams that run one sweep's launches concurrently
     for (LaunchGroup& g : P.groups)
-      for (int t = g.tile0; t < g.tile1; ++t) g.work += (int64_t)kWarp * P.tiles[t].nmax * P.tiles[t].nhops;
+      for (int t = g.tile0; t < g.tile1; ++t) {
+        const Tile& tl = P.tiles[t];
+        g.work += tl.unit ? (int64_t)tl.nhops * (14 * P.unit_shapes[tl.unit - 1].W + 40)
+                          : (int64_t)kWarp * tl.nmax * tl.nhops;
+      }
     // the long BDDs are one more launch (index -1 here): a warp walks each
     // level in turn, estimated like a tile level of 16 nodes per level
     int64_t long_work = 0;
@@ -616,6 +888,8 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     return at;
   };
   P.off.tiles = put(P.tiles.size() * sizeof(Tile));
+  P.off.unit_shapes = put(P.unit_shapes.size() * sizeof(UnitShape));
+  P.off.unit_runs = put(P.unit_runs.size() * 2);
   P.off.desc = put(P.desc.size() * 2);
   P.off.lohi8 = put(P.lohi8.size() * 2);
   P.off.slot_var = put(num_slots * 4);
@@ -679,6 +953,20 @@ dg_status validate_plan(const Plan& P) {
   if ((int64_t)P.desc.size() != NS || (int64_t)P.slot_var.size() != NS || (int64_t)P.slot_row.size() != NS ||
       (int64_t)P.slot_to_csr.size() != NS || (int64_t)P.lohi8.size() != P.sizes.num_nodes_padded)
     return bad("array sizes disagree with the plan sizes");
+  // unit shapes: window, states and runs in range
+  for (const UnitShape& s : P.unit_shapes) {
+    if (s.W < 2 || s.W > kUnitMaxW || s.W % 2 != 0 || s.k < 1 || s.start < 0 || s.start >= s.W || s.accept <= 0 ||
+        s.accept >= (1 << s.W) || s.nruns < 1 || s.run_base < 0 ||
+        (size_t)s.run_base + (size_t)s.nruns > P.unit_runs.size())
+      return bad("unit shape out of range");
+    int prev = 0;
+    for (int r = 0; r < s.nruns; ++r) {
+      const int e = P.unit_runs[s.run_base + r] >> 2;
+      if (e <= prev || e > s.k) return bad("unit shape runs not ascending");
+      prev = e;
+    }
+    if (prev != s.k) return bad("unit shape runs do not cover its levels");
+  }
   // tiles: contiguous bases, sane shapes, every lane's BDD well formed
   int64_t node_base = 0, slot_base = 0, real_nodes = 0, real_slots = 0;
   std::vector<int64_t> csr_seen(NL, 0);
@@ -689,6 +977,10 @@ dg_status validate_plan(const Plan& P) {
     if (tl.nbdd < 1 || tl.nbdd > kWarp || tl.nhops < 1 || tl.nmax < 3 || tl.nmax > kMaxNodesPerBdd + 2 ||
         tl.maxw < 1 || tl.maxw > kMaxWidth || tl.ring != ring_size(tl.maxw))
       return bad(at + "shape out of range");
+    if (tl.unit < 0 || tl.unit > (int32_t)P.unit_shapes.size() ||
+        (tl.unit && (P.unit_shapes[tl.unit - 1].k != tl.nhops || slot_base >= P.unit_slots)) ||
+        (!tl.unit && slot_base < P.unit_slots))
+      return bad(at + "unit shape does not fit the tile");
     for (int b = 0; b < kWarp; ++b) {
       int first = 2, level_w = 0, last_h = -1, row = -1;
       for (int h = 0; h < tl.nhops; ++h) {
@@ -719,6 +1011,10 @@ dg_status validate_plan(const Plan& P) {
       }
       if (b >= tl.nbdd) continue;
       if (last_h < 0) last_h = tl.nhops - 1;
+      if (tl.unit && last_h != tl.nhops - 1) return bad(at + "unit tile lane with fewer levels");
+      // a unit tile's lanes are sweeped by its shape alone: nodes as states
+      std::vector<int> state(1, tl.unit ? P.unit_shapes[tl.unit - 1].start : 0), next;
+      const uint16_t* run = tl.unit ? &P.unit_runs[P.unit_shapes[tl.unit - 1].run_base] : nullptr;
       // children: next level's nodes (no level skipped) or the bottom; the
       // last level only the terminals; at least one child not the bottom
       int f = 2;
@@ -736,6 +1032,30 @@ dg_status validate_plan(const Plan& P) {
             if (h == last_h ? !term : (c == (uint32_t)kTopCode || (!term && (c < (uint32_t)fn || c >= (uint32_t)(fn + wn)))))
               return bad(at + "child code outside the next level");
           }
+        }
+        if (tl.unit) {
+          const UnitShape& s = P.unit_shapes[tl.unit - 1];
+          if (h >= (*run >> 2)) ++run;
+          next.assign(wn, -1);
+          for (int r = 0; r < w; ++r) {
+            const uint32_t code = P.lohi8[node_base + (int64_t)(f + r - 2) * kWarp + b];
+            const int u = state[r];
+            if (u < 0 || (r > 0 && u >= state[r - 1])) return bad(at + "unit states not descending");
+            for (int beta = 0; beta < 2; ++beta) {
+              const uint32_t c = beta ? code >> 8 : code & 0xFFu;
+              if (c == (uint32_t)kBotCode) continue;
+              const int to = beta ? unit_o(*run & 3, u) : unit_z(*run & 3, u);
+              if (to < 0 || to >= s.W) return bad(at + "unit state outside the window");
+              if (c == (uint32_t)kTopCode) {
+                if (!((s.accept >> to) & 1)) return bad(at + "unit state not accepted");
+              } else if (next[c - fn] >= 0 && next[c - fn] != to) {
+                return bad(at + "unit states of a node differ");
+              } else {
+                next[c - fn] = to;
+              }
+            }
+          }
+          state.swap(next);
         }
         f = fn;
       }

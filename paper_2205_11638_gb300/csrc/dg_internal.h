@@ -45,9 +45,45 @@ struct Tile {
   int32_t nbdd;       // BDDs (lanes in use)
   int32_t maxw;       // widest level
   int32_t ring;       // ring size (power of two >= 2 * maxw) of the sweep-direction costs
-  int32_t pad1;
+  int32_t unit;       // 1 + index of the UnitShape all BDDs of the tile share, 0 for a mixed tile
 };
 static_assert(sizeof(Tile) == 32, "Tile is 32 bytes");
+
+// Unit rows: all coefficients +1 or -1.  Their BDDs are windows of partial
+// sums: a level holds states u = 0 .. W-1 ("sum minus the level's base") and
+// its two arcs shift u by at most one, so a lane keeps a whole level's path
+// costs in W registers and needs no child codes.  Level h maps state u to
+// the states of level h + 1 by its type:
+//            0-arc          1-arc
+//   kUp      u              u + 1            (coefficient +1)
+//   kDown    u              max(u - 1, 0)    (-1, the base absorbs: every completion is feasible)
+//   kSwap    max(u - 1, 0)  u                (+1 while the base follows the sum that is feasible anyway)
+//   kDrop    u              u - 1            (-1, below the window nothing is feasible)
+// A state outside the window is the bottom terminal.  After the last level
+// the states in `accept` are the top terminal, the others the bottom one.
+// Rows are normalised to '<=' or '=' (signs flipped where that makes it so),
+// and a row is a unit row only if its canonical BDD has exactly these states
+// with node ranks descending in u, so that the tie rules (smallest rank)
+// read "largest u first".
+enum UnitType : int { kUp = 0, kDown = 1, kSwap = 2, kDrop = 3 };
+constexpr int kUnitMaxW = 8;
+struct UnitShape {
+  int32_t W;         // states per level: 2, 4, 6 or 8 (the window rounded up)
+  int32_t k;         // levels
+  int32_t start;     // state of the root
+  int32_t accept;    // bit u: state u after the last level is the top terminal
+  int32_t run_base;  // first entry of unit_runs
+  int32_t nruns;     // runs of levels of one type: end level << 2 | type
+  int32_t pad[2];
+};
+static_assert(sizeof(UnitShape) == 32, "UnitShape is 32 bytes");
+
+// Shared memory of one unit tile (one warp's slice) in the sweeps: the path
+// costs of levels 1 .. k-1 and per level lambda, the averaging term and (mode
+// 1) omega and alpha.
+inline size_t unit_smem_bytes(int W, int k, int mode) {
+  return (size_t)kWarp * 4 * ((size_t)(k - 1) * W + (size_t)k * (mode ? 4 : 2));
+}
 
 inline int ring_size(int maxw) {
   int r = 2;
@@ -77,6 +113,8 @@ static_assert(sizeof(LongBdd) == 32, "LongBdd is 32 bytes");
 // Device view of an arena (all pointers inside the caller's buffer).
 struct DevArena {
   const Tile* tiles;
+  const UnitShape* unit_shapes;
+  const uint16_t* unit_runs;
   const uint16_t* desc;     // per slot: first node number | width << 8
   const uint16_t* lohi8;    // per node and lane: lo code | hi code << 8
   const int32_t* slot_var;  // variable of a slot, -1 for padding
@@ -121,6 +159,7 @@ struct DevArena {
   int64_t m;
   int64_t num_slots;
   int32_t num_tiles;
+  int32_t unit_slots;       // the unit tiles come first: their slots are [0, unit_slots)
   int32_t num_lb_chunks;
   int32_t num_long;
   int32_t long_slot_base;   // first slot of the long BDDs (after every tile's slots)
@@ -145,6 +184,9 @@ struct LaunchGroup {
   int8_t wpc_bwd;
   int8_t pad[2];
   int32_t meta_bytes;     // argmin records of the recording sweeps: 64 (nmax - 2), largest tile
+  int32_t unit_w;         // unit tiles: the largest W of the group (0: a group of mixed tiles)
+  int32_t unit_bytes0;    // unit tiles: shared memory per warp, mode 0
+  int32_t unit_bytes1;    // ... mode 1
 };
 
 // Tiles of one adjoint launch (the sweep's launch groups with the adjoint's
@@ -161,6 +203,9 @@ struct Plan {
   int64_t hop_histogram[64]{};
   // host images of the device arrays
   std::vector<Tile> tiles;
+  std::vector<UnitShape> unit_shapes;
+  std::vector<uint16_t> unit_runs;
+  int32_t unit_slots = 0;
   std::vector<LaunchGroup> groups;
   std::vector<AdjGroup> adj_groups;
   std::vector<uint16_t> desc;
@@ -194,7 +239,7 @@ struct Plan {
   int32_t long_slot_base = 0, long_cost_size = 0, long_stream = 0;
   // byte offsets of every array inside the arena
   struct Off {
-    size_t tiles, desc, lohi8, slot_var, slot_row, var_ptr, var_slots, var_ell, wide_vars, c, invdeg, inst_row_ptr,
+    size_t tiles, unit_shapes, unit_runs, desc, lohi8, slot_var, slot_row, var_ptr, var_slots, var_ell, wide_vars, c, invdeg, inst_row_ptr,
         inst_var_ptr,
         lb_chunks, inst_chunk_ptr, inst_unc, longs, long_code, long_lvl, long_in_ptr, long_in, long_order, S, Sbar, slot_avg, E, lb_part,
         long_d, long_t, nodecost, slot_invdeg, total;

@@ -65,6 +65,11 @@ struct StreamSet {
 };
 
 cudaError_t set_sweep_smem_limit(size_t bytes);
+cudaError_t set_unit_smem_limit(size_t bytes);
+// The launch of one group of unit tiles (kernels_unit.cu), wpc warps of
+// `region` bytes to a CTA.
+void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
+                 cudaStream_t st);
 // Dynamic shared memory one CTA may use; launchers put fewer warps in a CTA
 // when their tiles need more.
 void set_cta_smem_cap(size_t bytes);
@@ -74,10 +79,13 @@ void launch_sweep(int kind, const DevArena& A, const SweepArgs& a, int threads, 
 
 // S_i = sum_{k in J_i} M_ik in fixed slot order; with renorm, also
 // lambda_ij += alpha_ij * (c_i - sum_k (lambda_ik + M_ik)) computed in FP64.
-// With for_sweep, also the mode's averaging term of every slot into
-// A.slot_avg, where the next sweeps read it.
+// Before a sweep also the mode's averaging term into A.slot_avg for the slots
+// the sweep reads it from: those of the mixed tiles and the long BDDs before
+// a plain sweep (the unit tiles gather S or Sbar), every slot before a
+// recording one.
+enum class Scatter { kNone, kPlain, kAll };
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
-                     cudaStream_t st, bool for_sweep);
+                     cudaStream_t st, Scatter to);
 void launch_init(const DevArena& A, float* lam, float* M, cudaStream_t st);
 // per-instance FP64 lower bound from A.E and A.S
 void launch_lower_bound(const DevArena& A, double* lb_out, cudaStream_t st);

@@ -14,10 +14,11 @@ namespace dg {
 // With SCATTER every slot of the variable also receives the averaging term
 // the sweeps add (Sbar_i = S_i / |J_i| in mode 0, S_i in mode 1, which they
 // multiply by alpha_ij), so that a sweep reads it with the slot's other
-// inputs instead of gathering it per variable.
+// inputs instead of gathering it per variable.  Slots below scatter_from are
+// left out: the unit tiles' sweeps gather S or Sbar themselves.
 template <bool RENORM, bool SCATTER>
 __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* __restrict__ M, float* lam,
-                                                   const float* __restrict__ alpha, int mode) {
+                                                   const float* __restrict__ alpha, int mode, int scatter_from) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   float s = 0.f;
@@ -50,8 +51,11 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* __res
       const float t = mode == 1 ? s : sbar;
 #pragma unroll
       for (int r = 0; r < kEll; ++r)
-        if (q[r] >= 0) A.slot_avg[q[r]] = t;
-      for (int k = b; k < e; ++k) A.slot_avg[__ldg(A.var_slots + k)] = t;
+        if (q[r] >= scatter_from) A.slot_avg[q[r]] = t;
+      for (int k = b; k < e; ++k) {
+        const int qk = __ldg(A.var_slots + k);
+        if (qk >= scatter_from) A.slot_avg[qk] = t;
+      }
     }
     return;
   }
@@ -74,7 +78,7 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* __res
       const int q = __ldg(A.var_slots + k);
       const double w = mode == 1 ? (double)alpha[q] : (double)inv;
       lam[q] = (float)((double)lam[q] + w * r);
-      if (SCATTER) A.slot_avg[q] = t;
+      if (SCATTER && q >= scatter_from) A.slot_avg[q] = t;
     }
   }
 }
@@ -84,7 +88,8 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* __res
 // every lane adds them in slot order (the plain loop's order, so S is the
 // same to the bit); lane 0 stores S.
 template <bool SCATTER>
-__global__ void __launch_bounds__(256) k_reduce_wide(DevArena A, const float* __restrict__ M, int mode) {
+__global__ void __launch_bounds__(256) k_reduce_wide(DevArena A, const float* __restrict__ M, int mode,
+                                                     int scatter_from) {
   constexpr unsigned kAll = 0xffffffffu;
   const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (w >= A.num_wide) return;  // the whole warp
@@ -103,7 +108,10 @@ __global__ void __launch_bounds__(256) k_reduce_wide(DevArena A, const float* __
   }
   if (SCATTER) {
     const float t = mode == 1 ? s : sbar;
-    for (int k = b + lane; k < e; k += 32) A.slot_avg[__ldg(A.var_slots + k)] = t;
+    for (int k = b + lane; k < e; k += 32) {
+      const int qk = __ldg(A.var_slots + k);
+      if (qk >= scatter_from) A.slot_avg[qk] = t;
+    }
   }
 }
 
@@ -284,19 +292,21 @@ void launch_gather_var(const DevArena& A, const float* v, float* out_slot, cudaS
 }
 
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
-                     cudaStream_t st, bool for_sweep) {
+                     cudaStream_t st, Scatter to) {
   const int T = 256;
   const int G = (A.n + T - 1) / T;
   if (G == 0) return;
+  const int from = to == Scatter::kAll ? 0 : A.unit_slots;
+  const bool scatter = to != Scatter::kNone && from < A.num_slots;
   if (renorm)
-    for_sweep ? k_reduce_S<true, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode)
-              : k_reduce_S<true, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode);
+    scatter ? k_reduce_S<true, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from)
+            : k_reduce_S<true, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from);
   else {
-    for_sweep ? k_reduce_S<false, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode)
-              : k_reduce_S<false, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode);
+    scatter ? k_reduce_S<false, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from)
+            : k_reduce_S<false, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from);
     if (A.num_wide > 0)
-      for_sweep ? k_reduce_wide<true><<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, M, mode)
-                : k_reduce_wide<false><<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, M, mode);
+      scatter ? k_reduce_wide<true><<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, M, mode, from)
+              : k_reduce_wide<false><<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, M, mode, from);
   }
 }
 

@@ -423,9 +423,11 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
     const LaunchGroup& G = groups[g];
     constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
     constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
-    const size_t region = (size_t)(BWD ? (MODE == 1 ? G.region_bwd1 : G.region_bwd0)
-                                       : (MODE == 1 ? G.region_bytes : G.region_bytes0)) +
-                          (REC ? (size_t)G.meta_bytes : 0);
+    const bool unit = G.unit_w > 0 && !REC;
+    const size_t region = unit ? (size_t)(MODE == 1 ? G.unit_bytes1 : G.unit_bytes0)
+                               : (size_t)(BWD ? (MODE == 1 ? G.region_bwd1 : G.region_bwd0)
+                                              : (MODE == 1 ? G.region_bytes : G.region_bytes0)) +
+                                     (REC ? (size_t)G.meta_bytes : 0);
     int wpc = threads / kWarp;
     if (wpc > 4) wpc = 4;  // __launch_bounds__(128)
     const int tuned = REC ? 0 : (BWD ? G.wpc_bwd : G.wpc_fwd);
@@ -433,6 +435,10 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
       wpc = tuned;
     else
       wpc = best_warps_per_cta(region, wpc, g_cta_smem_cap);
+    if (unit) {
+      launch_unit(KIND, A, a, G, wpc, region, fork ? ss.of(G.stream) : ss.main);
+      continue;
+    }
     const int nt = G.tile1 - G.tile0;
     dim3 grid((nt + wpc - 1) / wpc), block(wpc * kWarp);
     k_sweep<KIND, MODE><<<grid, block, region * wpc, fork ? ss.of(G.stream) : ss.main>>>(A, a, (int)region, G.tile0,

@@ -92,7 +92,7 @@ dg_status lower_bound_noalloc(const DevArena& arena, const LaunchGroup* groups, 
   a.lam = const_cast<float*>(lam);
   a.E = A.E;
   launch_sweep(kEnergy, A, a, threads, groups, num_groups, ss);
-  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, false);
+  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, Scatter::kNone);
   launch_lower_bound(A, lb, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DG_ECUDA, std::string("dg_lower_bound_noalloc: ") + cudaGetErrorString(e));

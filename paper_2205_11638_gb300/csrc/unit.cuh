@@ -1,0 +1,208 @@
+// unit.cuh -- device building blocks of the unit tiles (UnitShape): one warp
+// owns a tile of up to 32 BDDs of one shape, lane b owns BDD b, and a level's
+// path costs are W registers of the lane.
+//
+// A unit row's BDD is a window of partial sums whose two arcs shift a state
+// by at most one, so App. B's recursions need no child codes, no gathers and
+// no per-node address arithmetic: SP(r, .) and SP(., T) of a level are W adds
+// and W mins over registers, the state shifts are register names (the level
+// type is the same for the whole warp), and only the costs of the direction
+// opposite to the sweep go through shared memory (written by a first pass,
+// one lane's own words, so without barriers).  Every cost is the value of the
+// node-by-node kernels bit for bit: the same FP32 additions along the same
+// arcs, and minima are exact in any order.
+#pragma once
+
+#include "sweep.cuh"
+
+namespace dg {
+
+// State reached from state u by the 0-arc / 1-arc of a level of type TYPE; -1
+// and W are outside the window.
+template <int TYPE>
+__device__ __forceinline__ constexpr int unit_z(int u) {
+  return TYPE == kSwap ? (u > 0 ? u - 1 : 0) : u;
+}
+template <int TYPE>
+__device__ __forceinline__ constexpr int unit_o(int u) {
+  return TYPE == kUp ? u + 1 : (TYPE == kSwap ? u : (TYPE == kDown ? (u > 0 ? u - 1 : 0) : u - 1));
+}
+
+template <int W>
+struct Costs {
+  float v[W];
+  __device__ __forceinline__ float at(int u) const { return u >= 0 && u < W ? v[u] : f_inf(); }  // u is a constant
+};
+
+// Costs of a level from the costs T of the level below: SP(., T) of state u.
+template <int W, int TYPE>
+__device__ __forceinline__ Costs<W> unit_up(const Costs<W>& T, float l) {
+  Costs<W> r;
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
+    const int o = unit_o<TYPE>(u);
+    r.v[u] = T.at(unit_z<TYPE>(u));
+    if (o >= 0 && o < W) r.v[u] = fminf(r.v[u], l + T.at(o));
+  }
+  return r;
+}
+
+// SP(r, .) of the next level from the costs R of a level.
+template <int W, int TYPE>
+__device__ __forceinline__ Costs<W> unit_down(const Costs<W>& R, float l) {
+  Costs<W> r;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    float b = f_inf();
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      if (unit_z<TYPE>(u) == w) b = fminf(b, R.v[u]);
+      if (unit_o<TYPE>(u) == w) b = fminf(b, R.v[u] + l);
+    }
+    r.v[w] = b;
+  }
+  return r;
+}
+
+// Minima over the level's states of SP(r, u) + SP(child, T) by the 0- and the
+// 1-arc.
+template <int W, int TYPE>
+__device__ __forceinline__ void unit_minima(const Costs<W>& R, const Costs<W>& T, float& b0, float& b1) {
+  b0 = b1 = f_inf();
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
+    b0 = fminf(b0, R.v[u] + T.at(unit_z<TYPE>(u)));
+    if (unit_o<TYPE>(u) >= 0 && unit_o<TYPE>(u) < W) b1 = fminf(b1, R.v[u] + T.at(unit_o<TYPE>(u)));
+  }
+}
+
+// The costs of a level in the warp's shared memory: 32 W floats per level,
+// in pieces of four (or two) states per lane, so that a lane moves them with
+// 16- (8-) byte accesses free of bank conflicts.
+template <int W>
+__device__ __forceinline__ void unit_store(float* row, const Costs<W>& c, int lane) {
+  if constexpr (W % 4 == 0) {
+#pragma unroll
+    for (int j = 0; j < W / 4; ++j)
+      reinterpret_cast<float4*>(row)[j * kWarp + lane] = make_float4(c.v[4 * j], c.v[4 * j + 1], c.v[4 * j + 2], c.v[4 * j + 3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < W / 2; ++j)
+      reinterpret_cast<float2*>(row)[j * kWarp + lane] = make_float2(c.v[2 * j], c.v[2 * j + 1]);
+  }
+}
+template <int W>
+__device__ __forceinline__ Costs<W> unit_load(const float* row, int lane) {
+  Costs<W> c;
+  if constexpr (W % 4 == 0) {
+#pragma unroll
+    for (int j = 0; j < W / 4; ++j) {
+      const float4 x = reinterpret_cast<const float4*>(row)[j * kWarp + lane];
+      c.v[4 * j] = x.x;
+      c.v[4 * j + 1] = x.y;
+      c.v[4 * j + 2] = x.z;
+      c.v[4 * j + 3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < W / 2; ++j) {
+      const float2 x = reinterpret_cast<const float2*>(row)[j * kWarp + lane];
+      c.v[2 * j] = x.x;
+      c.v[2 * j + 1] = x.y;
+    }
+  }
+  return c;
+}
+
+// SP(., T) below the last level, SP(r, .) of the first.
+template <int W>
+__device__ __forceinline__ Costs<W> unit_end(int accept) {
+  Costs<W> c;
+#pragma unroll
+  for (int u = 0; u < W; ++u) c.v[u] = (accept >> u) & 1 ? 0.0f : f_inf();
+  return c;
+}
+template <int W>
+__device__ __forceinline__ Costs<W> unit_root(int start) {
+  Costs<W> c;
+#pragma unroll
+  for (int u = 0; u < W; ++u) c.v[u] = u == start ? 0.0f : f_inf();
+  return c;
+}
+
+// One shape, as a warp holds it.
+struct UnitCtx {
+  int k, start, accept, nruns;
+  const uint16_t* runs;
+};
+
+// Calls f(type constant, level) for the levels first .. k-1 in ascending
+// order, run by run, so that the type is decided once per run.
+template <int T>
+struct TypeC {
+  static constexpr int value = T;
+};
+template <class F>
+__device__ __forceinline__ void unit_levels_down(const UnitCtx& s, int first, int last, F&& f) {
+  int h = first;
+  for (int r = 0; r < s.nruns; ++r) {
+    const unsigned run = __ldg(s.runs + r);
+    const int e = min((int)(run >> 2), last);
+    switch (run & 3u) {
+      case kUp:
+        for (; h < e; ++h) f(TypeC<kUp>{}, h);
+        break;
+      case kDown:
+        for (; h < e; ++h) f(TypeC<kDown>{}, h);
+        break;
+      case kSwap:
+        for (; h < e; ++h) f(TypeC<kSwap>{}, h);
+        break;
+      default:
+        for (; h < e; ++h) f(TypeC<kDrop>{}, h);
+        break;
+    }
+  }
+}
+// ... and for the levels k-1 .. first in descending order.
+template <class F>
+__device__ __forceinline__ void unit_levels_up(const UnitCtx& s, int first, F&& f) {
+  int h = s.k - 1;
+  for (int r = s.nruns - 1; r >= 0; --r) {
+    const unsigned run = __ldg(s.runs + r);
+    const int b = max(r > 0 ? (int)(__ldg(s.runs + r - 1) >> 2) : 0, first);
+    switch (run & 3u) {
+      case kUp:
+        for (; h >= b; --h) f(TypeC<kUp>{}, h);
+        break;
+      case kDown:
+        for (; h >= b; --h) f(TypeC<kDown>{}, h);
+        break;
+      case kSwap:
+        for (; h >= b; --h) f(TypeC<kSwap>{}, h);
+        break;
+      default:
+        for (; h >= b; --h) f(TypeC<kDrop>{}, h);
+        break;
+    }
+  }
+}
+
+// lambda^new of the update, every rounding spelled out as the mixed tiles'
+// kernel has it: M^new = omega (m1 - m0) rounded on its own, the mode-1 term
+// alpha S by one fused multiply-add.
+template <int MODE>
+__device__ __forceinline__ float unit_lambda_new(float l, float Mn, float al, float av) {
+  const float r = l - Mn;
+  return MODE == 1 ? __fmaf_rn(al, av, r) : r + av;
+}
+
+// Asynchronous 4-byte global -> shared copy (a gather: every lane its own
+// address), through L1.
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
+
+}  // namespace dg

@@ -1,0 +1,113 @@
+"""Unit tiles (rows with coefficients +1 and -1, all BDDs of a tile of one
+shape) against the mixed tiles' kernels.  Doubling a row's coefficients and
+right-hand side leaves its canonical BDD unchanged but makes it no unit row,
+so the doubled problem runs the general kernels on the same BDDs.  Both do
+the same FP32 additions along the same arcs and take exact minima, hence the
+results have to be equal bit for bit (no tolerance)."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from paper_2205_11638_gb300 import build, solver
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build.build()
+
+
+def _doubled(p):
+    return dict(p, coef=(2 * p["coef"]).astype(np.int32), rhs=(2 * p["rhs"]).astype(np.int32))
+
+
+def _random_unit_rows(seed, n=300, patterns=60):
+    """Random sign patterns of 1..14 terms, every sense and right-hand side,
+    each as 1, 31, 32, 33 or 70 rows over random variables."""
+    rng = np.random.default_rng(seed)
+    rows = []
+    while len(rows) < patterns * 60:
+        k = int(rng.integers(1, 15))
+        a = rng.choice([-1, 1], size=k) if rng.random() < 0.6 else np.full(k, rng.choice([-1, 1]))
+        sense = int(rng.integers(0, 3))
+        b = int(rng.integers(np.minimum(a, 0).sum(), np.maximum(a, 0).sum() + 1))
+        if not workloads._free_row((None, a, sense, b)):
+            continue
+        for _ in range(int(rng.choice([1, 31, 32, 33, 70]))):
+            rows.append((np.sort(rng.choice(n, size=k, replace=False)), a, sense, b))
+    rng.shuffle(rows)
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+CASES = {
+    "random_signs": lambda: _random_unit_rows(5),
+    "tracking": lambda: workloads.tracking(frames=8, dets=150, seed=41),
+    "matching": lambda: workloads.matching_quadratic(L=40, R=40, pairs=1500, seed=42),
+    "set_cover": lambda: workloads.set_cover(n=400, m=300, kmin=2, kmax=12, seed=43),
+    "one_row": lambda: workloads.single_rows_problem([(np.arange(3), np.ones(3, np.int64), 0, 1)], 3,
+                                                     np.array([-1.0, 0.5, -2.0])),
+}
+
+
+def _pair(name):
+    p = CASES[name]()
+    return p, solver.plan(p).bind(), solver.plan(_doubled(p)).bind()
+
+
+def _vectors(p, seed):
+    rng = np.random.default_rng(seed)
+    nnz = len(p["col"])
+    e = np.exp(rng.normal(size=nnz))
+    s = np.zeros(p["n"])
+    np.add.at(s, p["col"], e)
+    return [torch.as_tensor(x, dtype=torch.float32) for x in
+            (rng.normal(size=nnz), 0.1 * rng.normal(size=nnz), rng.uniform(0.1, 0.9, size=nnz), e / s[p["col"]])]
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("mode", [0, 1])
+def test_sweeps_equal_the_mixed_tiles(name, mode):
+    p, A, B = _pair(name)
+    v = _vectors(p, 7)
+    out = []
+    for X in (A, B):
+        lam, M, om, al = [X.from_csr(x) for x in v]
+        lb = X.iterate(lam, M, om if mode else None, al if mode else None, iters=5, lb=True)
+        assert torch.equal(X.from_csr(X.to_csr(lam)), lam)  # padding stays 0
+        out.append((X.to_csr(lam), X.to_csr(M), lb))
+    for a, b in zip(*out):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_scalar_damping_equals_the_mixed_tiles(name):
+    p = CASES[name]()
+    v = _vectors(p, 8)
+    out = []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q, omega=0.3).bind()
+        lam, M = X.from_csr(v[0]), X.from_csr(v[1])
+        X.iterate(lam, M, iters=3)
+        out.append((X.to_csr(lam), X.to_csr(M)))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_marginals_energies_and_minimisers_equal_the_mixed_tiles(name):
+    p, A, B = _pair(name)
+    v = _vectors(p, 9)
+    # many equal costs: ties between paths follow the same rule
+    tied = torch.round(v[0])
+    for x in (v[0], tied):
+        out = []
+        for X in (A, B):
+            lam, M = X.from_csr(x), X.from_csr(v[1])
+            m0, m1 = X.min_marginals(lam)
+            lb, E = X.lower_bound(lam, M, energies=True)
+            gl, gM = X.lb_seed(lam, M)
+            out.append([X.to_csr(m0), X.to_csr(m1), lb, E, X.to_csr(gl), X.to_csr(gM)])
+        for a, b in zip(*out):
+            assert torch.equal(a, b) and torch.isfinite(a).all()
