@@ -208,6 +208,12 @@ bool unit_candidate(const int8_t* a, int k, bool eq, int64_t rhs, const std::vec
     if (shift < 0 || shift > (a[h] > 0 ? 1 : 0)) return false;
     out.type[h] = (uint8_t)(a[h] > 0 ? (shift == 0 ? kUp : kSwap) : (eq ? kDrop : kDown));
   }
+  s.rows = -1;
+  for (int h = 0, b = 0; h < k; ++h)
+    if (h + 1 == k || out.type[h + 1] != out.type[h]) {
+      s.rows += (h + 1 - b + 1) / 2;
+      b = h + 1;
+    }
   // the shape's own feasibility, then every node and arc of the BDD
   std::vector<uint32_t> alive(k + 1);
   alive[k] = (uint32_t)s.accept;
@@ -573,7 +579,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     tile_order[t] = t;
   }
   auto tile_smem = [&](int t) {
-    return src[t].unit >= 0 ? unit_smem_bytes(units[src[t].unit].s.W, tile_nh[t], 1)
+    return src[t].unit >= 0 ? unit_smem_bytes(units[src[t].unit].s, 1)
                             : sweep_smem_bytes(tile_nmax[t], tile_nh[t], 1, ring_size(tile_maxw[t]));
   };
   std::stable_sort(tile_order.begin(), tile_order.end(), [&](int x, int y) {
@@ -670,7 +676,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     size_t gmax = 0;
     auto group_smem = [&](int t) {
       const Tile& tl = P.tiles[t];
-      return tl.unit ? unit_smem_bytes(P.unit_shapes[tl.unit - 1].W, tl.nhops, 1)
+      return tl.unit ? unit_smem_bytes(P.unit_shapes[tl.unit - 1], 1)
                      : sweep_smem_bytes(tl.nmax, tl.nhops, 1, tl.ring);
     };
     for (int t = 0; t <= T; ++t) {
@@ -697,8 +703,8 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
         if (tl.unit) {
           const UnitShape& s = P.unit_shapes[tl.unit - 1];
           g.unit_w = std::max(g.unit_w, s.W);
-          g.unit_bytes0 = std::max<int32_t>(g.unit_bytes0, (int32_t)unit_smem_bytes(s.W, s.k, 0));
-          g.unit_bytes1 = std::max<int32_t>(g.unit_bytes1, (int32_t)unit_smem_bytes(s.W, s.k, 1));
+          g.unit_bytes0 = std::max<int32_t>(g.unit_bytes0, (int32_t)unit_smem_bytes(s, 0));
+          g.unit_bytes1 = std::max<int32_t>(g.unit_bytes1, (int32_t)unit_smem_bytes(s, 1));
         }
         g.region_bwd1 = std::max<int32_t>(g.region_bwd1, (int32_t)sweep_smem_bytes_bwd(P.tiles[t].nmax, P.tiles[t].nhops, 1));
         g.region_bwd0 = std::max<int32_t>(g.region_bwd0, (int32_t)sweep_smem_bytes_bwd(P.tiles[t].nmax, P.tiles[t].nhops, 0));
@@ -959,13 +965,14 @@ dg_status validate_plan(const Plan& P) {
         s.accept >= (1 << s.W) || s.nruns < 1 || s.run_base < 0 ||
         (size_t)s.run_base + (size_t)s.nruns > P.unit_runs.size())
       return bad("unit shape out of range");
-    int prev = 0;
+    int prev = 0, rows = -1;
     for (int r = 0; r < s.nruns; ++r) {
       const int e = P.unit_runs[s.run_base + r] >> 2;
       if (e <= prev || e > s.k) return bad("unit shape runs not ascending");
+      rows += (e - prev + 1) / 2;
       prev = e;
     }
-    if (prev != s.k) return bad("unit shape runs do not cover its levels");
+    if (prev != s.k || rows != s.rows) return bad("unit shape runs do not cover its levels");
   }
   // tiles: contiguous bases, sane shapes, every lane's BDD well formed
   int64_t node_base = 0, slot_base = 0, real_nodes = 0, real_slots = 0;

@@ -74,15 +74,16 @@ struct UnitShape {
   int32_t accept;    // bit u: state u after the last level is the top terminal
   int32_t run_base;  // first entry of unit_runs
   int32_t nruns;     // runs of levels of one type: end level << 2 | type
-  int32_t pad[2];
+  int32_t rows;      // levels whose path costs a sweep keeps: every second one of a run
+  int32_t pad;
 };
 static_assert(sizeof(UnitShape) == 32, "UnitShape is 32 bytes");
 
 // Shared memory of one unit tile (one warp's slice) in the sweeps: the path
-// costs of levels 1 .. k-1 and per level lambda, the averaging term and (mode
-// 1) omega and alpha.
-inline size_t unit_smem_bytes(int W, int k, int mode) {
-  return (size_t)kWarp * 4 * ((size_t)(k - 1) * W + (size_t)k * (mode ? 4 : 2));
+// costs of `rows` levels and per level lambda, the averaging term and (mode 1)
+// omega and alpha.
+inline size_t unit_smem_bytes(const UnitShape& s, int mode) {
+  return (size_t)kWarp * 4 * ((size_t)s.rows * s.W + (size_t)s.k * (mode ? 4 : 2));
 }
 
 inline int ring_size(int maxw) {

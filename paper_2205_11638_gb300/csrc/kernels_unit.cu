@@ -20,149 +20,149 @@ namespace dg {
 
 namespace {
 
-// One tile.  KIND: kFwd, kBwd, kMinMarg, kEnergy, kSeed.
+// A warp's slice of shared memory: per level and lane lambda, (update sweeps)
+// the averaging term, (mode 1) omega and alpha, then the path costs of levels
+// 1 .. k-1, 32 W floats each.
+struct UnitSmem {
+  float *lam, *avg, *om, *al, *cost;
+};
+
+template <bool UPDATE, int MODE>
+__device__ __forceinline__ UnitSmem carve_unit(unsigned char* p, int ns) {
+  UnitSmem m;
+  m.lam = (float*)p;
+  m.avg = m.lam + ns;
+  m.om = m.avg + ns;
+  m.al = m.om + ns;
+  m.cost = !UPDATE ? m.avg : (MODE == 1 ? m.al + ns : m.om);
+  return m;
+}
+
+// Starts the copies of a tile's inputs.  The variable ids come first, into the
+// words of the averaging terms, so that gather_avg can follow as soon as they
+// are there: two memory latencies per tile whatever its length (loading the
+// ids into registers instead takes one per few levels).
+template <bool UPDATE, int MODE>
+__device__ __forceinline__ void stage_unit(const DevArena& A, const SweepArgs& a, const UnitSmem& m, int64_t sb,
+                                           int ns, int lane) {
+  if (UPDATE) {
+    copy_async(m.avg, A.slot_var + sb, ns * 4, lane);
+    cp_async_commit();
+  }
+  copy_async(m.lam, a.lam + sb, ns * 4, lane);
+  if (UPDATE && MODE == 1) {
+    copy_async(m.om, a.omega + sb, ns * 4, lane);
+    copy_async(m.al, a.alpha + sb, ns * 4, lane);
+  }
+  cp_async_commit();
+}
+
+// Replaces the staged variable ids by the averaging terms (S_i in mode 1,
+// S_i / |J_i| in mode 0), asynchronously: they are not needed before the
+// second pass.
+template <int MODE>
+__device__ __forceinline__ void gather_avg(const DevArena& A, const UnitSmem& m, int ns, int lane) {
+  const float* src = MODE == 1 ? A.S : A.Sbar;
+#pragma unroll 4
+  for (int q = lane; q < ns; q += kWarp) {
+    const int v = __float_as_int(m.avg[q]);
+    if (v >= 0) cp_async4(m.avg + q, src + v);
+  }
+  cp_async_commit();
+}
+
+// One tile whose inputs are on their way.  KIND: kFwd, kBwd, kMinMarg,
+// kEnergy, kSeed.
 template <int KIND, int MODE, int W>
 __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
-                                          unsigned char* smem, int lane) {
+                                          const UnitSmem& m, int lane) {
   constexpr bool UPDATE = KIND == kFwd || KIND == kBwd;
   const UnitCtx s{S.k, S.start, S.accept, S.nruns, A.unit_runs + S.run_base};
   const int64_t sb = T.slot_base;
-  const int k = s.k, ns = k * kWarp;
+  const int k = s.k;
   const bool real = lane < T.nbdd;
-  float* lam = (float*)smem;
-  float* avg = lam + ns;
-  float* om = avg + ns;
-  float* al = om + (MODE == 1 ? ns : 0);
-  float* cost = UPDATE ? al + ns : avg;  // level h >= 1 at cost + (h - 1) 32 W
-  if (MODE == 0) cost = UPDATE ? avg + ns : avg;
-  auto row = [&](int h) { return cost + (h - 1) * (kWarp * W); };
-
-  copy_async(lam, a.lam + sb, ns * 4, lane);
-  if (UPDATE && MODE == 1) {
-    copy_async(om, a.omega + sb, ns * 4, lane);
-    copy_async(al, a.alpha + sb, ns * 4, lane);
-  }
-  cp_async_commit();
-  if (UPDATE) {
-    // the averaging term of every slot, gathered per variable: it is not
-    // needed before the second pass
-    const float* src = MODE == 1 ? A.S : A.Sbar;
-    const int32_t* var = A.slot_var + sb + lane;
-#pragma unroll 4
-    for (int h = 0; h < k; ++h) {
-      const int v = __ldg(var + h * kWarp);
-      if (v >= 0) cp_async4(avg + h * kWarp + lane, src + v);
+  const float *lam = m.lam, *avg = m.avg, *om = m.om, *al = m.al;
+  auto energy = [&](const Costs<W>& t) {  // SP(r, T) = E^j
+    float e = f_inf();
+#pragma unroll
+    for (int u = 0; u < W; ++u)
+      if (u == s.start) e = t.v[u];
+    a.E[__ldg(A.slot_row + sb + lane)] = e;
+  };
+  // the update of level h from its minima; returns lambda^new
+  auto update = [&](int h, float l, float b0, float b1) -> float {
+    const int q = h * kWarp + lane;
+    const float m0 = b0, m1 = l + b1;
+    const float Mn = __fmul_rn(MODE == 1 ? om[q] : a.omega0, m1 - m0);
+    const float ln = unit_lambda_new<MODE>(l, Mn, MODE == 1 ? al[q] : 0.0f, avg[q]);
+    if (real) {
+      a.lam[sb + q] = ln;
+      a.M[sb + q] = Mn;
     }
-    cp_async_commit();
-    cp_async_wait_one();
-  } else {
-    cp_async_wait_all();
-  }
-  __syncwarp();
+    return ln;
+  };
 
   if (KIND == kFwd || KIND == kMinMarg) {
-    Costs<W> t = unit_end<W>(s.accept);
-    unit_levels_up(s, 1, [&](auto ty, int h) {
-      t = unit_up<W, decltype(ty)::value>(t, lam[h * kWarp + lane]);
-      unit_store<W>(row(h), t, lane);
-    });
-    if (UPDATE) {
-      cp_async_wait_all();
-      __syncwarp();
-    }
+    unit_first_up<W>(s, S.rows, lam, m.cost, lane);
+    if (UPDATE) cp_async_wait_all();  // every lane gathered its own averaging terms
     Costs<W> R = unit_root<W>(s.start);
-    unit_levels_down(s, 0, k, [&](auto ty, int h) {
+    unit_second_down<W>(s, lam, m.cost, lane, [&](auto ty, int h, const Costs<W>& t1) {
       constexpr int TY = decltype(ty)::value;
-      const Costs<W> t1 = h + 1 < k ? unit_load<W>(row(h + 1), lane) : unit_end<W>(s.accept);
       const int q = h * kWarp + lane;
       const float l = lam[q];
       float b0, b1;
       unit_minima<W, TY>(R, t1, b0, b1);
-      const float m0 = b0, m1 = l + b1;
       float ln = l;
       if (KIND == kMinMarg) {
         if (real) {
-          a.M[sb + q] = m0;
-          a.out2[sb + q] = m1;
+          a.M[sb + q] = b0;
+          a.out2[sb + q] = l + b1;
         }
       } else {
-        const float Mn = __fmul_rn(MODE == 1 ? om[q] : a.omega0, m1 - m0);
-        ln = unit_lambda_new<MODE>(l, Mn, MODE == 1 ? al[q] : 0.0f, avg[q]);
-        if (real) {
-          a.lam[sb + q] = ln;
-          a.M[sb + q] = Mn;
-        }
+        ln = update(h, l, b0, b1);
       }
       R = unit_down<W, TY>(R, ln);
     });
   } else if (KIND == kBwd) {
-    Costs<W> R = unit_root<W>(s.start);
-    unit_levels_down(s, 0, k - 1, [&](auto ty, int h) {
-      R = unit_down<W, decltype(ty)::value>(R, lam[h * kWarp + lane]);
-      unit_store<W>(row(h + 1), R, lane);
-    });
+    unit_first_down<W>(s, lam, m.cost, lane);
     cp_async_wait_all();
-    __syncwarp();
     Costs<W> t = unit_end<W>(s.accept);
-    unit_levels_up(s, 0, [&](auto ty, int h) {
+    unit_second_up<W>(s, S.rows, lam, m.cost, lane, [&](auto ty, int h, const Costs<W>& r) {
       constexpr int TY = decltype(ty)::value;
-      const Costs<W> r = h > 0 ? unit_load<W>(row(h), lane) : unit_root<W>(s.start);
-      const int q = h * kWarp + lane;
-      const float l = lam[q];
+      const float l = lam[h * kWarp + lane];
       float b0, b1;
       unit_minima<W, TY>(r, t, b0, b1);
-      const float m0 = b0, m1 = l + b1;
-      const float Mn = __fmul_rn(MODE == 1 ? om[q] : a.omega0, m1 - m0);
-      const float ln = unit_lambda_new<MODE>(l, Mn, MODE == 1 ? al[q] : 0.0f, avg[q]);
-      if (real) {
-        a.lam[sb + q] = ln;
-        a.M[sb + q] = Mn;
-      }
-      t = unit_up<W, TY>(t, ln);
+      t = unit_up<W, TY>(t, update(h, l, b0, b1));
     });
-    if (a.E != nullptr && real) {
-      float e = f_inf();  // SP(r, T) = E^j
-#pragma unroll
-      for (int u = 0; u < W; ++u)
-        if (u == s.start) e = t.v[u];
-      a.E[__ldg(A.slot_row + sb + lane)] = e;
-    }
-  } else {
+    if (a.E != nullptr && real) energy(t);
+  } else if (KIND == kEnergy) {
     Costs<W> t = unit_end<W>(s.accept);
-    unit_levels_up(s, 0, [&](auto ty, int h) {
-      t = unit_up<W, decltype(ty)::value>(t, lam[h * kWarp + lane]);
-      if (KIND == kSeed && h > 0) unit_store<W>(row(h), t, lane);
+    unit_runs_up(s, [&](auto ty, int b, int e) {
+      for (int h = e - 1; h >= b; --h) t = unit_up<W, decltype(ty)::value>(t, lam[h * kWarp + lane]);
     });
-    if (KIND == kEnergy && a.E != nullptr && real) {
-      float e = f_inf();
+    if (a.E != nullptr && real) energy(t);
+  } else {
+    // kSeed: walk the minimising path from the root, the 0-arc on ties
+    unit_first_up<W>(s, S.rows, lam, m.cost, lane);
+    int at = s.start;
+    unit_second_down<W>(s, lam, m.cost, lane, [&](auto ty, int h, const Costs<W>& t1) {
+      constexpr int TY = decltype(ty)::value;
+      const int q = h * kWarp + lane;
+      float c0 = f_inf(), c1 = f_inf();
+      int z = 0, o = 0;
 #pragma unroll
       for (int u = 0; u < W; ++u)
-        if (u == s.start) e = t.v[u];
-      a.E[__ldg(A.slot_row + sb + lane)] = e;
-    }
-    if (KIND == kSeed) {
-      // walk the minimising path from the root: 0-arc on ties
-      int at = s.start;
-      unit_levels_down(s, 0, k, [&](auto ty, int h) {
-        constexpr int TY = decltype(ty)::value;
-        const Costs<W> t1 = h + 1 < k ? unit_load<W>(row(h + 1), lane) : unit_end<W>(s.accept);
-        const int q = h * kWarp + lane;
-        float c0 = f_inf(), c1 = f_inf();
-        int z = 0, o = 0;
-#pragma unroll
-        for (int u = 0; u < W; ++u)
-          if (u == at) {
-            c0 = t1.at(unit_z<TY>(u));
-            c1 = t1.at(unit_o<TY>(u));
-            z = unit_z<TY>(u);
-            o = unit_o<TY>(u);
-          }
-        // an infinite cost is the bottom terminal (the path stays feasible)
-        const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= lam[q] + c1);
-        if (real) a.M[sb + q] = take0 ? 0.f : 1.f;
-        at = take0 ? z : o;
-      });
-    }
+        if (u == at) {
+          c0 = t1.at(unit_z<TY>(u));
+          c1 = t1.at(unit_o<TY>(u));
+          z = unit_z<TY>(u);
+          o = unit_o<TY>(u);
+        }
+      // an infinite cost is the bottom terminal (the path stays feasible)
+      const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= lam[q] + c1);
+      if (real) a.M[sb + q] = take0 ? 0.f : 1.f;
+      at = take0 ? z : o;
+    });
   }
 }
 
@@ -172,17 +172,29 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
   if (tile >= tile1) return;  // whole warp leaves; no CTA-wide barrier follows
+  constexpr bool UPDATE = KIND == kFwd || KIND == kBwd;
   const Tile T = A.tiles[tile];
+  const int ns = T.nhops * kWarp;
+  const UnitSmem m = carve_unit<UPDATE, MODE>(smem + (size_t)warp * region_bytes, ns);
+  stage_unit<UPDATE, MODE>(A, a, m, T.slot_base, ns, lane);
   const UnitShape S = A.unit_shapes[T.unit - 1];
-  unsigned char* p = smem + (size_t)warp * region_bytes;
+  if (UPDATE) {
+    cp_async_wait_one();
+    __syncwarp();
+    gather_avg<MODE>(A, m, ns, lane);
+    cp_async_wait_one();
+  } else {
+    cp_async_wait_all();
+  }
+  __syncwarp();
   if (S.W == 2)
-    unit_tile<KIND, MODE, 2>(A, a, T, S, p, lane);
+    unit_tile<KIND, MODE, 2>(A, a, T, S, m, lane);
   else if (WMAX >= 4 && S.W == 4)
-    unit_tile<KIND, MODE, 4>(A, a, T, S, p, lane);
+    unit_tile<KIND, MODE, 4>(A, a, T, S, m, lane);
   else if (WMAX >= 8 && S.W == 6)
-    unit_tile<KIND, MODE, 6>(A, a, T, S, p, lane);
+    unit_tile<KIND, MODE, 6>(A, a, T, S, m, lane);
   else if (WMAX >= 8)
-    unit_tile<KIND, MODE, 8>(A, a, T, S, p, lane);
+    unit_tile<KIND, MODE, 8>(A, a, T, S, m, lane);
 }
 
 template <int KIND, int MODE, int WMAX>

@@ -65,15 +65,25 @@ __device__ __forceinline__ Costs<W> unit_down(const Costs<W>& R, float l) {
 }
 
 // Minima over the level's states of SP(r, u) + SP(child, T) by the 0- and the
-// 1-arc.
+// 1-arc (as trees: a short chain between one level's update and the next).
 template <int W, int TYPE>
 __device__ __forceinline__ void unit_minima(const Costs<W>& R, const Costs<W>& T, float& b0, float& b1) {
-  b0 = b1 = f_inf();
+  float x0[W], x1[W];
 #pragma unroll
   for (int u = 0; u < W; ++u) {
-    b0 = fminf(b0, R.v[u] + T.at(unit_z<TYPE>(u)));
-    if (unit_o<TYPE>(u) >= 0 && unit_o<TYPE>(u) < W) b1 = fminf(b1, R.v[u] + T.at(unit_o<TYPE>(u)));
+    const int o = unit_o<TYPE>(u);
+    x0[u] = R.v[u] + T.at(unit_z<TYPE>(u));
+    x1[u] = o >= 0 && o < W ? R.v[u] + T.at(o) : f_inf();
   }
+#pragma unroll
+  for (int d = 1; d < W; d *= 2)
+#pragma unroll
+    for (int u = 0; u + d < W; u += 2 * d) {
+      x0[u] = fminf(x0[u], x0[u + d]);
+      x1[u] = fminf(x1[u], x1[u + d]);
+    }
+  b0 = x0[0];
+  b1 = x1[0];
 }
 
 // The costs of a level in the warp's shared memory: 32 W floats per level,
@@ -136,56 +146,124 @@ struct UnitCtx {
   const uint16_t* runs;
 };
 
-// Calls f(type constant, level) for the levels first .. k-1 in ascending
-// order, run by run, so that the type is decided once per run.
+// Calls f(type constant, first level, end level) for the runs in ascending or
+// descending order, so that a level's type is decided once per run.
 template <int T>
 struct TypeC {
   static constexpr int value = T;
 };
 template <class F>
-__device__ __forceinline__ void unit_levels_down(const UnitCtx& s, int first, int last, F&& f) {
-  int h = first;
-  for (int r = 0; r < s.nruns; ++r) {
-    const unsigned run = __ldg(s.runs + r);
-    const int e = min((int)(run >> 2), last);
-    switch (run & 3u) {
-      case kUp:
-        for (; h < e; ++h) f(TypeC<kUp>{}, h);
-        break;
-      case kDown:
-        for (; h < e; ++h) f(TypeC<kDown>{}, h);
-        break;
-      case kSwap:
-        for (; h < e; ++h) f(TypeC<kSwap>{}, h);
-        break;
-      default:
-        for (; h < e; ++h) f(TypeC<kDrop>{}, h);
-        break;
-    }
+__device__ __forceinline__ void unit_run(unsigned type, int b, int e, F& f) {
+  switch (type) {
+    case kUp: f(TypeC<kUp>{}, b, e); break;
+    case kDown: f(TypeC<kDown>{}, b, e); break;
+    case kSwap: f(TypeC<kSwap>{}, b, e); break;
+    default: f(TypeC<kDrop>{}, b, e); break;
   }
 }
-// ... and for the levels k-1 .. first in descending order.
 template <class F>
-__device__ __forceinline__ void unit_levels_up(const UnitCtx& s, int first, F&& f) {
-  int h = s.k - 1;
-  for (int r = s.nruns - 1; r >= 0; --r) {
+__device__ __forceinline__ void unit_runs_down(const UnitCtx& s, F&& f) {
+  int b = 0;
+  for (int r = 0; r < s.nruns; ++r) {
     const unsigned run = __ldg(s.runs + r);
-    const int b = max(r > 0 ? (int)(__ldg(s.runs + r - 1) >> 2) : 0, first);
-    switch (run & 3u) {
-      case kUp:
-        for (; h >= b; --h) f(TypeC<kUp>{}, h);
-        break;
-      case kDown:
-        for (; h >= b; --h) f(TypeC<kDown>{}, h);
-        break;
-      case kSwap:
-        for (; h >= b; --h) f(TypeC<kSwap>{}, h);
-        break;
-      default:
-        for (; h >= b; --h) f(TypeC<kDrop>{}, h);
-        break;
-    }
+    unit_run(run & 3u, b, (int)(run >> 2), f);
+    b = (int)(run >> 2);
   }
+}
+template <class F>
+__device__ __forceinline__ void unit_runs_up(const UnitCtx& s, F&& f) {
+  unsigned run = __ldg(s.runs + s.nruns - 1);
+  for (int r = s.nruns - 1; r >= 0; --r) {
+    const unsigned prev = r > 0 ? __ldg(s.runs + r - 1) : 0u;
+    unit_run(run & 3u, (int)(prev >> 2), (int)(run >> 2), f);
+    run = prev;
+  }
+}
+
+// The two-pass walks.  The first pass leaves the costs of every second level
+// of a run in shared memory, the second recomputes the others from their
+// neighbour (the same operations on the same values) right before it needs
+// them: half the shared memory per tile, which is what limits the warps per
+// SM, for two operations per recomputed state.
+
+// First pass of a forward sweep: SP(., T) of the levels at even distance from
+// their run's first level and of every run's end, in level order.
+template <int W>
+__device__ __forceinline__ void unit_first_up(const UnitCtx& s, int rows, const float* lam, float* cost, int lane) {
+  Costs<W> t = unit_end<W>(s.accept);
+  float* p = cost + rows * (kWarp * W);
+  unit_runs_up(s, [&](auto ty, int b, int e) {
+    if (e < s.k) unit_store<W>(p -= kWarp * W, t, lane);
+    for (int h = e - 1; h >= b; --h) {
+      if (h == 0) break;  // SP(root, T) is not used
+      t = unit_up<W, decltype(ty)::value>(t, lam[h * kWarp + lane]);
+      if (h > b && ((h - b) & 1) == 0) unit_store<W>(p -= kWarp * W, t, lane);
+    }
+  });
+}
+// Second pass: f(type constant, level h, SP(., T) of level h + 1) for every
+// level in ascending order.
+template <int W, class F>
+__device__ __forceinline__ void unit_second_down(const UnitCtx& s, const float* lam, const float* cost, int lane,
+                                                 F&& f) {
+  const float* p = cost;
+  unit_runs_down(s, [&](auto ty, int b, int e) {
+    constexpr int TY = decltype(ty)::value;
+    auto next = [&](int h) {
+      if (h == s.k) return unit_end<W>(s.accept);
+      const Costs<W> c = unit_load<W>(p, lane);
+      p += kWarp * W;
+      return c;
+    };
+    int h = b;
+    for (; h + 1 < e; h += 2) {
+      const Costs<W> t2 = next(h + 2);
+      const Costs<W> t1 = unit_up<W, TY>(t2, lam[(h + 1) * kWarp + lane]);
+      f(ty, h, t1);
+      f(ty, h + 1, t2);
+    }
+    if (h < e) f(ty, h, next(e));
+  });
+}
+
+// The same for a backward sweep: SP(r, .) of the levels at even distance from
+// their run's first level, then f(type constant, level h, SP(r, .) of level
+// h) in descending order.
+template <int W>
+__device__ __forceinline__ void unit_first_down(const UnitCtx& s, const float* lam, float* cost, int lane) {
+  Costs<W> R = unit_root<W>(s.start);
+  float* p = cost;
+  unit_runs_down(s, [&](auto ty, int b, int e) {
+    for (int h = b; h < e; ++h) {
+      if (h > 0 && ((h - b) & 1) == 0) {
+        unit_store<W>(p, R, lane);
+        p += kWarp * W;
+      }
+      if (h + 1 < s.k) R = unit_down<W, decltype(ty)::value>(R, lam[h * kWarp + lane]);
+    }
+  });
+}
+template <int W, class F>
+__device__ __forceinline__ void unit_second_up(const UnitCtx& s, int rows, const float* lam, const float* cost,
+                                               int lane, F&& f) {
+  const float* p = cost + rows * (kWarp * W);
+  unit_runs_up(s, [&](auto ty, int b, int e) {
+    constexpr int TY = decltype(ty)::value;
+    auto prev = [&](int h) {
+      return h == 0 ? unit_root<W>(s.start) : unit_load<W>(p -= kWarp * W, lane);
+    };
+    int h = e - 1;
+    if (((h - b) & 1) == 0) {
+      f(ty, h, prev(h));
+      --h;
+    }
+    for (; h > b; h -= 2) {
+      const Costs<W> r0 = prev(h - 1);
+      const Costs<W> r1 = unit_down<W, TY>(r0, lam[(h - 1) * kWarp + lane]);
+      f(ty, h, r1);
+      f(ty, h - 1, r0);
+    }
+  });
 }
 
 // lambda^new of the update, every rounding spelled out as the mixed tiles'
