@@ -20,134 +20,108 @@ namespace dg {
 
 namespace {
 
-// A warp's slice of shared memory: per level and lane lambda, (update sweeps)
-// the averaging term, (mode 1) omega and alpha, then the path costs of levels
-// 1 .. k-1, 32 W floats each.
-struct UnitSmem {
-  float *lam, *avg, *om, *al, *cost;
-};
-
+// A warp's slice of shared memory: per level 32 lambdas and (update sweeps) 32
+// averaging terms, (mode 1) 32 omegas and 32 alphas, so that one pointer walks
+// them all; then the path costs the sweep keeps, 32 W floats per level.
+constexpr int kAvg = kWarp, kOm = 2 * kWarp, kAl = 3 * kWarp;
 template <bool UPDATE, int MODE>
-__device__ __forceinline__ UnitSmem carve_unit(unsigned char* p, int ns) {
-  UnitSmem m;
-  m.lam = (float*)p;
-  m.avg = m.lam + ns;
-  m.om = m.avg + ns;
-  m.al = m.om + ns;
-  m.cost = !UPDATE ? m.avg : (MODE == 1 ? m.al + ns : m.om);
-  return m;
-}
+constexpr int kStride = kWarp * (!UPDATE ? 1 : (MODE == 1 ? 4 : 2));
 
-// Starts the copies of a tile's inputs.  The variable ids come first, into the
-// words of the averaging terms, so that gather_avg can follow as soon as they
-// are there: two memory latencies per tile whatever its length (loading the
-// ids into registers instead takes one per few levels).
-template <bool UPDATE, int MODE>
-__device__ __forceinline__ void stage_unit(const DevArena& A, const SweepArgs& a, const UnitSmem& m, int64_t sb,
-                                           int ns, int lane) {
-  if (UPDATE) {
-    copy_async(m.avg, A.slot_var + sb, ns * 4, lane);
-    cp_async_commit();
+// k rows of 128 bytes from src to every STRIDE-th float of dst, asynchronously.
+template <int STRIDE>
+__device__ __forceinline__ void copy_rows(float* dst, const void* src, int k, int lane, uint64_t pol) {
+  const char* g = reinterpret_cast<const char*>(src) + lane * 16;
+  char* d = reinterpret_cast<char*>(dst) + (lane >> 3) * (STRIDE * 4) + (lane & 7) * 16;
+  for (int h = lane >> 3; h < k; h += 4) {
+    cp_async16(d, g, pol);
+    d += 4 * STRIDE * 4;
+    g += 512;
   }
-  copy_async(m.lam, a.lam + sb, ns * 4, lane);
-  if (UPDATE && MODE == 1) {
-    copy_async(m.om, a.omega + sb, ns * 4, lane);
-    copy_async(m.al, a.alpha + sb, ns * 4, lane);
-  }
-  cp_async_commit();
-}
-
-// Replaces the staged variable ids by the averaging terms (S_i in mode 1,
-// S_i / |J_i| in mode 0), asynchronously: they are not needed before the
-// second pass.
-template <int MODE>
-__device__ __forceinline__ void gather_avg(const DevArena& A, const UnitSmem& m, int ns, int lane) {
-  const float* src = MODE == 1 ? A.S : A.Sbar;
-#pragma unroll 4
-  for (int q = lane; q < ns; q += kWarp) {
-    const int v = __float_as_int(m.avg[q]);
-    if (v >= 0) cp_async4(m.avg + q, src + v);
-  }
-  cp_async_commit();
 }
 
 // One tile whose inputs are on their way.  KIND: kFwd, kBwd, kMinMarg,
 // kEnergy, kSeed.
 template <int KIND, int MODE, int W>
 __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
-                                          const UnitSmem& m, int lane) {
+                                          float* smem, int lane) {
   constexpr bool UPDATE = KIND == kFwd || KIND == kBwd;
+  constexpr int STRIDE = kStride<UPDATE, MODE>;
   const UnitCtx s{S.k, S.start, S.accept, S.nruns, A.unit_runs + S.run_base};
-  const int64_t sb = T.slot_base;
-  const int k = s.k;
+  const int64_t sb = T.slot_base + lane;
   const bool real = lane < T.nbdd;
-  const float *lam = m.lam, *avg = m.avg, *om = m.om, *al = m.al;
+  const float* x0 = smem + lane;
+  float* cost = smem + s.k * STRIDE;
   auto energy = [&](const Costs<W>& t) {  // SP(r, T) = E^j
     float e = f_inf();
 #pragma unroll
     for (int u = 0; u < W; ++u)
       if (u == s.start) e = t.v[u];
-    a.E[__ldg(A.slot_row + sb + lane)] = e;
+    a.E[__ldg(A.slot_row + sb)] = e;
   };
-  // the update of level h from its minima; returns lambda^new
-  auto update = [&](int h, float l, float b0, float b1) -> float {
-    const int q = h * kWarp + lane;
+  // the update of a level from its minima; returns lambda^new
+  auto update = [&](const float* x, float* lam, float* M, float b0, float b1) -> float {
+    const float l = x[0];
     const float m0 = b0, m1 = l + b1;
-    const float Mn = __fmul_rn(MODE == 1 ? om[q] : a.omega0, m1 - m0);
-    const float ln = unit_lambda_new<MODE>(l, Mn, MODE == 1 ? al[q] : 0.0f, avg[q]);
+    const float Mn = __fmul_rn(MODE == 1 ? x[kOm] : a.omega0, m1 - m0);
+    const float ln = unit_lambda_new<MODE>(l, Mn, MODE == 1 ? x[kAl] : 0.0f, x[kAvg]);
     if (real) {
-      a.lam[sb + q] = ln;
-      a.M[sb + q] = Mn;
+      *lam = ln;
+      *M = Mn;
     }
     return ln;
   };
 
   if (KIND == kFwd || KIND == kMinMarg) {
-    unit_first_up<W>(s, S.rows, lam, m.cost, lane);
+    unit_first_up<W, STRIDE>(s, S.rows, x0, cost, lane);
     if (UPDATE) cp_async_wait_all();  // every lane gathered its own averaging terms
     Costs<W> R = unit_root<W>(s.start);
-    unit_second_down<W>(s, lam, m.cost, lane, [&](auto ty, int h, const Costs<W>& t1) {
+    float* g0 = (KIND == kFwd ? a.lam : a.out2) + sb;
+    float* g1 = a.M + sb;
+    unit_second_down<W, STRIDE>(s, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& t1) {
       constexpr int TY = decltype(ty)::value;
-      const int q = h * kWarp + lane;
-      const float l = lam[q];
-      float b0, b1;
+      float b0, b1, ln = x[0];
       unit_minima<W, TY>(R, t1, b0, b1);
-      float ln = l;
       if (KIND == kMinMarg) {
         if (real) {
-          a.M[sb + q] = b0;
-          a.out2[sb + q] = l + b1;
+          *g0 = ln + b1;
+          *g1 = b0;
         }
       } else {
-        ln = update(h, l, b0, b1);
+        ln = update(x, g0, g1, b0, b1);
       }
+      g0 += kWarp;
+      g1 += kWarp;
       R = unit_down<W, TY>(R, ln);
     });
   } else if (KIND == kBwd) {
-    unit_first_down<W>(s, lam, m.cost, lane);
+    unit_first_down<W, STRIDE>(s, x0, cost, lane);
     cp_async_wait_all();
     Costs<W> t = unit_end<W>(s.accept);
-    unit_second_up<W>(s, S.rows, lam, m.cost, lane, [&](auto ty, int h, const Costs<W>& r) {
+    float* g0 = a.lam + sb + s.k * kWarp;
+    float* g1 = a.M + sb + s.k * kWarp;
+    unit_second_up<W, STRIDE>(s, S.rows, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& r) {
       constexpr int TY = decltype(ty)::value;
-      const float l = lam[h * kWarp + lane];
       float b0, b1;
       unit_minima<W, TY>(r, t, b0, b1);
-      t = unit_up<W, TY>(t, update(h, l, b0, b1));
+      g0 -= kWarp;
+      g1 -= kWarp;
+      t = unit_up<W, TY>(t, update(x, g0, g1, b0, b1));
     });
     if (a.E != nullptr && real) energy(t);
   } else if (KIND == kEnergy) {
     Costs<W> t = unit_end<W>(s.accept);
+    const float* x = x0 + s.k * STRIDE;
     unit_runs_up(s, [&](auto ty, int b, int e) {
-      for (int h = e - 1; h >= b; --h) t = unit_up<W, decltype(ty)::value>(t, lam[h * kWarp + lane]);
+      for (int n = e - b; n > 0; --n) t = unit_up<W, decltype(ty)::value>(t, *(x -= STRIDE));
     });
     if (a.E != nullptr && real) energy(t);
   } else {
     // kSeed: walk the minimising path from the root, the 0-arc on ties
-    unit_first_up<W>(s, S.rows, lam, m.cost, lane);
+    unit_first_up<W, STRIDE>(s, S.rows, x0, cost, lane);
     int at = s.start;
-    unit_second_down<W>(s, lam, m.cost, lane, [&](auto ty, int h, const Costs<W>& t1) {
+    float* g1 = a.M + sb;
+    unit_second_down<W, STRIDE>(s, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& t1) {
       constexpr int TY = decltype(ty)::value;
-      const int q = h * kWarp + lane;
       float c0 = f_inf(), c1 = f_inf();
       int z = 0, o = 0;
 #pragma unroll
@@ -159,8 +133,9 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
           o = unit_o<TY>(u);
         }
       // an infinite cost is the bottom terminal (the path stays feasible)
-      const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= lam[q] + c1);
-      if (real) a.M[sb + q] = take0 ? 0.f : 1.f;
+      const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= x[0] + c1);
+      if (real) *g1 = take0 ? 0.f : 1.f;
+      g1 += kWarp;
       at = take0 ? z : o;
     });
   }
@@ -173,15 +148,40 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
   const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
   if (tile >= tile1) return;  // whole warp leaves; no CTA-wide barrier follows
   constexpr bool UPDATE = KIND == kFwd || KIND == kBwd;
+  constexpr int STRIDE = kStride<UPDATE, MODE>;
   const Tile T = A.tiles[tile];
-  const int ns = T.nhops * kWarp;
-  const UnitSmem m = carve_unit<UPDATE, MODE>(smem + (size_t)warp * region_bytes, ns);
-  stage_unit<UPDATE, MODE>(A, a, m, T.slot_base, ns, lane);
+  const int k = T.nhops;
+  float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
+  const uint64_t pol = l2_evict_first();
+  // the variable ids come first, into the words of the averaging terms, so
+  // that the gather can follow as soon as they are there: two memory latencies
+  // per tile whatever its length (ids loaded into registers a few levels at a
+  // time took one per few levels)
+  if (UPDATE) {
+    copy_rows<STRIDE>(m + kAvg, A.slot_var + T.slot_base, k, lane, pol);
+    cp_async_commit();
+  }
+  copy_rows<STRIDE>(m, a.lam + T.slot_base, k, lane, pol);
+  if (UPDATE && MODE == 1) {
+    copy_rows<STRIDE>(m + kOm, a.omega + T.slot_base, k, lane, pol);
+    copy_rows<STRIDE>(m + kAl, a.alpha + T.slot_base, k, lane, pol);
+  }
+  cp_async_commit();
   const UnitShape S = A.unit_shapes[T.unit - 1];
   if (UPDATE) {
     cp_async_wait_one();
     __syncwarp();
-    gather_avg<MODE>(A, m, ns, lane);
+    // the averaging terms (S_i in mode 1, S_i / |J_i| in mode 0) replace the
+    // ids; they are not needed before the second pass
+    const float* src = MODE == 1 ? A.S : A.Sbar;
+    float* q = m + kAvg + lane;
+#pragma unroll 2
+    for (int h = 0; h < k; ++h) {
+      const int v = __float_as_int(*q);
+      if (v >= 0) cp_async4(q, src + v);
+      q += STRIDE;
+    }
+    cp_async_commit();
     cp_async_wait_one();
   } else {
     cp_async_wait_all();

@@ -184,84 +184,112 @@ __device__ __forceinline__ void unit_runs_up(const UnitCtx& s, F&& f) {
 // of a run in shared memory, the second recomputes the others from their
 // neighbour (the same operations on the same values) right before it needs
 // them: half the shared memory per tile, which is what limits the warps per
-// SM, for two operations per recomputed state.
+// SM, for two operations per recomputed state.  x points at the lane's word of
+// level 0 in the staged inputs (lambda first), STRIDE floats per level; the
+// walks move pointers instead of indexing, because a level of a narrow row is
+// only some twenty operations.
 
 // First pass of a forward sweep: SP(., T) of the levels at even distance from
 // their run's first level and of every run's end, in level order.
-template <int W>
-__device__ __forceinline__ void unit_first_up(const UnitCtx& s, int rows, const float* lam, float* cost, int lane) {
+template <int W, int STRIDE>
+__device__ __forceinline__ void unit_first_up(const UnitCtx& s, int rows, const float* x, float* cost, int lane) {
   Costs<W> t = unit_end<W>(s.accept);
   float* p = cost + rows * (kWarp * W);
+  x += s.k * STRIDE;
   unit_runs_up(s, [&](auto ty, int b, int e) {
+    constexpr int TY = decltype(ty)::value;
     if (e < s.k) unit_store<W>(p -= kWarp * W, t, lane);
-    for (int h = e - 1; h >= b; --h) {
-      if (h == 0) break;  // SP(root, T) is not used
-      t = unit_up<W, decltype(ty)::value>(t, lam[h * kWarp + lane]);
-      if (h > b && ((h - b) & 1) == 0) unit_store<W>(p -= kWarp * W, t, lane);
+    int n = e - b;
+    if (n & 1) {
+      x -= STRIDE;
+      t = unit_up<W, TY>(t, x[0]);
+      if (--n > 0) unit_store<W>(p -= kWarp * W, t, lane);
+    }
+    for (; n > 0; n -= 2) {
+      t = unit_up<W, TY>(t, x[-STRIDE]);
+      x -= 2 * STRIDE;
+      t = unit_up<W, TY>(t, x[0]);
+      if (n > 2) unit_store<W>(p -= kWarp * W, t, lane);
     }
   });
 }
-// Second pass: f(type constant, level h, SP(., T) of level h + 1) for every
-// level in ascending order.
-template <int W, class F>
-__device__ __forceinline__ void unit_second_down(const UnitCtx& s, const float* lam, const float* cost, int lane,
+// Second pass: f(type constant, x of level h, SP(., T) of level h + 1) for
+// every level in ascending order.
+template <int W, int STRIDE, class F>
+__device__ __forceinline__ void unit_second_down(const UnitCtx& s, const float* x, const float* cost, int lane,
                                                  F&& f) {
   const float* p = cost;
   unit_runs_down(s, [&](auto ty, int b, int e) {
     constexpr int TY = decltype(ty)::value;
-    auto next = [&](int h) {
-      if (h == s.k) return unit_end<W>(s.accept);
-      const Costs<W> c = unit_load<W>(p, lane);
-      p += kWarp * W;
-      return c;
-    };
-    int h = b;
-    for (; h + 1 < e; h += 2) {
-      const Costs<W> t2 = next(h + 2);
-      const Costs<W> t1 = unit_up<W, TY>(t2, lam[(h + 1) * kWarp + lane]);
-      f(ty, h, t1);
-      f(ty, h + 1, t2);
+    const int last = e == s.k ? 2 : 0;  // levels left when SP(., T) of the next stored level is the terminals'
+    int n = e - b;
+    for (; n >= 2; n -= 2) {
+      Costs<W> t2 = unit_end<W>(s.accept);
+      if (n != last) {
+        t2 = unit_load<W>(p, lane);
+        p += kWarp * W;
+      }
+      const Costs<W> t1 = unit_up<W, TY>(t2, x[STRIDE]);
+      f(ty, x, t1);
+      f(ty, x + STRIDE, t2);
+      x += 2 * STRIDE;
     }
-    if (h < e) f(ty, h, next(e));
+    if (n > 0) {
+      Costs<W> t1 = unit_end<W>(s.accept);
+      if (last == 0) {
+        t1 = unit_load<W>(p, lane);
+        p += kWarp * W;
+      }
+      f(ty, x, t1);
+      x += STRIDE;
+    }
   });
 }
 
 // The same for a backward sweep: SP(r, .) of the levels at even distance from
-// their run's first level, then f(type constant, level h, SP(r, .) of level
-// h) in descending order.
-template <int W>
-__device__ __forceinline__ void unit_first_down(const UnitCtx& s, const float* lam, float* cost, int lane) {
+// their run's first level, then f(type constant, x of level h, SP(r, .) of
+// level h) in descending order.
+template <int W, int STRIDE>
+__device__ __forceinline__ void unit_first_down(const UnitCtx& s, const float* x, float* cost, int lane) {
   Costs<W> R = unit_root<W>(s.start);
   float* p = cost;
   unit_runs_down(s, [&](auto ty, int b, int e) {
-    for (int h = b; h < e; ++h) {
-      if (h > 0 && ((h - b) & 1) == 0) {
+    constexpr int TY = decltype(ty)::value;
+    int n = e - b;
+    for (bool stored = b > 0; n > 0; n -= 2, stored = true) {
+      if (stored) {
         unit_store<W>(p, R, lane);
         p += kWarp * W;
       }
-      if (h + 1 < s.k) R = unit_down<W, decltype(ty)::value>(R, lam[h * kWarp + lane]);
+      R = unit_down<W, TY>(R, x[0]);
+      if (n > 1) R = unit_down<W, TY>(R, x[STRIDE]);
+      x += (n > 1 ? 2 : 1) * STRIDE;
     }
   });
 }
-template <int W, class F>
-__device__ __forceinline__ void unit_second_up(const UnitCtx& s, int rows, const float* lam, const float* cost,
+template <int W, int STRIDE, class F>
+__device__ __forceinline__ void unit_second_up(const UnitCtx& s, int rows, const float* x, const float* cost,
                                                int lane, F&& f) {
   const float* p = cost + rows * (kWarp * W);
+  x += s.k * STRIDE;
   unit_runs_up(s, [&](auto ty, int b, int e) {
     constexpr int TY = decltype(ty)::value;
-    auto prev = [&](int h) {
-      return h == 0 ? unit_root<W>(s.start) : unit_load<W>(p -= kWarp * W, lane);
-    };
-    int h = e - 1;
-    if (((h - b) & 1) == 0) {
-      f(ty, h, prev(h));
-      --h;
+    const int first = b == 0 ? 2 : 0;  // levels left when SP(r, .) of the run's first level is the root's
+    int n = e - b;
+    if (n & 1) {
+      Costs<W> r0 = unit_root<W>(s.start);
+      if (n != 1 || b > 0) r0 = unit_load<W>(p -= kWarp * W, lane);
+      x -= STRIDE;
+      f(ty, x, r0);
+      --n;
     }
-    for (; h > b; h -= 2) {
-      const Costs<W> r0 = prev(h - 1);
-      const Costs<W> r1 = unit_down<W, TY>(r0, lam[(h - 1) * kWarp + lane]);
-      f(ty, h, r1);
-      f(ty, h - 1, r0);
+    for (; n > 0; n -= 2) {
+      Costs<W> r0 = unit_root<W>(s.start);
+      if (n != first) r0 = unit_load<W>(p -= kWarp * W, lane);
+      x -= 2 * STRIDE;
+      const Costs<W> r1 = unit_down<W, TY>(r0, x[0]);
+      f(ty, x + STRIDE, r1);
+      f(ty, x, r0);
     }
   });
 }
