@@ -97,7 +97,7 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
   a.omega0 = omega_of(opts);
   a.mode = mode;
   ar->avg_mode = mode;
-  launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kPlain);
+  launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kSweep);
   // every sweep hands its path costs to the next one (the S reductions
   // between them leave lambda alone), except into the first sweep, whose
   // lambda comes from the caller, and across a re-projection
@@ -108,13 +108,13 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
     a.cost_out = A.nodecost;
     a.cost_in = handed ? A.nodecost : nullptr;
     launch_sweep(kFwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kPlain);
+    launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kSweep);
     if (lb_out && it == iters - 1) a.E = A.E;
     handed = it + 1 < iters && !rn;
     a.cost_out = handed ? A.nodecost : nullptr;
     a.cost_in = A.nodecost;
     launch_sweep(kBwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_reduce_S(A, M, lam, alpha, mode, rn, st, it + 1 < iters ? Scatter::kPlain : Scatter::kNone);
+    launch_reduce_S(A, M, lam, alpha, mode, rn, st, it + 1 < iters ? Scatter::kSweep : Scatter::kNone);
   }
   if (lb_out) {
     if (iters == 0) {
@@ -132,8 +132,9 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
 // shared memory; every launch group's tiles must still fit one CTA.
 dg_status check_recording_fits(const dg_arena* ar, int mode, const char* where) {
   for (const LaunchGroup& g : ar->groups)
-    if ((size_t)(mode ? g.region_bwd1 : g.region_bwd0) + (size_t)g.meta_bytes > ar->cta_smem_cap ||
-        (size_t)(mode ? g.region_bytes : g.region_bytes0) + (size_t)g.meta_bytes > ar->cta_smem_cap)
+    if (g.unit_w == 0 &&
+        ((size_t)(mode ? g.region_bwd1 : g.region_bwd0) + (size_t)g.meta_bytes > ar->cta_smem_cap ||
+        (size_t)(mode ? g.region_bytes : g.region_bytes0) + (size_t)g.meta_bytes > ar->cta_smem_cap))
       return fail(DG_EINVAL, std::string(where) + ": a tile's recording sweep does not fit one CTA's shared memory");
   return DG_OK;
 }
@@ -354,6 +355,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.unit_shapes = (const UnitShape*)(b + P.off.unit_shapes);
   A.unit_runs = (const uint16_t*)(b + P.off.unit_runs);
   A.unit_slots = P.unit_slots;
+  A.unit_nodes = P.unit_nodes;
   A.desc = (const uint16_t*)(b + P.off.desc);
   A.lohi8 = (const uint16_t*)(b + P.off.lohi8);
   A.slot_var = (const int32_t*)(b + P.off.slot_var);
@@ -510,7 +512,7 @@ dg_status dg_autotune(dg_arena* ar, void* stream, float* lam, float* M, int32_t 
     return ms / reps;
   };
   ar->avg_mode = 0;
-  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, Scatter::kPlain);
+  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, Scatter::kSweep);
   // timed as dg_iterate runs them after its first sweep: each sweep takes
   // its opposite-direction costs from the one before
   a.cost_out = A.nodecost;
@@ -589,7 +591,7 @@ dg_status dg_sum_M(dg_arena* ar, void* stream, const float* M, float* lam, const
   ar->avg_mode = mode;
   // a reduction without re-projection leaves lambda, so a hand-off survives it
   if (!renorm) keep_costs(ar);
-  launch_reduce_S(ar->dev, M, lam, alpha, mode, renorm != 0, (cudaStream_t)stream, Scatter::kPlain);
+  launch_reduce_S(ar->dev, M, lam, alpha, mode, renorm != 0, (cudaStream_t)stream, Scatter::kSweep);
   return check_launch("dg_sum_M");
 }
 
@@ -797,7 +799,7 @@ void dg_graph_destroy(dg_graph_t* g) {
 namespace {
 
 struct BwdLayout {
-  size_t ck_lam, ck_M, rec_meta, rec_amin, rec_diff, seg_S, w_lam, w_M, sdot, sd_a, sd_b, slot_in, rec_lmeta,
+  size_t ck_lam, ck_M, rec_meta, rec_amin, rec_unit, rec_diff, seg_S, w_lam, w_M, sdot, sd_a, sd_b, var_in, slot_in, rec_lmeta,
       rec_lamin, long_a1, long_a2, total;
   size_t meta_stride;   // bytes of one sweep's node records
   size_t lmeta_stride;  // ... of the long BDDs' node records
@@ -819,9 +821,12 @@ BwdLayout backward_layout(const dg_arena* ar, int iters, int ckpt_every) {
   L.ck_lam = put((size_t)L.nseg * NS * 4);
   L.ck_M = put((size_t)L.nseg * NS * 4);
   // argmin records of every sweep of one segment (recording sweeps)
-  L.meta_stride = (size_t)ar->sizes.num_nodes_padded * 2;
+  // (per node and slot of the mixed tiles, a word per slot of the unit tiles)
+  const size_t US = (size_t)ar->dev.unit_slots;
+  L.meta_stride = ((size_t)ar->sizes.num_nodes_padded - (size_t)ar->dev.unit_nodes) * 2;
   L.rec_meta = put((size_t)2 * L.k * L.meta_stride);
-  L.rec_amin = put((size_t)2 * L.k * NS * 2);
+  L.rec_amin = put((size_t)2 * L.k * (NS - US) * 2);
+  L.rec_unit = put((size_t)2 * L.k * US * 4);
   L.rec_diff = put((size_t)2 * L.k * NS * 4);
   L.seg_S = put((size_t)2 * L.k * n * 4);
   L.w_lam = put(NS * 4);
@@ -829,7 +834,10 @@ BwdLayout backward_layout(const dg_arena* ar, int iters, int ckpt_every) {
   L.sdot = put(NS * 4);
   L.sd_a = put(n * 4);
   L.sd_b = put(n * 4);
-  L.slot_in = put(NS * 8);  // float2 per slot: the adjoint sweep's per-variable inputs
+  // the adjoint sweep's per-variable inputs: float2 per variable, and laid out
+  // per slot unless every slot belongs to a unit tile
+  L.var_in = put(n * 8);
+  L.slot_in = put(US < NS ? NS * 8 : 0);
   // long BDDs: node and slot records of every sweep of one segment, and the
   // per-node gradients of the adjoint
   const size_t lcost = (size_t)ar->dev.long_cost_size, lslots = NS - (size_t)ar->dev.long_slot_base;
@@ -864,12 +872,13 @@ dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, fl
   cudaError_t e = cudaSuccess;
   ar->avg_mode = mode;
   for (int sw = 0; sw < 2 * k; ++sw) {
-    launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, Scatter::kAll);
+    launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
     if (e == cudaSuccess && n)
       e = cudaMemcpyAsync(w + L.seg_S + (size_t)sw * n * 4, A.S, n * 4, cudaMemcpyDeviceToDevice, st);
     SweepArgs ra = fa;
     ra.rec_meta = (uint16_t*)(w + L.rec_meta + (size_t)sw * L.meta_stride);
-    ra.rec_amin = (uint16_t*)(w + L.rec_amin) + (size_t)sw * NS;
+    ra.rec_amin = (uint16_t*)(w + L.rec_amin) + (size_t)sw * (NS - (size_t)A.unit_slots);
+    ra.rec_unit = (uint32_t*)(w + L.rec_unit) + (size_t)sw * (size_t)A.unit_slots;
     ra.rec_diff = (float*)(w + L.rec_diff) + (size_t)sw * NS;
     ra.rec_lmeta = (int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
     ra.rec_lamin = (int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
@@ -955,6 +964,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
   float* sdot = (float*)(w + L.sdot);
   float* sd_next = (float*)(w + L.sd_a);
   float* sd_cur = (float*)(w + L.sd_b);
+  float2* var_in = (float2*)(w + L.var_in);
   float2* slot_in = (float2*)(w + L.slot_in);
   const int threads = threads_of(opts);
   SweepArgs fa{};
@@ -988,9 +998,9 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       f.cost_in = handed ? A.nodecost : nullptr;
       b.cost_in = A.nodecost;
       handed = true;
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kPlain);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
       launch_sweep(kFwd, A, f, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kPlain);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
       launch_sweep(kBwd, A, b, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
     }
   }
@@ -1009,8 +1019,9 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
   aa.g_alpha = g_alpha;
   aa.sdot = sdot;
   aa.slot_in = slot_in;
+  aa.var_in = var_in;
   // padding slots belong to no variable: their inputs stay 0
-  if (e == cudaSuccess && iters > 0) e = cudaMemsetAsync(slot_in, 0, NS * 8, st);
+  if (e == cudaSuccess && (size_t)A.unit_slots < NS) e = cudaMemsetAsync(slot_in, 0, NS * 8, st);
   aa.long_a1 = (float*)(w + L.long_a1);
   aa.long_a2 = (float*)(w + L.long_a2);
   const int last_sweep = 2 * iters - 1;
@@ -1023,11 +1034,12 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       cpy(w_M, ck_M + (size_t)c * NS, bNS);
     }
     for (int sw = 0; sw < (recorded ? 0 : nsw); ++sw) {
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kAll);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
       cpy(seg_S + (size_t)sw * n, A.S, bn);
       SweepArgs ra = fa;
       ra.rec_meta = (uint16_t*)(rec_meta + (size_t)sw * L.meta_stride);
-      ra.rec_amin = rec_amin + (size_t)sw * NS;
+      ra.rec_amin = rec_amin + (size_t)sw * (NS - (size_t)A.unit_slots);
+      ra.rec_unit = (uint32_t*)(w + L.rec_unit) + (size_t)sw * (size_t)A.unit_slots;
       ra.rec_diff = rec_diff + (size_t)sw * NS;
       ra.rec_lmeta = (int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
       ra.rec_lamin = (int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
@@ -1043,11 +1055,12 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
     // the per-slot inputs of the segment's last sweep: the S-dot handed over
     // from the adjoint of the segment after it (none after the last sweep)
     launch_slot_inputs(A, nullptr, 2 * it0 + nsw - 1 == last_sweep ? nullptr : sd_next, nullptr,
-                       seg_S + (size_t)(nsw - 1) * n, slot_in, st);
+                       seg_S + (size_t)(nsw - 1) * n, var_in, slot_in, st);
     for (int sw = nsw - 1; sw >= 0; --sw) {
       const int gsw = 2 * it0 + sw;
       aa.rec_meta = (const uint16_t*)(rec_meta + (size_t)sw * L.meta_stride);
-      aa.rec_amin = rec_amin + (size_t)sw * NS;
+      aa.rec_amin = rec_amin + (size_t)sw * (NS - (size_t)A.unit_slots);
+      aa.rec_unit = (const uint32_t*)(w + L.rec_unit) + (size_t)sw * (size_t)A.unit_slots;
       aa.rec_diff = rec_diff + (size_t)sw * NS;
       aa.rec_lmeta = (const int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
       aa.rec_lamin = (const int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
@@ -1058,7 +1071,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
                            streams_for(ar, st));
       // S-dot of this sweep, and the next adjoint sweep's per-slot inputs
       launch_slot_inputs(A, sdot, nullptr, sd_cur, sw > 0 ? seg_S + (size_t)(sw - 1) * n : nullptr,
-                         sw > 0 ? slot_in : nullptr, st);
+                         sw > 0 ? var_in : nullptr, sw > 0 ? slot_in : nullptr, st);
       std::swap(sd_next, sd_cur);
     }
   }

@@ -662,7 +662,10 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     P.max_tile_hops = std::max(P.max_tile_hops, nh);
     node_base += (int64_t)(nmax - 2) * kWarp;
     slot_base += tslots;
-    if (tile.unit) P.unit_slots = (int32_t)slot_base;
+    if (tile.unit) {
+      P.unit_slots = (int32_t)slot_base;
+      P.unit_nodes = (int32_t)node_base;
+    }
   }
   // launch groups: consecutive tiles whose footprints stay within 1/kGroupRatio
   // of the group's largest one
@@ -742,9 +745,11 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     }
   }
   for (const LaunchGroup& g : P.groups) {
-    AdjGroup a{g.tile0, g.tile1, 0, g.stream};
+    AdjGroup a{g.tile0, g.tile1, 0, g.stream, g.unit_w};
     for (int t = g.tile0; t < g.tile1; ++t)
-      a.region = std::max<int32_t>(a.region, (int32_t)adjoint_smem_bytes(P.tiles[t].nmax, P.tiles[t].nhops));
+      a.region = std::max<int32_t>(
+          a.region, (int32_t)(g.unit_w ? unit_adjoint_bytes(P.tiles[t].nhops)
+                                       : adjoint_smem_bytes(P.tiles[t].nmax, P.tiles[t].nhops)));
     P.adj_groups.push_back(a);
   }
   // ---- 2b. long BDDs: levels as consecutive slots after the tiles (each

@@ -86,6 +86,11 @@ inline size_t unit_smem_bytes(const UnitShape& s, int mode) {
   return (size_t)kWarp * 4 * ((size_t)s.rows * s.W + (size_t)s.k * (mode ? 4 : 2));
 }
 
+// ... and in the adjoint kernel: per level the staged inputs of kernels_unit.cu
+// (the gradient of lambda, the argmin word, m1 - m0, the weight, a pair per
+// variable and, in mode 1, omega).
+inline size_t unit_adjoint_bytes(int k) { return (size_t)kWarp * 4 * 7 * (size_t)k; }
+
 inline int ring_size(int maxw) {
   int r = 2;
   while (r < 2 * maxw) r <<= 1;
@@ -161,6 +166,7 @@ struct DevArena {
   int64_t num_slots;
   int32_t num_tiles;
   int32_t unit_slots;       // the unit tiles come first: their slots are [0, unit_slots)
+  int32_t unit_nodes;       // ... and their child codes [0, unit_nodes)
   int32_t num_lb_chunks;
   int32_t num_long;
   int32_t long_slot_base;   // first slot of the long BDDs (after every tile's slots)
@@ -194,8 +200,9 @@ struct LaunchGroup {
 // shared-memory footprint).
 struct AdjGroup {
   int32_t tile0, tile1;
-  int32_t region;  // per-warp slice (the same in both modes)
+  int32_t region;  // per-warp slice (the larger mode's)
   int32_t stream;
+  int32_t unit_w;  // unit tiles: the largest W of the group (0: mixed tiles)
 };
 
 struct Plan {
@@ -206,7 +213,7 @@ struct Plan {
   std::vector<Tile> tiles;
   std::vector<UnitShape> unit_shapes;
   std::vector<uint16_t> unit_runs;
-  int32_t unit_slots = 0;
+  int32_t unit_slots = 0, unit_nodes = 0;
   std::vector<LaunchGroup> groups;
   std::vector<AdjGroup> adj_groups;
   std::vector<uint16_t> desc;

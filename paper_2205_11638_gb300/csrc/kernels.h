@@ -40,6 +40,9 @@ struct SweepArgs {
   uint16_t* rec_meta;  // per node (layout of the child codes): in-arc parent | beta << 8 | hi-choice << 9
   uint16_t* rec_amin;  // per slot: argmin node of m0 | argmin node of m1 << 8
   float* rec_diff;     // per slot: m1 - m0
+  // (rec_meta and rec_amin hold the mixed tiles only, from node unit_nodes and
+  // slot unit_slots on; a unit tile's records are one word per slot)
+  uint32_t* rec_unit;
   // ... for the long BDDs: per node (cost scratch index) in-arc << 1 |
   // hi-choice, per long slot (from long_slot_base) the argmin nodes of m0, m1
   int32_t* rec_lmeta;
@@ -68,8 +71,11 @@ cudaError_t set_sweep_smem_limit(size_t bytes);
 cudaError_t set_unit_smem_limit(size_t bytes);
 // The launch of one group of unit tiles (kernels_unit.cu), wpc warps of
 // `region` bytes to a CTA.
+struct AdjArgs;
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
                  cudaStream_t st);
+void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
+                         cudaStream_t st);
 // Dynamic shared memory one CTA may use; launchers put fewer warps in a CTA
 // when their tiles need more.
 void set_cta_smem_cap(size_t bytes);
@@ -81,9 +87,8 @@ void launch_sweep(int kind, const DevArena& A, const SweepArgs& a, int threads, 
 // lambda_ij += alpha_ij * (c_i - sum_k (lambda_ik + M_ik)) computed in FP64.
 // Before a sweep also the mode's averaging term into A.slot_avg for the slots
 // the sweep reads it from: those of the mixed tiles and the long BDDs before
-// a plain sweep (the unit tiles gather S or Sbar), every slot before a
-// recording one.
-enum class Scatter { kNone, kPlain, kAll };
+// a sweep (the unit tiles gather S or Sbar themselves).
+enum class Scatter { kNone, kSweep };
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
                      cudaStream_t st, Scatter to);
 void launch_init(const DevArena& A, float* lam, float* M, cudaStream_t st);
@@ -96,6 +101,7 @@ struct AdjArgs {
   const uint16_t* rec_meta;  // the records of the sweep (SweepArgs::rec_*)
   const uint16_t* rec_amin;
   const float* rec_diff;
+  const uint32_t* rec_unit;
   const float* S_in;       // S at the start of the sweep (per variable)
   const float* omega;      // mode 1
   const float* alpha;      // mode 1
@@ -108,6 +114,8 @@ struct AdjArgs {
   // instead of gathering per variable (with DevArena::slot_invdeg for the
   // weights of mode 0); the long BDDs use the per-variable arrays above
   const float2* slot_in;
+  // the same per variable: the unit tiles gather it
+  const float2* var_in;
   float* g_lam;            // in: gradient of lambda after the sweep; out: before
   float* g_omega;          // accumulated (nullable: not computed)
   float* g_alpha;          // accumulated (nullable: not computed)
@@ -124,10 +132,11 @@ void launch_adjoint_sweep(bool forward, const DevArena& A, const AdjArgs& a, con
                           size_t cta_smem_cap, const StreamSet& ss);
 // Per variable i: s_i = sum over the slots q of i of x[q] (fixed order), or
 // sd_in[i] when x is NULL (0 when both are); out_var[i] = s_i (nullable);
-// and, when slot_in is not NULL, slot_in[q] = {s_i, S_var[i] (0 if NULL)}
-// for every slot q of i.
+// and, when var_in is not NULL, {s_i, S_var[i] (0 if NULL)} in var_in[i] and
+// in slot_in[q] for every slot q >= unit_slots of i (the unit tiles gather
+// var_in, the mixed tiles read slot_in).
 void launch_slot_inputs(const DevArena& A, const float* x, const float* sd_in, float* out_var, const float* S_var,
-                        float2* slot_in, cudaStream_t st);
+                        float2* var_in, float2* slot_in, cudaStream_t st);
 // A.slot_invdeg[q] = 1/|J_i| of the variable of slot q (0 for padding)
 void launch_fill_slot_invdeg(const DevArena& A, cudaStream_t st);
 // out_slot[q] = v[variable of q] (0 for padding slots)

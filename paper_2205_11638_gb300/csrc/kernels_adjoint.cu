@@ -78,7 +78,7 @@ __device__ __forceinline__ LevelIn load_level(const DevArena& A, const AdjArgs& 
   const int q = h * kWarp + lane;
   const float2 in = a.slot_in[sb + q];
   r.diff = a.rec_diff[sb + q];
-  r.amin = a.rec_amin[sb + q];
+  r.amin = a.rec_amin[sb - A.unit_slots + q];
   r.S = in.y;
   r.al = MODE == 1 ? a.alpha[sb + q] : A.slot_invdeg[sb + q];
   r.om = MODE == 1 ? a.omega[sb + q] : a.omega0;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(128) k_adjoint(DevArena A, AdjArgs a, int regi
 
   // ---- staging: child codes, the sweep's node records, the gradients -----
   copy_async(s.code + 2 * kWarp, A.lohi8 + T.node_base, (s.nmax - 2) * kWarp * 2, lane);
-  copy_async(s.meta + 2 * kWarp, a.rec_meta + T.node_base, (s.nmax - 2) * kWarp * 2, lane);
+  copy_async(s.meta + 2 * kWarp, a.rec_meta + (T.node_base - A.unit_nodes), (s.nmax - 2) * kWarp * 2, lane);
   copy_async(s.desc, A.desc + sb, ns * 2, lane);
   copy_async(s.gl, a.g_lam + sb, ns * 4, lane);
   cp_async_commit();
@@ -254,6 +254,10 @@ static void launch_adj(const DevArena& A, const AdjArgs& a, const AdjGroup* grou
     const AdjGroup& G = groups[g];
     const size_t region = (size_t)G.region;
     const int wpc = best_warps_per_cta(region, 4, cap);
+    if (G.unit_w > 0) {
+      launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, fork ? ss.of(G.stream) : ss.main);
+      continue;
+    }
     const int nt = G.tile1 - G.tile0;
     k_adjoint<FWD, MODE><<<(nt + wpc - 1) / wpc, wpc * kWarp, region * wpc, fork ? ss.of(G.stream) : ss.main>>>(
         A, a, (int)region, G.tile0, G.tile1);

@@ -212,7 +212,8 @@ __global__ void k_seed_M(DevArena A, float* gM) {
 // contributions) and the per-slot inputs of the next adjoint sweep.
 __global__ void __launch_bounds__(256) k_slot_inputs(DevArena A, const float* __restrict__ x,
                                                       const float* __restrict__ sd_in, float* out_var,
-                                                      const float* __restrict__ S_var, float2* slot_in) {
+                                                      const float* __restrict__ S_var, float2* var_in,
+                                                      float2* slot_in) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const int b = __ldg(A.var_ptr + i), e = __ldg(A.var_ptr + i + 1);
@@ -223,9 +224,14 @@ __global__ void __launch_bounds__(256) k_slot_inputs(DevArena A, const float* __
   else if (sd_in)
     s = sd_in[i];
   if (out_var) out_var[i] = s;
-  if (slot_in) {
+  if (var_in) {
     const float2 t = make_float2(s, S_var ? S_var[i] : 0.f);
-    for (int k = b; k < e; ++k) slot_in[__ldg(A.var_slots + k)] = t;
+    var_in[i] = t;
+    if (slot_in)
+      for (int k = b; k < e; ++k) {
+        const int q = __ldg(A.var_slots + k);
+        if (q >= A.unit_slots) slot_in[q] = t;
+      }
   }
 }
 
@@ -233,7 +239,8 @@ __global__ void __launch_bounds__(256) k_slot_inputs(DevArena A, const float* __
 // as in k_reduce_wide).
 __global__ void __launch_bounds__(256) k_slot_inputs_wide(DevArena A, const float* __restrict__ x,
                                                            const float* __restrict__ sd_in, float* out_var,
-                                                           const float* __restrict__ S_var, float2* slot_in) {
+                                                           const float* __restrict__ S_var, float2* var_in,
+                                                      float2* slot_in) {
   constexpr unsigned kAll = 0xffffffffu;
   const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (w >= A.num_wide) return;  // the whole warp
@@ -250,9 +257,14 @@ __global__ void __launch_bounds__(256) k_slot_inputs_wide(DevArena A, const floa
     s = sd_in[i];
   }
   if (out_var && lane == 0) out_var[i] = s;
-  if (slot_in) {
+  if (var_in) {
     const float2 t = make_float2(s, S_var ? S_var[i] : 0.f);
-    for (int k = b + lane; k < e; k += 32) slot_in[__ldg(A.var_slots + k)] = t;
+    if (lane == 0) var_in[i] = t;
+    if (slot_in)
+      for (int k = b + lane; k < e; k += 32) {
+        const int q = __ldg(A.var_slots + k);
+        if (q >= A.unit_slots) slot_in[q] = t;
+      }
   }
 }
 
@@ -277,12 +289,13 @@ __global__ void k_gather_var(DevArena A, const float* __restrict__ v, float* out
 }
 
 void launch_slot_inputs(const DevArena& A, const float* x, const float* sd_in, float* out_var, const float* S_var,
-                        float2* slot_in, cudaStream_t st) {
+                        float2* var_in, float2* slot_in, cudaStream_t st) {
   const int T = 256;
   const int G = (A.n + T - 1) / T;
-  if (G > 0) k_slot_inputs<<<G, T, 0, st>>>(A, x, sd_in, out_var, S_var, slot_in);
+  if (A.unit_slots >= A.num_slots) slot_in = nullptr;  // no slot reads it
+  if (G > 0) k_slot_inputs<<<G, T, 0, st>>>(A, x, sd_in, out_var, S_var, var_in, slot_in);
   if (A.num_wide > 0)
-    k_slot_inputs_wide<<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, x, sd_in, out_var, S_var, slot_in);
+    k_slot_inputs_wide<<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, x, sd_in, out_var, S_var, var_in, slot_in);
 }
 
 void launch_gather_var(const DevArena& A, const float* v, float* out_slot, cudaStream_t st) {
@@ -296,8 +309,8 @@ void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float*
   const int T = 256;
   const int G = (A.n + T - 1) / T;
   if (G == 0) return;
-  const int from = to == Scatter::kAll ? 0 : A.unit_slots;
-  const bool scatter = to != Scatter::kNone && from < A.num_slots;
+  const int from = A.unit_slots;
+  const bool scatter = to == Scatter::kSweep && from < A.num_slots;
   if (renorm)
     scatter ? k_reduce_S<true, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from)
             : k_reduce_S<true, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from);

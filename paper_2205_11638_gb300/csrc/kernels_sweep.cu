@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(128) k_sweep(DevArena A, SweepArgs a, int regi
   // choices of SP(., T) (for a forward sweep) or the in-arcs of SP(r, .)
   // (for a backward one); the rest of each record is rewritten below
   if (REC && cost_in) {
-    copy_async(s.meta + 2 * kWarp, a.meta_in + T.node_base, (s.nmax - 2) * kWarp * 2, lane);
+    copy_async(s.meta + 2 * kWarp, a.meta_in + (T.node_base - A.unit_nodes), (s.nmax - 2) * kWarp * 2, lane);
     cp_async_commit();
     cp_async_wait_all();
     __syncwarp();
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(128) k_sweep(DevArena A, SweepArgs a, int regi
         a.lam[sbase + q] = ln;
         a.M[sbase + q] = Mn;
         if (REC) {
-          a.rec_amin[sbase + q] = (uint16_t)(v0 | (v1 << 8));
+          a.rec_amin[sbase - A.unit_slots + q] = (uint16_t)(v0 | (v1 << 8));
           a.rec_diff[sbase + q] = m1 - m0;
         }
       }
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(128) k_sweep(DevArena A, SweepArgs a, int regi
       a.lam[sbase + q] = ln;
       a.M[sbase + q] = Mn;
       if (REC) {
-        a.rec_amin[sbase + q] = (uint16_t)(v0 | (v1 << 8));
+        a.rec_amin[sbase - A.unit_slots + q] = (uint16_t)(v0 | (v1 << 8));
         a.rec_diff[sbase + q] = m1 - m0;
       }
       #pragma unroll
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(128) k_sweep(DevArena A, SweepArgs a, int regi
     // the records of nodes 2 .. nmax-1, in the layout of the child codes
     __syncwarp();
     const uint32_t* src = reinterpret_cast<const uint32_t*>(s.meta + 2 * kWarp);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(a.rec_meta + T.node_base);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(a.rec_meta + (T.node_base - A.unit_nodes));
     for (int o = lane; o < (s.nmax - 2) * (kWarp / 2); o += kWarp) dst[o] = src[o];
   }
 
@@ -423,7 +423,7 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
     const LaunchGroup& G = groups[g];
     constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
     constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
-    const bool unit = G.unit_w > 0 && !REC;
+    const bool unit = G.unit_w > 0;
     const size_t region = unit ? (size_t)(MODE == 1 ? G.unit_bytes1 : G.unit_bytes0)
                                : (size_t)(BWD ? (MODE == 1 ? G.region_bwd1 : G.region_bwd0)
                                               : (MODE == 1 ? G.region_bytes : G.region_bytes0)) +

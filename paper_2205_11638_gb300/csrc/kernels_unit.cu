@@ -39,12 +39,15 @@ __device__ __forceinline__ void copy_rows(float* dst, const void* src, int k, in
   }
 }
 
-// One tile whose inputs are on their way.  KIND: kFwd, kBwd, kMinMarg,
-// kEnergy, kSeed.
+// One tile whose inputs are on their way.  KIND: kFwd, kBwd, their recording
+// variants kFwdRec and kBwdRec, kMinMarg, kEnergy, kSeed.
 template <int KIND, int MODE, int W>
 __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
                                           float* smem, int lane) {
-  constexpr bool UPDATE = KIND == kFwd || KIND == kBwd;
+  constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
+  constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
+  constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
+  constexpr bool UPDATE = FWD || BWD;
   constexpr int STRIDE = kStride<UPDATE, MODE>;
   const UnitCtx s{S.k, S.start, S.accept, S.nruns, A.unit_runs + S.run_base};
   const int64_t sb = T.slot_base + lane;
@@ -59,53 +62,82 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
     a.E[__ldg(A.slot_row + sb)] = e;
   };
   // the update of a level from its minima; returns lambda^new
-  auto update = [&](const float* x, float* lam, float* M, float b0, float b1) -> float {
+  // where the sweep leaves the level at hand
+  const int64_t first = sb + (BWD ? s.k * kWarp : 0);
+  float* g0 = (KIND == kMinMarg ? a.out2 : a.lam) + first;
+  float* g1 = a.M + first;
+  float* gd = REC ? a.rec_diff + first : nullptr;
+  uint32_t* gr = REC ? a.rec_unit + first : nullptr;
+  auto move = [&](int by) {
+    g0 += by;
+    g1 += by;
+    if (REC) {
+      gd += by;
+      gr += by;
+    }
+  };
+  auto update = [&](const float* x, float b0, float b1) -> float {
     const float l = x[0];
     const float m0 = b0, m1 = l + b1;
     const float Mn = __fmul_rn(MODE == 1 ? x[kOm] : a.omega0, m1 - m0);
     const float ln = unit_lambda_new<MODE>(l, Mn, MODE == 1 ? x[kAl] : 0.0f, x[kAvg]);
     if (real) {
-      *lam = ln;
-      *M = Mn;
+      *g0 = ln;
+      *g1 = Mn;
+      if (REC) *gd = m1 - m0;
     }
     return ln;
   };
 
-  if (KIND == kFwd || KIND == kMinMarg) {
+  if (FWD || KIND == kMinMarg) {
     unit_first_up<W, STRIDE>(s, S.rows, x0, cost, lane);
     if (UPDATE) cp_async_wait_all();  // every lane gathered its own averaging terms
     Costs<W> R = unit_root<W>(s.start);
-    float* g0 = (KIND == kFwd ? a.lam : a.out2) + sb;
-    float* g1 = a.M + sb;
     unit_second_down<W, STRIDE>(s, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& t1) {
       constexpr int TY = decltype(ty)::value;
-      float b0, b1, ln = x[0];
-      unit_minima<W, TY>(R, t1, b0, b1);
-      if (KIND == kMinMarg) {
-        if (real) {
-          *g0 = ln + b1;
-          *g1 = b0;
-        }
+      float b0, b1;
+      const float l = x[0];
+      if (REC) {
+        // the out-arcs under the incoming lambda, the in-arcs under the new one
+        uint32_t rec = 0;
+        unit_minima_rec<W, TY>(R, t1, b0, b1, rec);
+        unit_up_rec<W, TY>(t1, l, rec);
+        R = unit_down_rec<W, TY>(R, update(x, b0, b1), rec);
+        if (real) *gr = rec;
       } else {
-        ln = update(x, g0, g1, b0, b1);
+        unit_minima<W, TY>(R, t1, b0, b1);
+        float ln = l;
+        if (KIND == kMinMarg) {
+          if (real) {
+            *g0 = l + b1;
+            *g1 = b0;
+          }
+        } else {
+          ln = update(x, b0, b1);
+        }
+        R = unit_down<W, TY>(R, ln);
       }
-      g0 += kWarp;
-      g1 += kWarp;
-      R = unit_down<W, TY>(R, ln);
+      move(kWarp);
     });
-  } else if (KIND == kBwd) {
+  } else if (BWD) {
     unit_first_down<W, STRIDE>(s, x0, cost, lane);
     cp_async_wait_all();
     Costs<W> t = unit_end<W>(s.accept);
-    float* g0 = a.lam + sb + s.k * kWarp;
-    float* g1 = a.M + sb + s.k * kWarp;
     unit_second_up<W, STRIDE>(s, S.rows, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& r) {
       constexpr int TY = decltype(ty)::value;
       float b0, b1;
-      unit_minima<W, TY>(r, t, b0, b1);
-      g0 -= kWarp;
-      g1 -= kWarp;
-      t = unit_up<W, TY>(t, update(x, g0, g1, b0, b1));
+      move(-kWarp);
+      if (REC) {
+        // the in-arcs under the incoming lambda, the out-arcs under the new one
+        uint32_t rec = 0;
+        unit_minima_rec<W, TY>(r, t, b0, b1, rec);
+        unit_down_rec<W, TY>(r, x[0], rec);
+        t = unit_up_rec<W, TY>(t, update(x, b0, b1), rec);
+        if (real) *gr = rec;
+      } else {
+        unit_minima<W, TY>(r, t, b0, b1);
+        t = unit_up<W, TY>(t, update(x, b0, b1));
+      }
     });
     if (a.E != nullptr && real) energy(t);
   } else if (KIND == kEnergy) {
@@ -119,7 +151,6 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
     // kSeed: walk the minimising path from the root, the 0-arc on ties
     unit_first_up<W, STRIDE>(s, S.rows, x0, cost, lane);
     int at = s.start;
-    float* g1 = a.M + sb;
     unit_second_down<W, STRIDE>(s, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& t1) {
       constexpr int TY = decltype(ty)::value;
       float c0 = f_inf(), c1 = f_inf();
@@ -147,7 +178,7 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
   if (tile >= tile1) return;  // whole warp leaves; no CTA-wide barrier follows
-  constexpr bool UPDATE = KIND == kFwd || KIND == kBwd;
+  constexpr bool UPDATE = KIND == kFwd || KIND == kBwd || KIND == kFwdRec || KIND == kBwdRec;
   constexpr int STRIDE = kStride<UPDATE, MODE>;
   const Tile T = A.tiles[tile];
   const int k = T.nhops;
@@ -197,6 +228,183 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
     unit_tile<KIND, MODE, 8>(A, a, T, S, m, lane);
 }
 
+// ---- adjoint of a recording sweep (see kernels_adjoint.cu) -----------------
+// Per level and lane, staged: the gradient of lambda, the argmin word, m1 - m0,
+// the averaging weight, {S-dot of the next sweep, S at the sweep's start} of
+// the slot's variable (its id first, as in the sweeps), (mode 1) omega.
+constexpr int kJRec = kWarp, kJDiff = 2 * kWarp, kJAl = 3 * kWarp, kJIn = 4 * kWarp, kJOm = 6 * kWarp;
+
+template <int FWD, int MODE, int W>
+__device__ __forceinline__ void unit_adjoint_tile(const AdjArgs& a, const Tile& T, const UnitCtx& s, float* smem,
+                                                  int lane) {
+  constexpr int STRIDE = kWarp * (MODE == 1 ? 7 : 6);
+  const bool real = lane < T.nbdd;
+  float* x = smem + lane + (FWD ? (s.k - 1) * STRIDE : 0);
+  int64_t q = T.slot_base + lane + (FWD ? (s.k - 1) * kWarp : 0);
+  // the update of a level reversed (g: gradient of lambda^new with the path
+  // costs' share); returns the gradient d of m1 (that of m0 is -d).  The
+  // running parameter gradients are read one level ahead.
+  const bool want_a = a.g_alpha != nullptr, want_w = a.g_omega != nullptr;
+  float ga = want_a && real ? a.g_alpha[q] : 0.0f, gw = want_w && real ? a.g_omega[q] : 0.0f;
+  int left = s.k;
+  auto reverse = [&](float* y, float g) -> float {
+    const int64_t at = q;
+    const float ca = ga, cw = gw;
+    q += FWD ? -kWarp : kWarp;
+    if (--left > 0) {
+      if (want_a && real) ga = a.g_alpha[q];
+      if (want_w && real) gw = a.g_omega[q];
+    }
+    const float2 in = *reinterpret_cast<const float2*>(y - lane + kJIn + 2 * lane);
+    const float seed = a.seed_M && real ? a.seed_M[at] : 0.0f;
+    const float Mt = seed + in.x - g;
+    const float d = (MODE == 1 ? y[kJOm] : a.omega0) * Mt;
+    if (real) {
+      a.sdot[at] = y[kJAl] * g;
+      if (want_a) a.g_alpha[at] = ca + g * in.y;
+      if (want_w) a.g_omega[at] = cw + Mt * y[kJDiff];
+    }
+    y[0] = g + d;
+    y[kJDiff] = d;
+    return d;
+  };
+  Costs<W> G;
+#pragma unroll
+  for (int u = 0; u < W; ++u) G.v[u] = 0.0f;
+  if (FWD) {
+    // SP(r, .) of level h + 1 was relaxed from level h with lambda^new_h
+    unit_runs_up(s, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int n = e - b; n > 0; --n) {
+        const uint32_t rec = __float_as_uint(x[kJRec]);
+        float g = x[0];
+        G = unit_route_in<W, TY>(G, rec, g);
+        unit_seed_in<W>(G, rec, reverse(x, g));
+        x -= STRIDE;
+      }
+    });
+    // SP(., T) under lambda^old: its gradient flows top-down
+    x += STRIDE;
+#pragma unroll
+    for (int u = 0; u < W; ++u) G.v[u] = 0.0f;
+    unit_runs_down(s, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int n = e - b; n > 0; --n) {
+        const uint32_t rec = __float_as_uint(x[kJRec]);
+        float g = x[0];
+        Costs<W> N;
+#pragma unroll
+        for (int u = 0; u < W; ++u) N.v[u] = 0.0f;
+        unit_seed_out<W, TY>(N, rec, x[kJDiff]);
+        unit_route_out<W, TY>(G, rec, N, g);
+        G = N;
+        x[0] = g;
+        x += STRIDE;
+      }
+    });
+  } else {
+    // SP(., T) of level h was recomputed with lambda^new_h
+    unit_runs_down(s, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int n = e - b; n > 0; --n) {
+        const uint32_t rec = __float_as_uint(x[kJRec]);
+        float g = x[0];
+        Costs<W> N;
+#pragma unroll
+        for (int u = 0; u < W; ++u) N.v[u] = 0.0f;
+        unit_route_out<W, TY>(G, rec, N, g);
+        unit_seed_out<W, TY>(N, rec, reverse(x, g));
+        G = N;
+        x += STRIDE;
+      }
+    });
+    // SP(r, .) under lambda^old: its gradient flows bottom-up
+    x -= STRIDE;
+#pragma unroll
+    for (int u = 0; u < W; ++u) G.v[u] = 0.0f;
+    unit_runs_up(s, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int n = e - b; n > 0; --n) {
+        const uint32_t rec = __float_as_uint(x[kJRec]);
+        float g = x[0];
+        G = unit_route_in<W, TY>(G, rec, g);
+        unit_seed_in<W>(G, rec, x[kJDiff]);
+        x[0] = g;
+        x -= STRIDE;
+      }
+    });
+  }
+  float* out = a.g_lam + T.slot_base + lane;
+  x = smem + lane;
+  if (real)
+    for (int h = 0; h < s.k; ++h) out[h * kWarp] = x[h * STRIDE];
+}
+
+template <int FWD, int MODE, int WMAX>
+__global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int region_bytes, int tile0, int tile1) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int STRIDE = kWarp * (MODE == 1 ? 7 : 6);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
+  if (tile >= tile1) return;  // whole warp leaves; no CTA-wide barrier follows
+  const Tile T = A.tiles[tile];
+  const int k = T.nhops;
+  float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
+  const uint64_t pol = l2_evict_first();
+  copy_rows<STRIDE>(m + kJIn, A.slot_var + T.slot_base, k, lane, pol);
+  cp_async_commit();
+  copy_rows<STRIDE>(m, a.g_lam + T.slot_base, k, lane, pol);
+  copy_rows<STRIDE>(m + kJRec, a.rec_unit + T.slot_base, k, lane, pol);
+  copy_rows<STRIDE>(m + kJDiff, a.rec_diff + T.slot_base, k, lane, pol);
+  copy_rows<STRIDE>(m + kJAl, (MODE == 1 ? a.alpha : A.slot_invdeg) + T.slot_base, k, lane, pol);
+  if (MODE == 1) copy_rows<STRIDE>(m + kJOm, a.omega + T.slot_base, k, lane, pol);
+  cp_async_commit();
+  const UnitShape S = A.unit_shapes[T.unit - 1];
+  cp_async_wait_one();
+  __syncwarp();
+  for (int h = 0; h < k; ++h) {
+    // the pairs replace the ids: every lane reads its id before any is overwritten
+    float* in = m + h * STRIDE + kJIn;
+    const int v = __float_as_int(in[lane]);
+    __syncwarp();
+    if (v >= 0) cp_async8(in + 2 * lane, a.var_in + v);
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncwarp();
+  const UnitCtx s{S.k, S.start, S.accept, S.nruns, A.unit_runs + S.run_base};
+  if (S.W == 2)
+    unit_adjoint_tile<FWD, MODE, 2>(a, T, s, m, lane);
+  else if (WMAX >= 4 && S.W == 4)
+    unit_adjoint_tile<FWD, MODE, 4>(a, T, s, m, lane);
+  else if (WMAX >= 8 && S.W == 6)
+    unit_adjoint_tile<FWD, MODE, 6>(a, T, s, m, lane);
+  else if (WMAX >= 8)
+    unit_adjoint_tile<FWD, MODE, 8>(a, T, s, m, lane);
+}
+
+template <int FWD, int MODE>
+void launch_adjoint_group(const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
+                          cudaStream_t st) {
+  const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc, r = (int)region;
+  if (G.unit_w <= 2)
+    k_unit_adjoint<FWD, MODE, 2><<<grid, wpc * kWarp, region * wpc, st>>>(A, a, r, G.tile0, G.tile1);
+  else if (G.unit_w <= 4)
+    k_unit_adjoint<FWD, MODE, 4><<<grid, wpc * kWarp, region * wpc, st>>>(A, a, r, G.tile0, G.tile1);
+  else
+    k_unit_adjoint<FWD, MODE, 8><<<grid, wpc * kWarp, region * wpc, st>>>(A, a, r, G.tile0, G.tile1);
+}
+
+template <int FWD, int MODE>
+cudaError_t set_adjoint_attr(int b) {
+  cudaError_t e = cudaFuncSetAttribute(k_unit_adjoint<FWD, MODE, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_unit_adjoint<FWD, MODE, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_unit_adjoint<FWD, MODE, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  return e;
+}
+
 template <int KIND, int MODE, int WMAX>
 void launch_w(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, cudaStream_t st) {
   const int nt = G.tile1 - G.tile0;
@@ -230,6 +438,14 @@ cudaError_t set_unit_smem_limit(size_t bytes) {
   if (e == cudaSuccess) e = set_attr<kFwd, 1>(b);
   if (e == cudaSuccess) e = set_attr<kBwd, 0>(b);
   if (e == cudaSuccess) e = set_attr<kBwd, 1>(b);
+  if (e == cudaSuccess) e = set_attr<kFwdRec, 0>(b);
+  if (e == cudaSuccess) e = set_attr<kFwdRec, 1>(b);
+  if (e == cudaSuccess) e = set_attr<kBwdRec, 0>(b);
+  if (e == cudaSuccess) e = set_attr<kBwdRec, 1>(b);
+  if (e == cudaSuccess) e = set_adjoint_attr<1, 0>(b);
+  if (e == cudaSuccess) e = set_adjoint_attr<1, 1>(b);
+  if (e == cudaSuccess) e = set_adjoint_attr<0, 0>(b);
+  if (e == cudaSuccess) e = set_adjoint_attr<0, 1>(b);
   if (e == cudaSuccess) e = set_attr<kMinMarg, 0>(b);
   if (e == cudaSuccess) e = set_attr<kEnergy, 0>(b);
   if (e == cudaSuccess) e = set_attr<kSeed, 0>(b);
@@ -242,10 +458,26 @@ void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGr
   switch (kind) {
     case kFwd: m1 ? launch_group<kFwd, 1>(A, a, G, wpc, region, st) : launch_group<kFwd, 0>(A, a, G, wpc, region, st); break;
     case kBwd: m1 ? launch_group<kBwd, 1>(A, a, G, wpc, region, st) : launch_group<kBwd, 0>(A, a, G, wpc, region, st); break;
+    case kFwdRec:
+      m1 ? launch_group<kFwdRec, 1>(A, a, G, wpc, region, st) : launch_group<kFwdRec, 0>(A, a, G, wpc, region, st);
+      break;
+    case kBwdRec:
+      m1 ? launch_group<kBwdRec, 1>(A, a, G, wpc, region, st) : launch_group<kBwdRec, 0>(A, a, G, wpc, region, st);
+      break;
     case kMinMarg: launch_group<kMinMarg, 0>(A, a, G, wpc, region, st); break;
     case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, st); break;
     default: launch_group<kSeed, 0>(A, a, G, wpc, region, st); break;
   }
+}
+
+void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
+                         cudaStream_t st) {
+  if (forward)
+    a.mode == 1 ? launch_adjoint_group<1, 1>(A, a, G, wpc, region, st)
+                : launch_adjoint_group<1, 0>(A, a, G, wpc, region, st);
+  else
+    a.mode == 1 ? launch_adjoint_group<0, 1>(A, a, G, wpc, region, st)
+                : launch_adjoint_group<0, 0>(A, a, G, wpc, region, st);
 }
 
 }  // namespace dg

@@ -86,6 +86,155 @@ __device__ __forceinline__ void unit_minima(const Costs<W>& R, const Costs<W>& T
   b1 = x1[0];
 }
 
+// Argmin records of one level of a recording sweep, one 32-bit word per slot:
+//   bits 0..7    SP(state u, T) leaves u by its 1-arc
+//   bits 8..16   in-arc of SP(r, w) on the next level: two bits for w = 0, one
+//                for each other state, the index of the candidate in
+//                unit_in_arc's order
+//   bits 17..19  argmin state of m0, bits 20..22 of m1
+// The candidates of a state are ordered as the tie rule wants them, by (parent
+// rank, beta); ranks descend in the state number.
+constexpr int kRecIn = 8, kRecV0 = 17, kRecV1 = 20;
+__device__ __forceinline__ constexpr int unit_in_shift(int w) { return kRecIn + (w == 0 ? 0 : w + 1); }
+
+// Calls f(candidate index, parent state, beta) for the arcs into state w.
+template <int W, int TYPE, class F>
+__device__ __forceinline__ void unit_in_arcs(int w, F&& f) {
+  if (TYPE == kUp) {
+    f(0, w, 0);
+    if (w > 0) f(1, w - 1, 1);
+  } else if (TYPE == kSwap) {
+    if (w + 1 < W) f(0, w + 1, 0);
+    f(1, w, w == 0 ? 0 : 1);
+    if (w == 0) f(2, 0, 1);
+  } else {
+    if (w + 1 < W) f(0, w + 1, 1);
+    f(1, w, 0);
+    if (TYPE == kDown && w == 0) f(2, 0, 1);
+  }
+}
+
+// unit_down that also records the in-arcs (the first strictly smallest
+// candidate).
+template <int W, int TYPE>
+__device__ __forceinline__ Costs<W> unit_down_rec(const Costs<W>& R, float l, uint32_t& rec) {
+  Costs<W> r;
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    float b = f_inf();
+    uint32_t c = 0;
+    unit_in_arcs<W, TYPE>(w, [&](int i, int u, int beta) {
+      const float x = beta ? R.v[u] + l : R.v[u];
+      if (x < b) {
+        b = x;
+        c = (uint32_t)i << unit_in_shift(w);
+      }
+    });
+    r.v[w] = b;
+    rec |= c;
+  }
+  return r;
+}
+
+// unit_up that also records the out-arcs (the 0-arc on ties).
+template <int W, int TYPE>
+__device__ __forceinline__ Costs<W> unit_up_rec(const Costs<W>& T, float l, uint32_t& rec) {
+  Costs<W> r;
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
+    const int o = unit_o<TYPE>(u);
+    const float tl = T.at(unit_z<TYPE>(u));
+    const float th = o >= 0 && o < W ? l + T.at(o) : f_inf();
+    const bool take0 = tl <= th;
+    r.v[u] = take0 ? tl : th;
+    rec |= take0 ? 0u : 1u << u;
+  }
+  return r;
+}
+
+// unit_minima that also records the argmin states (the largest on ties).
+template <int W, int TYPE>
+__device__ __forceinline__ void unit_minima_rec(const Costs<W>& R, const Costs<W>& T, float& b0, float& b1,
+                                                uint32_t& rec) {
+  b0 = b1 = f_inf();
+  uint32_t v0 = 0, v1 = 0;
+#pragma unroll
+  for (int u = W - 1; u >= 0; --u) {
+    const int o = unit_o<TYPE>(u);
+    const float x0 = R.v[u] + T.at(unit_z<TYPE>(u));
+    if (x0 < b0) {
+      b0 = x0;
+      v0 = u;
+    }
+    if (o >= 0 && o < W) {
+      const float x1 = R.v[u] + T.at(o);
+      if (x1 < b1) {
+        b1 = x1;
+        v1 = u;
+      }
+    }
+  }
+  rec |= v0 << kRecV0 | v1 << kRecV1;
+}
+
+// Gradients G of SP(r, .) on the next level to the parents' level along the
+// recorded in-arcs; g receives those that entered by a 1-arc.
+template <int W, int TYPE>
+__device__ __forceinline__ Costs<W> unit_route_in(const Costs<W>& G, uint32_t rec, float& g) {
+  Costs<W> r;
+#pragma unroll
+  for (int u = 0; u < W; ++u) r.v[u] = 0.0f;
+#pragma unroll
+  for (int w = W - 1; w >= 0; --w) {
+    const uint32_t c = rec >> unit_in_shift(w) & (w == 0 ? 3u : 1u);
+    unit_in_arcs<W, TYPE>(w, [&](int i, int u, int beta) {
+      const float x = c == (uint32_t)i ? G.v[w] : 0.0f;
+      r.v[u] += x;
+      if (beta) g += x;
+    });
+  }
+  return r;
+}
+
+// Gradients G of SP(., T) of a level to the children's level (added to r)
+// along the recorded out-arcs; g receives those that left by a 1-arc.
+template <int W, int TYPE>
+__device__ __forceinline__ void unit_route_out(const Costs<W>& G, uint32_t rec, Costs<W>& r, float& g) {
+#pragma unroll
+  for (int u = W - 1; u >= 0; --u) {
+    const bool hi = (rec >> u) & 1u;
+    const int z = unit_z<TYPE>(u), o = unit_o<TYPE>(u);
+    r.v[z] += hi ? 0.0f : G.v[u];
+    if (o >= 0 && o < W) {
+      const float x = hi ? G.v[u] : 0.0f;
+      r.v[o] += x;
+      g += x;
+    }
+  }
+}
+
+// The gradients of the min-marginals (m1: d, m0: -d) at the argmin states:
+// SP(r, .) of the level, SP(., T) of the children's level.
+template <int W>
+__device__ __forceinline__ void unit_seed_in(Costs<W>& r, uint32_t rec, float d) {
+  const int v0 = (rec >> kRecV0) & 7u, v1 = (rec >> kRecV1) & 7u;
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
+    if (v0 == u) r.v[u] -= d;
+    if (v1 == u) r.v[u] += d;
+  }
+}
+template <int W, int TYPE>
+__device__ __forceinline__ void unit_seed_out(Costs<W>& r, uint32_t rec, float d) {
+  const int v0 = (rec >> kRecV0) & 7u, v1 = (rec >> kRecV1) & 7u;
+#pragma unroll
+  for (int u = 0; u < W; ++u) {
+    const int o = unit_o<TYPE>(u);
+    if (v0 == u) r.v[unit_z<TYPE>(u)] -= d;
+    if (o >= 0 && o < W && v1 == u) r.v[o] += d;
+  }
+}
+
 // The costs of a level in the warp's shared memory: 32 W floats per level,
 // in pieces of four (or two) states per lane, so that a lane moves them with
 // 16- (8-) byte accesses free of bank conflicts.
@@ -308,6 +457,10 @@ __device__ __forceinline__ float unit_lambda_new(float l, float Mn, float al, fl
 __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 

@@ -111,3 +111,33 @@ def test_marginals_energies_and_minimisers_equal_the_mixed_tiles(name):
             out.append([X.to_csr(m0), X.to_csr(m1), lb, E, X.to_csr(gl), X.to_csr(gM)])
         for a, b in zip(*out):
             assert torch.equal(a, b) and torch.isfinite(a).all()
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("tied", [False, True])
+def test_gradients_equal_the_mixed_tiles(name, mode, tied):
+    """Recording sweeps and adjoint: the same argmins (many equal path costs
+    when tied), so the gradients differ by the rounding of sums alone: at most
+    64 roundings per sweep on the way of a value, 6 sweeps, 2^-24 each, against
+    the largest gradient."""
+    p, A, B = _pair(name)
+    v = _vectors(p, 10)
+    lam0 = torch.round(v[0]) if tied else v[0]
+    g = [torch.as_tensor(np.random.default_rng(s).normal(size=len(p["col"])), dtype=torch.float32) for s in (1, 2)]
+    for iters, every in ((1, 1), (3, 2)):
+        out = []
+        for X in (A, B):
+            lam, M, om, al = [X.from_csr(x) for x in (lam0, *v[1:])]
+            gl, gM = [X.from_csr(x) for x in g]
+            res = X.backward(lam, M, om if mode else None, al if mode else None, iters, every, gl, gM)
+            w, _ = X.iterate_checkpointed(lam, M, om if mode else None, al if mode else None, iters, every)
+            res2 = X.backward_checkpointed(om if mode else None, al if mode else None, iters, every, gl, gM, w)
+            for a, b in zip(res, res2):
+                assert torch.equal(X.to_csr(a), X.to_csr(b))
+            out.append([X.to_csr(t) for t in (*res, lam, M)])
+        for a, b in zip(out[0][:4], out[1][:4]):
+            assert torch.isfinite(a).all()
+            assert (a - b).abs().max() <= 64 * 6 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
+        for a, b in zip(out[0][4:], out[1][4:]):
+            assert torch.equal(a, b)
