@@ -314,6 +314,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   cp(P.off.long_in_ptr, P.long_in_ptr.data(), P.long_in_ptr.size() * 4);
   cp(P.off.long_in, P.long_in.data(), P.long_in.size() * 4);
   cp(P.off.long_order, P.long_order.data(), P.long_order.size() * 4);
+  cp(P.off.long_items, P.long_items.data(), P.long_items.size() * sizeof(LongItem));
   cudaError_t e = cudaMemcpyAsync(arena_dev, h.data(), image, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync((char*)arena_dev + P.off.S, 0, P.off.total - P.off.S, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -323,9 +324,11 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
     cudaGetDevice(&dev);
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return cuda_fail(e, "dg_bind: device attribute");
-    if ((size_t)optin < P.smem_sweep) return fail(DG_EINVAL, "dg_bind: tiles need more shared memory than a CTA has");
+    if ((size_t)optin < std::max<size_t>(P.smem_sweep, (size_t)std::max(P.long_unit_smem[1], P.long_unit_adj_smem)))
+      return fail(DG_EINVAL, "dg_bind: tiles need more shared memory than a CTA has");
     e = set_sweep_smem_limit((size_t)optin);  // same limit for every arena of the process
     if (e == cudaSuccess) e = set_unit_smem_limit((size_t)optin);
+    if (e == cudaSuccess) e = set_long_unit_smem_limit((size_t)optin);
     if (e == cudaSuccess) e = set_adjoint_smem_limit((size_t)optin);
     set_cta_smem_cap((size_t)optin);
     if (e != cudaSuccess) return cuda_fail(e, "dg_bind: shared-memory limit");
@@ -398,18 +401,24 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.long_cost_size = P.long_cost_size;
   A.long_stream = P.long_stream;
   A.num_long_narrow = P.num_long_narrow;
+  A.num_long_unit = P.num_long_unit;
+  A.long_items = (const LongItem*)(b + P.off.long_items);
+  A.num_long_items = (int32_t)P.long_items.size();
+  for (int mode = 0; mode < 2; ++mode) A.long_unit_smem[mode] = P.long_unit_smem[mode];
+  A.long_unit_adj_smem = P.long_unit_adj_smem;
   {
     // lanes per narrow long BDD: the widest level's power of two (or the
     // option's, if larger); by default doubled (fewer BDDs per warp) while
     // that leaves fewer than four warps per SM
     int G = 1, maxw = 1, sms = 1;
-    for (int32_t i = 0; i < P.num_long_narrow; ++i) maxw = std::max(maxw, P.longs[P.long_order[i]].maxw);
+    for (int32_t i = P.num_long_unit; i < P.num_long_narrow; ++i) maxw = std::max(maxw, P.longs[P.long_order[i]].maxw);
     while (G < maxw) G <<= 1;
     if (P.long_lanes > 0) {
       G = std::max(G, (int)P.long_lanes);
     } else {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ar->device);
-      while (G < kWarp && (int64_t)(P.num_long_narrow + kWarp / G - 1) / (kWarp / G) < 4LL * sms) G <<= 1;
+      const int64_t packed = P.num_long_narrow - P.num_long_unit;
+      while (G < kWarp && (packed + kWarp / G - 1) / (kWarp / G) < 4LL * sms) G <<= 1;
     }
     A.long_lanes = G;
   }
@@ -800,10 +809,11 @@ namespace {
 
 struct BwdLayout {
   size_t ck_lam, ck_M, rec_meta, rec_amin, rec_unit, rec_diff, seg_S, w_lam, w_M, sdot, sd_a, sd_b, var_in, slot_in, rec_lmeta,
-      rec_lamin, long_a1, long_a2, total;
+      rec_lamin, rec_lunit, long_a1, long_a2, total;
   size_t meta_stride;   // bytes of one sweep's node records
   size_t lmeta_stride;  // ... of the long BDDs' node records
   size_t lamin_stride;  // ... of the long BDDs' slot records
+  size_t lunit_stride;  // ... of the long unit BDDs' level records
   int nseg, k;
 };
 
@@ -845,6 +855,9 @@ BwdLayout backward_layout(const dg_arena* ar, int iters, int ckpt_every) {
   L.lamin_stride = lslots * 8;
   L.rec_lmeta = put((size_t)2 * L.k * L.lmeta_stride);
   L.rec_lamin = put((size_t)2 * L.k * L.lamin_stride);
+  // ... of the long unit BDDs four words per long slot (none without them)
+  L.lunit_stride = ar->dev.num_long_unit > 0 ? lslots * 16 : 0;
+  L.rec_lunit = put((size_t)2 * L.k * L.lunit_stride);
   L.long_a1 = put(lcost * 4);
   L.long_a2 = put(lcost * 4);
   L.total = o;
@@ -882,6 +895,7 @@ dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, fl
     ra.rec_diff = (float*)(w + L.rec_diff) + (size_t)sw * NS;
     ra.rec_lmeta = (int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
     ra.rec_lamin = (int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
+    ra.rec_lunit = (uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
     // each recording sweep hands its path costs (and records) to the next
     ra.cost_out = A.nodecost;
     if (sw > 0) {
@@ -1043,6 +1057,8 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       ra.rec_diff = rec_diff + (size_t)sw * NS;
       ra.rec_lmeta = (int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
       ra.rec_lamin = (int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
+      ra.rec_lunit = (uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
+    ra.rec_lunit = (uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
       ra.cost_out = A.nodecost;  // handed on from recording sweep to recording sweep
       if (sw > 0) {
         ra.cost_in = A.nodecost;
@@ -1064,6 +1080,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       aa.rec_diff = rec_diff + (size_t)sw * NS;
       aa.rec_lmeta = (const int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
       aa.rec_lamin = (const int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
+      aa.rec_lunit = (const uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
       aa.S_in = seg_S + (size_t)sw * n;
       aa.seed_M = gsw == last_sweep ? g_M_T : nullptr;
       aa.sdot_next = gsw == last_sweep ? nullptr : sd_next;

@@ -166,7 +166,7 @@ inline int unit_o(int t, int u) {
 // row (see UnitShape) whose states are the nodes of its canonical BDD
 // (level_keys, k levels).  Every arc of the BDD is compared with the shape.
 bool unit_candidate(const int8_t* a, int k, bool eq, int64_t rhs, const std::vector<std::vector<uint64_t>>& level_keys,
-                    UnitRow& out) {
+                    int max_w, UnitRow& out) {
   // sums from which every completion is feasible act like clamp[g] ('<='),
   // those outside the alive range like the bottom
   std::vector<int64_t> pos(k + 1, 0), neg(k + 1, 0);
@@ -194,14 +194,15 @@ bool unit_candidate(const int8_t* a, int k, bool eq, int64_t rhs, const std::vec
   int64_t W = 1;
   for (int g = 0; g < k; ++g) W = std::max(W, hi[g] - base[g] + 1);
   W = std::max(W, hi[k] - base[k] + 1);
-  if (W > kUnitMaxW) return false;
+  if (W > max_w) return false;
   UnitShape& s = out.s;
-  s.W = (int32_t)((W + 1) / 2 * 2);
+  s.W = 2;
+  while (s.W < W) s.W += max_w > kUnitMaxW ? s.W : 2;  // the long rows' windows are powers of two
   s.k = k;
   s.start = (int32_t)(l[0] - base[0]);
   s.accept = 0;
   for (int u = 0; u < s.W; ++u)
-    if (eq ? base[k] + u == rhs : base[k] + u <= rhs) s.accept |= 1 << u;
+    if (eq ? base[k] + u == rhs : base[k] + u <= rhs) s.accept = (int32_t)((uint32_t)s.accept | 1u << u);
   out.type.assign(k, 0);
   for (int h = 0; h < k; ++h) {
     const int64_t shift = base[h + 1] - base[h];
@@ -251,16 +252,16 @@ bool unit_candidate(const int8_t* a, int k, bool eq, int64_t rhs, const std::vec
 }
 
 bool unit_row(const int32_t* a, int k, int sense, int64_t rhs, const std::vector<std::vector<uint64_t>>& level_keys,
-              UnitRow& out) {
+              int max_w, UnitRow& out) {
   std::vector<int8_t> sign(k);
   for (int h = 0; h < k; ++h) {
     if (a[h] != 1 && a[h] != -1) return false;
     sign[h] = (int8_t)(sense == 1 ? -a[h] : a[h]);
   }
-  if (sense != 2) return unit_candidate(sign.data(), k, false, sense == 1 ? -rhs : rhs, level_keys, out);
-  if (unit_candidate(sign.data(), k, true, rhs, level_keys, out)) return true;
+  if (sense != 2) return unit_candidate(sign.data(), k, false, sense == 1 ? -rhs : rhs, level_keys, max_w, out);
+  if (unit_candidate(sign.data(), k, true, rhs, level_keys, max_w, out)) return true;
   for (int h = 0; h < k; ++h) sign[h] = (int8_t)-sign[h];
-  return unit_candidate(sign.data(), k, true, -rhs, level_keys, out);
+  return unit_candidate(sign.data(), k, true, -rhs, level_keys, max_w, out);
 }
 
 // A row's BDD as the builder keeps it for later rows with the same terms.
@@ -378,8 +379,10 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
         built.maxw = sc.maxw;
         built.unit = -1;
         UnitRow u;
-        if (sc.nodes <= kMaxNodesPerBdd && sc.maxw <= kUnitMaxW &&
-            unit_row(R->coef + b, k, R->sense[j], R->rhs[j], built.level_keys, u)) {
+        const bool tile = sc.nodes <= kMaxNodesPerBdd && sc.maxw <= kMaxWidth;
+        const int max_w = tile ? kUnitMaxW : kLongUnitMaxW;
+        if (sc.maxw <= max_w && (tile || k <= kLongUnitMaxK) &&
+            unit_row(R->coef + b, k, R->sense[j], R->rhs[j], built.level_keys, max_w, u)) {
           std::string uk((const char*)&u.s, sizeof(UnitShape));
           uk.append((const char*)u.type.data(), u.type.size());
           auto at = unit_index.emplace(uk, (int)pt.units.size());
@@ -835,8 +838,62 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     P.long_order.clear();
     for (size_t b = 0; b < P.longs.size(); ++b)
       if (P.longs[b].maxw <= kWarp) P.long_order.push_back((int32_t)b);
-    std::stable_sort(P.long_order.begin(), P.long_order.end(),
-                     [&](int32_t x, int32_t y) { return P.longs[x].k > P.longs[y].k; });
+    // ... the unit ones by kind before the others
+    std::unordered_map<std::string, int> kind_index;
+    std::vector<int> kind(P.longs.size(), INT32_MAX);
+    for (int32_t b : P.long_order) {
+      const int u = unit_of_row[P.longs[b].row];
+      if (u < 0) continue;
+      const UnitRow& U = units[u];
+      const bool one = std::count(U.type.begin(), U.type.end(), U.type[0]) == (std::ptrdiff_t)U.type.size();
+      std::string uk((const char*)&U.s.W, 4);
+      uk.append((const char*)&U.s.start, 4);
+      uk.append((const char*)&U.s.accept, 4);
+      uk.append((const char*)U.type.data(), one ? 1 : U.type.size());
+      kind[b] = kind_index.emplace(uk, (int)kind_index.size()).first->second;
+    }
+    std::stable_sort(P.long_order.begin(), P.long_order.end(), [&](int32_t x, int32_t y) {
+      return kind[x] != kind[y] ? kind[x] < kind[y] : P.longs[x].k > P.longs[y].k;
+    });
+    P.num_long_unit = 0;
+    for (int32_t b : P.long_order) P.num_long_unit += kind[b] != INT32_MAX;
+    P.long_items.clear();
+    for (int32_t i = 0; i < P.num_long_unit;) {
+      const int k0 = kind[P.long_order[i]];
+      int32_t e = i;
+      while (e < P.num_long_unit && kind[P.long_order[e]] == k0) ++e;
+      const UnitRow& U = units[unit_of_row[P.longs[P.long_order[i]].row]];
+      const int G = U.s.W, kmax = P.longs[P.long_order[i]].k;
+      // BDDs per warp: as many as lanes allow while that leaves at least four
+      // warps per SM (a warp's levels are a chain of dependent steps, which
+      // other warps hide), and as fit shared memory
+      int nseg = kWarp / G;
+      while (nseg > 1 && ((int64_t)(e - i) < 4LL * 152 * nseg || long_unit_bytes(nseg, G, kmax, 1) > 64 * 1024 ||
+                          long_unit_adjoint_bytes(nseg, kmax) > 64 * 1024))
+        nseg /= 2;
+      const int32_t run_base = (int32_t)P.unit_runs.size();
+      for (int h = 0; h < U.s.k; ++h)
+        if (h + 1 == U.s.k || U.type[h + 1] != U.type[h]) P.unit_runs.push_back((uint16_t)((h + 1) << 2 | U.type[h]));
+      for (int32_t x = i; x < e; x += nseg) {
+        LongItem it{};
+        it.first = x;
+        it.nseg = std::min(nseg, e - x);
+        it.G = G;
+        it.kmax = P.longs[P.long_order[x]].k;
+        it.start = U.s.start;
+        it.accept = (uint32_t)U.s.accept;
+        it.run_base = run_base;
+        it.nruns = (int32_t)P.unit_runs.size() - run_base;
+        P.long_items.push_back(it);
+        for (int mode = 0; mode < 2; ++mode)
+          P.long_unit_smem[mode] = std::max<int32_t>(P.long_unit_smem[mode], (int32_t)long_unit_bytes(it.nseg, G, it.kmax, mode));
+        P.long_unit_adj_smem = std::max<int32_t>(P.long_unit_adj_smem, (int32_t)long_unit_adjoint_bytes(it.nseg, it.kmax));
+      }
+      i = e;
+    }
+    // the longest items first
+    std::stable_sort(P.long_items.begin(), P.long_items.end(),
+                     [](const LongItem& x, const LongItem& y) { return x.kmax > y.kmax; });
     P.num_long_narrow = (int32_t)P.long_order.size();
     P.long_lanes = opts ? opts->long_lanes : 0;
     for (size_t b = 0; b < P.longs.size(); ++b)
@@ -922,6 +979,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
   P.off.long_in_ptr = put(P.long_in_ptr.size() * 4);
   P.off.long_in = put(P.long_in.size() * 4);
   P.off.long_order = put(P.long_order.size() * 4);
+  P.off.long_items = put(P.long_items.size() * sizeof(LongItem));
   P.off.S = put((size_t)n * 4);
   P.off.Sbar = put((size_t)n * 4);
   P.off.slot_avg = put((size_t)num_slots * 4);
@@ -1145,6 +1203,55 @@ dg_status validate_plan(const Plan& P) {
       return bad("long BDD order malformed");
     if (P.long_lanes < 0 || P.long_lanes > kWarp || (P.long_lanes & (P.long_lanes - 1)) != 0)
       return bad("lanes per narrow long BDD not a power of two up to 32");
+    // the unit ones: every item's BDDs have its shape, state for node
+    if (P.num_long_unit < 0 || P.num_long_unit > P.num_long_narrow) return bad("long unit BDDs not narrow");
+    std::vector<char> in_item(P.num_long_unit, 0);
+    for (const LongItem& it : P.long_items) {
+      if (it.G < 2 || it.G > kLongUnitMaxW || (it.G & (it.G - 1)) != 0 || it.nseg < 1 || it.nseg * it.G > kWarp ||
+          it.first < 0 || it.first + it.nseg > P.num_long_unit || it.start < 0 || it.start >= it.G || it.nruns < 1 ||
+          it.run_base < 0 || (size_t)it.run_base + (size_t)it.nruns > P.unit_runs.size() ||
+          long_unit_bytes(it.nseg, it.G, it.kmax, 0) > (size_t)P.long_unit_smem[0] ||
+          long_unit_bytes(it.nseg, it.G, it.kmax, 1) > (size_t)P.long_unit_smem[1] ||
+          long_unit_adjoint_bytes(it.nseg, it.kmax) > (size_t)P.long_unit_adj_smem)
+        return bad("long unit item out of range");
+      for (int x = it.first; x < it.first + it.nseg; ++x) {
+        const LongBdd& L = P.longs[P.long_order[x]];
+        if (in_item[x]++ || L.k > it.kmax) return bad("long unit item lists a BDD twice or too long a one");
+        const int32_t* lvl = P.long_lvl.data() + L.lvl_base;
+        std::vector<int> state(1, it.start), next;
+        const uint16_t* run = &P.unit_runs[it.run_base];
+        int left = it.nruns;
+        for (int h = 0; h < L.k; ++h) {
+          if (left > 1 && h >= (*run >> 2)) {
+            ++run;
+            --left;
+          }
+          next.assign(h + 1 < L.k ? lvl[h + 2] - lvl[h + 1] : 0, -1);
+          for (int v = lvl[h]; v < lvl[h + 1]; ++v) {
+            const int u = state[v - lvl[h]];
+            if (u < 0 || (v > lvl[h] && u >= state[v - lvl[h] - 1])) return bad("long unit states not descending");
+            const int2 cc = P.long_code[L.code_base + v - 2];
+            for (int beta = 0; beta < 2; ++beta) {
+              const int c = beta ? cc.y : cc.x;
+              if (c == (int)kBotCode) continue;
+              const int to = beta ? unit_o(*run & 3, u) : unit_z(*run & 3, u);
+              if (to < 0 || to >= it.G) return bad("long unit state outside the window");
+              if (c == (int)kTopCode) {
+                if (!((it.accept >> to) & 1)) return bad("long unit state not accepted");
+              } else if (next[c - lvl[h + 1]] >= 0 && next[c - lvl[h + 1]] != to) {
+                return bad("long unit states of a node differ");
+              } else {
+                next[c - lvl[h + 1]] = to;
+              }
+            }
+          }
+          state.swap(next);
+        }
+        if (left > 1) return bad("long unit item's BDD shorter than its runs");
+      }
+    }
+    for (char c : in_item)
+      if (!c) return bad("long unit BDD in no item");
     std::vector<char> listed(P.longs.size(), 0);
     for (size_t i = 0; i < P.long_order.size(); ++i) {
       const int32_t b = P.long_order[i];

@@ -11,6 +11,12 @@
 
 #include "dg.h"
 
+#ifdef __CUDACC__
+#define DG_HD __host__ __device__
+#else
+#define DG_HD
+#endif
+
 namespace dg {
 
 // Node numbers inside a BDD: 0 is the top terminal, 1 the bottom terminal,
@@ -116,6 +122,39 @@ struct LongBdd {
 };
 static_assert(sizeof(LongBdd) == 32, "LongBdd is 32 bytes");
 
+// Long unit rows (see UnitShape; up to 32 states a level): a segment of G
+// lanes sweeps one BDD, lane s holding state s, and one warp (work item) takes
+// `nseg` BDDs of one kind: the same level types, start and accepted states
+// (any lengths when all levels have one type, else the same length).
+struct LongItem {
+  int32_t first;     // its BDDs: long_order[first .. first + nseg)
+  int32_t nseg;
+  int32_t G;         // 2, 4, 8, 16 or 32
+  int32_t kmax;      // levels of the longest
+  int32_t start;
+  uint32_t accept;
+  int32_t run_base;  // unit_runs entries (the last run's end is read as "to the end")
+  int32_t nruns;
+};
+static_assert(sizeof(LongItem) == 32, "LongItem is 32 bytes");
+constexpr int kLongUnitMaxW = 32;
+constexpr int kLongUnitMaxK = 1400;  // levels whose path costs fit a CTA's shared memory at 32 states
+// Row stride (floats) of a per-level array of one BDD in shared memory: whole
+// 16-byte pieces.
+DG_HD inline int long_unit_stride(int kmax) { return (kmax + 3) / 4 * 4; }
+// Shared memory of one item in the sweeps: the path costs of levels 0 .. kmax
+// and per BDD lambda, the averaging term and (mode 1) omega and alpha ...
+inline size_t long_unit_bytes(int nseg, int G, int kmax, int mode) {
+  const size_t b = 4 * ((size_t)nseg * (mode ? 4 : 2) * long_unit_stride(kmax) + (size_t)(kmax + 1) * nseg * G);
+  return (b + 127) / 128 * 128;
+}
+// ... and in the adjoint: per level and BDD the gradient of lambda, m1 - m0,
+// the weight, omega, the variable id, a pair per variable and four record
+// words.
+inline size_t long_unit_adjoint_bytes(int nseg, int kmax) {
+  return (size_t)nseg * 11 * 4 * long_unit_stride(kmax);
+}
+
 // Device view of an arena (all pointers inside the caller's buffer).
 struct DevArena {
   const Tile* tiles;
@@ -146,6 +185,7 @@ struct DevArena {
   // the long BDDs whose levels have at most 32 nodes ("narrow"; longest
   // first), then the others (ascending): indices into `longs`
   const int32_t* long_order;
+  const LongItem* long_items;  // work items of the long unit BDDs (the head of long_order)
   float* long_d;               // scratch per node of long BDDs: SP(r, .)
   float* long_t;               // ... SP(., T)
   // scratch per node and lane of the tiles (layout of lohi8): SP(r, .) as a
@@ -173,6 +213,10 @@ struct DevArena {
   int32_t long_cost_size;   // entries of long_d / long_t
   int32_t long_stream;      // stream of the fork/join set the long BDDs run on
   int32_t num_long_narrow;  // narrow long BDDs (the head of long_order)
+  int32_t num_long_unit;    // ... of them, the unit ones (its very head)
+  int32_t num_long_items;
+  int32_t long_unit_smem[2];  // shared memory of the largest work item, mode 0 and 1
+  int32_t long_unit_adj_smem;
   int32_t long_lanes;       // lanes per narrow BDD in the plain sweeps (a power of two, set at bind)
 };
 
@@ -240,7 +284,9 @@ struct Plan {
   std::vector<int2> long_code;
   std::vector<int32_t> long_lvl, long_in_ptr, long_in;
   std::vector<int32_t> long_order;  // see DevArena::long_order
-  int32_t num_long_narrow = 0;
+  int32_t num_long_narrow = 0, num_long_unit = 0;
+  std::vector<LongItem> long_items;
+  int32_t long_unit_smem[2] = {0, 0}, long_unit_adj_smem = 0;
   int32_t long_lanes = 0;           // dg_options::long_lanes (0: chosen at bind)
   std::vector<int64_t> long_rank_ptr;  // per long BDD, first entry of long_lo / long_hi
   std::vector<int32_t> long_lo, long_hi;  // child ranks as in lo8 / hi8 (-2 bottom, -1 top)
@@ -249,7 +295,7 @@ struct Plan {
   struct Off {
     size_t tiles, unit_shapes, unit_runs, desc, lohi8, slot_var, slot_row, var_ptr, var_slots, var_ell, wide_vars, c, invdeg, inst_row_ptr,
         inst_var_ptr,
-        lb_chunks, inst_chunk_ptr, inst_unc, longs, long_code, long_lvl, long_in_ptr, long_in, long_order, S, Sbar, slot_avg, E, lb_part,
+        lb_chunks, inst_chunk_ptr, inst_unc, longs, long_code, long_lvl, long_in_ptr, long_in, long_order, long_items, S, Sbar, slot_avg, E, lb_part,
         long_d, long_t, nodecost, slot_invdeg, total;
   } off{};
   size_t smem_sweep = 0;   // dynamic smem of the sweep kernels

@@ -47,6 +47,9 @@ struct SweepArgs {
   // hi-choice, per long slot (from long_slot_base) the argmin nodes of m0, m1
   int32_t* rec_lmeta;
   int2* rec_lamin;
+  // ... and for the long unit BDDs per long slot (from long_slot_base) the
+  // out-arc bits of the level, the in-arc bits of the next, and argmin states
+  uint4* rec_lunit;
 };
 
 // The caller's stream plus kStreams - 1 auxiliary streams of an arena: the
@@ -124,6 +127,7 @@ struct AdjArgs {
   // SP(., T) and SP(r, .)
   const int32_t* rec_lmeta;
   const int2* rec_lamin;
+  const uint4* rec_lunit;
   float* long_a1;
   float* long_a2;
 };
@@ -156,6 +160,9 @@ void launch_param_transform_bwd(const DevArena& A, const float* alpha, const flo
 
 // Long BDDs, one warp per BDD (kernels_long.cu); each is a single launch on
 // the given stream, or nothing when the arena has no long BDDs.
+cudaError_t set_long_unit_smem_limit(size_t bytes);
+void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st);
+void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st);
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st);
 void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, cudaStream_t st);
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st);

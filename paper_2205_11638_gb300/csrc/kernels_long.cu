@@ -469,8 +469,9 @@ __global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
     // the plain sweeps take the wide long BDDs here (k_long_narrow the others)
     if (b >= A.num_long - A.num_long_narrow) return;  // whole warp leaves
     b = A.long_order[A.num_long_narrow + b];
-  } else if (b >= A.num_long) {
-    return;
+  } else {
+    if (b >= A.num_long - A.num_long_unit) return;
+    b = A.long_order[A.num_long_unit + b];
   }
   const LongCtx c = long_ctx(A, b);
   const int64_t sb = c.B.slot_base;
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(128) k_long_narrow(DevArena A, SweepArgs a) {
   constexpr bool FWD = KIND == kFwd;
   const int lane = threadIdx.x & 31;
   const int G = A.long_lanes;
-  const int first = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (kWarp / G);
+  const int first = A.num_long_unit + (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (kWarp / G);
   if (first >= A.num_long_narrow) return;  // whole warp leaves
   Seg g;
   g.s = lane & (G - 1);
@@ -684,8 +685,9 @@ __global__ void __launch_bounds__(128) k_long_smoothed(DevArena A, const float* 
 template <int FWD, int MODE>
 __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
   const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= A.num_long) return;
+  int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= A.num_long - A.num_long_unit) return;
+  b = A.long_order[A.num_long_unit + b];
   const LongCtx c = long_ctx(A, b);
   const int64_t sb = c.B.slot_base;
   const int k = c.B.k;
@@ -804,14 +806,16 @@ namespace {
 constexpr int kLongWarps = 4;  // BDDs (warps) per CTA
 
 int long_grid(const DevArena& A) { return (A.num_long + kLongWarps - 1) / kLongWarps; }
+// ... without the unit ones (kernels_long_unit.cu)
+int long_grid_other(const DevArena& A) { return (A.num_long - A.num_long_unit + kLongWarps - 1) / kLongWarps; }
 
 template <int KIND>
 void launch_long_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  int grid = long_grid(A);
+  int grid = long_grid_other(A);
   if constexpr (KIND == kFwd || KIND == kBwd) {
-    if (A.num_long_narrow > 0) {
+    if (A.num_long_narrow > A.num_long_unit) {
       const int per = kWarp / A.long_lanes;
-      const int warps = (A.num_long_narrow + per - 1) / per;
+      const int warps = (A.num_long_narrow - A.num_long_unit + per - 1) / per;
       const int ng = (warps + kLongWarps - 1) / kLongWarps;
       if (a.mode == 1)
         k_long_narrow<KIND, 1><<<ng, kLongWarps * kWarp, 0, st>>>(A, a);
@@ -830,15 +834,16 @@ void launch_long_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
 }  // namespace
 
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (A.num_long == 0) return;
+  if (A.num_long_items > 0) launch_long_unit(kind, A, a, st);
+  if (A.num_long == A.num_long_unit) return;
   switch (kind) {
     case kFwd: launch_long_kind<kFwd>(A, a, st); break;
     case kBwd: launch_long_kind<kBwd>(A, a, st); break;
     case kFwdRec: launch_long_kind<kFwdRec>(A, a, st); break;
     case kBwdRec: launch_long_kind<kBwdRec>(A, a, st); break;
-    case kMinMarg: k_long_sweep<kMinMarg, 0><<<long_grid(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
-    case kEnergy: k_long_sweep<kEnergy, 0><<<long_grid(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
-    default: k_long_sweep<kSeed, 0><<<long_grid(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
+    case kMinMarg: k_long_sweep<kMinMarg, 0><<<long_grid_other(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
+    case kEnergy: k_long_sweep<kEnergy, 0><<<long_grid_other(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
+    default: k_long_sweep<kSeed, 0><<<long_grid_other(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
   }
 }
 
@@ -848,8 +853,9 @@ void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float*
 }
 
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st) {
-  if (A.num_long == 0) return;
-  const int g = long_grid(A), t = kLongWarps * kWarp;
+  if (A.num_long_items > 0) launch_long_unit_adjoint(forward, A, a, st);
+  if (A.num_long == A.num_long_unit) return;
+  const int g = long_grid_other(A), t = kLongWarps * kWarp;
   if (forward)
     a.mode == 1 ? k_long_adjoint<1, 1><<<g, t, 0, st>>>(A, a) : k_long_adjoint<1, 0><<<g, t, 0, st>>>(A, a);
   else

@@ -1,0 +1,660 @@
+// kernels_long_unit.cu -- the long unit rows (LongItem): long cardinality and
+// assignment rows, whose BDDs are too large for a tile lane but have at most
+// 32 states a level that two shifts connect (see UnitShape).
+//
+// The levels of one BDD are a chain (the paper's long subproblems: the update
+// of a level needs the path costs under the lambda of the level before), so a
+// sweep's time is the levels times the latency of one step, and everything
+// else has to be out of that chain.  A segment of G lanes holds a level, lane
+// s its state s; a step is one shuffle to the neighbour state, the segment's
+// minima and the update.  All inputs of a work item are staged in shared
+// memory before the walk (asynchronous copies; the averaging terms gathered
+// through the staged variable ids), the costs opposite to the sweep are
+// recomputed into shared memory by a first walk, and each step's words are
+// read one step ahead.  New lambda and M replace the staged inputs and leave
+// in one coalesced pass.  The loops over explicit children and in-arcs in
+// global memory (kernels_long.cu) take half a microsecond a level.
+//
+// Same FP32 operations, tie rules and records as there: results are equal bit
+// for bit, gradients up to the rounding of sums.
+#include "kernels.h"
+#include "unit.cuh"
+
+namespace dg {
+
+namespace {
+
+constexpr unsigned kAll = 0xFFFFFFFFu;
+
+// The segment of a lane.
+template <int G>
+struct LSeg {
+  int base, s;
+  bool act;   // a BDD of the item
+  int row;    // ... its index (0 where there is none)
+};
+
+template <int G>
+__device__ __forceinline__ float seg_min(float x) {
+  if constexpr (G == 32) {
+    // one reduction instead of five shuffles, over an order-preserving map
+    const int i = __float_as_int(x);
+    const int m = __reduce_min_sync(kAll, i ^ ((i >> 31) & 0x7FFFFFFF));
+    return __int_as_float(m ^ ((m >> 31) & 0x7FFFFFFF));
+  } else {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) x = fminf(x, __shfl_xor_sync(kAll, x, o));
+    return x;
+  }
+}
+template <int G>
+__device__ __forceinline__ float seg_sum(float x) {
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) x += __shfl_xor_sync(kAll, x, o);
+  return x;
+}
+template <int G>
+__device__ __forceinline__ uint32_t seg_bits(bool p, int base) {
+  return (__ballot_sync(kAll, p) >> base) & (G == 32 ? kAll : (1u << (G & 31)) - 1u);
+}
+
+template <int G, int TYPE>
+__device__ __forceinline__ int lz(int s) {
+  return TYPE == kSwap ? max(s - 1, 0) : s;
+}
+template <int G, int TYPE>
+__device__ __forceinline__ int lo_(int s) {  // may be -1 or G: no such state
+  return TYPE == kUp ? s + 1 : (TYPE == kSwap ? s : (TYPE == kDown ? max(s - 1, 0) : s - 1));
+}
+
+// Value of the neighbour state the arcs come from (down) or lead to (up), inf
+// outside the window.
+template <int G, int TYPE>
+__device__ __forceinline__ float from_neighbour(float R, const LSeg<G>& g, float none) {
+  const int n = TYPE == kUp ? g.s - 1 : g.s + 1;
+  const float x = __shfl_sync(kAll, R, g.base + (n & (G - 1)));
+  return n >= 0 && n < G ? x : none;
+}
+
+// SP(., T) of the two children of the lane's state, from the level below.
+template <int G, int TYPE>
+__device__ __forceinline__ void children(float t, const LSeg<G>& g, float& tz, float& to) {
+  const int n = TYPE == kUp ? g.s + 1 : g.s - 1;
+  float x = __shfl_sync(kAll, t, g.base + (n & (G - 1)));
+  if (TYPE == kDown || TYPE == kSwap) x = n < 0 ? t : x;  // the lowest state absorbs
+  else x = n >= 0 && n < G ? x : f_inf();
+  tz = TYPE == kSwap ? x : t;
+  to = TYPE == kSwap ? t : x;
+}
+
+// SP(r, .) of the lane's state on the next level.
+template <int G, int TYPE>
+__device__ __forceinline__ float down(float R, float n, float l, int s) {
+  if (TYPE == kSwap) return fminf(s == 0 ? fminf(R, R + l) : R + l, n);
+  const float r = fminf(R, n + l);
+  return TYPE == kDown && s == 0 ? fminf(r, R + l) : r;
+}
+// ... with the index of the in-arc in unit_in_arcs' order.
+template <int G, int TYPE>
+__device__ __forceinline__ float down_rec(float R, float n, float l, int s, int& c) {
+  float x0, x1, x2 = f_inf();
+  if (TYPE == kUp) {
+    x0 = R;
+    x1 = n + l;
+  } else if (TYPE == kSwap) {
+    x0 = n;
+    x1 = s == 0 ? R : R + l;
+    if (s == 0) x2 = R + l;
+  } else {
+    x0 = n + l;
+    x1 = R;
+    if (TYPE == kDown && s == 0) x2 = R + l;
+  }
+  float b = f_inf();
+  c = 0;
+  if (x0 < b) b = x0;
+  if (x1 < b) {
+    b = x1;
+    c = 1;
+  }
+  if (x2 < b) {
+    b = x2;
+    c = 2;
+  }
+  return b;
+}
+
+// Runs of one level type over [0, kmax): the last run ends there.
+template <class F>
+__device__ __forceinline__ void runs_down(const DevArena& A, const LongItem& it, F&& f) {
+  int b = 0;
+  for (int r = 0; r < it.nruns; ++r) {
+    const unsigned run = __ldg(A.unit_runs + it.run_base + r);
+    const int e = r + 1 < it.nruns ? (int)(run >> 2) : it.kmax;
+    unit_run(run & 3u, b, e, f);
+    b = e;
+  }
+}
+template <class F>
+__device__ __forceinline__ void runs_up(const DevArena& A, const LongItem& it, F&& f) {
+  int e = it.kmax;
+  for (int r = it.nruns - 1; r >= 0; --r) {
+    const unsigned run = __ldg(A.unit_runs + it.run_base + r);
+    const int b = r > 0 ? (int)(__ldg(A.unit_runs + it.run_base + r - 1) >> 2) : 0;
+    unit_run(run & 3u, b, e, f);
+    e = b;
+  }
+}
+
+// k floats (whole 16-byte pieces; slot ranges are padded to 32) to shared memory.
+__device__ __forceinline__ void copy_row(float* dst, const void* src, int k, int lane, uint64_t pol) {
+  for (int p = lane; p < (k + 3) / 4; p += kWarp) cp_async16(dst + 4 * p, (const char*)src + 16 * p, pol);
+}
+
+template <int KIND, int MODE, int G>
+__device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArgs& a, const LongItem& it, float* smem,
+                                               int lane) {
+  constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
+  constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
+  constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
+  constexpr bool UPDATE = FWD || BWD;
+  const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST, TS = it.nseg * G;
+  float* lam = smem;
+  float* avg = lam + nrow;
+  float* om = avg + nrow;
+  float* al = om + (MODE == 1 ? nrow : 0);
+  float* cost = al + (MODE == 1 ? nrow : 0);
+
+  // ---- staging -------------------------------------------------------------
+  const uint64_t pol = l2_evict_first();
+  if (UPDATE) {
+    for (int r = 0; r < it.nseg; ++r) {
+      const LongBdd B = A.longs[A.long_order[it.first + r]];
+      copy_row(avg + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
+    }
+    cp_async_commit();
+  }
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd B = A.longs[A.long_order[it.first + r]];
+    copy_row(lam + r * ST, a.lam + B.slot_base, B.k, lane, pol);
+    if (UPDATE && MODE == 1) {
+      copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
+      copy_row(al + r * ST, a.alpha + B.slot_base, B.k, lane, pol);
+    }
+  }
+  cp_async_commit();
+  if (UPDATE) {
+    cp_async_wait_one();
+    __syncwarp();
+    const float* src = MODE == 1 ? A.S : A.Sbar;
+    for (int r = 0; r < it.nseg; ++r) {
+      const int k = A.longs[A.long_order[it.first + r]].k;
+#pragma unroll 4
+      for (int h = lane; h < k; h += kWarp) {
+        const int v = __float_as_int(avg[r * ST + h]);
+        cp_async4(avg + r * ST + h, src + v);
+      }
+    }
+    cp_async_commit();
+  }
+  cp_async_wait_all();
+  __syncwarp();
+
+  // ---- the walk --------------------------------------------------------------
+  LSeg<G> g;
+  g.s = lane & (G - 1);
+  g.base = lane - g.s;
+  g.act = lane / G < it.nseg;
+  g.row = g.act ? lane / G : 0;
+  const LongBdd B = A.longs[A.long_order[it.first + g.row]];
+  const int k = B.k;
+  float* ml = lam + g.row * ST;
+  float* ma = avg + g.row * ST;
+  const float* mo = om + g.row * ST;
+  const float* mw = al + g.row * ST;
+  float* mt = cost + g.row * G + g.s;  // level h at mt[h TS]
+  const float end = (it.accept >> g.s) & 1u ? 0.0f : f_inf();
+  const float root = g.s == it.start ? 0.0f : f_inf();
+
+  auto first_up = [&]() -> float {  // SP(., T) of every level; returns level 0's
+    float t = end;
+    if (g.act) mt[k * TS] = end;
+    float l = ml[it.kmax - 1];
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = e - 1; h >= b; --h) {
+        const float ln = ml[max(h - 1, 0)];
+        float tz, to;
+        children<G, TY>(t, g, tz, to);
+        if (h < k) t = fminf(tz, l + to);
+        if (g.act && h < k) mt[h * TS] = t;
+        l = ln;
+      }
+    });
+    return t;
+  };
+  // the update of a level from its minima, by every lane of the segment
+  auto update = [&](int h, float l, float av, float b0, float b1, float w, float alpha) -> float {
+    const float m0 = b0, m1 = l + b1;
+    const float Mn = __fmul_rn(MODE == 1 ? w : a.omega0, m1 - m0);
+    const float ln = unit_lambda_new<MODE>(l, Mn, alpha, av);
+    if (g.act && g.s == 0 && h < k) {
+      ml[h] = ln;
+      ma[h] = Mn;
+      if (REC) a.rec_diff[(int64_t)B.slot_base + h] = m1 - m0;
+    }
+    return ln;
+  };
+  auto record = [&](int h, bool hi, int c, float x0, float m0, float x1, float m1) {
+    const uint32_t tb = seg_bits<G>(hi, g.base), rb = seg_bits<G>((c & 1) != 0, g.base);
+    const uint32_t ex = seg_bits<G>(c == 2, g.base) & 1u;
+    // the argmins: the largest state on ties
+    const uint32_t b0 = seg_bits<G>(x0 == m0, g.base), b1 = seg_bits<G>(x1 == m1, g.base);
+    const int v0 = b0 ? 31 - __clz((int)b0) : 0, v1 = b1 ? 31 - __clz((int)b1) : 0;
+    if (g.act && g.s == 0 && h < k)
+      a.rec_lunit[(int64_t)B.slot_base + h - A.long_slot_base] =
+          make_uint4(tb, rb, (uint32_t)v0 | (uint32_t)v1 << 8 | ex << 16, 0u);
+  };
+
+  if (FWD || KIND == kMinMarg) {
+    first_up();
+    __syncwarp();
+    float R = root;
+    float l = ml[0], av = ma[0], w = MODE == 1 ? mo[0] : 0.0f, alpha = MODE == 1 ? mw[0] : 0.0f;
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      const int zi = lz<G, TY>(g.s) - g.s, oi = lo_<G, TY>(g.s) - g.s;
+      const bool ov = lo_<G, TY>(g.s) >= 0 && lo_<G, TY>(g.s) < G;
+      auto child = [&](int h, float& tz, float& to) {
+        const float* p = mt + min(h + 1, k) * TS;
+        tz = p[zi];
+        to = p[ov ? oi : 0];
+      };
+      float tz, to;
+      child(b, tz, to);
+      for (int h = b; h < e; ++h) {
+        const int hn = min(h + 1, it.kmax - 1);
+        float tzn, ton;
+        const float l1 = ml[hn], av1 = ma[hn], w1 = MODE == 1 ? mo[hn] : 0.0f, al1 = MODE == 1 ? mw[hn] : 0.0f;
+        child(hn, tzn, ton);
+        const float n = from_neighbour<G, TY>(R, g, f_inf());
+        const float x0 = R + tz, x1 = ov ? R + to : f_inf();
+        const float b0 = seg_min<G>(x0), b1 = seg_min<G>(x1);
+        if (KIND == kMinMarg) {
+          if (g.act && g.s == 0 && h < k) {
+            ml[h] = l + b1;
+            ma[h] = b0;
+          }
+          R = down<G, TY>(R, n, l, g.s);
+        } else {
+          const float ln = update(h, l, av, b0, b1, w, alpha);
+          if (REC) {
+            int c;
+            const bool hi = !(tz <= (ov ? l + to : f_inf()));
+            R = down_rec<G, TY>(R, n, ln, g.s, c);
+            record(h, hi, c, x0, b0, x1, b1);
+          } else {
+            R = down<G, TY>(R, n, ln, g.s);
+          }
+        }
+        l = l1;
+        av = av1;
+        w = w1;
+        alpha = al1;
+        tz = tzn;
+        to = ton;
+      }
+    });
+  } else if (BWD) {
+    float R = root;
+    {
+      float l = ml[0];
+      runs_down(A, it, [&](auto ty, int b, int e) {
+        constexpr int TY = decltype(ty)::value;
+        for (int h = b; h < e; ++h) {
+          const float ln = ml[min(h + 1, it.kmax - 1)];
+          if (g.act && h < k) mt[h * TS] = R;
+          R = down<G, TY>(R, from_neighbour<G, TY>(R, g, f_inf()), l, g.s);
+          l = ln;
+        }
+      });
+    }
+    __syncwarp();
+    float t = end;
+    const int h0 = it.kmax - 1;
+    float l = ml[h0], av = ma[h0], w = MODE == 1 ? mo[h0] : 0.0f, alpha = MODE == 1 ? mw[h0] : 0.0f;
+    float r = mt[min(h0, k - 1) * TS];
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      const int ni = TY == kUp ? -1 : 1;
+      const bool nv = g.s + ni >= 0 && g.s + ni < G;
+      for (int h = e - 1; h >= b; --h) {
+        const int hn = max(h - 1, 0);
+        const float l1 = ml[hn], av1 = ma[hn], w1 = MODE == 1 ? mo[hn] : 0.0f, al1 = MODE == 1 ? mw[hn] : 0.0f;
+        const float r1 = mt[min(hn, k - 1) * TS];
+        float tz, to;
+        children<G, TY>(t, g, tz, to);
+        const float x0 = r + tz, x1 = r + to;
+        const float b0 = seg_min<G>(x0), b1 = seg_min<G>(x1);
+        const float ln = update(h, l, av, b0, b1, w, alpha);
+        if (REC) {
+          int c;
+          const float n = nv ? mt[min(h, k - 1) * TS + ni] : f_inf();
+          down_rec<G, TY>(r, n, l, g.s, c);
+          const float th = ln + to;
+          const bool hi = !(tz <= th);
+          if (h < k) t = hi ? th : tz;
+          record(h, hi, c, x0, b0, x1, b1);
+        } else if (h < k) {
+          t = fminf(tz, ln + to);
+        }
+        l = l1;
+        av = av1;
+        w = w1;
+        alpha = al1;
+        r = r1;
+      }
+    });
+    if (a.E != nullptr && g.act && g.s == it.start) a.E[B.row] = t;  // E^j = SP(r, T)
+  } else {
+    const float t = first_up();
+    if (KIND == kEnergy) {
+      if (a.E != nullptr && g.act && g.s == it.start) a.E[B.row] = t;
+    } else {
+      // kSeed: walk the minimising path from the root, the 0-arc on ties
+      __syncwarp();
+      int at = it.start;
+      const float* row = cost + g.row * G;
+      runs_down(A, it, [&](auto ty, int b, int e) {
+        constexpr int TY = decltype(ty)::value;
+        for (int h = b; h < min(e, k); ++h) {
+          const int z = lz<G, TY>(at), o = lo_<G, TY>(at);
+          const float* p = row + (h + 1) * TS;
+          const float c0 = p[z], c1 = o >= 0 && o < G ? p[o] : f_inf();
+          // an infinite cost is the bottom terminal (the path stays feasible)
+          const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= ml[h] + c1);
+          if (g.act && g.s == 0) ma[h] = take0 ? 0.f : 1.f;
+          at = take0 ? z : max(min(o, G - 1), 0);
+        }
+      });
+    }
+  }
+
+  // ---- the new state ---------------------------------------------------------
+  if (KIND == kEnergy) return;
+  __syncwarp();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd Br = A.longs[A.long_order[it.first + r]];
+    float* o0 = (KIND == kMinMarg ? a.out2 : a.lam) + Br.slot_base;
+    float* o1 = a.M + Br.slot_base;
+    for (int h = lane; h < Br.k; h += kWarp) {
+      if (KIND != kSeed) o0[h] = lam[r * ST + h];
+      o1[h] = avg[r * ST + h];
+    }
+  }
+}
+
+template <int KIND, int MODE>
+__global__ void __launch_bounds__(32) k_long_unit(DevArena A, SweepArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x;
+  const LongItem it = A.long_items[blockIdx.x];
+  float* p = reinterpret_cast<float*>(smem);
+  switch (it.G) {
+    case 2: long_unit_item<KIND, MODE, 2>(A, a, it, p, lane); break;
+    case 4: long_unit_item<KIND, MODE, 4>(A, a, it, p, lane); break;
+    case 8: long_unit_item<KIND, MODE, 8>(A, a, it, p, lane); break;
+    case 16: long_unit_item<KIND, MODE, 16>(A, a, it, p, lane); break;
+    default: long_unit_item<KIND, MODE, 32>(A, a, it, p, lane); break;
+  }
+}
+
+// Adjoint of a recording sweep: the reverse of the walk with the gradients of
+// a level's path costs on the segment's lanes (see kernels_adjoint.cu for the
+// steps and kernels_unit.cu for the routing along the recorded arcs).
+template <int FWD, int MODE, int G>
+__device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const AdjArgs& a, const LongItem& it,
+                                                       float* smem, int lane) {
+  const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST;
+  uint4* rec = reinterpret_cast<uint4*>(smem);
+  float2* in = reinterpret_cast<float2*>(rec + nrow);
+  float* gl = reinterpret_cast<float*>(in + nrow);
+  float* df = gl + nrow;
+  float* al = df + nrow;
+  float* om = al + nrow;
+  float* id = om + nrow;
+  const uint64_t pol = l2_evict_first();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd B = A.longs[A.long_order[it.first + r]];
+    copy_row(id + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
+  }
+  cp_async_commit();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd B = A.longs[A.long_order[it.first + r]];
+    copy_row(gl + r * ST, a.g_lam + B.slot_base, B.k, lane, pol);
+    copy_row(df + r * ST, a.rec_diff + B.slot_base, B.k, lane, pol);
+    copy_row(al + r * ST, (MODE == 1 ? a.alpha : A.slot_invdeg) + B.slot_base, B.k, lane, pol);
+    if (MODE == 1) copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
+    const uint4* src = a.rec_lunit + (B.slot_base - A.long_slot_base);
+    for (int h = lane; h < B.k; h += kWarp) cp_async16(rec + r * ST + h, src + h, pol);
+  }
+  cp_async_commit();
+  cp_async_wait_one();
+  __syncwarp();
+  for (int r = 0; r < it.nseg; ++r) {
+    const int k = A.longs[A.long_order[it.first + r]].k;
+#pragma unroll 4
+    for (int h = lane; h < k; h += kWarp) cp_async8(in + r * ST + h, a.var_in + __float_as_int(id[r * ST + h]));
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncwarp();
+
+  LSeg<G> g;
+  g.s = lane & (G - 1);
+  g.base = lane - g.s;
+  g.act = lane / G < it.nseg;
+  g.row = g.act ? lane / G : 0;
+  const LongBdd B = A.longs[A.long_order[it.first + g.row]];
+  const int k = B.k;
+  const bool own = g.act && g.s == 0;
+  float* mg = gl + g.row * ST;
+  float* md = df + g.row * ST;
+  float* mw = al + g.row * ST;
+  const float* mo = om + g.row * ST;
+  float2* mi = in + g.row * ST;
+  const uint4* mr = rec + g.row * ST;
+  const float* seed = a.seed_M ? a.seed_M + B.slot_base : nullptr;
+
+  // the update of level h reversed; returns the gradient of m1
+  auto reverse = [&](int h, float x) -> float {
+    const float2 v = mi[h];
+    const float Mt = (seed ? seed[h] : 0.0f) + v.x - x;
+    const float d = (MODE == 1 ? mo[h] : a.omega0) * Mt;
+    __syncwarp();
+    if (own && h < k) {
+      mi[h] = make_float2(Mt * md[h], x * v.y);  // omega-dot, alpha-dot
+      mw[h] = mw[h] * x;                         // contribution to S-dot
+      md[h] = d;
+      mg[h] = x + d;
+    }
+    return d;
+  };
+  // gradient of SP(r, .) from level h + 1 to level h; gs: what entered by 1-arcs
+  auto route_in = [&](auto ty, float G2, const uint4& w, float& gs) -> float {
+    constexpr int TY = decltype(ty)::value;
+    const int c = (int)((w.y >> g.s) & 1u) | (g.s == 0 ? (int)((w.z >> 16) & 1u) << 1 : 0);
+    float stay, moved, hi;
+    if (TY == kUp) {
+      stay = c == 0 ? G2 : 0.0f;
+      moved = hi = c == 1 ? G2 : 0.0f;
+    } else {
+      moved = c == 0 ? G2 : 0.0f;
+      stay = c != 0 ? G2 : 0.0f;
+      hi = TY == kSwap ? (c == (g.s == 0 ? 2 : 1) ? G2 : 0.0f) : (c != 1 ? G2 : 0.0f);
+    }
+    const int n = TY == kUp ? g.s + 1 : g.s - 1;
+    const float x = __shfl_sync(kAll, moved, g.base + (n & (G - 1)));
+    gs = seg_sum<G>(hi);
+    return stay + (n >= 0 && n < G ? x : 0.0f);
+  };
+  // gradient of SP(., T) from level h to level h + 1; gs: what left by 1-arcs
+  auto route_out = [&](auto ty, float G1, const uint4& w, float& gs) -> float {
+    constexpr int TY = decltype(ty)::value;
+    const bool hi = (w.x >> g.s) & 1u;
+    const float hp = hi ? G1 : 0.0f, lp = hi ? 0.0f : G1;
+    const float moved = TY == kSwap ? lp : hp;
+    float r = TY == kSwap ? hp : lp;
+    const int n = TY == kUp ? g.s - 1 : g.s + 1;
+    const float x = __shfl_sync(kAll, moved, g.base + (n & (G - 1)));
+    if (n >= 0 && n < G) r += x;
+    if ((TY == kDown || TY == kSwap) && g.s == 0) r += moved;  // the lowest state absorbs
+    gs = seg_sum<G>(hp);
+    return r;
+  };
+  auto seed_in = [&](float x, const uint4& w, float d) {
+    if (g.s == (int)(w.z & 255u)) x -= d;
+    if (g.s == (int)(w.z >> 8 & 255u)) x += d;
+    return x;
+  };
+  auto seed_out = [&](auto ty, float x, const uint4& w, float d) {
+    constexpr int TY = decltype(ty)::value;
+    if (g.s == lz<G, TY>((int)(w.z & 255u))) x -= d;
+    if (g.s == lo_<G, TY>((int)(w.z >> 8 & 255u))) x += d;
+    return x;
+  };
+  const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+  float x = 0.0f;
+  if (FWD) {
+    // SP(r, .) of level h + 1 was relaxed from level h with lambda^new_h
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      for (int h = e - 1; h >= b; --h) {
+        const bool on = h < k;
+        const uint4 w = on ? mr[h] : none;
+        float gs;
+        const float y = route_in(ty, x, w, gs);
+        const float d = reverse(min(h, k - 1), mg[min(h, k - 1)] + gs);
+        x = on ? seed_in(y, w, d) : 0.0f;
+      }
+    });
+  } else {
+    // SP(., T) of level h was recomputed with lambda^new_h
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      for (int h = b; h < e; ++h) {
+        const bool on = h < k;
+        const uint4 w = on ? mr[h] : none;
+        float gs;
+        const float y = route_out(ty, x, w, gs);
+        const float d = reverse(min(h, k - 1), mg[min(h, k - 1)] + gs);
+        x = on ? seed_out(ty, y, w, d) : 0.0f;
+      }
+    });
+  }
+  __syncwarp();
+  x = 0.0f;
+  if (FWD) {
+    // SP(., T) under lambda^old: its gradient flows top-down
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      for (int h = b; h < e; ++h) {
+        const bool on = h < k;
+        const uint4 w = on ? mr[h] : none;
+        float gs;
+        const float y = route_out(ty, x, w, gs);
+        x = seed_out(ty, y, w, on ? md[h] : 0.0f);
+        if (own && on) mg[h] += gs;
+      }
+    });
+  } else {
+    // SP(r, .) under lambda^old: its gradient flows bottom-up
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      for (int h = e - 1; h >= b; --h) {
+        const bool on = h < k;
+        const uint4 w = on ? mr[h] : none;
+        float gs;
+        const float y = route_in(ty, x, w, gs);
+        x = on ? seed_in(y, w, md[h]) : 0.0f;
+        if (own && on) mg[h] += gs;
+      }
+    });
+  }
+  __syncwarp();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd Br = A.longs[A.long_order[it.first + r]];
+    const int64_t q = Br.slot_base;
+    for (int h = lane; h < Br.k; h += kWarp) {
+      const float2 v = in[r * ST + h];
+      a.sdot[q + h] = al[r * ST + h];
+      a.g_lam[q + h] = gl[r * ST + h];
+      if (a.g_omega) a.g_omega[q + h] += v.x;
+      if (a.g_alpha) a.g_alpha[q + h] += v.y;
+    }
+  }
+}
+
+template <int FWD, int MODE>
+__global__ void __launch_bounds__(32) k_long_unit_adjoint(DevArena A, AdjArgs a) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x;
+  const LongItem it = A.long_items[blockIdx.x];
+  float* p = reinterpret_cast<float*>(smem);
+  switch (it.G) {
+    case 2: long_unit_adjoint_item<FWD, MODE, 2>(A, a, it, p, lane); break;
+    case 4: long_unit_adjoint_item<FWD, MODE, 4>(A, a, it, p, lane); break;
+    case 8: long_unit_adjoint_item<FWD, MODE, 8>(A, a, it, p, lane); break;
+    case 16: long_unit_adjoint_item<FWD, MODE, 16>(A, a, it, p, lane); break;
+    default: long_unit_adjoint_item<FWD, MODE, 32>(A, a, it, p, lane); break;
+  }
+}
+
+template <int KIND>
+void launch_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
+  if (a.mode == 1)
+    k_long_unit<KIND, 1><<<A.num_long_items, kWarp, A.long_unit_smem[1], st>>>(A, a);
+  else
+    k_long_unit<KIND, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a);
+}
+
+}  // namespace
+
+cudaError_t set_long_unit_smem_limit(size_t bytes) {
+  const int b = (int)bytes;
+  constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(k_long_unit<kFwd, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kFwd, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kBwd, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kBwd, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kFwdRec, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kFwdRec, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kBwdRec, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kBwdRec, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kMinMarg, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kEnergy, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit<kSeed, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit_adjoint<0, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit_adjoint<0, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit_adjoint<1, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_unit_adjoint<1, 1>, attr, b);
+  return e;
+}
+
+void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st) {
+  switch (kind) {
+    case kFwd: launch_kind<kFwd>(A, a, st); break;
+    case kBwd: launch_kind<kBwd>(A, a, st); break;
+    case kFwdRec: launch_kind<kFwdRec>(A, a, st); break;
+    case kBwdRec: launch_kind<kBwdRec>(A, a, st); break;
+    case kMinMarg: k_long_unit<kMinMarg, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a); break;
+    case kEnergy: k_long_unit<kEnergy, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a); break;
+    default: k_long_unit<kSeed, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a); break;
+  }
+}
+
+void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st) {
+  const int G = A.num_long_items, b = A.long_unit_adj_smem;
+  if (forward)
+    a.mode == 1 ? k_long_unit_adjoint<1, 1><<<G, kWarp, b, st>>>(A, a) : k_long_unit_adjoint<1, 0><<<G, kWarp, b, st>>>(A, a);
+  else
+    a.mode == 1 ? k_long_unit_adjoint<0, 1><<<G, kWarp, b, st>>>(A, a) : k_long_unit_adjoint<0, 0><<<G, kWarp, b, st>>>(A, a);
+}
+
+}  // namespace dg

@@ -1,5 +1,6 @@
-"""Unit tiles (rows with coefficients +1 and -1, all BDDs of a tile of one
-shape) against the mixed tiles' kernels.  Doubling a row's coefficients and
+"""Unit rows (coefficients +1 and -1), in tiles of one shape and, beyond a tile
+lane, as long unit rows, against the kernels of the mixed tiles and of the
+other long BDDs.  Doubling a row's coefficients and
 right-hand side leaves its canonical BDD unchanged but makes it no unit row,
 so the doubled problem runs the general kernels on the same BDDs.  Both do
 the same FP32 additions along the same arcs and take exact minima, hence the
@@ -41,7 +42,38 @@ def _random_unit_rows(seed, n=300, patterns=60):
     return workloads.single_rows_problem(rows, n, rng.normal(size=n))
 
 
+def _long_unit_rows(seed, n=700):
+    """Long rows of both layouts' limits: cardinality rows of several lengths,
+    senses and widths (up to 32 states a level; one of 33, which stays with
+    the general loops), clauses of random signs (two to four states, level
+    types alternating), and short rows next to them."""
+    rng = np.random.default_rng(seed)
+    rows = []
+
+    def add(a, sense, b, copies):
+        for _ in range(copies):
+            rows.append((np.sort(rng.choice(n, size=len(a), replace=False)), np.asarray(a, np.int64), sense, b))
+    for k in (128, 130, 257, 300, 511):
+        add(np.ones(k), workloads.LE, 1, 3)
+        add(np.ones(k), workloads.GE, 1, 2)
+        add(np.ones(k), workloads.EQ, 1, 2)
+    for b in (2, 5, 12, 31, 32):
+        add(np.ones(150 + b), workloads.LE, b, 2)
+        add(np.ones(150 + b), workloads.EQ, b, 1)
+        add(np.ones(140), workloads.GE, b, 1)
+    for b in (1, 3):
+        for copies in (1, 4):
+            a = rng.choice([-1, 1], size=260)
+            add(a, workloads.GE, b - int((a < 0).sum()), copies)
+    for r in workloads.random_rows(200, kmax=6, n=n, amax=1, seed=seed + 1):
+        if workloads._free_row(r):
+            rows.append(r)
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
 CASES = {
+    "long_rows": lambda: _long_unit_rows(6),
+    "assignment": lambda: workloads.assignment(L=50, R=300, cand=260, seed=44),
     "random_signs": lambda: _random_unit_rows(5),
     "tracking": lambda: workloads.tracking(frames=8, dets=150, seed=41),
     "matching": lambda: workloads.matching_quadratic(L=40, R=40, pairs=1500, seed=42),
