@@ -74,6 +74,11 @@ StreamSet streams_for(const dg_arena* ar, cudaStream_t main) {
   s.main = main;
   return s;
 }
+Chain chain_for(const dg_arena* ar, cudaStream_t main) {
+  Chain c;
+  c.ss = streams_for(ar, main);
+  return c;
+}
 
 dg_status check_launch(const char* where) {
   cudaError_t e = cudaGetLastError();
@@ -82,9 +87,9 @@ dg_status check_launch(const char* where) {
 }
 
 // Enqueues `iters` iterations (forward sweep, S, backward sweep, S per
-// iteration) on st.  The first S reduction makes the snapshot of the
+// iteration) on the chain's stream.  The first S reduction makes the snapshot of the
 // incoming M.
-dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, const float* omega, const float* alpha,
+dg_status enqueue_iterate(dg_arena* ar, Chain& ch, float* lam, float* M, const float* omega, const float* alpha,
                           int mode, int iters, double* lb_out, const dg_options* opts) {
   const DevArena& A = ar->dev;
   const int threads = threads_of(opts);
@@ -97,7 +102,9 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
   a.omega0 = omega_of(opts);
   a.mode = mode;
   ar->avg_mode = mode;
-  launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kSweep);
+  // only the last reduction stores what later calls may read
+  const int need = mode == 1 ? kNeedS : kNeedSbar;
+  launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, iters > 0 ? need : kNeedS | kNeedSbar);
   // every sweep hands its path costs to the next one (the S reductions
   // between them leave lambda alone), except into the first sweep, whose
   // lambda comes from the caller, and across a re-projection
@@ -107,23 +114,24 @@ dg_status enqueue_iterate(dg_arena* ar, cudaStream_t st, float* lam, float* M, c
     a.E = nullptr;
     a.cost_out = A.nodecost;
     a.cost_in = handed ? A.nodecost : nullptr;
-    launch_sweep(kFwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_reduce_S(A, M, lam, alpha, mode, false, st, Scatter::kSweep);
+    launch_sweep(kFwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), ch);
+    launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, need);
     if (lb_out && it == iters - 1) a.E = A.E;
     handed = it + 1 < iters && !rn;
     a.cost_out = handed ? A.nodecost : nullptr;
     a.cost_in = A.nodecost;
-    launch_sweep(kBwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_reduce_S(A, M, lam, alpha, mode, rn, st, it + 1 < iters ? Scatter::kSweep : Scatter::kNone);
+    launch_sweep(kBwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), ch);
+    launch_reduce_S(A, M, lam, alpha, mode, rn, ch, it + 1 < iters ? Scatter::kSweep : Scatter::kNone,
+                    it + 1 < iters ? need : kNeedS | kNeedSbar);
   }
   if (lb_out) {
     if (iters == 0) {
       SweepArgs e{};
       e.lam = lam;
       e.E = A.E;
-      launch_sweep(kEnergy, A, e, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
+      launch_sweep(kEnergy, A, e, threads, ar->groups.data(), (int)ar->groups.size(), ch);
     }
-    launch_lower_bound(A, lb_out, st);
+    launch_lower_bound(A, lb_out, ch);
   }
   return check_launch("dg_iterate");
 }
@@ -493,7 +501,8 @@ dg_status dg_iterate(dg_arena* ar, void* stream, float* lam, float* M, const flo
   if (opts && opts->block_threads != 0 && (opts->block_threads % 32 != 0 || opts->block_threads > 512))
     return fail(DG_EINVAL, "dg_iterate: block_threads must be a multiple of 32 in [32, 512]");
   if (dg_status s = check_vectors("dg_iterate", lam, M, omega, alpha)) return s;
-  return enqueue_iterate(ar, (cudaStream_t)stream, lam, M, omega, alpha, mode, iters, lb_out, opts);
+  Chain ch = chain_for(ar, (cudaStream_t)stream);
+  return enqueue_iterate(ar, ch, lam, M, omega, alpha, mode, iters, lb_out, opts);
 }
 
 dg_status dg_autotune(dg_arena* ar, void* stream, float* lam, float* M, int32_t reps, float* tuned_ms) {
@@ -521,16 +530,18 @@ dg_status dg_autotune(dg_arena* ar, void* stream, float* lam, float* M, int32_t 
     return ms / reps;
   };
   ar->avg_mode = 0;
-  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, Scatter::kSweep);
+  Chain ch = chain_for(ar, st);
+  launch_reduce_S(A, M, nullptr, nullptr, 0, false, ch, Scatter::kSweep);
   // timed as dg_iterate runs them after its first sweep: each sweep takes
   // its opposite-direction costs from the one before
   a.cost_out = A.nodecost;
-  launch_sweep(kFwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
+  launch_sweep(kFwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), ch);
   a.cost_in = A.nodecost;
-  launch_sweep(kBwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
+  launch_sweep(kBwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), ch);
   auto pair = [&] {
-    launch_sweep(kFwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-    launch_sweep(kBwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
+    Chain ch = chain_for(ar, st);
+    launch_sweep(kFwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), ch);
+    launch_sweep(kBwd, A, a, 128, ar->groups.data(), (int)ar->groups.size(), ch);
   };
   // start from the occupancy choice, made explicit
   for (LaunchGroup& G : ar->groups) {
@@ -600,7 +611,8 @@ dg_status dg_sum_M(dg_arena* ar, void* stream, const float* M, float* lam, const
   ar->avg_mode = mode;
   // a reduction without re-projection leaves lambda, so a hand-off survives it
   if (!renorm) keep_costs(ar);
-  launch_reduce_S(ar->dev, M, lam, alpha, mode, renorm != 0, (cudaStream_t)stream, Scatter::kSweep);
+  Chain ch = chain_for(ar, (cudaStream_t)stream);
+  launch_reduce_S(ar->dev, M, lam, alpha, mode, renorm != 0, ch, Scatter::kSweep);
   return check_launch("dg_sum_M");
 }
 
@@ -633,8 +645,8 @@ dg_status dg_sweep(dg_arena* ar, void* stream, float* lam, float* M, const float
   a.E = want_energy ? ar->dev.E : nullptr;
   a.cost_out = (flags & DG_SWEEP_COSTS_OUT) ? ar->dev.nodecost : nullptr;
   a.cost_in = (flags & DG_SWEEP_COSTS_IN) ? ar->dev.nodecost : nullptr;
-  launch_sweep(forward ? kFwd : kBwd, ar->dev, a, threads_of(opts), ar->groups.data(), (int)ar->groups.size(),
-               streams_for(ar, (cudaStream_t)stream));
+  Chain ch = chain_for(ar, (cudaStream_t)stream);
+  launch_sweep(forward ? kFwd : kBwd, ar->dev, a, threads_of(opts), ar->groups.data(), (int)ar->groups.size(), ch);
   if (flags & DG_SWEEP_COSTS_OUT) {
     ar->costs_epoch = ar->epoch;
     ar->costs_dir = dir;
@@ -647,7 +659,8 @@ dg_status dg_bound_from_energies(dg_arena* ar, void* stream, double* lb_out) {
   if (dg_status s = check_state(ar)) return s;
   if (!lb_out) return fail(DG_EINVAL, "dg_bound_from_energies: null output");
   keep_costs(ar);
-  launch_lower_bound(ar->dev, lb_out, (cudaStream_t)stream);
+  Chain ch = chain_for(ar, (cudaStream_t)stream);
+  launch_lower_bound(ar->dev, lb_out, ch);
   return check_launch("dg_bound_from_energies");
 }
 
@@ -659,8 +672,8 @@ dg_status dg_min_marginals(dg_arena* ar, void* stream, const float* lam, float* 
   a.lam = const_cast<float*>(lam);
   a.M = m0;
   a.out2 = m1;
-  launch_sweep(kMinMarg, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(),
-               streams_for(ar, (cudaStream_t)stream));
+  Chain ch = chain_for(ar, (cudaStream_t)stream);
+  launch_sweep(kMinMarg, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(), ch);
   return check_launch("dg_min_marginals");
 }
 
@@ -672,10 +685,10 @@ dg_status dg_lower_bound(dg_arena* ar, void* stream, const float* lam, const flo
   SweepArgs a{};
   a.lam = const_cast<float*>(lam);
   a.E = ar->dev.E;
-  launch_sweep(kEnergy, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(),
-               streams_for(ar, st));
-  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, st, Scatter::kNone);
-  launch_lower_bound(ar->dev, lb, st);
+  Chain ch = chain_for(ar, st);
+  launch_sweep(kEnergy, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(), ch);
+  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, ch, Scatter::kNone);
+  launch_lower_bound(ar->dev, lb, ch);
   if (E_per_row) {
     cudaError_t e = cudaMemcpyAsync(E_per_row, ar->dev.E, (size_t)ar->dev.m * 4, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e, "dg_lower_bound copy");
@@ -687,8 +700,8 @@ dg_status dg_lower_bound_noalloc(dg_arena* ar, void* stream, const float* lam, c
   if (dg_status s = check_state(ar)) return s;
   if (missing(ar, lam) || missing(ar, M) || !lb) return fail(DG_EINVAL, "dg_lower_bound_noalloc: null pointer");
   if (dg_status s = check_vectors("dg_lower_bound_noalloc", lam, M)) return s;
-  return lower_bound_noalloc(ar->dev, ar->groups.data(), (int)ar->groups.size(), threads_of(nullptr),
-                             streams_for(ar, (cudaStream_t)stream), lam, M, lb);
+  Chain ch = chain_for(ar, (cudaStream_t)stream);
+  return lower_bound_noalloc(ar->dev, ar->groups.data(), (int)ar->groups.size(), threads_of(nullptr), ch, lam, M, lb);
 }
 
 dg_status dg_lb_seed(dg_arena* ar, void* stream, const float* lam, const float* M, float* g_lam, float* g_M) {
@@ -700,9 +713,9 @@ dg_status dg_lb_seed(dg_arena* ar, void* stream, const float* lam, const float* 
   SweepArgs a{};
   a.lam = const_cast<float*>(lam);
   a.M = g_lam;
-  launch_sweep(kSeed, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(),
-               streams_for(ar, st));
-  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, st, Scatter::kNone);
+  Chain ch = chain_for(ar, st);
+  launch_sweep(kSeed, ar->dev, a, threads_of(nullptr), ar->groups.data(), (int)ar->groups.size(), ch);
+  launch_reduce_S(ar->dev, M, nullptr, nullptr, 0, false, ch, Scatter::kNone);
   launch_seed_M(ar->dev, g_M, st);
   return check_launch("dg_lb_seed");
 }
@@ -763,7 +776,8 @@ dg_status dg_graph_create(dg_arena* ar, void* stream, float* lam, float* M, cons
   if (!st) return fail(DG_EINVAL, "dg_graph_create: capture needs a non-default stream");
   cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(e, "dg_graph_create: begin capture");
-  dg_status s = enqueue_iterate(ar, st, lam, M, omega, alpha, mode, iters, lb_out, opts);
+  Chain ch = chain_for(ar, st);
+  dg_status s = enqueue_iterate(ar, ch, lam, M, omega, alpha, mode, iters, lb_out, opts);
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(st, &g);
   if (s != DG_OK) {
@@ -870,10 +884,11 @@ BwdLayout backward_layout(const dg_arena* ar, int iters, int ckpt_every) {
 // enqueue_iterate (the recording sweeps compute the same values), so lam, M
 // and the bound are bit-identical to k plain iterations.  With lb_out the last
 // backward sweep writes the energies and the bound follows.
-dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, float* M, const float* omega,
+dg_status enqueue_recorded_segment(dg_arena* ar, Chain& ch, float* lam, float* M, const float* omega,
                                    const float* alpha, int mode, int k, const BwdLayout& L, char* w, double* lb_out,
                                    const dg_options* opts) {
-  const DevArena& A = ar->dev;
+  DevArena A = ar->dev;
+  float* const own_S = A.S;
   const size_t NS = (size_t)ar->sizes.num_slots, n = (size_t)ar->sizes.n;
   SweepArgs fa{};
   fa.lam = lam;
@@ -882,12 +897,10 @@ dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, fl
   fa.alpha = alpha;
   fa.omega0 = omega_of(opts);
   fa.mode = mode;
-  cudaError_t e = cudaSuccess;
   ar->avg_mode = mode;
   for (int sw = 0; sw < 2 * k; ++sw) {
-    launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
-    if (e == cudaSuccess && n)
-      e = cudaMemcpyAsync(w + L.seg_S + (size_t)sw * n * 4, A.S, n * 4, cudaMemcpyDeviceToDevice, st);
+    A.S = (float*)(w + L.seg_S) + (size_t)sw * n;  // the sweep's snapshot stays there
+    launch_reduce_S(A, M, nullptr, nullptr, mode, false, ch, Scatter::kSweep);
     SweepArgs ra = fa;
     ra.rec_meta = (uint16_t*)(w + L.rec_meta + (size_t)sw * L.meta_stride);
     ra.rec_amin = (uint16_t*)(w + L.rec_amin) + (size_t)sw * (NS - (size_t)A.unit_slots);
@@ -905,11 +918,11 @@ dg_status enqueue_recorded_segment(dg_arena* ar, cudaStream_t st, float* lam, fl
     }
     if (lb_out && sw == 2 * k - 1) ra.E = A.E;
     launch_sweep(sw % 2 == 0 ? kFwdRec : kBwdRec, A, ra, threads_of(opts), ar->groups.data(), (int)ar->groups.size(),
-                 streams_for(ar, st));
+                 ch);
   }
-  launch_reduce_S(A, M, nullptr, nullptr, mode, false, st, Scatter::kNone);
-  if (lb_out) launch_lower_bound(A, lb_out, st);
-  if (e != cudaSuccess) return cuda_fail(e, "recorded segment copies");
+  A.S = own_S;
+  launch_reduce_S(A, M, nullptr, nullptr, mode, false, ch, Scatter::kNone);
+  if (lb_out) launch_lower_bound(A, lb_out, ch);
   return check_launch("recorded segment");
 }
 
@@ -953,9 +966,11 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
   const DevArena& A = ar->dev;
   if (iters > 0) ar->avg_mode = mode;
   const size_t NS = (size_t)ar->sizes.num_slots, n = (size_t)ar->sizes.n;
-  const size_t bNS = NS * 4, bn = n * 4;
+  const size_t bNS = NS * 4;
   cudaError_t e = cudaSuccess;
+  Chain ch = chain_for(ar, st);
   auto cpy = [&](void* d, const void* src, size_t bytes) {
+    ch.linked = false;
     if (e == cudaSuccess && bytes) e = cudaMemcpyAsync(d, src, bytes, cudaMemcpyDeviceToDevice, st);
   };
   if (g_omega) e = cudaMemsetAsync(g_omega, 0, bNS, st);
@@ -1001,7 +1016,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
     if (c + 1 == L.nseg) {
       // the last segment runs as recording sweeps right away
       if (e != cudaSuccess) return cuda_fail(e, "dg_backward copies");
-      if (dg_status s = enqueue_recorded_segment(ar, st, w_lam, w_M, omega, alpha, mode, iters - c * L.k, L, w,
+      if (dg_status s = enqueue_recorded_segment(ar, ch, w_lam, w_M, omega, alpha, mode, iters - c * L.k, L, w,
                                                  nullptr, opts))
         return s;
       break;
@@ -1012,10 +1027,10 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       f.cost_in = handed ? A.nodecost : nullptr;
       b.cost_in = A.nodecost;
       handed = true;
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
-      launch_sweep(kFwd, A, f, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
-      launch_sweep(kBwd, A, b, threads, ar->groups.data(), (int)ar->groups.size(), streams_for(ar, st));
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, ch, Scatter::kSweep);
+      launch_sweep(kFwd, A, f, threads, ar->groups.data(), (int)ar->groups.size(), ch);
+      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, ch, Scatter::kSweep);
+      launch_sweep(kBwd, A, b, threads, ar->groups.data(), (int)ar->groups.size(), ch);
     }
   }
   // 2. segments newest first: recompute every sweep of the segment as a
@@ -1048,8 +1063,9 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       cpy(w_M, ck_M + (size_t)c * NS, bNS);
     }
     for (int sw = 0; sw < (recorded ? 0 : nsw); ++sw) {
-      launch_reduce_S(A, w_M, nullptr, nullptr, mode, false, st, Scatter::kSweep);
-      cpy(seg_S + (size_t)sw * n, A.S, bn);
+      DevArena B = A;  // the sweep's snapshot of S is kept
+      B.S = seg_S + (size_t)sw * n;
+      launch_reduce_S(B, w_M, nullptr, nullptr, mode, false, ch, Scatter::kSweep);
       SweepArgs ra = fa;
       ra.rec_meta = (uint16_t*)(rec_meta + (size_t)sw * L.meta_stride);
       ra.rec_amin = rec_amin + (size_t)sw * (NS - (size_t)A.unit_slots);
@@ -1065,13 +1081,15 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
         ra.meta_in = (const uint16_t*)(rec_meta + (size_t)(sw - 1) * L.meta_stride);
         ra.lmeta_in = (const int32_t*)(w + L.rec_lmeta + (size_t)(sw - 1) * L.lmeta_stride);
       }
-      launch_sweep(sw % 2 == 0 ? kFwdRec : kBwdRec, A, ra, threads, ar->groups.data(), (int)ar->groups.size(),
-                   streams_for(ar, st));
+      launch_sweep(sw % 2 == 0 ? kFwdRec : kBwdRec, B, ra, threads, ar->groups.data(), (int)ar->groups.size(),
+                   ch);
     }
+    // as every call that sweeps, leave the last snapshot in the arena
+    if (!recorded && c == 0) cpy(A.S, seg_S + (size_t)(nsw - 1) * n, n * 4);
     // the per-slot inputs of the segment's last sweep: the S-dot handed over
     // from the adjoint of the segment after it (none after the last sweep)
     launch_slot_inputs(A, nullptr, 2 * it0 + nsw - 1 == last_sweep ? nullptr : sd_next, nullptr,
-                       seg_S + (size_t)(nsw - 1) * n, var_in, slot_in, st);
+                       seg_S + (size_t)(nsw - 1) * n, var_in, slot_in, ch);
     for (int sw = nsw - 1; sw >= 0; --sw) {
       const int gsw = 2 * it0 + sw;
       aa.rec_meta = (const uint16_t*)(rec_meta + (size_t)sw * L.meta_stride);
@@ -1085,10 +1103,10 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       aa.seed_M = gsw == last_sweep ? g_M_T : nullptr;
       aa.sdot_next = gsw == last_sweep ? nullptr : sd_next;
       launch_adjoint_sweep(sw % 2 == 0, A, aa, ar->adj_groups.data(), (int)ar->adj_groups.size(), ar->cta_smem_cap,
-                           streams_for(ar, st));
+                           ch);
       // S-dot of this sweep, and the next adjoint sweep's per-slot inputs
       launch_slot_inputs(A, sdot, nullptr, sd_cur, sw > 0 ? seg_S + (size_t)(sw - 1) * n : nullptr,
-                         sw > 0 ? var_in : nullptr, sw > 0 ? slot_in : nullptr, st);
+                         sw > 0 ? var_in : nullptr, sw > 0 ? slot_in : nullptr, ch);
       std::swap(sd_next, sd_cur);
     }
   }
@@ -1139,7 +1157,9 @@ dg_status dg_iterate_checkpointed(dg_arena* ar, void* stream, float* lam, float*
   cudaStream_t st = (cudaStream_t)stream;
   const size_t bNS = (size_t)ar->sizes.num_slots * 4;
   char* w = (char*)workspace;
+  Chain ch = chain_for(ar, st);
   for (int c = 0; c < L.nseg; ++c) {
+    ch.linked = false;
     cudaError_t e = cudaMemcpyAsync(w + L.ck_lam + (size_t)c * bNS, lam, bNS, cudaMemcpyDeviceToDevice, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(w + L.ck_M + (size_t)c * bNS, M, bNS, cudaMemcpyDeviceToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e, "dg_iterate_checkpointed copies");
@@ -1147,12 +1167,12 @@ dg_status dg_iterate_checkpointed(dg_arena* ar, void* stream, float* lam, float*
     if (c + 1 == L.nseg) {
       // the last segment's argmin records stay in the workspace, so that
       // dg_backward_checkpointed does not recompute that segment
-      if (dg_status s = enqueue_recorded_segment(ar, st, lam, M, omega, alpha, mode, k, L, w, lb_out, opts)) return s;
-    } else if (dg_status s = enqueue_iterate(ar, st, lam, M, omega, alpha, mode, k, nullptr, opts)) {
+      if (dg_status s = enqueue_recorded_segment(ar, ch, lam, M, omega, alpha, mode, k, L, w, lb_out, opts)) return s;
+    } else if (dg_status s = enqueue_iterate(ar, ch, lam, M, omega, alpha, mode, k, nullptr, opts)) {
       return s;
     }
   }
-  if (iters == 0) return enqueue_iterate(ar, st, lam, M, omega, alpha, mode, 0, lb_out, opts);
+  if (iters == 0) return enqueue_iterate(ar, ch, lam, M, omega, alpha, mode, 0, lb_out, opts);
   return DG_OK;
 }
 

@@ -70,21 +70,72 @@ struct StreamSet {
   void end() const;    // join
 };
 
+// One API call's work on a stream.  Kernels that begin with grid_wait() (below)
+// are launched through chain_launch: each may start while the one before it
+// drains, set up whatever does not depend on it (tile and shape records,
+// variable ids, slot lists) and only then wait for it, which hides the launch
+// latency that small instances consist of.  `linked`: the stream's last
+// operation is such a kernel of this call; anything else enqueued in between
+// (a copy, a fork) resets it.  Every chained kernel waits before it ends, so
+// that the end of one implies the end of all before it.
+struct Chain {
+  StreamSet ss;
+  bool linked = false;
+};
+template <class... P, class... X>
+void chain_launch(Chain& c, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, X... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = c.ss.main;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = c.linked ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  c.linked = true;
+}
+#ifdef __CUDACC__
+// Waits until the kernels before this one in its chain have ended and their
+// results are visible (at once when it was not launched into a chain).  Data
+// they wrote is read after it, by loads that are not read-only-cached.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the chain start once every block has come here.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
+// Whether a sweep's launches form one chain on the caller's stream instead of
+// forking onto the arena's streams: arenas of unit tiles only with one launch
+// group or up to kChainTiles tiles, and arenas of long unit BDDs only.  A small
+// arena's time is launch latency, which the chain hides (20 iterations of
+// tracking, us per iteration chained / forked: 50 frames, 9,500 tiles 52 / 57;
+// 4 batched instances, 5,000 tiles 25 / 36); a large one's launch groups share
+// the SMs better side by side, large shared-memory tiles next to narrow ones,
+// than one after another (100 frames, 19,000 tiles 88 / 82; 500 frames, 96,000
+// tiles 438 / 370).
+constexpr int kChainTiles = 16384;
+inline bool chained_sweeps(const DevArena& A, int num_groups) {
+  if (num_groups == 0) return A.num_long == A.num_long_unit;
+  return A.unit_slots == A.num_slots && (num_groups == 1 || A.num_tiles <= kChainTiles);
+}
+
 cudaError_t set_sweep_smem_limit(size_t bytes);
 cudaError_t set_unit_smem_limit(size_t bytes);
 // The launch of one group of unit tiles (kernels_unit.cu), wpc warps of
 // `region` bytes to a CTA.
 struct AdjArgs;
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
-                 cudaStream_t st);
+                 Chain& ch, bool late);
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
-                         cudaStream_t st);
+                         Chain& ch, bool late);
 // Dynamic shared memory one CTA may use; launchers put fewer warps in a CTA
 // when their tiles need more.
 void set_cta_smem_cap(size_t bytes);
 int best_warps_per_cta(size_t region, int max_wpc, size_t cta_cap);
 void launch_sweep(int kind, const DevArena& A, const SweepArgs& a, int threads, const LaunchGroup* groups,
-                  int num_groups, const StreamSet& ss);
+                  int num_groups, Chain& ch);
 
 // S_i = sum_{k in J_i} M_ik in fixed slot order; with renorm, also
 // lambda_ij += alpha_ij * (c_i - sum_k (lambda_ik + M_ik)) computed in FP64.
@@ -92,11 +143,12 @@ void launch_sweep(int kind, const DevArena& A, const SweepArgs& a, int threads, 
 // the sweep reads it from: those of the mixed tiles and the long BDDs before
 // a sweep (the unit tiles gather S or Sbar themselves).
 enum class Scatter { kNone, kSweep };
+constexpr int kNeedS = 1, kNeedSbar = 2;  // which of S and Sbar the reduction stores
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
-                     cudaStream_t st, Scatter to);
+                     Chain& ch, Scatter to, int need = kNeedS | kNeedSbar);
 void launch_init(const DevArena& A, float* lam, float* M, cudaStream_t st);
 // per-instance FP64 lower bound from A.E and A.S
-void launch_lower_bound(const DevArena& A, double* lb_out, cudaStream_t st);
+void launch_lower_bound(const DevArena& A, double* lb_out, Chain& ch);
 void launch_seed_M(const DevArena& A, float* g_M, cudaStream_t st);
 
 // Backpropagation through one sweep (kernels_adjoint.cu).
@@ -133,14 +185,14 @@ struct AdjArgs {
 };
 cudaError_t set_adjoint_smem_limit(size_t bytes);
 void launch_adjoint_sweep(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup* groups, int num_groups,
-                          size_t cta_smem_cap, const StreamSet& ss);
+                          size_t cta_smem_cap, Chain& ch);
 // Per variable i: s_i = sum over the slots q of i of x[q] (fixed order), or
 // sd_in[i] when x is NULL (0 when both are); out_var[i] = s_i (nullable);
 // and, when var_in is not NULL, {s_i, S_var[i] (0 if NULL)} in var_in[i] and
 // in slot_in[q] for every slot q >= unit_slots of i (the unit tiles gather
 // var_in, the mixed tiles read slot_in).
 void launch_slot_inputs(const DevArena& A, const float* x, const float* sd_in, float* out_var, const float* S_var,
-                        float2* var_in, float2* slot_in, cudaStream_t st);
+                        float2* var_in, float2* slot_in, Chain& ch);
 // A.slot_invdeg[q] = 1/|J_i| of the variable of slot q (0 for padding)
 void launch_fill_slot_invdeg(const DevArena& A, cudaStream_t st);
 // out_slot[q] = v[variable of q] (0 for padding slots)
@@ -161,14 +213,14 @@ void launch_param_transform_bwd(const DevArena& A, const float* alpha, const flo
 // Long BDDs, one warp per BDD (kernels_long.cu); each is a single launch on
 // the given stream, or nothing when the arena has no long BDDs.
 cudaError_t set_long_unit_smem_limit(size_t bytes);
-void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st);
-void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st);
+void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, Chain& ch);
+void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, Chain& ch);
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st);
 void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, cudaStream_t st);
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st);
 
 // dg_lower_bound with its intermediates in a static device array (noalloc.cu).
 dg_status lower_bound_noalloc(const DevArena& arena, const LaunchGroup* groups, int num_groups, int threads,
-                              const StreamSet& ss, const float* lam, const float* M, double* lb);
+                              Chain& ch, const float* lam, const float* M, double* lb);
 
 }  // namespace dg

@@ -246,16 +246,29 @@ cudaError_t set_adjoint_smem_limit(size_t bytes) {
 
 template <int FWD, int MODE>
 static void launch_adj(const DevArena& A, const AdjArgs& a, const AdjGroup* groups, int num_groups, size_t cap,
-                       const StreamSet& ss) {
-  const bool fork = num_groups + (A.num_long > 0 ? 1 : 0) > 1 && ss.ready;
+                       Chain& ch) {
+  const bool chained = chained_sweeps(A, num_groups);
+  const StreamSet& ss = ch.ss;
+  const bool fork = !chained && num_groups + (A.num_long > 0 ? 1 : 0) > 1 && ss.ready;
   if (fork) ss.begin();
-  launch_long_adjoint(FWD != 0, A, a, fork ? ss.of(A.long_stream) : ss.main);
+  if (!chained) {
+    ch.linked = false;
+    launch_long_adjoint(FWD != 0, A, a, fork ? ss.of(A.long_stream) : ss.main);
+  } else if (A.num_long_items > 0) {
+    launch_long_unit_adjoint(FWD != 0, A, a, ch);
+  }
   for (int g = 0; g < num_groups; ++g) {
     const AdjGroup& G = groups[g];
     const size_t region = (size_t)G.region;
     const int wpc = best_warps_per_cta(region, 4, cap);
     if (G.unit_w > 0) {
-      launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, fork ? ss.of(G.stream) : ss.main);
+      if (chained) {
+        launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, ch, g > 0);
+      } else {
+        Chain own;
+        own.ss.main = fork ? ss.of(G.stream) : ss.main;
+        launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, own, false);
+      }
       continue;
     }
     const int nt = G.tile1 - G.tile0;
@@ -266,7 +279,7 @@ static void launch_adj(const DevArena& A, const AdjArgs& a, const AdjGroup* grou
 }
 
 void launch_adjoint_sweep(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup* groups, int num_groups,
-                          size_t cta_smem_cap, const StreamSet& st) {
+                          size_t cta_smem_cap, Chain& st) {
   if (forward)
     a.mode == 1 ? launch_adj<1, 1>(A, a, groups, num_groups, cta_smem_cap, st)
                 : launch_adj<1, 0>(A, a, groups, num_groups, cta_smem_cap, st);

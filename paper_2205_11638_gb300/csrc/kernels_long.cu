@@ -834,7 +834,11 @@ void launch_long_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
 }  // namespace
 
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (A.num_long_items > 0) launch_long_unit(kind, A, a, st);
+  if (A.num_long_items > 0) {
+    Chain ch;
+    ch.ss.main = st;
+    launch_long_unit(kind, A, a, ch);
+  }
   if (A.num_long == A.num_long_unit) return;
   switch (kind) {
     case kFwd: launch_long_kind<kFwd>(A, a, st); break;
@@ -853,7 +857,11 @@ void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float*
 }
 
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st) {
-  if (A.num_long_items > 0) launch_long_unit_adjoint(forward, A, a, st);
+  if (A.num_long_items > 0) {
+    Chain ch;
+    ch.ss.main = st;
+    launch_long_unit_adjoint(forward, A, a, ch);
+  }
   if (A.num_long == A.num_long_unit) return;
   const int g = long_grid_other(A), t = kLongWarps * kWarp;
   if (forward)

@@ -174,6 +174,8 @@ __device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArg
     }
     cp_async_commit();
   }
+  grid_wait();
+  grid_trigger();
   for (int r = 0; r < it.nseg; ++r) {
     const LongBdd B = A.longs[A.long_order[it.first + r]];
     copy_row(lam + r * ST, a.lam + B.slot_base, B.k, lane, pol);
@@ -429,6 +431,8 @@ __device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const 
     copy_row(id + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
   }
   cp_async_commit();
+  grid_wait();
+  grid_trigger();
   for (int r = 0; r < it.nseg; ++r) {
     const LongBdd B = A.longs[A.long_order[it.first + r]];
     copy_row(gl + r * ST, a.g_lam + B.slot_base, B.k, lane, pol);
@@ -607,11 +611,9 @@ __global__ void __launch_bounds__(32) k_long_unit_adjoint(DevArena A, AdjArgs a)
 }
 
 template <int KIND>
-void launch_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (a.mode == 1)
-    k_long_unit<KIND, 1><<<A.num_long_items, kWarp, A.long_unit_smem[1], st>>>(A, a);
-  else
-    k_long_unit<KIND, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a);
+void launch_kind(const DevArena& A, const SweepArgs& a, Chain& ch) {
+  chain_launch(ch, a.mode == 1 ? k_long_unit<KIND, 1> : k_long_unit<KIND, 0>, A.num_long_items, kWarp,
+               A.long_unit_smem[a.mode == 1], A, a);
 }
 
 }  // namespace
@@ -637,24 +639,22 @@ cudaError_t set_long_unit_smem_limit(size_t bytes) {
   return e;
 }
 
-void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st) {
+void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, Chain& ch) {
   switch (kind) {
-    case kFwd: launch_kind<kFwd>(A, a, st); break;
-    case kBwd: launch_kind<kBwd>(A, a, st); break;
-    case kFwdRec: launch_kind<kFwdRec>(A, a, st); break;
-    case kBwdRec: launch_kind<kBwdRec>(A, a, st); break;
-    case kMinMarg: k_long_unit<kMinMarg, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a); break;
-    case kEnergy: k_long_unit<kEnergy, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a); break;
-    default: k_long_unit<kSeed, 0><<<A.num_long_items, kWarp, A.long_unit_smem[0], st>>>(A, a); break;
+    case kFwd: launch_kind<kFwd>(A, a, ch); break;
+    case kBwd: launch_kind<kBwd>(A, a, ch); break;
+    case kFwdRec: launch_kind<kFwdRec>(A, a, ch); break;
+    case kBwdRec: launch_kind<kBwdRec>(A, a, ch); break;
+    case kMinMarg: chain_launch(ch, k_long_unit<kMinMarg, 0>, A.num_long_items, kWarp, A.long_unit_smem[0], A, a); break;
+    case kEnergy: chain_launch(ch, k_long_unit<kEnergy, 0>, A.num_long_items, kWarp, A.long_unit_smem[0], A, a); break;
+    default: chain_launch(ch, k_long_unit<kSeed, 0>, A.num_long_items, kWarp, A.long_unit_smem[0], A, a); break;
   }
 }
 
-void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st) {
-  const int G = A.num_long_items, b = A.long_unit_adj_smem;
-  if (forward)
-    a.mode == 1 ? k_long_unit_adjoint<1, 1><<<G, kWarp, b, st>>>(A, a) : k_long_unit_adjoint<1, 0><<<G, kWarp, b, st>>>(A, a);
-  else
-    a.mode == 1 ? k_long_unit_adjoint<0, 1><<<G, kWarp, b, st>>>(A, a) : k_long_unit_adjoint<0, 0><<<G, kWarp, b, st>>>(A, a);
+void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, Chain& ch) {
+  auto k = forward ? (a.mode == 1 ? k_long_unit_adjoint<1, 1> : k_long_unit_adjoint<1, 0>)
+                   : (a.mode == 1 ? k_long_unit_adjoint<0, 1> : k_long_unit_adjoint<0, 0>);
+  chain_launch(ch, k, A.num_long_items, kWarp, A.long_unit_adj_smem, A, a);
 }
 
 }  // namespace dg

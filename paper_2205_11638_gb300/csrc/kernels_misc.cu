@@ -7,59 +7,116 @@
 
 namespace dg {
 
-// S_i = sum_{j in J_i} M_ij over the variable's slots in fixed order.  With
-// renorm the same pass re-projects lambda onto sum_j (lambda_ij + M_ij) = c_i
-// (the invariant of the proof of Prop. 1): the FP64 residual
-// r_i = c_i - sum_j (lambda_ij + M_ij) is spread with the averaging weights.
-// With SCATTER every slot of the variable also receives the averaging term
-// the sweeps add (Sbar_i = S_i / |J_i| in mode 0, S_i in mode 1, which they
-// multiply by alpha_ij), so that a sweep reads it with the slot's other
-// inputs instead of gathering it per variable.  Slots below scatter_from are
-// left out: the unit tiles' sweeps gather S or Sbar themselves.
-template <bool RENORM, bool SCATTER>
-__global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* __restrict__ M, float* lam,
-                                                   const float* __restrict__ alpha, int mode, int scatter_from) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.n) return;
+// x[q] summed over the slots of one variable in fixed order: the first kEll
+// slots (q, from the ELL columns, -1 past the end), then var_slots[b .. e).
+// The loads of a batch are all issued before its first addition; the order of
+// the additions is the plain loop's.
+__device__ __forceinline__ float sum_slots(const DevArena& A, const float* x, const int (&q)[kEll], int b, int e) {
+  float v[kEll], s = 0.f;
+#pragma unroll
+  for (int r = 0; r < kEll; ++r) v[r] = q[r] >= 0 ? x[q[r]] : 0.f;
+#pragma unroll
+  for (int r = 0; r < kEll; ++r)
+    if (q[r] >= 0) s += v[r];
+  constexpr int kB = 8;
+  for (int k = b; k < e; k += kB) {
+    int p[kB];
+    float w[kB];
+#pragma unroll
+    for (int j = 0; j < kB; ++j) p[j] = k + j < e ? __ldg(A.var_slots + k + j) : -1;
+#pragma unroll
+    for (int j = 0; j < kB; ++j) w[j] = p[j] >= 0 ? x[p[j]] : 0.f;
+#pragma unroll
+    for (int j = 0; j < kB; ++j)
+      if (p[j] >= 0) s += w[j];
+  }
+  return s;
+}
+
+// ... by a warp, for the wide variables: the lanes load 32 values at a time
+// and every lane adds them in slot order (the same sum to the bit).
+__device__ __forceinline__ float sum_slots_warp(const DevArena& A, const float* x, int b, int e, int lane) {
   float s = 0.f;
-  if (!RENORM) {
-    // the first kEll slots come from the ELL columns (coalesced, no var_ptr
-    // needed), all loaded before their M values, which are all loaded before
-    // the first addition; the order of additions is the plain loop's
-    int q[kEll];
+  for (int c = b; c < e; c += 32) {
+    const float v = c + lane < e ? x[__ldg(A.var_slots + c + lane)] : 0.f;
+    const int cnt = min(32, e - c);
+    for (int j = 0; j < cnt; ++j) s += __shfl_sync(0xffffffffu, v, j);
+  }
+  return s;
+}
+
+// The first kEll slots of variable i; returns whether there are more.
+__device__ __forceinline__ bool ell_slots(const DevArena& A, int i, int (&q)[kEll]) {
 #pragma unroll
-    for (int r = 0; r < kEll; ++r) q[r] = __ldg(A.var_ell + (int64_t)r * A.n + i);
-    const bool more = q[kEll - 1] <= -2;
-    if (more) q[kEll - 1] = -2 - q[kEll - 1];
-    float mv[kEll];
-#pragma unroll
-    for (int r = 0; r < kEll; ++r) mv[r] = q[r] >= 0 ? M[q[r]] : 0.f;
-#pragma unroll
-    for (int r = 0; r < kEll; ++r)
-      if (q[r] >= 0) s += mv[r];
-    int b = 0, e = 0;
-    if (more) {
+  for (int r = 0; r < kEll; ++r) q[r] = __ldg(A.var_ell + (int64_t)r * A.n + i);
+  const bool more = q[kEll - 1] <= -2;
+  if (more) q[kEll - 1] = -2 - q[kEll - 1];
+  return more;
+}
+
+// S_i = sum_{j in J_i} M_ij over the variable's slots in fixed order.  Blocks
+// below nblk take a variable per thread, the others a wide variable (more than
+// kWide slots) per warp.  `need`: which of S and Sbar to store.  With SCATTER
+// every slot in [from, to) of the variable also receives the averaging term a
+// sweep adds (Sbar_i = S_i / |J_i| in mode 0, S_i in mode 1, which it
+// multiplies by alpha_ij); the unit rows' sweeps gather S or Sbar instead,
+// which halves the reduction's random accesses.
+template <bool SCATTER>
+__global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* M, int mode, int need, int from, int to,
+                                                   int nblk) {
+  const bool wide = (int)blockIdx.x >= nblk;
+  const int lane = threadIdx.x & 31;
+  const int x = (wide ? (int)blockIdx.x - nblk : (int)blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
+  int i, b = 0, e = 0, q[kEll] = {-1, -1, -1, -1};
+  bool mine = true;
+  if (wide) {
+    const int w = x >> 5;
+    mine = w < A.num_wide;  // uniform in the warp
+    i = mine ? __ldg(A.wide_vars + w) : 0;
+    b = mine ? __ldg(A.var_ptr + i) : 0;
+    e = mine ? __ldg(A.var_ptr + i + 1) : 0;
+  } else {
+    i = x;
+    mine = i < A.n;
+    if (mine && ell_slots(A, i, q)) {
       b = __ldg(A.var_ptr + i) + kEll;
       e = __ldg(A.var_ptr + i + 1);
-      if (e - b > kWide - kEll) return;  // a wide variable: k_reduce_wide's
-      for (int k = b; k < e; ++k) s += M[__ldg(A.var_slots + k)];
+      mine = e - b <= kWide - kEll;  // else a wide variable
     }
-    const float sbar = __ldg(A.invdeg + i) * s;
-    A.S[i] = s;
-    A.Sbar[i] = sbar;
-    if (SCATTER) {
-      const float t = mode == 1 ? s : sbar;
+  }
+  grid_wait();
+  grid_trigger();
+  if (!mine) return;
+  const float s = wide ? sum_slots_warp(A, M, b, e, lane) : sum_slots(A, M, q, b, e);
+  const float sbar = __ldg(A.invdeg + i) * s;
+  if (!wide || lane == 0) {
+    if (need & kNeedS) A.S[i] = s;
+    if (need & kNeedSbar) A.Sbar[i] = sbar;
+  }
+  if (SCATTER) {
+    const float t = mode == 1 ? s : sbar;
+    if (!wide) {
 #pragma unroll
       for (int r = 0; r < kEll; ++r)
-        if (q[r] >= scatter_from) A.slot_avg[q[r]] = t;
-      for (int k = b; k < e; ++k) {
-        const int qk = __ldg(A.var_slots + k);
-        if (qk >= scatter_from) A.slot_avg[qk] = t;
-      }
+        if (q[r] >= from && q[r] < to) A.slot_avg[q[r]] = t;
     }
-    return;
+    for (int k = b + (wide ? lane : 0); k < e; k += wide ? 32 : 1) {
+      const int p = __ldg(A.var_slots + k);
+      if (p >= from && p < to) A.slot_avg[p] = t;
+    }
   }
+}
+
+// The reduction with the re-projection of lambda onto sum_j (lambda_ij + M_ij)
+// = c_i (the invariant of the proof of Prop. 1): the FP64 residual
+// r_i = c_i - sum_j (lambda_ij + M_ij) is spread with the averaging weights.
+template <bool SCATTER>
+__global__ void __launch_bounds__(256) k_reduce_renorm(DevArena A, const float* __restrict__ M, float* lam,
+                                                        const float* __restrict__ alpha, int mode, int from, int to) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= A.n) return;
   const int b = __ldg(A.var_ptr + i), e = __ldg(A.var_ptr + i + 1);
+  float s = 0.f;
   double tot = 0.0;
   for (int k = b; k < e; ++k) {
     const int q = __ldg(A.var_slots + k);
@@ -78,39 +135,7 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* __res
       const int q = __ldg(A.var_slots + k);
       const double w = mode == 1 ? (double)alpha[q] : (double)inv;
       lam[q] = (float)((double)lam[q] + w * r);
-      if (SCATTER && q >= scatter_from) A.slot_avg[q] = t;
-    }
-  }
-}
-
-// k_reduce_S<false, SCATTER> for the wide variables (more than kWide slots),
-// one warp each: the lanes load 32 of the variable's M values at a time and
-// every lane adds them in slot order (the plain loop's order, so S is the
-// same to the bit); lane 0 stores S.
-template <bool SCATTER>
-__global__ void __launch_bounds__(256) k_reduce_wide(DevArena A, const float* __restrict__ M, int mode,
-                                                     int scatter_from) {
-  constexpr unsigned kAll = 0xffffffffu;
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (w >= A.num_wide) return;  // the whole warp
-  const int i = __ldg(A.wide_vars + w);
-  const int b = __ldg(A.var_ptr + i), e = __ldg(A.var_ptr + i + 1);
-  float s = 0.f;
-  for (int c = b; c < e; c += 32) {
-    const float v = c + lane < e ? M[__ldg(A.var_slots + c + lane)] : 0.f;
-    const int cnt = min(32, e - c);
-    for (int j = 0; j < cnt; ++j) s += __shfl_sync(kAll, v, j);
-  }
-  const float sbar = __ldg(A.invdeg + i) * s;
-  if (lane == 0) {
-    A.S[i] = s;
-    A.Sbar[i] = sbar;
-  }
-  if (SCATTER) {
-    const float t = mode == 1 ? s : sbar;
-    for (int k = b + lane; k < e; k += 32) {
-      const int qk = __ldg(A.var_slots + k);
-      if (qk >= scatter_from) A.slot_avg[qk] = t;
+      if (SCATTER && q >= from && q < to) A.slot_avg[q] = t;
     }
   }
 }
@@ -136,6 +161,8 @@ __global__ void k_init(DevArena A, float* lam, float* M) {
 // error, both float32), and only the per-thread results are combined in
 // FP64, in a fixed order (deterministic for a given layout).
 __global__ void __launch_bounds__(256) k_lb_partial(DevArena A) {
+  grid_wait();
+  grid_trigger();
   const int4 ch = __ldg(A.lb_chunks + blockIdx.x);
   float hi = 0.f, lo = 0.f;
   // variables no row covers have S_i = 0 (an empty sum), so min(0, S_i) adds
@@ -186,6 +213,8 @@ __global__ void __launch_bounds__(256) k_lb_partial(DevArena A) {
 // One CTA per instance sums the instance's chunk partials (strided per
 // thread, then a fixed tree): deterministic for a given layout.
 __global__ void __launch_bounds__(256) k_lb_final(DevArena A, double* lb) {
+  grid_wait();
+  grid_trigger();
   const int k = blockIdx.x;
   double t = 0.0;
   for (int c = A.inst_chunk_ptr[k] + threadIdx.x; c < A.inst_chunk_ptr[k + 1]; c += blockDim.x) t += A.lb_part[c];
@@ -209,62 +238,53 @@ __global__ void k_seed_M(DevArena A, float* gM) {
 }
 
 // Between two adjoint sweeps: the S-dot of a variable (sum of its slots'
-// contributions) and the per-slot inputs of the next adjoint sweep.
-__global__ void __launch_bounds__(256) k_slot_inputs(DevArena A, const float* __restrict__ x,
-                                                      const float* __restrict__ sd_in, float* out_var,
-                                                      const float* __restrict__ S_var, float2* var_in,
-                                                      float2* slot_in) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= A.n) return;
-  const int b = __ldg(A.var_ptr + i), e = __ldg(A.var_ptr + i + 1);
-  if (e - b > kWide) return;  // a wide variable: k_slot_inputs_wide's
+// contributions) and the inputs of the next adjoint sweep.  Blocks as in
+// k_reduce_S.
+__global__ void __launch_bounds__(256) k_slot_inputs(DevArena A, const float* x, const float* sd_in, float* out_var,
+                                                      const float* S_var, float2* var_in, float2* slot_in, int nblk) {
+  const bool wide = (int)blockIdx.x >= nblk;
+  const int lane = threadIdx.x & 31;
+  const int t = (wide ? (int)blockIdx.x - nblk : (int)blockIdx.x) * (int)blockDim.x + (int)threadIdx.x;
+  int i, b = 0, e = 0, q[kEll] = {-1, -1, -1, -1};
+  bool mine = true;
+  if (wide) {
+    const int w = t >> 5;
+    mine = w < A.num_wide;
+    i = mine ? __ldg(A.wide_vars + w) : 0;
+    b = mine ? __ldg(A.var_ptr + i) : 0;
+    e = mine ? __ldg(A.var_ptr + i + 1) : 0;
+  } else {
+    i = t;
+    mine = i < A.n;
+    if (mine && ell_slots(A, i, q)) {
+      b = __ldg(A.var_ptr + i) + kEll;
+      e = __ldg(A.var_ptr + i + 1);
+      mine = e - b <= kWide - kEll;
+    }
+  }
+  grid_wait();
+  grid_trigger();
+  if (!mine) return;
   float s = 0.f;
   if (x)
-    for (int k = b; k < e; ++k) s += x[__ldg(A.var_slots + k)];
+    s = wide ? sum_slots_warp(A, x, b, e, lane) : sum_slots(A, x, q, b, e);
   else if (sd_in)
     s = sd_in[i];
-  if (out_var) out_var[i] = s;
+  if (out_var && (!wide || lane == 0)) out_var[i] = s;
   if (var_in) {
-    const float2 t = make_float2(s, S_var ? S_var[i] : 0.f);
-    var_in[i] = t;
-    if (slot_in)
-      for (int k = b; k < e; ++k) {
-        const int q = __ldg(A.var_slots + k);
-        if (q >= A.unit_slots) slot_in[q] = t;
+    const float2 v = make_float2(s, S_var ? S_var[i] : 0.f);
+    if (!wide || lane == 0) var_in[i] = v;
+    if (slot_in) {
+      if (!wide) {
+#pragma unroll
+        for (int r = 0; r < kEll; ++r)
+          if (q[r] >= A.unit_slots) slot_in[q[r]] = v;
       }
-  }
-}
-
-// k_slot_inputs for the wide variables, one warp each (the sum in slot order
-// as in k_reduce_wide).
-__global__ void __launch_bounds__(256) k_slot_inputs_wide(DevArena A, const float* __restrict__ x,
-                                                           const float* __restrict__ sd_in, float* out_var,
-                                                           const float* __restrict__ S_var, float2* var_in,
-                                                      float2* slot_in) {
-  constexpr unsigned kAll = 0xffffffffu;
-  const int w = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (w >= A.num_wide) return;  // the whole warp
-  const int i = __ldg(A.wide_vars + w);
-  const int b = __ldg(A.var_ptr + i), e = __ldg(A.var_ptr + i + 1);
-  float s = 0.f;
-  if (x) {
-    for (int c = b; c < e; c += 32) {
-      const float v = c + lane < e ? x[__ldg(A.var_slots + c + lane)] : 0.f;
-      const int cnt = min(32, e - c);
-      for (int j = 0; j < cnt; ++j) s += __shfl_sync(kAll, v, j);
+      for (int k = b + (wide ? lane : 0); k < e; k += wide ? 32 : 1) {
+        const int p = __ldg(A.var_slots + k);
+        if (p >= A.unit_slots) slot_in[p] = v;
+      }
     }
-  } else if (sd_in) {
-    s = sd_in[i];
-  }
-  if (out_var && lane == 0) out_var[i] = s;
-  if (var_in) {
-    const float2 t = make_float2(s, S_var ? S_var[i] : 0.f);
-    if (lane == 0) var_in[i] = t;
-    if (slot_in)
-      for (int k = b + lane; k < e; k += 32) {
-        const int q = __ldg(A.var_slots + k);
-        if (q >= A.unit_slots) slot_in[q] = t;
-      }
   }
 }
 
@@ -288,14 +308,23 @@ __global__ void k_gather_var(DevArena A, const float* __restrict__ v, float* out
   out[q] = var >= 0 ? v[var] : 0.f;
 }
 
+// Threads per block of the per-variable kernels, blocks over all variables and
+// over the wide ones (a warp each).
+constexpr int kVarThreads = 256;
+static int var_blocks(const DevArena& A) { return (A.n + kVarThreads - 1) / kVarThreads; }
+static int wide_blocks(const DevArena& A) { return (A.num_wide + kVarThreads / 32 - 1) / (kVarThreads / 32); }
+// The slots whose averaging term the sweeps read per slot: the mixed tiles',
+// and the long BDDs' unless all of them are unit rows.
+static int scatter_to(const DevArena& A) {
+  return A.num_long == A.num_long_unit ? A.long_slot_base : (int)A.num_slots;
+}
+
 void launch_slot_inputs(const DevArena& A, const float* x, const float* sd_in, float* out_var, const float* S_var,
-                        float2* var_in, float2* slot_in, cudaStream_t st) {
-  const int T = 256;
-  const int G = (A.n + T - 1) / T;
-  if (A.unit_slots >= A.num_slots) slot_in = nullptr;  // no slot reads it
-  if (G > 0) k_slot_inputs<<<G, T, 0, st>>>(A, x, sd_in, out_var, S_var, var_in, slot_in);
-  if (A.num_wide > 0)
-    k_slot_inputs_wide<<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, x, sd_in, out_var, S_var, var_in, slot_in);
+                        float2* var_in, float2* slot_in, Chain& ch) {
+  if (A.unit_slots >= scatter_to(A)) slot_in = nullptr;  // no slot reads it
+  const int G = var_blocks(A);
+  if (G > 0)
+    chain_launch(ch, k_slot_inputs, G + wide_blocks(A), kVarThreads, 0, A, x, sd_in, out_var, S_var, var_in, slot_in, G);
 }
 
 void launch_gather_var(const DevArena& A, const float* v, float* out_slot, cudaStream_t st) {
@@ -305,21 +334,18 @@ void launch_gather_var(const DevArena& A, const float* v, float* out_slot, cudaS
 }
 
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
-                     cudaStream_t st, Scatter to) {
-  const int T = 256;
-  const int G = (A.n + T - 1) / T;
+                     Chain& ch, Scatter to, int need) {
+  const int G = var_blocks(A);
   if (G == 0) return;
-  const int from = A.unit_slots;
-  const bool scatter = to == Scatter::kSweep && from < A.num_slots;
-  if (renorm)
-    scatter ? k_reduce_S<true, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from)
-            : k_reduce_S<true, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from);
-  else {
-    scatter ? k_reduce_S<false, true><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from)
-            : k_reduce_S<false, false><<<G, T, 0, st>>>(A, M, lam, alpha, mode, from);
-    if (A.num_wide > 0)
-      scatter ? k_reduce_wide<true><<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, M, mode, from)
-              : k_reduce_wide<false><<<(A.num_wide + 7) / 8, 256, 0, st>>>(A, M, mode, from);
+  const int from = A.unit_slots, end = scatter_to(A);
+  const bool scatter = to == Scatter::kSweep && from < end;
+  if (renorm) {
+    ch.linked = false;
+    scatter ? k_reduce_renorm<true><<<G, kVarThreads, 0, ch.ss.main>>>(A, M, lam, alpha, mode, from, end)
+            : k_reduce_renorm<false><<<G, kVarThreads, 0, ch.ss.main>>>(A, M, lam, alpha, mode, from, end);
+  } else {
+    chain_launch(ch, scatter ? k_reduce_S<true> : k_reduce_S<false>, G + wide_blocks(A), kVarThreads, 0, A, M, mode,
+                 need, from, end, G);
   }
 }
 
@@ -329,9 +355,9 @@ void launch_init(const DevArena& A, float* lam, float* M, cudaStream_t st) {
   if (G > 0) k_init<<<(unsigned)G, T, 0, st>>>(A, lam, M);
 }
 
-void launch_lower_bound(const DevArena& A, double* lb, cudaStream_t st) {
-  if (A.num_lb_chunks > 0) k_lb_partial<<<A.num_lb_chunks, 256, 0, st>>>(A);
-  k_lb_final<<<A.num_inst, 256, 0, st>>>(A, lb);
+void launch_lower_bound(const DevArena& A, double* lb, Chain& ch) {
+  if (A.num_lb_chunks > 0) chain_launch(ch, k_lb_partial, A.num_lb_chunks, 256, 0, A);
+  chain_launch(ch, k_lb_final, A.num_inst, 256, 0, A, lb);
 }
 
 void launch_seed_M(const DevArena& A, float* gM, cudaStream_t st) {

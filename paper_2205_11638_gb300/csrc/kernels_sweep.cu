@@ -414,11 +414,18 @@ void StreamSet::end() const {
 
 template <int KIND, int MODE>
 static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, const LaunchGroup* groups,
-                          int num_groups, const StreamSet& ss) {
-  const bool fork = num_groups + (A.num_long > 0 ? 1 : 0) > 1 && ss.ready;
+                          int num_groups, Chain& ch) {
+  const bool chained = chained_sweeps(A, num_groups);
+  const StreamSet& ss = ch.ss;
+  const bool fork = !chained && num_groups + (A.num_long > 0 ? 1 : 0) > 1 && ss.ready;
   if (fork) ss.begin();
-  // the long BDDs first: their launch is a few warps walking long chains
-  launch_long_sweep(KIND, A, a, fork ? ss.of(A.long_stream) : ss.main);
+  if (!chained) {
+    // the long BDDs first: their launch is a few warps walking long chains
+    ch.linked = false;
+    launch_long_sweep(KIND, A, a, fork ? ss.of(A.long_stream) : ss.main);
+  } else if (A.num_long_items > 0) {
+    launch_long_unit(KIND, A, a, ch);
+  }
   for (int g = 0; g < num_groups; ++g) {
     const LaunchGroup& G = groups[g];
     constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
@@ -436,7 +443,13 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
     else
       wpc = best_warps_per_cta(region, wpc, g_cta_smem_cap);
     if (unit) {
-      launch_unit(KIND, A, a, G, wpc, region, fork ? ss.of(G.stream) : ss.main);
+      if (chained) {
+        launch_unit(KIND, A, a, G, wpc, region, ch, g > 0);
+      } else {
+        Chain own;
+        own.ss.main = fork ? ss.of(G.stream) : ss.main;
+        launch_unit(KIND, A, a, G, wpc, region, own, false);
+      }
       continue;
     }
     const int nt = G.tile1 - G.tile0;
@@ -451,7 +464,7 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
 // sweeps one tile with its own slice of the group's shared memory.  Only
 // the update sweeps read omega/alpha, so only they have a mode-1 variant.
 void launch_sweep(int kind, const DevArena& A, const SweepArgs& a, int threads, const LaunchGroup* groups,
-                  int num_groups, const StreamSet& st) {
+                  int num_groups, Chain& st) {
   const bool m1 = a.mode == 1;
   switch (kind) {
     case kFwd:

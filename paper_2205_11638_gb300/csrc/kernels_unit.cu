@@ -173,7 +173,8 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
 }
 
 template <int KIND, int MODE, int WMAX>
-__global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int region_bytes, int tile0, int tile1) {
+__global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int region_bytes, int tile0, int tile1,
+                                              int late) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
@@ -184,6 +185,10 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
   const int k = T.nhops;
   float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
   const uint64_t pol = l2_evict_first();
+  // A late group of a sweep starts when the group before it has waited for the
+  // kernel before the sweep (its trigger comes after), so only at its end does
+  // it wait: for that group.
+  if (late) grid_trigger();
   // the variable ids come first, into the words of the averaging terms, so
   // that the gather can follow as soon as they are there: two memory latencies
   // per tile whatever its length (ids loaded into registers a few levels at a
@@ -192,13 +197,17 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
     copy_rows<STRIDE>(m + kAvg, A.slot_var + T.slot_base, k, lane, pol);
     cp_async_commit();
   }
+  const UnitShape S = A.unit_shapes[T.unit - 1];
+  if (!late) {
+    grid_wait();
+    grid_trigger();
+  }
   copy_rows<STRIDE>(m, a.lam + T.slot_base, k, lane, pol);
   if (UPDATE && MODE == 1) {
     copy_rows<STRIDE>(m + kOm, a.omega + T.slot_base, k, lane, pol);
     copy_rows<STRIDE>(m + kAl, a.alpha + T.slot_base, k, lane, pol);
   }
   cp_async_commit();
-  const UnitShape S = A.unit_shapes[T.unit - 1];
   if (UPDATE) {
     cp_async_wait_one();
     __syncwarp();
@@ -226,6 +235,7 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
     unit_tile<KIND, MODE, 6>(A, a, T, S, m, lane);
   else if (WMAX >= 8)
     unit_tile<KIND, MODE, 8>(A, a, T, S, m, lane);
+  if (late) grid_wait();
 }
 
 // ---- adjoint of a recording sweep (see kernels_adjoint.cu) -----------------
@@ -341,7 +351,8 @@ __device__ __forceinline__ void unit_adjoint_tile(const AdjArgs& a, const Tile& 
 }
 
 template <int FWD, int MODE, int WMAX>
-__global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int region_bytes, int tile0, int tile1) {
+__global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int region_bytes, int tile0, int tile1,
+                                                      int late) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int STRIDE = kWarp * (MODE == 1 ? 7 : 6);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -351,15 +362,20 @@ __global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int
   const int k = T.nhops;
   float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
   const uint64_t pol = l2_evict_first();
+  if (late) grid_trigger();  // see k_unit
   copy_rows<STRIDE>(m + kJIn, A.slot_var + T.slot_base, k, lane, pol);
   cp_async_commit();
+  const UnitShape S = A.unit_shapes[T.unit - 1];
+  if (!late) {
+    grid_wait();
+    grid_trigger();
+  }
   copy_rows<STRIDE>(m, a.g_lam + T.slot_base, k, lane, pol);
   copy_rows<STRIDE>(m + kJRec, a.rec_unit + T.slot_base, k, lane, pol);
   copy_rows<STRIDE>(m + kJDiff, a.rec_diff + T.slot_base, k, lane, pol);
   copy_rows<STRIDE>(m + kJAl, (MODE == 1 ? a.alpha : A.slot_invdeg) + T.slot_base, k, lane, pol);
   if (MODE == 1) copy_rows<STRIDE>(m + kJOm, a.omega + T.slot_base, k, lane, pol);
   cp_async_commit();
-  const UnitShape S = A.unit_shapes[T.unit - 1];
   cp_async_wait_one();
   __syncwarp();
   for (int h = 0; h < k; ++h) {
@@ -381,18 +397,16 @@ __global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int
     unit_adjoint_tile<FWD, MODE, 6>(a, T, s, m, lane);
   else if (WMAX >= 8)
     unit_adjoint_tile<FWD, MODE, 8>(a, T, s, m, lane);
+  if (late) grid_wait();
 }
 
 template <int FWD, int MODE>
-void launch_adjoint_group(const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
-                          cudaStream_t st) {
-  const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc, r = (int)region;
-  if (G.unit_w <= 2)
-    k_unit_adjoint<FWD, MODE, 2><<<grid, wpc * kWarp, region * wpc, st>>>(A, a, r, G.tile0, G.tile1);
-  else if (G.unit_w <= 4)
-    k_unit_adjoint<FWD, MODE, 4><<<grid, wpc * kWarp, region * wpc, st>>>(A, a, r, G.tile0, G.tile1);
-  else
-    k_unit_adjoint<FWD, MODE, 8><<<grid, wpc * kWarp, region * wpc, st>>>(A, a, r, G.tile0, G.tile1);
+void launch_adjoint_group(const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region, Chain& ch,
+                          bool late) {
+  const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc;
+  auto k = G.unit_w <= 2 ? k_unit_adjoint<FWD, MODE, 2>
+                         : (G.unit_w <= 4 ? k_unit_adjoint<FWD, MODE, 4> : k_unit_adjoint<FWD, MODE, 8>);
+  chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1, late ? 1 : 0);
 }
 
 template <int FWD, int MODE>
@@ -405,21 +419,12 @@ cudaError_t set_adjoint_attr(int b) {
   return e;
 }
 
-template <int KIND, int MODE, int WMAX>
-void launch_w(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, cudaStream_t st) {
-  const int nt = G.tile1 - G.tile0;
-  k_unit<KIND, MODE, WMAX><<<(nt + wpc - 1) / wpc, wpc * kWarp, region * wpc, st>>>(A, a, (int)region, G.tile0, G.tile1);
-}
-
 template <int KIND, int MODE>
-void launch_group(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
-                  cudaStream_t st) {
-  if (G.unit_w <= 2)
-    launch_w<KIND, MODE, 2>(A, a, G, wpc, region, st);
-  else if (G.unit_w <= 4)
-    launch_w<KIND, MODE, 4>(A, a, G, wpc, region, st);
-  else
-    launch_w<KIND, MODE, 8>(A, a, G, wpc, region, st);
+void launch_group(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, Chain& ch,
+                  bool late) {
+  const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc;
+  auto k = G.unit_w <= 2 ? k_unit<KIND, MODE, 2> : (G.unit_w <= 4 ? k_unit<KIND, MODE, 4> : k_unit<KIND, MODE, 8>);
+  chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1, late ? 1 : 0);
 }
 
 template <int KIND, int MODE>
@@ -453,31 +458,31 @@ cudaError_t set_unit_smem_limit(size_t bytes) {
 }
 
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
-                 cudaStream_t st) {
+                 Chain& ch, bool late) {
   const bool m1 = a.mode == 1;
   switch (kind) {
-    case kFwd: m1 ? launch_group<kFwd, 1>(A, a, G, wpc, region, st) : launch_group<kFwd, 0>(A, a, G, wpc, region, st); break;
-    case kBwd: m1 ? launch_group<kBwd, 1>(A, a, G, wpc, region, st) : launch_group<kBwd, 0>(A, a, G, wpc, region, st); break;
+    case kFwd: m1 ? launch_group<kFwd, 1>(A, a, G, wpc, region, ch, late) : launch_group<kFwd, 0>(A, a, G, wpc, region, ch, late); break;
+    case kBwd: m1 ? launch_group<kBwd, 1>(A, a, G, wpc, region, ch, late) : launch_group<kBwd, 0>(A, a, G, wpc, region, ch, late); break;
     case kFwdRec:
-      m1 ? launch_group<kFwdRec, 1>(A, a, G, wpc, region, st) : launch_group<kFwdRec, 0>(A, a, G, wpc, region, st);
+      m1 ? launch_group<kFwdRec, 1>(A, a, G, wpc, region, ch, late) : launch_group<kFwdRec, 0>(A, a, G, wpc, region, ch, late);
       break;
     case kBwdRec:
-      m1 ? launch_group<kBwdRec, 1>(A, a, G, wpc, region, st) : launch_group<kBwdRec, 0>(A, a, G, wpc, region, st);
+      m1 ? launch_group<kBwdRec, 1>(A, a, G, wpc, region, ch, late) : launch_group<kBwdRec, 0>(A, a, G, wpc, region, ch, late);
       break;
-    case kMinMarg: launch_group<kMinMarg, 0>(A, a, G, wpc, region, st); break;
-    case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, st); break;
-    default: launch_group<kSeed, 0>(A, a, G, wpc, region, st); break;
+    case kMinMarg: launch_group<kMinMarg, 0>(A, a, G, wpc, region, ch, late); break;
+    case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, ch, late); break;
+    default: launch_group<kSeed, 0>(A, a, G, wpc, region, ch, late); break;
   }
 }
 
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
-                         cudaStream_t st) {
+                         Chain& ch, bool late) {
   if (forward)
-    a.mode == 1 ? launch_adjoint_group<1, 1>(A, a, G, wpc, region, st)
-                : launch_adjoint_group<1, 0>(A, a, G, wpc, region, st);
+    a.mode == 1 ? launch_adjoint_group<1, 1>(A, a, G, wpc, region, ch, late)
+                : launch_adjoint_group<1, 0>(A, a, G, wpc, region, ch, late);
   else
-    a.mode == 1 ? launch_adjoint_group<0, 1>(A, a, G, wpc, region, st)
-                : launch_adjoint_group<0, 0>(A, a, G, wpc, region, st);
+    a.mode == 1 ? launch_adjoint_group<0, 1>(A, a, G, wpc, region, ch, late)
+                : launch_adjoint_group<0, 0>(A, a, G, wpc, region, ch, late);
 }
 
 }  // namespace dg

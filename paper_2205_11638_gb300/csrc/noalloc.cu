@@ -67,8 +67,7 @@ size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 }  // namespace
 
 dg_status lower_bound_noalloc(const DevArena& arena, const LaunchGroup* groups, int num_groups, int threads,
-                              const StreamSet& ss, const float* lam, const float* M, double* lb) {
-  cudaStream_t st = ss.main;
+                              Chain& ch, const float* lam, const float* M, double* lb) {
   const size_t bE = up256((size_t)arena.m * 4), bS = up256((size_t)arena.n * 4);
   const size_t bP = up256((size_t)arena.num_lb_chunks * 8);
   const size_t bL = up256((size_t)arena.long_cost_size * 4);
@@ -91,9 +90,9 @@ dg_status lower_bound_noalloc(const DevArena& arena, const LaunchGroup* groups, 
   SweepArgs a{};
   a.lam = const_cast<float*>(lam);
   a.E = A.E;
-  launch_sweep(kEnergy, A, a, threads, groups, num_groups, ss);
-  launch_reduce_S(A, M, nullptr, nullptr, 0, false, st, Scatter::kNone);
-  launch_lower_bound(A, lb, st);
+  launch_sweep(kEnergy, A, a, threads, groups, num_groups, ch);
+  launch_reduce_S(A, M, nullptr, nullptr, 0, false, ch, Scatter::kNone);
+  launch_lower_bound(A, lb, ch);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DG_ECUDA, std::string("dg_lower_bound_noalloc: ") + cudaGetErrorString(e));
   return DG_OK;
