@@ -128,6 +128,8 @@ cudaError_t set_unit_smem_limit(size_t bytes);
 struct AdjArgs;
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
                  Chain& ch, bool late);
+void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, const LaunchGroup& G,
+                          int wpc, size_t region, cudaStream_t st);
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
                          Chain& ch, bool late);
 // Dynamic shared memory one CTA may use; launchers put fewer warps in a CTA

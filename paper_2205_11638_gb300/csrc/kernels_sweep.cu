@@ -346,8 +346,12 @@ void launch_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a,
   launch_long_smoothed(A, lam, a_s, E_a, marg, fork ? ss.of(A.long_stream) : ss.main);
   for (int g = 0; g < num_groups; ++g) {
     const LaunchGroup& G = groups[g];
-    const size_t region = (size_t)G.region_bwd0;
+    const size_t region = (size_t)(G.unit_w ? G.unit_bytes0 : G.region_bwd0);
     const int wpc = best_warps_per_cta(region, 4, g_cta_smem_cap);
+    if (G.unit_w) {
+      launch_unit_smoothed(A, lam, a_s, E_a, marg, G, wpc, region, fork ? ss.of(G.stream) : ss.main);
+      continue;
+    }
     const int nt = G.tile1 - G.tile0;
     k_smoothed<<<(nt + wpc - 1) / wpc, wpc * kWarp, region * wpc, fork ? ss.of(G.stream) : ss.main>>>(
         A, lam, a_s, E_a, marg, (int)region, G.tile0, G.tile1);

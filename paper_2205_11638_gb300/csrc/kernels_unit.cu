@@ -238,6 +238,197 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
   if (late) grid_wait();
 }
 
+// ---- smoothed subproblems --------------------------------------------------
+// E_a = -a log Z, Z = sum over feasible x of exp(<w, x>), w = -lambda / a, and
+// the marginals P(x_i = 1): the walks of a forward sweep with sums of products
+// in place of minima of sums.  A level's two weights 1 and exp(w) are divided
+// by the larger (its logarithm joins log Z), so that they are 1 and
+// exp(-|w|): one exponential per level and one fused multiply-add per arc,
+// where sums in the logarithmic domain take an exponential and a logarithm per
+// arc.  A product of weights is at least exp(-sum |w|) and a sum over paths at
+// most 2^k, so with sum |w| <= 40 and k <= 60 nothing leaves the range of
+// float32 (not the product of a prefix' and a suffix' sum either); a tile with
+// a row beyond that takes the logarithmic walk.
+struct SumProd {  // x: exp(-|w|), negative when w > 0 (the 0-arc then has it)
+  template <int W>
+  static __device__ __forceinline__ Costs<W> end(int accept) {
+    Costs<W> c;
+#pragma unroll
+    for (int u = 0; u < W; ++u) c.v[u] = (accept >> u) & 1 ? 1.0f : 0.0f;
+    return c;
+  }
+  static __device__ __forceinline__ float q0(float x) { return x < 0.0f ? -x : 1.0f; }
+  static __device__ __forceinline__ float q1(float x) { return x < 0.0f ? 1.0f : x; }
+  template <int W, int TYPE>
+  static __device__ __forceinline__ Costs<W> up(const Costs<W>& T, float x) {
+    const float a0 = q0(x), a1 = q1(x);
+    Costs<W> r;
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      const int o = unit_o<TYPE>(u);
+      r.v[u] = a0 * T.v[unit_z<TYPE>(u)];
+      if (o >= 0 && o < W) r.v[u] = fmaf(a1, T.v[o], r.v[u]);
+    }
+    return r;
+  }
+  template <int W, int TYPE>
+  static __device__ __forceinline__ Costs<W> down(const Costs<W>& F, float x) {
+    const float a0 = q0(x), a1 = q1(x);
+    Costs<W> r;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      float b = 0.0f;
+#pragma unroll
+      for (int u = 0; u < W; ++u) {
+        if (unit_z<TYPE>(u) == w) b = fmaf(a0, F.v[u], b);
+        if (unit_o<TYPE>(u) == w) b = fmaf(a1, F.v[u], b);
+      }
+      r.v[w] = b;
+    }
+    return r;
+  }
+  // the paths through the level's 1-arcs
+  template <int W, int TYPE>
+  static __device__ __forceinline__ float through(const Costs<W>& F, const Costs<W>& T, float x) {
+    float s = 0.0f;
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      const int o = unit_o<TYPE>(u);
+      if (o >= 0 && o < W) s = fmaf(F.v[u], T.v[o], s);
+    }
+    return q1(x) * s;
+  }
+  static __device__ __forceinline__ float share(float s, float Z) { return s / Z; }
+};
+
+// log(exp(x) + exp(y)) with -inf as the empty sum.
+__device__ __forceinline__ float lse2(float x, float y) {
+  const float m = fmaxf(x, y);
+  if (m == -f_inf()) return m;
+  return m + log1pf(expf(-fabsf(x - y)));
+}
+
+struct LogSum {  // x: w; everything a logarithm
+  template <int W>
+  static __device__ __forceinline__ Costs<W> end(int accept) {
+    Costs<W> c;
+#pragma unroll
+    for (int u = 0; u < W; ++u) c.v[u] = (accept >> u) & 1 ? 0.0f : -f_inf();
+    return c;
+  }
+  template <int W, int TYPE>
+  static __device__ __forceinline__ Costs<W> up(const Costs<W>& T, float x) {
+    Costs<W> r;
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      const int o = unit_o<TYPE>(u);
+      r.v[u] = T.v[unit_z<TYPE>(u)];
+      if (o >= 0 && o < W) r.v[u] = lse2(r.v[u], x + T.v[o]);
+    }
+    return r;
+  }
+  template <int W, int TYPE>
+  static __device__ __forceinline__ Costs<W> down(const Costs<W>& F, float x) {
+    Costs<W> r;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      float b = -f_inf();
+#pragma unroll
+      for (int u = 0; u < W; ++u) {
+        if (unit_z<TYPE>(u) == w) b = lse2(b, F.v[u]);
+        if (unit_o<TYPE>(u) == w) b = lse2(b, F.v[u] + x);
+      }
+      r.v[w] = b;
+    }
+    return r;
+  }
+  template <int W, int TYPE>
+  static __device__ __forceinline__ float through(const Costs<W>& F, const Costs<W>& T, float x) {
+    float s = -f_inf();
+#pragma unroll
+    for (int u = 0; u < W; ++u) {
+      const int o = unit_o<TYPE>(u);
+      if (o >= 0 && o < W) s = lse2(s, F.v[u] + x + T.v[o]);
+    }
+    return s;
+  }
+  static __device__ __forceinline__ float share(float s, float Z) { return expf(s - Z); }
+};
+
+template <class OP, int W>
+__device__ __forceinline__ float smoothed_walk(const UnitCtx& s, int rows, const float* x0, float* cost, float* out,
+                                               bool real, int lane) {
+  const Costs<W> t = unit_first_up<W, kWarp, OP>(s, rows, x0, cost, lane);
+  float Z = 0.0f;
+#pragma unroll
+  for (int u = 0; u < W; ++u)
+    if (u == s.start) Z = t.v[u];
+  Costs<W> F = OP::template end<W>(1 << s.start);
+  unit_second_down<W, kWarp, OP>(s, x0, cost, lane, [&](auto ty, const float* x, const Costs<W>& t1) {
+    constexpr int TY = decltype(ty)::value;
+    const float m = OP::share(OP::template through<W, TY>(F, t1, x[0]), Z);
+    if (real) *out = m;
+    out += kWarp;
+    F = OP::template down<W, TY>(F, x[0]);
+  });
+  return Z;
+}
+
+template <int W>
+__device__ __forceinline__ void smoothed_tile(const DevArena& A, float a_s, float* E_a, float* marg, const Tile& T,
+                                              const UnitShape& S, float* smem, int lane) {
+  const UnitCtx s{S.k, S.start, S.accept, S.nruns, A.unit_runs + S.run_base};
+  const int64_t sb = T.slot_base + lane;
+  const bool real = lane < T.nbdd;
+  float* x0 = smem + lane;
+  float* cost = smem + s.k * kWarp;
+  const float inv_a = 1.0f / a_s;
+  float range = 0.0f;
+  for (int h = 0; h < s.k; ++h) range += fabsf(x0[h * kWarp] * inv_a);
+  // (not a number: out of range too)
+  if (s.k <= 60 && __all_sync(0xffffffffu, !real || range <= 40.0f)) {
+    float off = 0.0f, err = 0.0f;  // sum of the logarithms divided out, and its rounding (TwoSum)
+    for (int h = 0; h < s.k; ++h) {
+      const float w = -x0[h * kWarp] * inv_a;
+      const float e = expf(-fabsf(w));
+      x0[h * kWarp] = w > 0.0f ? -e : e;
+      const float d = fmaxf(w, 0.0f), t = off + d, b = t - off;
+      err += (off - (t - b)) + (d - b);
+      off = t;
+    }
+    const float Z = smoothed_walk<SumProd, W>(s, S.rows, x0, cost, marg + sb, real, lane);
+    if (E_a && real) E_a[__ldg(A.slot_row + sb)] = -a_s * (off + (err + logf(Z)));
+  } else {
+    for (int h = 0; h < s.k; ++h) x0[h * kWarp] = -x0[h * kWarp] * inv_a;
+    const float Z = smoothed_walk<LogSum, W>(s, S.rows, x0, cost, marg + sb, real, lane);
+    if (E_a && real) E_a[__ldg(A.slot_row + sb)] = -a_s * Z;
+  }
+}
+
+template <int WMAX>
+__global__ void __launch_bounds__(128) k_unit_smoothed(DevArena A, const float* lam, float a_s, float* E_a, float* marg,
+                                                       int region_bytes, int tile0, int tile1) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
+  if (tile >= tile1) return;  // whole warp leaves; no CTA-wide barrier follows
+  const Tile T = A.tiles[tile];
+  float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
+  copy_rows<kWarp>(m, lam + T.slot_base, T.nhops, lane, l2_evict_first());
+  cp_async_commit();
+  const UnitShape S = A.unit_shapes[T.unit - 1];
+  cp_async_wait_all();
+  __syncwarp();
+  if (S.W == 2)
+    smoothed_tile<2>(A, a_s, E_a, marg, T, S, m, lane);
+  else if (WMAX >= 4 && S.W == 4)
+    smoothed_tile<4>(A, a_s, E_a, marg, T, S, m, lane);
+  else if (WMAX >= 8 && S.W == 6)
+    smoothed_tile<6>(A, a_s, E_a, marg, T, S, m, lane);
+  else if (WMAX >= 8)
+    smoothed_tile<8>(A, a_s, E_a, marg, T, S, m, lane);
+}
+
 // ---- adjoint of a recording sweep (see kernels_adjoint.cu) -----------------
 // Per level and lane, staged: the gradient of lambda, the argmin word, m1 - m0,
 // the averaging weight, {S-dot of the next sweep, S at the sweep's start} of
@@ -451,6 +642,9 @@ cudaError_t set_unit_smem_limit(size_t bytes) {
   if (e == cudaSuccess) e = set_adjoint_attr<1, 1>(b);
   if (e == cudaSuccess) e = set_adjoint_attr<0, 0>(b);
   if (e == cudaSuccess) e = set_adjoint_attr<0, 1>(b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit_smoothed<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit_smoothed<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit_smoothed<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess) e = set_attr<kMinMarg, 0>(b);
   if (e == cudaSuccess) e = set_attr<kEnergy, 0>(b);
   if (e == cudaSuccess) e = set_attr<kSeed, 0>(b);
@@ -473,6 +667,13 @@ void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGr
     case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, ch, late); break;
     default: launch_group<kSeed, 0>(A, a, G, wpc, region, ch, late); break;
   }
+}
+
+void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, const LaunchGroup& G,
+                          int wpc, size_t region, cudaStream_t st) {
+  const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc;
+  auto k = G.unit_w <= 2 ? k_unit_smoothed<2> : (G.unit_w <= 4 ? k_unit_smoothed<4> : k_unit_smoothed<8>);
+  k<<<grid, wpc * kWarp, region * wpc, st>>>(A, lam, a_s, E_a, marg, (int)region, G.tile0, G.tile1);
 }
 
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,

@@ -273,6 +273,17 @@ __device__ __forceinline__ Costs<W> unit_load(const float* row, int lane) {
   return c;
 }
 
+// What the two-pass walks compute: path costs (minima of sums), or the sums
+// over paths of the smoothed subproblems (kernels_unit.cu).
+struct MinPlus {
+  template <int W>
+  static __device__ __forceinline__ Costs<W> end(int accept);
+  template <int W, int TYPE>
+  static __device__ __forceinline__ Costs<W> up(const Costs<W>& T, float l) {
+    return unit_up<W, TYPE>(T, l);
+  }
+};
+
 // SP(., T) below the last level, SP(r, .) of the first.
 template <int W>
 __device__ __forceinline__ Costs<W> unit_end(int accept) {
@@ -287,6 +298,11 @@ __device__ __forceinline__ Costs<W> unit_root(int start) {
 #pragma unroll
   for (int u = 0; u < W; ++u) c.v[u] = u == start ? 0.0f : f_inf();
   return c;
+}
+
+template <int W>
+__device__ __forceinline__ Costs<W> MinPlus::end(int accept) {
+  return unit_end<W>(accept);
 }
 
 // One shape, as a warp holds it.
@@ -339,10 +355,11 @@ __device__ __forceinline__ void unit_runs_up(const UnitCtx& s, F&& f) {
 // only some twenty operations.
 
 // First pass of a forward sweep: SP(., T) of the levels at even distance from
-// their run's first level and of every run's end, in level order.
-template <int W, int STRIDE>
-__device__ __forceinline__ void unit_first_up(const UnitCtx& s, int rows, const float* x, float* cost, int lane) {
-  Costs<W> t = unit_end<W>(s.accept);
+// their run's first level and of every run's end, in level order; returns those
+// of level 0.
+template <int W, int STRIDE, class OP = MinPlus>
+__device__ __forceinline__ Costs<W> unit_first_up(const UnitCtx& s, int rows, const float* x, float* cost, int lane) {
+  Costs<W> t = OP::template end<W>(s.accept);
   float* p = cost + rows * (kWarp * W);
   x += s.k * STRIDE;
   unit_runs_up(s, [&](auto ty, int b, int e) {
@@ -351,20 +368,21 @@ __device__ __forceinline__ void unit_first_up(const UnitCtx& s, int rows, const 
     int n = e - b;
     if (n & 1) {
       x -= STRIDE;
-      t = unit_up<W, TY>(t, x[0]);
+      t = OP::template up<W, TY>(t, x[0]);
       if (--n > 0) unit_store<W>(p -= kWarp * W, t, lane);
     }
     for (; n > 0; n -= 2) {
-      t = unit_up<W, TY>(t, x[-STRIDE]);
+      t = OP::template up<W, TY>(t, x[-STRIDE]);
       x -= 2 * STRIDE;
-      t = unit_up<W, TY>(t, x[0]);
+      t = OP::template up<W, TY>(t, x[0]);
       if (n > 2) unit_store<W>(p -= kWarp * W, t, lane);
     }
   });
+  return t;
 }
 // Second pass: f(type constant, x of level h, SP(., T) of level h + 1) for
 // every level in ascending order.
-template <int W, int STRIDE, class F>
+template <int W, int STRIDE, class OP = MinPlus, class F>
 __device__ __forceinline__ void unit_second_down(const UnitCtx& s, const float* x, const float* cost, int lane,
                                                  F&& f) {
   const float* p = cost;
@@ -373,18 +391,18 @@ __device__ __forceinline__ void unit_second_down(const UnitCtx& s, const float* 
     const int last = e == s.k ? 2 : 0;  // levels left when SP(., T) of the next stored level is the terminals'
     int n = e - b;
     for (; n >= 2; n -= 2) {
-      Costs<W> t2 = unit_end<W>(s.accept);
+      Costs<W> t2 = OP::template end<W>(s.accept);
       if (n != last) {
         t2 = unit_load<W>(p, lane);
         p += kWarp * W;
       }
-      const Costs<W> t1 = unit_up<W, TY>(t2, x[STRIDE]);
+      const Costs<W> t1 = OP::template up<W, TY>(t2, x[STRIDE]);
       f(ty, x, t1);
       f(ty, x + STRIDE, t2);
       x += 2 * STRIDE;
     }
     if (n > 0) {
-      Costs<W> t1 = unit_end<W>(s.accept);
+      Costs<W> t1 = OP::template end<W>(s.accept);
       if (last == 0) {
         t1 = unit_load<W>(p, lane);
         p += kWarp * W;

@@ -173,3 +173,29 @@ def test_gradients_equal_the_mixed_tiles(name, mode, tied):
             assert (a - b).abs().max() <= 64 * 6 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
         for a, b in zip(out[0][4:], out[1][4:]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("scale", [1.0, 30.0])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_smoothed_dual_against_float64(name, scale):
+    """Energies and marginals of the smoothed subproblems on unit rows: the
+    walk over sums of products (scale 1) and, with path costs beyond its range,
+    the logarithmic one (scale 30), against the oracle.  Both make at most four
+    roundings per level and state on a logarithm of size up to the row's costs:
+    tolerance 4 levels 2^-24 relative to that size for E, absolute on the
+    marginals (a logarithm's error is a factor's relative error)."""
+    import oracle
+    p = CASES[name]()
+    O = oracle.Oracle(p)
+    A = solver.plan(p).bind()
+    lam = A.from_csr(scale * _vectors(p, 11)[0])
+    lam_c = A.to_csr(lam).double().cpu().numpy()
+    rp, absl = p["row_ptr"], np.abs(lam_c)
+    for a in (1.0, 10.0):
+        E, marg = A.smoothed_dual(lam, a)
+        oE, om = O.smoothed(lam_c, a)
+        size = np.add.reduceat(absl, rp[:-1]) / a + np.diff(rp)  # bound on the logarithms in a row
+        tol = 4 * np.diff(rp) * 2.0 ** -24 * size + 1e-6
+        assert torch.isfinite(E).all() and torch.isfinite(marg).all()
+        assert (np.abs(E.double().cpu().numpy() - oE) <= a * tol).all()
+        assert (np.abs(A.to_csr(marg).double().cpu().numpy() - om) <= np.repeat(tol, np.diff(rp))).all()
