@@ -867,7 +867,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       // BDDs per warp: as many as lanes allow while that leaves at least four
       // warps per SM (a warp's levels are a chain of dependent steps, which
       // other warps hide), and as fit shared memory
-      int nseg = kWarp / G;
+      int nseg = G <= kUnitMaxW ? kWarp : kWarp / G;
       while (nseg > 1 && ((int64_t)(e - i) < 4LL * 152 * nseg || long_unit_bytes(nseg, G, kmax, 1) > 64 * 1024 ||
                           long_unit_adjoint_bytes(nseg, kmax) > 64 * 1024))
         nseg /= 2;
@@ -1207,7 +1207,8 @@ dg_status validate_plan(const Plan& P) {
     if (P.num_long_unit < 0 || P.num_long_unit > P.num_long_narrow) return bad("long unit BDDs not narrow");
     std::vector<char> in_item(P.num_long_unit, 0);
     for (const LongItem& it : P.long_items) {
-      if (it.G < 2 || it.G > kLongUnitMaxW || (it.G & (it.G - 1)) != 0 || it.nseg < 1 || it.nseg * it.G > kWarp ||
+      if (it.G < 2 || it.G > kLongUnitMaxW || (it.G & (it.G - 1)) != 0 || it.nseg < 1 ||
+          it.nseg > (it.G <= kUnitMaxW ? kWarp : kWarp / it.G) ||
           it.first < 0 || it.first + it.nseg > P.num_long_unit || it.start < 0 || it.start >= it.G || it.nruns < 1 ||
           it.run_base < 0 || (size_t)it.run_base + (size_t)it.nruns > P.unit_runs.size() ||
           long_unit_bytes(it.nseg, it.G, it.kmax, 0) > (size_t)P.long_unit_smem[0] ||

@@ -122,9 +122,10 @@ struct LongBdd {
 };
 static_assert(sizeof(LongBdd) == 32, "LongBdd is 32 bytes");
 
-// Long unit rows (see UnitShape; up to 32 states a level): a segment of G
-// lanes sweeps one BDD, lane s holding state s, and one warp (work item) takes
-// `nseg` BDDs of one kind: the same level types, start and accepted states
+// Long unit rows (see UnitShape; up to 32 states a level, G of them with the
+// window rounded up): one warp (work item) sweeps `nseg` BDDs of one kind, each
+// by one lane holding a level's states in registers (G up to kUnitMaxW) or by
+// a segment of G lanes, lane s holding state s: the same level types, start and accepted states
 // (any lengths when all levels have one type, else the same length).
 struct LongItem {
   int32_t first;     // its BDDs: long_order[first .. first + nseg)

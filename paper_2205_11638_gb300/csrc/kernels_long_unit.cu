@@ -5,9 +5,12 @@
 // The levels of one BDD are a chain (the paper's long subproblems: the update
 // of a level needs the path costs under the lambda of the level before), so a
 // sweep's time is the levels times the latency of one step, and everything
-// else has to be out of that chain.  A segment of G lanes holds a level, lane
-// s its state s; a step is one shuffle to the neighbour state, the segment's
-// minima and the update.  All inputs of a work item are staged in shared
+// else has to be out of that chain.  Up to 8 states a level are one lane's
+// registers, as in the unit tiles: a step is some twenty instructions on a
+// short chain, and the BDDs are spread thinly over the warps, since a warp that
+// is alone on its scheduler waits for every instruction.  Wider levels are held
+// by a segment of G lanes, lane s its state s: a step is one shuffle to the
+// neighbour state, the segment's minima and the update.  All inputs of a work item are staged in shared
 // memory before the walk (asynchronous copies; the averaging terms gathered
 // through the staged variable ids), the costs opposite to the sweep are
 // recomputed into shared memory by a first walk, and each step's words are
@@ -151,58 +154,16 @@ __device__ __forceinline__ void copy_row(float* dst, const void* src, int k, int
   for (int p = lane; p < (k + 3) / 4; p += kWarp) cp_async16(dst + 4 * p, (const char*)src + 16 * p, pol);
 }
 
+// The walk of a sweep with a level's states on the lanes of a segment: lam and
+// avg (the staged inputs) receive the new lambda and M (kMinMarg: m1 and m0,
+// kSeed: the minimising assignment in avg).
 template <int KIND, int MODE, int G>
-__device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArgs& a, const LongItem& it, float* smem,
-                                               int lane) {
+__device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs& a, const LongItem& it, float* lam,
+                                              float* avg, const float* om, const float* al, float* cost, int lane) {
   constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
   constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
   constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
-  constexpr bool UPDATE = FWD || BWD;
-  const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST, TS = it.nseg * G;
-  float* lam = smem;
-  float* avg = lam + nrow;
-  float* om = avg + nrow;
-  float* al = om + (MODE == 1 ? nrow : 0);
-  float* cost = al + (MODE == 1 ? nrow : 0);
-
-  // ---- staging -------------------------------------------------------------
-  const uint64_t pol = l2_evict_first();
-  if (UPDATE) {
-    for (int r = 0; r < it.nseg; ++r) {
-      const LongBdd B = A.longs[A.long_order[it.first + r]];
-      copy_row(avg + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
-    }
-    cp_async_commit();
-  }
-  grid_wait();
-  grid_trigger();
-  for (int r = 0; r < it.nseg; ++r) {
-    const LongBdd B = A.longs[A.long_order[it.first + r]];
-    copy_row(lam + r * ST, a.lam + B.slot_base, B.k, lane, pol);
-    if (UPDATE && MODE == 1) {
-      copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
-      copy_row(al + r * ST, a.alpha + B.slot_base, B.k, lane, pol);
-    }
-  }
-  cp_async_commit();
-  if (UPDATE) {
-    cp_async_wait_one();
-    __syncwarp();
-    const float* src = MODE == 1 ? A.S : A.Sbar;
-    for (int r = 0; r < it.nseg; ++r) {
-      const int k = A.longs[A.long_order[it.first + r]].k;
-#pragma unroll 4
-      for (int h = lane; h < k; h += kWarp) {
-        const int v = __float_as_int(avg[r * ST + h]);
-        cp_async4(avg + r * ST + h, src + v);
-      }
-    }
-    cp_async_commit();
-  }
-  cp_async_wait_all();
-  __syncwarp();
-
-  // ---- the walk --------------------------------------------------------------
+  const int ST = long_unit_stride(it.kmax), TS = it.nseg * G;
   LSeg<G> g;
   g.s = lane & (G - 1);
   g.base = lane - g.s;
@@ -381,6 +342,251 @@ __device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArg
       });
     }
   }
+}
+
+// ... with a level's states in the registers of the BDD's lane.
+template <int KIND, int MODE, int W>
+__device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a, const LongItem& it, float* lam,
+                                           float* avg, const float* om, const float* al, float* cost, int lane) {
+  constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
+  constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
+  constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
+  const int ST = long_unit_stride(it.kmax);
+  const bool act = lane < it.nseg;
+  const int row = act ? lane : 0;
+  const LongBdd B = A.longs[A.long_order[it.first + row]];
+  const int k = act ? B.k : 0;  // a lane without a BDD walks nothing
+  float* ml = lam + row * ST;
+  float* ma = avg + row * ST;
+  const float* mo = om + row * ST;
+  const float* mw = al + row * ST;
+  float* mt = cost + row * W;  // level h at mt[h TS], the terminals' at level k
+  const int TS = it.nseg * W, last = max(k - 1, 0);
+  auto put = [&](int h, const Costs<W>& c) {
+    if constexpr (W == 2) {
+      *reinterpret_cast<float2*>(mt + h * TS) = make_float2(c.v[0], c.v[1]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < W / 4; ++j)
+        reinterpret_cast<float4*>(mt + h * TS)[j] = make_float4(c.v[4 * j], c.v[4 * j + 1], c.v[4 * j + 2], c.v[4 * j + 3]);
+    }
+  };
+  auto get = [&](int h) {
+    Costs<W> c;
+    if constexpr (W == 2) {
+      const float2 x = *reinterpret_cast<const float2*>(mt + h * TS);
+      c.v[0] = x.x;
+      c.v[1] = x.y;
+    } else {
+#pragma unroll
+      for (int j = 0; j < W / 4; ++j) {
+        const float4 x = reinterpret_cast<const float4*>(mt + h * TS)[j];
+        c.v[4 * j] = x.x;
+        c.v[4 * j + 1] = x.y;
+        c.v[4 * j + 2] = x.z;
+        c.v[4 * j + 3] = x.w;
+      }
+    }
+    return c;
+  };
+  const Costs<W> end = unit_end<W>((int)it.accept);
+  const Costs<W> root = unit_root<W>(it.start);
+  // a level's inputs, read one level ahead
+  struct In {
+    float l, av, w, al;
+  };
+  auto input = [&](int h) {
+    const int x = min(max(h, 0), last);
+    return In{ml[x], ma[x], MODE == 1 ? mo[x] : a.omega0, MODE == 1 ? mw[x] : 0.0f};
+  };
+  auto first_up = [&]() {
+    Costs<W> t = end;
+    if (act) put(k, end);
+    float l = ml[last];
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = e - 1; h >= b; --h) {
+        const float l1 = ml[min(max(h - 1, 0), last)];
+        if (h < k) {
+          t = unit_up<W, TY>(t, l);
+          put(h, t);
+        }
+        l = l1;
+      }
+    });
+    return t;
+  };
+  auto update = [&](int h, const In& x, float b0, float b1) -> float {
+    const float m0 = b0, m1 = x.l + b1;
+    const float Mn = __fmul_rn(x.w, m1 - m0);
+    const float ln = unit_lambda_new<MODE>(x.l, Mn, x.al, x.av);
+    ml[h] = ln;
+    ma[h] = Mn;
+    if (REC) a.rec_diff[(int64_t)B.slot_base + h] = m1 - m0;
+    return ln;
+  };
+  auto energy = [&](const Costs<W>& t) {  // E^j = SP(r, T)
+    if (a.E == nullptr || !act) return;
+    float e = f_inf();
+#pragma unroll
+    for (int u = 0; u < W; ++u)
+      if (u == it.start) e = t.v[u];
+    a.E[B.row] = e;
+  };
+  uint4* rec_out = REC ? a.rec_lunit + (B.slot_base - A.long_slot_base) : nullptr;
+
+  if (FWD || KIND == kMinMarg) {
+    first_up();
+    Costs<W> R = root;
+    In in = input(0);
+    Costs<W> t1 = get(min(1, k));
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = b; h < e; ++h) {
+        const In nxt = input(h + 1);
+        const Costs<W> t2 = get(min(h + 2, k));
+        if (h < k) {
+          float b0, b1;
+          if (REC) {
+            uint32_t rec = 0;
+            unit_minima_rec<W, TY>(R, t1, b0, b1, rec);
+            unit_up_rec<W, TY>(t1, in.l, rec);
+            R = unit_down_rec<W, TY>(R, update(h, in, b0, b1), rec);
+            rec_out[h].x = rec;
+          } else {
+            unit_minima<W, TY>(R, t1, b0, b1);
+            float ln = in.l;
+            if (KIND == kMinMarg) {
+              ml[h] = in.l + b1;
+              ma[h] = b0;
+            } else {
+              ln = update(h, in, b0, b1);
+            }
+            R = unit_down<W, TY>(R, ln);
+          }
+        }
+        in = nxt;
+        t1 = t2;
+      }
+    });
+  } else if (BWD) {
+    {
+      Costs<W> R = root;
+      float l = ml[0];
+      runs_down(A, it, [&](auto ty, int b, int e) {
+        constexpr int TY = decltype(ty)::value;
+        for (int h = b; h < e; ++h) {
+          const float l1 = ml[min(h + 1, last)];
+          if (h < k) {
+            put(h, R);
+            R = unit_down<W, TY>(R, l);
+          }
+          l = l1;
+        }
+      });
+    }
+    Costs<W> t = end;
+    In in = input(it.kmax - 1);
+    Costs<W> r = get(min(it.kmax - 1, last));
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = e - 1; h >= b; --h) {
+        const In nxt = input(h - 1);
+        const Costs<W> r1 = get(min(max(h - 1, 0), last));
+        if (h < k) {
+          float b0, b1;
+          if (REC) {
+            uint32_t rec = 0;
+            unit_minima_rec<W, TY>(r, t, b0, b1, rec);
+            unit_down_rec<W, TY>(r, in.l, rec);
+            t = unit_up_rec<W, TY>(t, update(h, in, b0, b1), rec);
+            rec_out[h].x = rec;
+          } else {
+            unit_minima<W, TY>(r, t, b0, b1);
+            t = unit_up<W, TY>(t, update(h, in, b0, b1));
+          }
+        }
+        in = nxt;
+        r = r1;
+      }
+    });
+    energy(t);
+  } else {
+    const Costs<W> t = first_up();
+    if (KIND == kEnergy) {
+      energy(t);
+    } else {
+      // kSeed: walk the minimising path from the root, the 0-arc on ties
+      int at = it.start;
+      runs_down(A, it, [&](auto ty, int b, int e) {
+        constexpr int TY = decltype(ty)::value;
+        for (int h = b; h < min(e, k); ++h) {
+          const int z = lz<W, TY>(at), o = lo_<W, TY>(at);
+          const float* p = mt + (h + 1) * TS;
+          const float c0 = p[z], c1 = o >= 0 && o < W ? p[o] : f_inf();
+          // an infinite cost is the bottom terminal (the path stays feasible)
+          const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= ml[h] + c1);
+          ma[h] = take0 ? 0.f : 1.f;
+          at = take0 ? z : max(min(o, W - 1), 0);
+        }
+      });
+    }
+  }
+}
+
+template <int KIND, int MODE, int G>
+__device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArgs& a, const LongItem& it, float* smem,
+                                               int lane) {
+  constexpr bool UPDATE = KIND == kFwd || KIND == kBwd || KIND == kFwdRec || KIND == kBwdRec;
+  const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST;
+  float* lam = smem;
+  float* avg = lam + nrow;
+  float* om = avg + nrow;
+  float* al = om + (MODE == 1 ? nrow : 0);
+  float* cost = al + (MODE == 1 ? nrow : 0);
+
+  // ---- staging -------------------------------------------------------------
+  const uint64_t pol = l2_evict_first();
+  if (UPDATE) {
+    for (int r = 0; r < it.nseg; ++r) {
+      const LongBdd B = A.longs[A.long_order[it.first + r]];
+      copy_row(avg + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
+    }
+    cp_async_commit();
+  }
+  grid_wait();
+  grid_trigger();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd B = A.longs[A.long_order[it.first + r]];
+    copy_row(lam + r * ST, a.lam + B.slot_base, B.k, lane, pol);
+    if (UPDATE && MODE == 1) {
+      copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
+      copy_row(al + r * ST, a.alpha + B.slot_base, B.k, lane, pol);
+    }
+  }
+  cp_async_commit();
+  if (UPDATE) {
+    cp_async_wait_one();
+    __syncwarp();
+    const float* src = MODE == 1 ? A.S : A.Sbar;
+    for (int r = 0; r < it.nseg; ++r) {
+      const int k = A.longs[A.long_order[it.first + r]].k;
+#pragma unroll 4
+      for (int h = lane; h < k; h += kWarp) {
+        const int v = __float_as_int(avg[r * ST + h]);
+        cp_async4(avg + r * ST + h, src + v);
+      }
+    }
+    cp_async_commit();
+  }
+  cp_async_wait_all();
+  __syncwarp();
+
+  // ---- the walk --------------------------------------------------------------
+  if constexpr (G <= kUnitMaxW)
+    walk_lanes<KIND, MODE, G>(A, a, it, lam, avg, om, al, cost, lane);
+  else
+    walk_segments<KIND, MODE, G>(A, a, it, lam, avg, om, al, cost, lane);
 
   // ---- the new state ---------------------------------------------------------
   if (KIND == kEnergy) return;
@@ -411,49 +617,15 @@ __global__ void __launch_bounds__(32) k_long_unit(DevArena A, SweepArgs a) {
   }
 }
 
-// Adjoint of a recording sweep: the reverse of the walk with the gradients of
-// a level's path costs on the segment's lanes (see kernels_adjoint.cu for the
-// steps and kernels_unit.cu for the routing along the recorded arcs).
+// The reverse walk with the gradients of a level's path costs on the lanes of
+// a segment.  Replaces, per level, the gradient of lambda^new by lambda^old's
+// (gl), the weight by the contribution to S-dot (al), and the pair by the
+// contributions to omega-dot and alpha-dot (in).
 template <int FWD, int MODE, int G>
-__device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const AdjArgs& a, const LongItem& it,
-                                                       float* smem, int lane) {
-  const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST;
-  uint4* rec = reinterpret_cast<uint4*>(smem);
-  float2* in = reinterpret_cast<float2*>(rec + nrow);
-  float* gl = reinterpret_cast<float*>(in + nrow);
-  float* df = gl + nrow;
-  float* al = df + nrow;
-  float* om = al + nrow;
-  float* id = om + nrow;
-  const uint64_t pol = l2_evict_first();
-  for (int r = 0; r < it.nseg; ++r) {
-    const LongBdd B = A.longs[A.long_order[it.first + r]];
-    copy_row(id + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
-  }
-  cp_async_commit();
-  grid_wait();
-  grid_trigger();
-  for (int r = 0; r < it.nseg; ++r) {
-    const LongBdd B = A.longs[A.long_order[it.first + r]];
-    copy_row(gl + r * ST, a.g_lam + B.slot_base, B.k, lane, pol);
-    copy_row(df + r * ST, a.rec_diff + B.slot_base, B.k, lane, pol);
-    copy_row(al + r * ST, (MODE == 1 ? a.alpha : A.slot_invdeg) + B.slot_base, B.k, lane, pol);
-    if (MODE == 1) copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
-    const uint4* src = a.rec_lunit + (B.slot_base - A.long_slot_base);
-    for (int h = lane; h < B.k; h += kWarp) cp_async16(rec + r * ST + h, src + h, pol);
-  }
-  cp_async_commit();
-  cp_async_wait_one();
-  __syncwarp();
-  for (int r = 0; r < it.nseg; ++r) {
-    const int k = A.longs[A.long_order[it.first + r]].k;
-#pragma unroll 4
-    for (int h = lane; h < k; h += kWarp) cp_async8(in + r * ST + h, a.var_in + __float_as_int(id[r * ST + h]));
-  }
-  cp_async_commit();
-  cp_async_wait_all();
-  __syncwarp();
-
+__device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArgs& a, const LongItem& it,
+                                                 const uint4* rec, float2* in, float* gl, float* df, float* al,
+                                                 const float* om, int lane) {
+  const int ST = long_unit_stride(it.kmax);
   LSeg<G> g;
   g.s = lane & (G - 1);
   g.base = lane - g.s;
@@ -581,6 +753,174 @@ __device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const 
       }
     });
   }
+}
+
+// ... in the registers of the BDD's lane.
+template <int FWD, int MODE, int W>
+__device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& a, const LongItem& it,
+                                              const uint4* rec, float2* in, float* gl, float* df, float* al,
+                                              const float* om, int lane) {
+  const int ST = long_unit_stride(it.kmax);
+  const bool act = lane < it.nseg;
+  const int row = act ? lane : 0;
+  const LongBdd B = A.longs[A.long_order[it.first + row]];
+  const int k = act ? B.k : 0, last = max(k - 1, 0);
+  float* mg = gl + row * ST;
+  float* md = df + row * ST;
+  float* mw = al + row * ST;
+  const float* mo = om + row * ST;
+  float2* mi = in + row * ST;
+  const uint4* mr = rec + row * ST;
+  const float* seed = a.seed_M ? a.seed_M + B.slot_base : nullptr;
+  struct In {  // a level's inputs, read one level ahead
+    uint32_t rec;
+    float g, df, w, om, seed;
+    float2 v;
+  };
+  auto input = [&](int h) {
+    const int x = min(max(h, 0), last);
+    return In{mr[x].x, mg[x], md[x], mw[x], MODE == 1 ? mo[x] : a.omega0, seed && act ? seed[x] : 0.0f, mi[x]};
+  };
+  auto reverse = [&](int h, const In& x, float g) -> float {
+    const float Mt = x.seed + x.v.x - g;
+    const float d = x.om * Mt;
+    mi[h] = make_float2(Mt * x.df, g * x.v.y);
+    mw[h] = x.w * g;
+    md[h] = d;
+    mg[h] = g + d;
+    return d;
+  };
+  Costs<W> x;
+  auto clear = [&](Costs<W>& c) {
+#pragma unroll
+    for (int u = 0; u < W; ++u) c.v[u] = 0.0f;
+  };
+  clear(x);
+  if (FWD) {
+    // SP(r, .) of level h + 1 was relaxed from level h with lambda^new_h
+    In v = input(it.kmax - 1);
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = e - 1; h >= b; --h) {
+        const In nxt = input(h - 1);
+        if (h < k) {
+          float g = v.g;
+          x = unit_route_in<W, TY>(x, v.rec, g);
+          unit_seed_in<W>(x, v.rec, reverse(h, v, g));
+        }
+        v = nxt;
+      }
+    });
+    // SP(., T) under lambda^old: its gradient flows top-down
+    clear(x);
+    uint32_t rc = mr[0].x;
+    float d = md[0];
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = b; h < e; ++h) {
+        const int n = min(h + 1, last);
+        const uint32_t rc1 = mr[n].x;
+        const float d1 = md[n];
+        if (h < k) {
+          Costs<W> y;
+          clear(y);
+          float g = 0.0f;
+          unit_seed_out<W, TY>(y, rc, d);
+          unit_route_out<W, TY>(x, rc, y, g);
+          x = y;
+          mg[h] += g;
+        }
+        rc = rc1;
+        d = d1;
+      }
+    });
+  } else {
+    // SP(., T) of level h was recomputed with lambda^new_h
+    In v = input(0);
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = b; h < e; ++h) {
+        const In nxt = input(h + 1);
+        if (h < k) {
+          Costs<W> y;
+          clear(y);
+          float g = v.g;
+          unit_route_out<W, TY>(x, v.rec, y, g);
+          unit_seed_out<W, TY>(y, v.rec, reverse(h, v, g));
+          x = y;
+        }
+        v = nxt;
+      }
+    });
+    // SP(r, .) under lambda^old: its gradient flows bottom-up
+    clear(x);
+    uint32_t rc = mr[last].x;
+    float d = md[last];
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      constexpr int TY = decltype(ty)::value;
+      for (int h = e - 1; h >= b; --h) {
+        if (h >= k) continue;
+        const int n = max(h - 1, 0);
+        const uint32_t rc1 = mr[n].x;
+        const float d1 = md[n];
+        float g = 0.0f;
+        x = unit_route_in<W, TY>(x, rc, g);
+        unit_seed_in<W>(x, rc, d);
+        mg[h] += g;
+        rc = rc1;
+        d = d1;
+      }
+    });
+  }
+}
+
+// Adjoint of a recording sweep: the reverse of the walk with the gradients of
+// a level's path costs on the segment's lanes (see kernels_adjoint.cu for the
+// steps and kernels_unit.cu for the routing along the recorded arcs).
+template <int FWD, int MODE, int G>
+__device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const AdjArgs& a, const LongItem& it,
+                                                       float* smem, int lane) {
+  const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST;
+  uint4* rec = reinterpret_cast<uint4*>(smem);
+  float2* in = reinterpret_cast<float2*>(rec + nrow);
+  float* gl = reinterpret_cast<float*>(in + nrow);
+  float* df = gl + nrow;
+  float* al = df + nrow;
+  float* om = al + nrow;
+  float* id = om + nrow;
+  const uint64_t pol = l2_evict_first();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd B = A.longs[A.long_order[it.first + r]];
+    copy_row(id + r * ST, A.slot_var + B.slot_base, B.k, lane, pol);
+  }
+  cp_async_commit();
+  grid_wait();
+  grid_trigger();
+  for (int r = 0; r < it.nseg; ++r) {
+    const LongBdd B = A.longs[A.long_order[it.first + r]];
+    copy_row(gl + r * ST, a.g_lam + B.slot_base, B.k, lane, pol);
+    copy_row(df + r * ST, a.rec_diff + B.slot_base, B.k, lane, pol);
+    copy_row(al + r * ST, (MODE == 1 ? a.alpha : A.slot_invdeg) + B.slot_base, B.k, lane, pol);
+    if (MODE == 1) copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
+    const uint4* src = a.rec_lunit + (B.slot_base - A.long_slot_base);
+    for (int h = lane; h < B.k; h += kWarp) cp_async16(rec + r * ST + h, src + h, pol);
+  }
+  cp_async_commit();
+  cp_async_wait_one();
+  __syncwarp();
+  for (int r = 0; r < it.nseg; ++r) {
+    const int k = A.longs[A.long_order[it.first + r]].k;
+#pragma unroll 4
+    for (int h = lane; h < k; h += kWarp) cp_async8(in + r * ST + h, a.var_in + __float_as_int(id[r * ST + h]));
+  }
+  cp_async_commit();
+  cp_async_wait_all();
+  __syncwarp();
+
+  if constexpr (G <= kUnitMaxW)
+    adjoint_lanes<FWD, MODE, G>(A, a, it, rec, in, gl, df, al, om, lane);
+  else
+    adjoint_segments<FWD, MODE, G>(A, a, it, rec, in, gl, df, al, om, lane);
   __syncwarp();
   for (int r = 0; r < it.nseg; ++r) {
     const LongBdd Br = A.longs[A.long_order[it.first + r]];
