@@ -143,10 +143,11 @@ constexpr int kLongUnitMaxK = 1400;  // levels whose path costs fit a CTA's shar
 // Row stride (floats) of a per-level array of one BDD in shared memory: whole
 // 16-byte pieces.
 DG_HD inline int long_unit_stride(int kmax) { return (kmax + 3) / 4 * 4; }
-// Shared memory of one item in the sweeps: the path costs of levels 0 .. kmax
-// and per BDD lambda, the averaging term and (mode 1) omega and alpha ...
+// Shared memory of one item in the sweeps: per BDD lambda, the averaging term
+// and (mode 1) omega and alpha, then the path costs of levels 0 .. kmax; one
+// level more at both ends (read ahead, not used) ...
 inline size_t long_unit_bytes(int nseg, int G, int kmax, int mode) {
-  const size_t b = 4 * ((size_t)nseg * (mode ? 4 : 2) * long_unit_stride(kmax) + (size_t)(kmax + 1) * nseg * G);
+  const size_t b = 4 * (4 + (size_t)nseg * (mode ? 4 : 2) * long_unit_stride(kmax) + (size_t)(kmax + 2) * nseg * G);
   return (b + 127) / 128 * 128;
 }
 // ... and in the adjoint: per level and BDD the gradient of lambda, m1 - m0,

@@ -344,24 +344,25 @@ __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs
   }
 }
 
-// ... with a level's states in the registers of the BDD's lane.
+// ... with a level's states in the registers of the BDD's lane.  Lanes beyond
+// the item's BDDs repeat another lane's (same addresses, same values), so that
+// nothing diverges; only past the shortest BDD's levels (kmin) are the steps
+// guarded.  Reads one level ahead may go one level past either end: the arrays
+// have that much room.
 template <int KIND, int MODE, int W>
 __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a, const LongItem& it, float* lam,
                                            float* avg, const float* om, const float* al, float* cost, int lane) {
   constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
   constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
   constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
-  const int ST = long_unit_stride(it.kmax);
-  const bool act = lane < it.nseg;
-  const int row = act ? lane : 0;
+  const int ST = long_unit_stride(it.kmax), row = lane % it.nseg, TS = it.nseg * W;
   const LongBdd B = A.longs[A.long_order[it.first + row]];
-  const int k = act ? B.k : 0;  // a lane without a BDD walks nothing
+  const int k = B.k, kmin = __reduce_min_sync(kAll, k);
   float* ml = lam + row * ST;
   float* ma = avg + row * ST;
   const float* mo = om + row * ST;
   const float* mw = al + row * ST;
   float* mt = cost + row * W;  // level h at mt[h TS], the terminals' at level k
-  const int TS = it.nseg * W, last = max(k - 1, 0);
   auto put = [&](int h, const Costs<W>& c) {
     if constexpr (W == 2) {
       *reinterpret_cast<float2*>(mt + h * TS) = make_float2(c.v[0], c.v[1]);
@@ -391,28 +392,43 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
   };
   const Costs<W> end = unit_end<W>((int)it.accept);
   const Costs<W> root = unit_root<W>(it.start);
-  // a level's inputs, read one level ahead
-  struct In {
+  struct In {  // a level's inputs
     float l, av, w, al;
   };
   auto input = [&](int h) {
-    const int x = min(max(h, 0), last);
-    return In{ml[x], ma[x], MODE == 1 ? mo[x] : a.omega0, MODE == 1 ? mw[x] : 0.0f};
+    return In{ml[h], ma[h], MODE == 1 ? mo[h] : a.omega0, MODE == 1 ? mw[h] : 0.0f};
+  };
+  // step(type, level) for the levels in ascending / descending order, of a BDD
+  // shorter than the level none
+  auto down_levels = [&](auto&& step) {
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      const int m = min(e, kmin);
+      int h = b;
+#pragma unroll 2
+      for (; h < m; ++h) step(ty, h, true);
+      for (; h < e; ++h) step(ty, h, h < k);
+    });
+  };
+  auto up_levels = [&](auto&& step) {
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      const int m = max(b, kmin);
+      int h = e - 1;
+      for (; h >= m; --h) step(ty, h, h < k);
+#pragma unroll 2
+      for (; h >= b; --h) step(ty, h, true);
+    });
   };
   auto first_up = [&]() {
     Costs<W> t = end;
-    if (act) put(k, end);
-    float l = ml[last];
-    runs_up(A, it, [&](auto ty, int b, int e) {
-      constexpr int TY = decltype(ty)::value;
-      for (int h = e - 1; h >= b; --h) {
-        const float l1 = ml[min(max(h - 1, 0), last)];
-        if (h < k) {
-          t = unit_up<W, TY>(t, l);
-          put(h, t);
-        }
-        l = l1;
+    put(k, end);
+    float l = ml[it.kmax - 1];
+    up_levels([&](auto ty, int h, bool on) {
+      const float l1 = ml[h - 1];
+      if (on) {
+        t = unit_up<W, decltype(ty)::value>(t, l);
+        put(h, t);
       }
+      l = l1;
     });
     return t;
   };
@@ -426,7 +442,7 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
     return ln;
   };
   auto energy = [&](const Costs<W>& t) {  // E^j = SP(r, T)
-    if (a.E == nullptr || !act) return;
+    if (a.E == nullptr) return;
     float e = f_inf();
 #pragma unroll
     for (int u = 0; u < W; ++u)
@@ -437,78 +453,75 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
 
   if (FWD || KIND == kMinMarg) {
     first_up();
+    __syncwarp();
     Costs<W> R = root;
     In in = input(0);
-    Costs<W> t1 = get(min(1, k));
-    runs_down(A, it, [&](auto ty, int b, int e) {
+    Costs<W> t1 = get(1);
+    down_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      for (int h = b; h < e; ++h) {
-        const In nxt = input(h + 1);
-        const Costs<W> t2 = get(min(h + 2, k));
-        if (h < k) {
-          float b0, b1;
-          if (REC) {
-            uint32_t rec = 0;
-            unit_minima_rec<W, TY>(R, t1, b0, b1, rec);
-            unit_up_rec<W, TY>(t1, in.l, rec);
-            R = unit_down_rec<W, TY>(R, update(h, in, b0, b1), rec);
-            rec_out[h].x = rec;
+      const In nxt = input(h + 1);
+      const Costs<W> t2 = get(h + 2);
+      __syncwarp();
+      if (on) {
+        float b0, b1;
+        if (REC) {
+          uint32_t rec = 0;
+          unit_minima_rec<W, TY>(R, t1, b0, b1, rec);
+          unit_up_rec<W, TY>(t1, in.l, rec);
+          R = unit_down_rec<W, TY>(R, update(h, in, b0, b1), rec);
+          rec_out[h].x = rec;
+        } else {
+          unit_minima<W, TY>(R, t1, b0, b1);
+          float ln = in.l;
+          if (KIND == kMinMarg) {
+            ml[h] = in.l + b1;
+            ma[h] = b0;
           } else {
-            unit_minima<W, TY>(R, t1, b0, b1);
-            float ln = in.l;
-            if (KIND == kMinMarg) {
-              ml[h] = in.l + b1;
-              ma[h] = b0;
-            } else {
-              ln = update(h, in, b0, b1);
-            }
-            R = unit_down<W, TY>(R, ln);
+            ln = update(h, in, b0, b1);
           }
+          R = unit_down<W, TY>(R, ln);
         }
-        in = nxt;
-        t1 = t2;
       }
+      in = nxt;
+      t1 = t2;
     });
   } else if (BWD) {
     {
       Costs<W> R = root;
       float l = ml[0];
-      runs_down(A, it, [&](auto ty, int b, int e) {
-        constexpr int TY = decltype(ty)::value;
-        for (int h = b; h < e; ++h) {
-          const float l1 = ml[min(h + 1, last)];
-          if (h < k) {
-            put(h, R);
-            R = unit_down<W, TY>(R, l);
-          }
-          l = l1;
+      down_levels([&](auto ty, int h, bool on) {
+        const float l1 = ml[h + 1];
+        if (on) {
+          put(h, R);
+          R = unit_down<W, decltype(ty)::value>(R, l);
         }
+        l = l1;
       });
     }
+    __syncwarp();
     Costs<W> t = end;
     In in = input(it.kmax - 1);
-    Costs<W> r = get(min(it.kmax - 1, last));
-    runs_up(A, it, [&](auto ty, int b, int e) {
+    Costs<W> r = get(it.kmax - 1);
+    up_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      for (int h = e - 1; h >= b; --h) {
-        const In nxt = input(h - 1);
-        const Costs<W> r1 = get(min(max(h - 1, 0), last));
-        if (h < k) {
-          float b0, b1;
-          if (REC) {
-            uint32_t rec = 0;
-            unit_minima_rec<W, TY>(r, t, b0, b1, rec);
-            unit_down_rec<W, TY>(r, in.l, rec);
-            t = unit_up_rec<W, TY>(t, update(h, in, b0, b1), rec);
-            rec_out[h].x = rec;
-          } else {
-            unit_minima<W, TY>(r, t, b0, b1);
-            t = unit_up<W, TY>(t, update(h, in, b0, b1));
-          }
+      const In nxt = input(h - 1);
+      const Costs<W> r1 = get(max(h - 1, 0));
+      __syncwarp();
+      if (on) {
+        float b0, b1;
+        if (REC) {
+          uint32_t rec = 0;
+          unit_minima_rec<W, TY>(r, t, b0, b1, rec);
+          unit_down_rec<W, TY>(r, in.l, rec);
+          t = unit_up_rec<W, TY>(t, update(h, in, b0, b1), rec);
+          rec_out[h].x = rec;
+        } else {
+          unit_minima<W, TY>(r, t, b0, b1);
+          t = unit_up<W, TY>(t, update(h, in, b0, b1));
         }
-        in = nxt;
-        r = r1;
       }
+      in = nxt;
+      r = r1;
     });
     energy(t);
   } else {
@@ -517,18 +530,18 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
       energy(t);
     } else {
       // kSeed: walk the minimising path from the root, the 0-arc on ties
+      __syncwarp();
       int at = it.start;
-      runs_down(A, it, [&](auto ty, int b, int e) {
+      down_levels([&](auto ty, int h, bool on) {
         constexpr int TY = decltype(ty)::value;
-        for (int h = b; h < min(e, k); ++h) {
-          const int z = lz<W, TY>(at), o = lo_<W, TY>(at);
-          const float* p = mt + (h + 1) * TS;
-          const float c0 = p[z], c1 = o >= 0 && o < W ? p[o] : f_inf();
-          // an infinite cost is the bottom terminal (the path stays feasible)
-          const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= ml[h] + c1);
-          ma[h] = take0 ? 0.f : 1.f;
-          at = take0 ? z : max(min(o, W - 1), 0);
-        }
+        if (!on) return;
+        const int z = lz<W, TY>(at), o = lo_<W, TY>(at);
+        const float* p = mt + (h + 1) * TS;
+        const float c0 = p[z], c1 = o >= 0 && o < W ? p[o] : f_inf();
+        // an infinite cost is the bottom terminal (the path stays feasible)
+        const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= ml[h] + c1);
+        ma[h] = take0 ? 0.f : 1.f;
+        at = take0 ? z : max(min(o, W - 1), 0);
       });
     }
   }
@@ -539,7 +552,7 @@ __device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArg
                                                int lane) {
   constexpr bool UPDATE = KIND == kFwd || KIND == kBwd || KIND == kFwdRec || KIND == kBwdRec;
   const int ST = long_unit_stride(it.kmax), nrow = it.nseg * ST;
-  float* lam = smem;
+  float* lam = smem + 4;  // room for the level before the first
   float* avg = lam + nrow;
   float* om = avg + nrow;
   float* al = om + (MODE == 1 ? nrow : 0);
@@ -755,16 +768,14 @@ __device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArg
   }
 }
 
-// ... in the registers of the BDD's lane.
+// ... in the registers of the BDD's lane (lanes and levels as in walk_lanes).
 template <int FWD, int MODE, int W>
 __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& a, const LongItem& it,
                                               const uint4* rec, float2* in, float* gl, float* df, float* al,
                                               const float* om, int lane) {
-  const int ST = long_unit_stride(it.kmax);
-  const bool act = lane < it.nseg;
-  const int row = act ? lane : 0;
+  const int ST = long_unit_stride(it.kmax), row = lane % it.nseg;
   const LongBdd B = A.longs[A.long_order[it.first + row]];
-  const int k = act ? B.k : 0, last = max(k - 1, 0);
+  const int k = B.k, kmin = __reduce_min_sync(kAll, k), last = k - 1;
   float* mg = gl + row * ST;
   float* md = df + row * ST;
   float* mw = al + row * ST;
@@ -772,6 +783,22 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
   float2* mi = in + row * ST;
   const uint4* mr = rec + row * ST;
   const float* seed = a.seed_M ? a.seed_M + B.slot_base : nullptr;
+  auto down_levels = [&](auto&& step) {
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      const int m = min(e, kmin);
+      int h = b;
+      for (; h < m; ++h) step(ty, h, true);
+      for (; h < e; ++h) step(ty, h, h < k);
+    });
+  };
+  auto up_levels = [&](auto&& step) {
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      const int m = max(b, kmin);
+      int h = e - 1;
+      for (; h >= m; --h) step(ty, h, h < k);
+      for (; h >= b; --h) step(ty, h, true);
+    });
+  };
   struct In {  // a level's inputs, read one level ahead
     uint32_t rec;
     float g, df, w, om, seed;
@@ -779,7 +806,7 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
   };
   auto input = [&](int h) {
     const int x = min(max(h, 0), last);
-    return In{mr[x].x, mg[x], md[x], mw[x], MODE == 1 ? mo[x] : a.omega0, seed && act ? seed[x] : 0.0f, mi[x]};
+    return In{mr[x].x, mg[x], md[x], mw[x], MODE == 1 ? mo[x] : a.omega0, seed ? seed[x] : 0.0f, mi[x]};
   };
   auto reverse = [&](int h, const In& x, float g) -> float {
     const float Mt = x.seed + x.v.x - g;
@@ -799,76 +826,77 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
   if (FWD) {
     // SP(r, .) of level h + 1 was relaxed from level h with lambda^new_h
     In v = input(it.kmax - 1);
-    runs_up(A, it, [&](auto ty, int b, int e) {
+    up_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      for (int h = e - 1; h >= b; --h) {
-        const In nxt = input(h - 1);
-        if (h < k) {
-          float g = v.g;
-          x = unit_route_in<W, TY>(x, v.rec, g);
-          unit_seed_in<W>(x, v.rec, reverse(h, v, g));
-        }
-        v = nxt;
+      const In nxt = input(h - 1);
+      __syncwarp();
+      if (on) {
+        float g = v.g;
+        x = unit_route_in<W, TY>(x, v.rec, g);
+        unit_seed_in<W>(x, v.rec, reverse(h, v, g));
       }
+      v = nxt;
     });
+    __syncwarp();
     // SP(., T) under lambda^old: its gradient flows top-down
     clear(x);
     uint32_t rc = mr[0].x;
-    float d = md[0];
-    runs_down(A, it, [&](auto ty, int b, int e) {
+    float d = md[0], g0 = mg[0];
+    down_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      for (int h = b; h < e; ++h) {
-        const int n = min(h + 1, last);
-        const uint32_t rc1 = mr[n].x;
-        const float d1 = md[n];
-        if (h < k) {
-          Costs<W> y;
-          clear(y);
-          float g = 0.0f;
-          unit_seed_out<W, TY>(y, rc, d);
-          unit_route_out<W, TY>(x, rc, y, g);
-          x = y;
-          mg[h] += g;
-        }
+      const int n = min(h + 1, last);
+      const uint32_t rc1 = mr[n].x;
+      const float d1 = md[n], g1 = mg[n];
+      __syncwarp();
+      if (on) {
+        Costs<W> y;
+        clear(y);
+        float g = 0.0f;
+        unit_seed_out<W, TY>(y, rc, d);
+        unit_route_out<W, TY>(x, rc, y, g);
+        x = y;
+        mg[h] = g0 + g;
         rc = rc1;
         d = d1;
+        g0 = g1;
       }
     });
   } else {
     // SP(., T) of level h was recomputed with lambda^new_h
     In v = input(0);
-    runs_down(A, it, [&](auto ty, int b, int e) {
+    down_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      for (int h = b; h < e; ++h) {
-        const In nxt = input(h + 1);
-        if (h < k) {
-          Costs<W> y;
-          clear(y);
-          float g = v.g;
-          unit_route_out<W, TY>(x, v.rec, y, g);
-          unit_seed_out<W, TY>(y, v.rec, reverse(h, v, g));
-          x = y;
-        }
-        v = nxt;
+      const In nxt = input(h + 1);
+      __syncwarp();
+      if (on) {
+        Costs<W> y;
+        clear(y);
+        float g = v.g;
+        unit_route_out<W, TY>(x, v.rec, y, g);
+        unit_seed_out<W, TY>(y, v.rec, reverse(h, v, g));
+        x = y;
       }
+      v = nxt;
     });
+    __syncwarp();
     // SP(r, .) under lambda^old: its gradient flows bottom-up
     clear(x);
     uint32_t rc = mr[last].x;
-    float d = md[last];
-    runs_up(A, it, [&](auto ty, int b, int e) {
+    float d = md[last], g0 = mg[last];
+    up_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      for (int h = e - 1; h >= b; --h) {
-        if (h >= k) continue;
-        const int n = max(h - 1, 0);
-        const uint32_t rc1 = mr[n].x;
-        const float d1 = md[n];
+      const int n = max(h - 1, 0);
+      const uint32_t rc1 = mr[n].x;
+      const float d1 = md[n], g1 = mg[n];
+      __syncwarp();
+      if (on) {
         float g = 0.0f;
         x = unit_route_in<W, TY>(x, rc, g);
         unit_seed_in<W>(x, rc, d);
-        mg[h] += g;
+        mg[h] = g0 + g;
         rc = rc1;
         d = d1;
+        g0 = g1;
       }
     });
   }
