@@ -336,6 +336,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
       return fail(DG_EINVAL, "dg_bind: tiles need more shared memory than a CTA has");
     e = set_sweep_smem_limit((size_t)optin);  // same limit for every arena of the process
     if (e == cudaSuccess) e = set_unit_smem_limit((size_t)optin);
+    if (e == cudaSuccess) e = set_long_smem_limit((size_t)optin - 1024);  // next to the reductions' words
     if (e == cudaSuccess) e = set_long_unit_smem_limit((size_t)optin);
     if (e == cudaSuccess) e = set_adjoint_smem_limit((size_t)optin);
     set_cta_smem_cap((size_t)optin);
@@ -414,6 +415,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.num_long_items = (int32_t)P.long_items.size();
   for (int mode = 0; mode < 2; ++mode) A.long_unit_smem[mode] = P.long_unit_smem[mode];
   A.long_unit_adj_smem = P.long_unit_adj_smem;
+  A.long_wide_smem = P.long_wide_smem;
   {
     // lanes per narrow long BDD: the widest level's power of two (or the
     // option's, if larger); by default doubled (fewer BDDs per warp) while

@@ -896,8 +896,13 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
                      [](const LongItem& x, const LongItem& y) { return x.kmax > y.kmax; });
     P.num_long_narrow = (int32_t)P.long_order.size();
     P.long_lanes = opts ? opts->long_lanes : 0;
+    size_t wide = 0;
     for (size_t b = 0; b < P.longs.size(); ++b)
-      if (P.longs[b].maxw > kWarp) P.long_order.push_back((int32_t)b);
+      if (P.longs[b].maxw > kWarp) {
+        P.long_order.push_back((int32_t)b);
+        wide = std::max(wide, (size_t)(P.longs[b].nn + 2) * 8);
+      }
+    P.long_wide_smem = wide <= 200 * 1024 ? (int32_t)wide : 0;
   }
   const int64_t num_slots = slot_base;
   if (num_slots >= (int64_t)INT32_MAX || node_base >= (int64_t)INT32_MAX)

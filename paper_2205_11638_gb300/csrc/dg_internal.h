@@ -217,6 +217,7 @@ struct DevArena {
   int32_t num_long_narrow;  // narrow long BDDs (the head of long_order)
   int32_t num_long_unit;    // ... of them, the unit ones (its very head)
   int32_t num_long_items;
+  int32_t long_wide_smem;   // shared memory of the largest wide long BDD's path costs (0: one does not fit)
   int32_t long_unit_smem[2];  // shared memory of the largest work item, mode 0 and 1
   int32_t long_unit_adj_smem;
   int32_t long_lanes;       // lanes per narrow BDD in the plain sweeps (a power of two, set at bind)
@@ -288,7 +289,7 @@ struct Plan {
   std::vector<int32_t> long_order;  // see DevArena::long_order
   int32_t num_long_narrow = 0, num_long_unit = 0;
   std::vector<LongItem> long_items;
-  int32_t long_unit_smem[2] = {0, 0}, long_unit_adj_smem = 0;
+  int32_t long_unit_smem[2] = {0, 0}, long_unit_adj_smem = 0, long_wide_smem = 0;
   int32_t long_lanes = 0;           // dg_options::long_lanes (0: chosen at bind)
   std::vector<int64_t> long_rank_ptr;  // per long BDD, first entry of long_lo / long_hi
   std::vector<int32_t> long_lo, long_hi;  // child ranks as in lo8 / hi8 (-2 bottom, -1 top)

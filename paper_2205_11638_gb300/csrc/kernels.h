@@ -115,6 +115,8 @@ __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.la
 // the SMs better side by side, large shared-memory tiles next to narrow ones,
 // than one after another (100 frames, 19,000 tiles 88 / 82; 500 frames, 96,000
 // tiles 438 / 370).
+// Kinds of long BDDs an arena has (unit rows, others).
+inline int long_launches(const DevArena& A) { return (A.num_long_items > 0) + (A.num_long > A.num_long_unit); }
 constexpr int kChainTiles = 16384;
 inline bool chained_sweeps(const DevArena& A, int num_groups) {
   if (num_groups == 0) return A.num_long == A.num_long_unit;
@@ -214,6 +216,7 @@ void launch_param_transform_bwd(const DevArena& A, const float* alpha, const flo
 
 // Long BDDs, one warp per BDD (kernels_long.cu); each is a single launch on
 // the given stream, or nothing when the arena has no long BDDs.
+cudaError_t set_long_smem_limit(size_t bytes);
 cudaError_t set_long_unit_smem_limit(size_t bytes);
 void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, Chain& ch);
 void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, Chain& ch);

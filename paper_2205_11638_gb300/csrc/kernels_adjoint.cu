@@ -249,11 +249,16 @@ static void launch_adj(const DevArena& A, const AdjArgs& a, const AdjGroup* grou
                        Chain& ch) {
   const bool chained = chained_sweeps(A, num_groups);
   const StreamSet& ss = ch.ss;
-  const bool fork = !chained && num_groups + (A.num_long > 0 ? 1 : 0) > 1 && ss.ready;
+  const bool fork = !chained && num_groups + long_launches(A) > 1 && ss.ready;
   if (fork) ss.begin();
   if (!chained) {
     ch.linked = false;
     launch_long_adjoint(FWD != 0, A, a, fork ? ss.of(A.long_stream) : ss.main);
+    if (A.num_long_items > 0) {
+      Chain own;
+      own.ss.main = fork ? ss.of(A.long_stream + (A.num_long > A.num_long_unit ? 1 : 0)) : ss.main;
+      launch_long_unit_adjoint(FWD != 0, A, a, own);
+    }
   } else if (A.num_long_items > 0) {
     launch_long_unit_adjoint(FWD != 0, A, a, ch);
   }

@@ -5,11 +5,14 @@
 // subproblems as the sequential part of the method (its conclusion): App. B's
 // recursions over one BDD visit its levels one after another.
 //
-// Execution model: one warp per BDD; the nodes of a level are spread over the
-// lanes (node f + lane, f + lane + 32, ...), the levels are walked in turn
-// with a __syncwarp between them.  The min-marginals of a level (App. B:
+// Execution model: one team of threads per BDD, a warp for BDDs of at most 32
+// nodes a level and a block of 256 threads for wider ones (a level of 169 nodes
+// took a warp six rounds of dependent loads); the nodes of a level are spread
+// over the team (node f + id, f + id + size, ...), the levels are walked in
+// turn with a barrier of the team between them.  The min-marginals of a level (App. B:
 // m^beta = min over the level's nodes of SP(r, v) + SP(s^beta(v), T), plus
-// lambda for beta = 1) are lane minima combined by warp shuffles; SP(r, .)
+// lambda for beta = 1) are the threads' minima combined by shuffles (and, in a block, one round
+// through shared memory); SP(r, .)
 // of a level is a pull over each node's in-arc list, SP(., T) over its two
 // children, so no two lanes write the same node and nothing needs atomics.
 // Path costs live in the arena's scratch (long_d, long_t, indexed by node
@@ -84,6 +87,77 @@ __device__ __forceinline__ float warp_lse(float x) {
   return x;
 }
 
+// The threads that walk one BDD together.
+struct WarpTeam {
+  static constexpr int kSize = kWarp;
+  int id;
+  __device__ __forceinline__ void sync() const { __syncwarp(); }
+  __device__ __forceinline__ void min2(float& a, float& b) {
+    a = warp_min(a);
+    b = warp_min(b);
+  }
+  __device__ __forceinline__ void argmin(float& v, int& n) { warp_argmin(v, n); }
+  __device__ __forceinline__ float sum(float x) { return warp_sum(x); }
+};
+struct BlockTeam {
+  static constexpr int kSize = 256, kWarps = kSize / kWarp;
+  int id;
+  float* sh;  // [2][2][kWarps]; the halves take turns, so one barrier per reduction
+  int half = 0;
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+  __device__ __forceinline__ float* turn() {
+    half ^= 1;
+    return sh + half * 2 * kWarps;
+  }
+  __device__ __forceinline__ void min2(float& a, float& b) {
+    float* p = turn();
+    a = warp_min(a);
+    b = warp_min(b);
+    if ((id & 31) == 0) {
+      p[id >> 5] = a;
+      p[kWarps + (id >> 5)] = b;
+    }
+    __syncthreads();
+    a = p[0];
+    b = p[kWarps];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+      a = fminf(a, p[w]);
+      b = fminf(b, p[kWarps + w]);
+    }
+  }
+  __device__ __forceinline__ void argmin(float& v, int& n) {
+    float* p = turn();
+    warp_argmin(v, n);
+    if ((id & 31) == 0) {
+      p[id >> 5] = v;
+      p[kWarps + (id >> 5)] = __int_as_float(n);
+    }
+    __syncthreads();
+    v = p[0];
+    n = __float_as_int(p[kWarps]);
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) {
+      const float v2 = p[w];
+      const int n2 = __float_as_int(p[kWarps + w]);
+      if (v2 < v || (v2 == v && n2 < n)) {
+        v = v2;
+        n = n2;
+      }
+    }
+  }
+  __device__ __forceinline__ float sum(float x) {
+    float* p = turn();
+    x = warp_sum(x);
+    if ((id & 31) == 0) p[id >> 5] = x;
+    __syncthreads();
+    x = p[0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) x += p[w];
+    return x;
+  }
+};
+
 // One warp's view of its BDD; every array is indexed by node number.
 struct LongCtx {
   LongBdd B;
@@ -123,26 +197,27 @@ __device__ __forceinline__ float long_lambda_new(float l, float Mn, float al, fl
 // recording sweep before it made in the same comparisons (keep: kLHi, the
 // out-arc choices of SP(., T), for a forward sweep; the in-arcs of SP(r, .)
 // for a backward one), the rest cleared for the sweep to write.
+template <class TEAM>
 __device__ __forceinline__ void long_take_records(const LongCtx& c, const int32_t* prev, int32_t* meta, int32_t keep,
-                                                  int lane) {
+                                                  TEAM& tm) {
   const int e = c.lvl[c.B.k];
-  for (int n = 2 + lane; n < e; n += kWarp) meta[n] = prev[n] & keep;
-  __syncwarp();
+  for (int n = 2 + tm.id; n < e; n += TEAM::kSize) meta[n] = prev[n] & keep;
+  tm.sync();
 }
 
 // SP(., T) of every node under lam, levels bottom-up.  REC: the record of
 // every node is rewritten with its hi-choice (0-arc on ties).
-template <bool REC>
-__device__ void long_cost_to_top(const LongCtx& c, const float* lam, int32_t* meta, int lane) {
-  if (lane == 0) {
+template <bool REC, class TEAM>
+__device__ void long_cost_to_top(const LongCtx& c, const float* lam, int32_t* meta, TEAM& tm) {
+  if (tm.id == 0) {
     c.t[kTopCode] = 0.0f;
     c.t[kBotCode] = f_inf();
   }
-  __syncwarp();
+  tm.sync();
   for (int h = c.B.k - 1; h >= 0; --h) {
     const float l = lam[c.B.slot_base + h];
     const int e = c.lvl[h + 1];
-    for (int n = c.lvl[h] + lane; n < e; n += kWarp) {
+    for (int n = c.lvl[h] + tm.id; n < e; n += TEAM::kSize) {
       const int2 cc = c.code[n];
       const float tl = c.t[cc.x], th = l + c.t[cc.y];
       if (REC) {
@@ -153,7 +228,7 @@ __device__ void long_cost_to_top(const LongCtx& c, const float* lam, int32_t* me
         c.t[n] = fminf(tl, th);
       }
     }
-    __syncwarp();
+    tm.sync();
   }
 }
 
@@ -183,30 +258,30 @@ __device__ __forceinline__ void relax_pull(const LongCtx& c, int n, float l, int
 
 // SP(r, .) of every node under lam, levels top-down.  REC: records rewritten
 // with the argmin in-arc (hi-choice cleared; the backward sweep sets it).
-template <bool REC>
-__device__ void long_cost_from_root(const LongCtx& c, const float* lam, int32_t* meta, int lane) {
-  if (lane == 0) {
+template <bool REC, class TEAM>
+__device__ void long_cost_from_root(const LongCtx& c, const float* lam, int32_t* meta, TEAM& tm) {
+  if (tm.id == 0) {
     c.d[2] = 0.0f;
     if (REC) meta[2] = 0;
   }
-  __syncwarp();
+  tm.sync();
   for (int h = 0; h + 1 < c.B.k; ++h) {
     const float l = lam[c.B.slot_base + h];
     const int e = c.lvl[h + 2];
-    for (int n = c.lvl[h + 1] + lane; n < e; n += kWarp) relax_pull<REC, false>(c, n, l, meta);
-    __syncwarp();
+    for (int n = c.lvl[h + 1] + tm.id; n < e; n += TEAM::kSize) relax_pull<REC, false>(c, n, l, meta);
+    tm.sync();
   }
 }
 
 // m0, m1 of level h: minima over its nodes of SP(r, v) + SP(child, T) by the
 // 0- and the 1-arc (lambda not yet added); REC: argmin nodes v0, v1.
-template <bool REC>
-__device__ __forceinline__ void level_minima(const LongCtx& c, int h, int lane, float& b0, float& b1, int& v0,
+template <bool REC, class TEAM>
+__device__ __forceinline__ void level_minima(const LongCtx& c, int h, TEAM& tm, float& b0, float& b1, int& v0,
                                              int& v1) {
   b0 = b1 = f_inf();
   v0 = v1 = INT_MAX;
   const int e = c.lvl[h + 1];
-  for (int n = c.lvl[h] + lane; n < e; n += kWarp) {
+  for (int n = c.lvl[h] + tm.id; n < e; n += TEAM::kSize) {
     const int2 cc = c.code[n];
     const float dv = c.d[n];
     const float x0 = dv + c.t[cc.x], x1 = dv + c.t[cc.y];
@@ -225,15 +300,14 @@ __device__ __forceinline__ void level_minima(const LongCtx& c, int h, int lane, 
     }
   }
   if (REC) {
-    warp_argmin(b0, v0);
-    warp_argmin(b1, v1);
+    tm.argmin(b0, v0);
+    tm.argmin(b1, v1);
     // a level without a finite candidate cannot occur in a planned arena (it
     // would force a variable); the first node keeps the record in range
     if (v0 == INT_MAX) v0 = c.lvl[h];
     if (v1 == INT_MAX) v1 = c.lvl[h];
   } else {
-    b0 = warp_min(b0);
-    b1 = warp_min(b1);
+    tm.min2(b0, b1);
   }
 }
 
@@ -458,22 +532,12 @@ __device__ __forceinline__ void narrow_up(const DevArena& A, const SweepArgs& a,
 
 }  // namespace
 
-template <int KIND, int MODE>
-__global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
+// One BDD's sweep by its team.
+template <int KIND, int MODE, class TEAM>
+__device__ __forceinline__ void long_sweep(const DevArena& A, const SweepArgs& a, const LongCtx& c, TEAM& tm) {
   constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
   constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
   constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
-  const int lane = threadIdx.x & 31;
-  int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (KIND == kFwd || KIND == kBwd) {
-    // the plain sweeps take the wide long BDDs here (k_long_narrow the others)
-    if (b >= A.num_long - A.num_long_narrow) return;  // whole warp leaves
-    b = A.long_order[A.num_long_narrow + b];
-  } else {
-    if (b >= A.num_long - A.num_long_unit) return;
-    b = A.long_order[A.num_long_unit + b];
-  }
-  const LongCtx c = long_ctx(A, b);
   const int64_t sb = c.B.slot_base;
   const int k = c.B.k;
   int32_t* meta = REC ? a.rec_lmeta + c.B.cost_base : nullptr;
@@ -481,29 +545,32 @@ __global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
 
   if (FWD || KIND == kMinMarg) {
     if (!handed)
-      long_cost_to_top<REC>(c, a.lam, meta, lane);
+      long_cost_to_top<REC>(c, a.lam, meta, tm);
     else if (REC)
-      long_take_records(c, a.lmeta_in + c.B.cost_base, meta, kLHi, lane);
-    if (lane == 0) c.d[2] = 0.0f;
-    __syncwarp();
+      long_take_records(c, a.lmeta_in + c.B.cost_base, meta, kLHi, tm);
+    if (tm.id == 0) c.d[2] = 0.0f;
+    tm.sync();
     for (int h = 0; h < k; ++h) {
       float b0, b1;
       int v0, v1;
-      level_minima<REC>(c, h, lane, b0, b1, v0, v1);
+      // (read before the minima's barrier: thread 0 writes lambda after it)
       const int64_t q = sb + h;
       const float l = a.lam[q];
+      const bool upd = KIND != kMinMarg;
+      const float om = MODE == 1 && upd ? a.omega[q] : a.omega0, al = MODE == 1 && upd ? a.alpha[q] : 0.0f;
+      const float av = upd ? A.slot_avg[q] : 0.0f;
+      level_minima<REC>(c, h, tm, b0, b1, v0, v1);
       const float m0 = b0, m1 = l + b1;
       float ln = l;
       if (KIND == kMinMarg) {
-        if (lane == 0) {
+        if (tm.id == 0) {
           a.M[q] = m0;
           a.out2[q] = m1;
         }
       } else {
-        const float om = MODE == 1 ? a.omega[q] : a.omega0;
         const float Mn = __fmul_rn(om, m1 - m0);
-        ln = long_lambda_new<MODE>(l, Mn, MODE == 1 ? a.alpha[q] : 0.0f, A.slot_avg[q]);
-        if (lane == 0) {
+        ln = long_lambda_new<MODE>(l, Mn, al, av);
+        if (tm.id == 0) {
           a.lam[q] = ln;
           a.M[q] = Mn;
           if (REC) {
@@ -514,31 +581,32 @@ __global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
       }
       if (h + 1 < k) {
         const int e = c.lvl[h + 2];
-        for (int n = c.lvl[h + 1] + lane; n < e; n += kWarp) relax_pull<REC, true>(c, n, ln, meta);
+        for (int n = c.lvl[h + 1] + tm.id; n < e; n += TEAM::kSize) relax_pull<REC, true>(c, n, ln, meta);
       }
-      __syncwarp();
+      tm.sync();
     }
   } else if (BWD) {
     if (!handed)
-      long_cost_from_root<REC>(c, a.lam, meta, lane);
+      long_cost_from_root<REC>(c, a.lam, meta, tm);
     else if (REC)
-      long_take_records(c, a.lmeta_in + c.B.cost_base, meta, ~kLHi, lane);
-    if (lane == 0) {
+      long_take_records(c, a.lmeta_in + c.B.cost_base, meta, ~kLHi, tm);
+    if (tm.id == 0) {
       c.t[kTopCode] = 0.0f;
       c.t[kBotCode] = f_inf();
     }
-    __syncwarp();
+    tm.sync();
     for (int h = k - 1; h >= 0; --h) {
       float b0, b1;
       int v0, v1;
-      level_minima<REC>(c, h, lane, b0, b1, v0, v1);
       const int64_t q = sb + h;
       const float l = a.lam[q];
+      const float om = MODE == 1 ? a.omega[q] : a.omega0, al = MODE == 1 ? a.alpha[q] : 0.0f;
+      const float av = A.slot_avg[q];
+      level_minima<REC>(c, h, tm, b0, b1, v0, v1);
       const float m0 = b0, m1 = l + b1;
-      const float om = MODE == 1 ? a.omega[q] : a.omega0;
       const float Mn = __fmul_rn(om, m1 - m0);
-      const float ln = long_lambda_new<MODE>(l, Mn, MODE == 1 ? a.alpha[q] : 0.0f, A.slot_avg[q]);
-      if (lane == 0) {
+      const float ln = long_lambda_new<MODE>(l, Mn, al, av);
+      if (tm.id == 0) {
         a.lam[q] = ln;
         a.M[q] = Mn;
         if (REC) {
@@ -547,7 +615,7 @@ __global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
         }
       }
       const int e = c.lvl[h + 1];
-      for (int n = c.lvl[h] + lane; n < e; n += kWarp) {
+      for (int n = c.lvl[h] + tm.id; n < e; n += TEAM::kSize) {
         const int2 cc = c.code[n];
         const float tl = c.t[cc.x], th = ln + c.t[cc.y];
         if (REC) {
@@ -558,14 +626,14 @@ __global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
           c.t[n] = fminf(tl, th);
         }
       }
-      __syncwarp();
+      tm.sync();
     }
   } else {
     // kEnergy / kSeed: SP(., T) under lambda
-    long_cost_to_top<false>(c, a.lam, nullptr, lane);
+    long_cost_to_top<false>(c, a.lam, nullptr, tm);
   }
 
-  if (KIND == kSeed && lane == 0) {
+  if (KIND == kSeed && tm.id == 0) {
     // walk the minimising path from the root: 0-arc on ties
     int n = 2;
     for (int h = 0; h < k; ++h) {
@@ -576,7 +644,49 @@ __global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
       n = take0 ? cc.x : cc.y;
     }
   }
-  if ((BWD || KIND == kEnergy) && a.E != nullptr && lane == 0) a.E[c.B.row] = c.t[2];  // E^j = SP(r, T)
+  if ((BWD || KIND == kEnergy) && a.E != nullptr && tm.id == 0) a.E[c.B.row] = c.t[2];  // E^j = SP(r, T)
+}
+
+template <int KIND, int MODE>
+__global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
+  // BDDs of at most 32 nodes a level that are no unit rows (their plain sweeps
+  // run in k_long_narrow)
+  WarpTeam tm{(int)threadIdx.x & 31};
+  const int b = A.num_long_unit + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= A.num_long_narrow) return;  // whole warp leaves
+  long_sweep<KIND, MODE>(A, a, long_ctx(A, A.long_order[b]), tm);
+}
+
+// The wide long BDDs, a block each.  Their path costs stay in shared memory
+// when they fit (smem): read from the arena's scratch when the sweep before
+// left them, written back at the end for the sweep after.
+template <int KIND, int MODE>
+__global__ void __launch_bounds__(BlockTeam::kSize) k_long_wide(DevArena A, SweepArgs a, int smem) {
+  constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
+  constexpr bool BWD = KIND == kBwd || KIND == kBwdRec;
+  extern __shared__ __align__(16) float costs[];
+  __shared__ float sh[4 * BlockTeam::kWarps];
+  BlockTeam tm{(int)threadIdx.x, sh};
+  LongCtx c = long_ctx(A, A.long_order[A.num_long_narrow + blockIdx.x]);
+  const int nn = c.B.nn + 2;
+  float *gd = c.d, *gt = c.t;
+  if (smem) {
+    c.d = costs;
+    c.t = costs + nn;
+    if ((FWD || BWD) && a.cost_in != nullptr) {
+      const float* src = FWD ? gt : gd;
+      float* dst = FWD ? c.t : c.d;
+      for (int n = tm.id; n < nn; n += BlockTeam::kSize) dst[n] = src[n];
+      __syncthreads();
+    }
+  }
+  long_sweep<KIND, MODE>(A, a, c, tm);
+  if (smem && (FWD || BWD)) {
+    __syncthreads();
+    const float* src = FWD ? c.d : c.t;
+    float* dst = FWD ? gd : gt;
+    for (int n = tm.id; n < nn; n += BlockTeam::kSize) dst[n] = src[n];
+  }
 }
 
 // Plain forward / backward sweep of the narrow long BDDs (the head of
@@ -682,23 +792,18 @@ __global__ void __launch_bounds__(128) k_long_smoothed(DevArena A, const float* 
 // gradients of SP(., T) and SP(r, .) per node in the backward workspace
 // (long_a1, long_a2) and every routing step a pull (each node gathers from
 // its two children or its in-arcs).
-template <int FWD, int MODE>
-__global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
-  const int lane = threadIdx.x & 31;
-  int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= A.num_long - A.num_long_unit) return;
-  b = A.long_order[A.num_long_unit + b];
-  const LongCtx c = long_ctx(A, b);
+template <int FWD, int MODE, class TEAM>
+__device__ __forceinline__ void long_adjoint(const DevArena& A, const AdjArgs& a, const LongCtx& c, TEAM& tm) {
   const int64_t sb = c.B.slot_base;
   const int k = c.B.k;
   const int32_t* meta = a.rec_lmeta + c.B.cost_base;
   float* A1 = a.long_a1 + c.B.cost_base;  // gradient of SP(., T)
   float* A2 = a.long_a2 + c.B.cost_base;  // gradient of SP(r, .)
-  for (int n = lane; n < c.B.nn + 2; n += kWarp) {
+  for (int n = tm.id; n < c.B.nn + 2; n += TEAM::kSize) {
     A1[n] = 0.0f;
     A2[n] = 0.0f;
   }
-  __syncwarp();
+  tm.sync();
 
   // the update of level h reversed (g = gradient of lambda^new_h with the
   // path-cost contributions of its level added); lane 0 writes
@@ -711,7 +816,7 @@ __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
     const float md = (a.seed_M ? a.seed_M[q] : 0.0f) + (a.sdot_next ? a.sdot_next[v] : 0.0f);
     const float Mt = md - g;
     const float dm1 = om * Mt, dm0 = -om * Mt;
-    if (lane == 0) {
+    if (tm.id == 0) {
       const int2 am = a.rec_lamin[q - A.long_slot_base];
       a.sdot[q] = al * g;
       if (a.g_alpha) a.g_alpha[q] = a.g_alpha[q] + g * S;
@@ -722,18 +827,18 @@ __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
       A2[am.y] += dm1;
       A1[c.code[am.y].y] += dm1;
     }
-    __syncwarp();
+    tm.sync();
   };
   // gradients of SP(., T) of level h leave along the argmin out-arcs: those
   // of the 1-arcs are returned (their sum), level h + 1 pulls them in
   auto route_out = [&](int h) -> float {
     float part = 0.0f;
     const int e = c.lvl[h + 1];
-    for (int n = c.lvl[h] + lane; n < e; n += kWarp)
+    for (int n = c.lvl[h] + tm.id; n < e; n += TEAM::kSize)
       if (meta[n] & kLHi) part += A1[n];
     if (h + 1 < k) {
       const int e2 = c.lvl[h + 2];
-      for (int w = c.lvl[h + 1] + lane; w < e2; w += kWarp) {
+      for (int w = c.lvl[h + 1] + tm.id; w < e2; w += TEAM::kSize) {
         float acc = A1[w];
         const int ie = c.inp[w + 1];
         for (int i = c.inp[w]; i < ie; ++i) {
@@ -743,7 +848,7 @@ __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
         A1[w] = acc;
       }
     }
-    return warp_sum(part);
+    return tm.sum(part);
   };
   // gradients of SP(r, .) of level h (>= 1) go to the argmin parents on level
   // h - 1 (pull over the parents' children, ascending); those entering by a
@@ -751,10 +856,10 @@ __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
   auto route_in = [&](int h) -> float {
     float part = 0.0f;
     const int e = c.lvl[h + 1];
-    for (int n = c.lvl[h] + lane; n < e; n += kWarp)
+    for (int n = c.lvl[h] + tm.id; n < e; n += TEAM::kSize)
       if (meta[n] & kLBeta) part += A2[n];
     const int ep = c.lvl[h];
-    for (int n = c.lvl[h - 1] + lane; n < ep; n += kWarp) {
+    for (int n = c.lvl[h - 1] + tm.id; n < ep; n += TEAM::kSize) {
       const int2 cc = c.code[n];
       float acc = A2[n];
       const bool tlo = cc.x >= 2 && (meta[cc.x] >> 1) == (n << 1);
@@ -768,7 +873,7 @@ __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
       }
       A2[n] = acc;
     }
-    return warp_sum(part);
+    return tm.sum(part);
   };
 
   if (FWD) {
@@ -776,29 +881,44 @@ __global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
       float g = a.g_lam[sb + h];
       // SP(r, .) of level h+1 was relaxed from level h with lambda^new_h
       if (h + 1 < k) g += route_in(h + 1);
-      __syncwarp();
+      tm.sync();
       reverse_level(h, g);
     }
     // SP(., T) under lambda^old: its gradient flows top-down
     for (int h = 0; h < k; ++h) {
       const float part = route_out(h);
-      if (lane == 0) a.g_lam[sb + h] += part;
-      __syncwarp();
+      if (tm.id == 0) a.g_lam[sb + h] += part;
+      tm.sync();
     }
   } else {
     for (int h = 0; h < k; ++h) {
       // SP(., T) of level h was recomputed with lambda^new_h
       const float g = a.g_lam[sb + h] + route_out(h);
-      __syncwarp();
+      tm.sync();
       reverse_level(h, g);
     }
     // SP(r, .) under lambda^old: its gradient flows bottom-up
     for (int h = k - 1; h >= 1; --h) {
       const float part = route_in(h);
-      if (lane == 0) a.g_lam[sb + h - 1] += part;
-      __syncwarp();
+      if (tm.id == 0) a.g_lam[sb + h - 1] += part;
+      tm.sync();
     }
   }
+}
+
+template <int FWD, int MODE>
+__global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
+  WarpTeam tm{(int)threadIdx.x & 31};
+  const int b = A.num_long_unit + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= A.num_long_narrow) return;
+  long_adjoint<FWD, MODE>(A, a, long_ctx(A, A.long_order[b]), tm);
+}
+
+template <int FWD, int MODE>
+__global__ void __launch_bounds__(BlockTeam::kSize) k_long_wide_adjoint(DevArena A, AdjArgs a) {
+  __shared__ float sh[4 * BlockTeam::kWarps];
+  BlockTeam tm{(int)threadIdx.x, sh};
+  long_adjoint<FWD, MODE>(A, a, long_ctx(A, A.long_order[A.num_long_narrow + blockIdx.x]), tm);
 }
 
 namespace {
@@ -806,14 +926,19 @@ namespace {
 constexpr int kLongWarps = 4;  // BDDs (warps) per CTA
 
 int long_grid(const DevArena& A) { return (A.num_long + kLongWarps - 1) / kLongWarps; }
-// ... without the unit ones (kernels_long_unit.cu)
-int long_grid_other(const DevArena& A) { return (A.num_long - A.num_long_unit + kLongWarps - 1) / kLongWarps; }
+// ... of the narrow ones that are no unit rows (kernels_long_unit.cu)
+int long_grid_narrow(const DevArena& A) { return (A.num_long_narrow - A.num_long_unit + kLongWarps - 1) / kLongWarps; }
+
+template <int KIND, int MODE>
+void launch_wide(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
+  const int g = A.num_long - A.num_long_narrow;
+  if (g > 0) k_long_wide<KIND, MODE><<<g, BlockTeam::kSize, A.long_wide_smem, st>>>(A, a, A.long_wide_smem);
+}
 
 template <int KIND>
 void launch_long_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  int grid = long_grid_other(A);
-  if constexpr (KIND == kFwd || KIND == kBwd) {
-    if (A.num_long_narrow > A.num_long_unit) {
+  if (A.num_long_narrow > A.num_long_unit) {
+    if constexpr (KIND == kFwd || KIND == kBwd) {
       const int per = kWarp / A.long_lanes;
       const int warps = (A.num_long_narrow - A.num_long_unit + per - 1) / per;
       const int ng = (warps + kLongWarps - 1) / kLongWarps;
@@ -821,34 +946,64 @@ void launch_long_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
         k_long_narrow<KIND, 1><<<ng, kLongWarps * kWarp, 0, st>>>(A, a);
       else
         k_long_narrow<KIND, 0><<<ng, kLongWarps * kWarp, 0, st>>>(A, a);
+    } else if (a.mode == 1) {
+      k_long_sweep<KIND, 1><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
+    } else {
+      k_long_sweep<KIND, 0><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
     }
-    grid = (A.num_long - A.num_long_narrow + kLongWarps - 1) / kLongWarps;
-    if (grid == 0) return;
   }
-  if (a.mode == 1)
-    k_long_sweep<KIND, 1><<<grid, kLongWarps * kWarp, 0, st>>>(A, a);
-  else
-    k_long_sweep<KIND, 0><<<grid, kLongWarps * kWarp, 0, st>>>(A, a);
+  a.mode == 1 ? launch_wide<KIND, 1>(A, a, st) : launch_wide<KIND, 0>(A, a, st);
+}
+
+// kMinMarg, kEnergy, kSeed: no omega, no alpha
+template <int KIND>
+void launch_long_plain(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
+  if (A.num_long_narrow > A.num_long_unit)
+    k_long_sweep<KIND, 0><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
+  launch_wide<KIND, 0>(A, a, st);
+}
+
+template <int FWD>
+void launch_adjoint_kind(const DevArena& A, const AdjArgs& a, cudaStream_t st) {
+  const int g = A.num_long_narrow - A.num_long_unit, gw = A.num_long - A.num_long_narrow;
+  if (g > 0)
+    a.mode == 1 ? k_long_adjoint<FWD, 1><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a)
+                : k_long_adjoint<FWD, 0><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
+  if (gw > 0)
+    a.mode == 1 ? k_long_wide_adjoint<FWD, 1><<<gw, BlockTeam::kSize, 0, st>>>(A, a)
+                : k_long_wide_adjoint<FWD, 0><<<gw, BlockTeam::kSize, 0, st>>>(A, a);
 }
 
 }  // namespace
 
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (A.num_long_items > 0) {
-    Chain ch;
-    ch.ss.main = st;
-    launch_long_unit(kind, A, a, ch);
-  }
   if (A.num_long == A.num_long_unit) return;
   switch (kind) {
     case kFwd: launch_long_kind<kFwd>(A, a, st); break;
     case kBwd: launch_long_kind<kBwd>(A, a, st); break;
     case kFwdRec: launch_long_kind<kFwdRec>(A, a, st); break;
     case kBwdRec: launch_long_kind<kBwdRec>(A, a, st); break;
-    case kMinMarg: k_long_sweep<kMinMarg, 0><<<long_grid_other(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
-    case kEnergy: k_long_sweep<kEnergy, 0><<<long_grid_other(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
-    default: k_long_sweep<kSeed, 0><<<long_grid_other(A), kLongWarps * kWarp, 0, st>>>(A, a); break;
+    case kMinMarg: launch_long_plain<kMinMarg>(A, a, st); break;
+    case kEnergy: launch_long_plain<kEnergy>(A, a, st); break;
+    default: launch_long_plain<kSeed>(A, a, st); break;
   }
+}
+
+cudaError_t set_long_smem_limit(size_t bytes) {
+  const int b = (int)bytes;
+  constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(k_long_wide<kFwd, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kFwd, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kBwd, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kBwd, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kFwdRec, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kFwdRec, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kBwdRec, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kBwdRec, 1>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kMinMarg, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kEnergy, 0>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_long_wide<kSeed, 0>, attr, b);
+  return e;
 }
 
 void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, cudaStream_t st) {
@@ -857,17 +1012,7 @@ void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float*
 }
 
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st) {
-  if (A.num_long_items > 0) {
-    Chain ch;
-    ch.ss.main = st;
-    launch_long_unit_adjoint(forward, A, a, ch);
-  }
-  if (A.num_long == A.num_long_unit) return;
-  const int g = long_grid_other(A), t = kLongWarps * kWarp;
-  if (forward)
-    a.mode == 1 ? k_long_adjoint<1, 1><<<g, t, 0, st>>>(A, a) : k_long_adjoint<1, 0><<<g, t, 0, st>>>(A, a);
-  else
-    a.mode == 1 ? k_long_adjoint<0, 1><<<g, t, 0, st>>>(A, a) : k_long_adjoint<0, 0><<<g, t, 0, st>>>(A, a);
+  forward ? launch_adjoint_kind<1>(A, a, st) : launch_adjoint_kind<0>(A, a, st);
 }
 
 }  // namespace dg

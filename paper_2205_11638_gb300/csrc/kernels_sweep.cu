@@ -421,12 +421,18 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
                           int num_groups, Chain& ch) {
   const bool chained = chained_sweeps(A, num_groups);
   const StreamSet& ss = ch.ss;
-  const bool fork = !chained && num_groups + (A.num_long > 0 ? 1 : 0) > 1 && ss.ready;
+  const bool fork = !chained && num_groups + long_launches(A) > 1 && ss.ready;
   if (fork) ss.begin();
   if (!chained) {
     // the long BDDs first: their launch is a few warps walking long chains
     ch.linked = false;
     launch_long_sweep(KIND, A, a, fork ? ss.of(A.long_stream) : ss.main);
+    if (A.num_long_items > 0) {
+      // side by side with the other long BDDs' walks
+      Chain own;
+      own.ss.main = fork ? ss.of(A.long_stream + (A.num_long > A.num_long_unit ? 1 : 0)) : ss.main;
+      launch_long_unit(KIND, A, a, own);
+    }
   } else if (A.num_long_items > 0) {
     launch_long_unit(KIND, A, a, ch);
   }
