@@ -33,8 +33,7 @@ constexpr unsigned kAll = 0xFFFFFFFFu;
 template <int G>
 struct LSeg {
   int base, s;
-  bool act;   // a BDD of the item
-  int row;    // ... its index (0 where there is none)
+  int row;  // its BDD, among the item's
 };
 
 template <int G>
@@ -156,7 +155,10 @@ __device__ __forceinline__ void copy_row(float* dst, const void* src, int k, int
 
 // The walk of a sweep with a level's states on the lanes of a segment: lam and
 // avg (the staged inputs) receive the new lambda and M (kMinMarg: m1 and m0,
-// kSeed: the minimising assignment in avg).
+// kSeed: the minimising assignment in avg).  Segments beyond the item's BDDs
+// repeat another one (same addresses, same values); steps are guarded only
+// past the shortest BDD's levels (kmin).  Reads one level ahead may go one
+// level past either end: the arrays have that much room.
 template <int KIND, int MODE, int G>
 __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs& a, const LongItem& it, float* lam,
                                               float* avg, const float* om, const float* al, float* cost, int lane) {
@@ -167,54 +169,73 @@ __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs
   LSeg<G> g;
   g.s = lane & (G - 1);
   g.base = lane - g.s;
-  g.act = lane / G < it.nseg;
-  g.row = g.act ? lane / G : 0;
+  g.row = (lane / G) % it.nseg;
   const LongBdd B = A.longs[A.long_order[it.first + g.row]];
-  const int k = B.k;
+  const int k = B.k, kmin = __reduce_min_sync(kAll, k);
   float* ml = lam + g.row * ST;
   float* ma = avg + g.row * ST;
   const float* mo = om + g.row * ST;
   const float* mw = al + g.row * ST;
-  float* mt = cost + g.row * G + g.s;  // level h at mt[h TS]
+  float* mt = cost + g.row * G + g.s;  // level h at mt[h TS], the terminals' at level k
   const float end = (it.accept >> g.s) & 1u ? 0.0f : f_inf();
   const float root = g.s == it.start ? 0.0f : f_inf();
-
+  auto down_levels = [&](auto&& step) {
+    runs_down(A, it, [&](auto ty, int b, int e) {
+      const int m = min(e, kmin);
+      int h = b;
+      for (; h < m; ++h) step(ty, h, true);
+      for (; h < e; ++h) step(ty, h, h < k);
+    });
+  };
+  auto up_levels = [&](auto&& step) {
+    runs_up(A, it, [&](auto ty, int b, int e) {
+      const int m = max(b, kmin);
+      int h = e - 1;
+      for (; h >= m; --h) step(ty, h, h < k);
+      for (; h >= b; --h) step(ty, h, true);
+    });
+  };
+  struct In {  // a level's inputs
+    float l, av, w, al;
+  };
+  auto input = [&](int h) {
+    return In{ml[h], ma[h], MODE == 1 ? mo[h] : a.omega0, MODE == 1 ? mw[h] : 0.0f};
+  };
   auto first_up = [&]() -> float {  // SP(., T) of every level; returns level 0's
     float t = end;
-    if (g.act) mt[k * TS] = end;
+    mt[k * TS] = end;
     float l = ml[it.kmax - 1];
-    runs_up(A, it, [&](auto ty, int b, int e) {
-      constexpr int TY = decltype(ty)::value;
-      for (int h = e - 1; h >= b; --h) {
-        const float ln = ml[max(h - 1, 0)];
-        float tz, to;
-        children<G, TY>(t, g, tz, to);
-        if (h < k) t = fminf(tz, l + to);
-        if (g.act && h < k) mt[h * TS] = t;
-        l = ln;
+    up_levels([&](auto ty, int h, bool on) {
+      const float l1 = ml[h - 1];
+      float tz, to;
+      children<G, decltype(ty)::value>(t, g, tz, to);
+      if (on) {
+        t = fminf(tz, l + to);
+        mt[h * TS] = t;
       }
+      l = l1;
     });
     return t;
   };
   // the update of a level from its minima, by every lane of the segment
-  auto update = [&](int h, float l, float av, float b0, float b1, float w, float alpha) -> float {
-    const float m0 = b0, m1 = l + b1;
-    const float Mn = __fmul_rn(MODE == 1 ? w : a.omega0, m1 - m0);
-    const float ln = unit_lambda_new<MODE>(l, Mn, alpha, av);
-    if (g.act && g.s == 0 && h < k) {
+  auto update = [&](int h, const In& x, bool on, float b0, float b1) -> float {
+    const float m0 = b0, m1 = x.l + b1;
+    const float Mn = __fmul_rn(x.w, m1 - m0);
+    const float ln = unit_lambda_new<MODE>(x.l, Mn, x.al, x.av);
+    if (g.s == 0 && on) {
       ml[h] = ln;
       ma[h] = Mn;
       if (REC) a.rec_diff[(int64_t)B.slot_base + h] = m1 - m0;
     }
     return ln;
   };
-  auto record = [&](int h, bool hi, int c, float x0, float m0, float x1, float m1) {
+  auto record = [&](int h, bool on, bool hi, int c, float x0, float m0, float x1, float m1) {
     const uint32_t tb = seg_bits<G>(hi, g.base), rb = seg_bits<G>((c & 1) != 0, g.base);
     const uint32_t ex = seg_bits<G>(c == 2, g.base) & 1u;
     // the argmins: the largest state on ties
     const uint32_t b0 = seg_bits<G>(x0 == m0, g.base), b1 = seg_bits<G>(x1 == m1, g.base);
     const int v0 = b0 ? 31 - __clz((int)b0) : 0, v1 = b1 ? 31 - __clz((int)b1) : 0;
-    if (g.act && g.s == 0 && h < k)
+    if (g.s == 0 && on)
       a.rec_lunit[(int64_t)B.slot_base + h - A.long_slot_base] =
           make_uint4(tb, rb, (uint32_t)v0 | (uint32_t)v1 << 8 | ex << 16, 0u);
   };
@@ -223,122 +244,106 @@ __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs
     first_up();
     __syncwarp();
     float R = root;
-    float l = ml[0], av = ma[0], w = MODE == 1 ? mo[0] : 0.0f, alpha = MODE == 1 ? mw[0] : 0.0f;
+    In in = input(0);
     runs_down(A, it, [&](auto ty, int b, int e) {
       constexpr int TY = decltype(ty)::value;
-      const int zi = lz<G, TY>(g.s) - g.s, oi = lo_<G, TY>(g.s) - g.s;
-      const bool ov = lo_<G, TY>(g.s) >= 0 && lo_<G, TY>(g.s) < G;
-      auto child = [&](int h, float& tz, float& to) {
-        const float* p = mt + min(h + 1, k) * TS;
-        tz = p[zi];
-        to = p[ov ? oi : 0];
-      };
-      float tz, to;
-      child(b, tz, to);
-      for (int h = b; h < e; ++h) {
-        const int hn = min(h + 1, it.kmax - 1);
-        float tzn, ton;
-        const float l1 = ml[hn], av1 = ma[hn], w1 = MODE == 1 ? mo[hn] : 0.0f, al1 = MODE == 1 ? mw[hn] : 0.0f;
-        child(hn, tzn, ton);
+      const int oi = lo_<G, TY>(g.s);
+      const bool ov = oi >= 0 && oi < G;
+      const float* pz = mt + lz<G, TY>(g.s) - g.s;
+      const float* po = mt + (ov ? oi : g.s) - g.s;
+      float tz = pz[(b + 1) * TS], to = po[(b + 1) * TS];
+      auto step = [&](int h, bool on) {
+        const In nxt = input(h + 1);
+        const float tz1 = pz[(h + 2) * TS], to1 = po[(h + 2) * TS];
         const float n = from_neighbour<G, TY>(R, g, f_inf());
         const float x0 = R + tz, x1 = ov ? R + to : f_inf();
         const float b0 = seg_min<G>(x0), b1 = seg_min<G>(x1);
         if (KIND == kMinMarg) {
-          if (g.act && g.s == 0 && h < k) {
-            ml[h] = l + b1;
+          if (g.s == 0 && on) {
+            ml[h] = in.l + b1;
             ma[h] = b0;
           }
-          R = down<G, TY>(R, n, l, g.s);
+          R = down<G, TY>(R, n, in.l, g.s);
         } else {
-          const float ln = update(h, l, av, b0, b1, w, alpha);
+          const float ln = update(h, in, on, b0, b1);
           if (REC) {
             int c;
-            const bool hi = !(tz <= (ov ? l + to : f_inf()));
+            const bool hi = !(tz <= (ov ? in.l + to : f_inf()));
             R = down_rec<G, TY>(R, n, ln, g.s, c);
-            record(h, hi, c, x0, b0, x1, b1);
+            record(h, on, hi, c, x0, b0, x1, b1);
           } else {
             R = down<G, TY>(R, n, ln, g.s);
           }
         }
-        l = l1;
-        av = av1;
-        w = w1;
-        alpha = al1;
-        tz = tzn;
-        to = ton;
-      }
+        in = nxt;
+        tz = tz1;
+        to = to1;
+      };
+      const int m = min(e, kmin);
+      int h = b;
+      for (; h < m; ++h) step(h, true);
+      for (; h < e; ++h) step(h, h < k);
     });
   } else if (BWD) {
-    float R = root;
     {
+      float R = root;
       float l = ml[0];
-      runs_down(A, it, [&](auto ty, int b, int e) {
+      down_levels([&](auto ty, int h, bool on) {
         constexpr int TY = decltype(ty)::value;
-        for (int h = b; h < e; ++h) {
-          const float ln = ml[min(h + 1, it.kmax - 1)];
-          if (g.act && h < k) mt[h * TS] = R;
-          R = down<G, TY>(R, from_neighbour<G, TY>(R, g, f_inf()), l, g.s);
-          l = ln;
-        }
+        const float l1 = ml[h + 1];
+        if (on) mt[h * TS] = R;
+        R = down<G, TY>(R, from_neighbour<G, TY>(R, g, f_inf()), l, g.s);
+        l = l1;
       });
     }
     __syncwarp();
     float t = end;
-    const int h0 = it.kmax - 1;
-    float l = ml[h0], av = ma[h0], w = MODE == 1 ? mo[h0] : 0.0f, alpha = MODE == 1 ? mw[h0] : 0.0f;
-    float r = mt[min(h0, k - 1) * TS];
-    runs_up(A, it, [&](auto ty, int b, int e) {
+    In in = input(it.kmax - 1);
+    float r = mt[(it.kmax - 1) * TS];
+    up_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
-      const int ni = TY == kUp ? -1 : 1;
-      const bool nv = g.s + ni >= 0 && g.s + ni < G;
-      for (int h = e - 1; h >= b; --h) {
-        const int hn = max(h - 1, 0);
-        const float l1 = ml[hn], av1 = ma[hn], w1 = MODE == 1 ? mo[hn] : 0.0f, al1 = MODE == 1 ? mw[hn] : 0.0f;
-        const float r1 = mt[min(hn, k - 1) * TS];
-        float tz, to;
-        children<G, TY>(t, g, tz, to);
-        const float x0 = r + tz, x1 = r + to;
-        const float b0 = seg_min<G>(x0), b1 = seg_min<G>(x1);
-        const float ln = update(h, l, av, b0, b1, w, alpha);
-        if (REC) {
-          int c;
-          const float n = nv ? mt[min(h, k - 1) * TS + ni] : f_inf();
-          down_rec<G, TY>(r, n, l, g.s, c);
-          const float th = ln + to;
-          const bool hi = !(tz <= th);
-          if (h < k) t = hi ? th : tz;
-          record(h, hi, c, x0, b0, x1, b1);
-        } else if (h < k) {
-          t = fminf(tz, ln + to);
-        }
-        l = l1;
-        av = av1;
-        w = w1;
-        alpha = al1;
-        r = r1;
+      const In nxt = input(h - 1);
+      const float r1 = mt[max(h - 1, 0) * TS];
+      float tz, to;
+      children<G, TY>(t, g, tz, to);
+      const float x0 = r + tz, x1 = r + to;
+      const float b0 = seg_min<G>(x0), b1 = seg_min<G>(x1);
+      const float ln = update(h, in, on, b0, b1);
+      const float th = ln + to;
+      if (REC) {
+        constexpr int ni = TY == kUp ? -1 : 1;
+        const bool nv = g.s + ni >= 0 && g.s + ni < G;
+        int c;
+        down_rec<G, TY>(r, nv ? mt[h * TS + ni] : f_inf(), in.l, g.s, c);
+        const bool hi = !(tz <= th);
+        record(h, on, hi, c, x0, b0, x1, b1);
+        if (on) t = hi ? th : tz;
+      } else if (on) {
+        t = fminf(tz, th);
       }
+      in = nxt;
+      r = r1;
     });
-    if (a.E != nullptr && g.act && g.s == it.start) a.E[B.row] = t;  // E^j = SP(r, T)
+    if (a.E != nullptr && g.s == it.start) a.E[B.row] = t;  // E^j = SP(r, T)
   } else {
     const float t = first_up();
     if (KIND == kEnergy) {
-      if (a.E != nullptr && g.act && g.s == it.start) a.E[B.row] = t;
+      if (a.E != nullptr && g.s == it.start) a.E[B.row] = t;
     } else {
       // kSeed: walk the minimising path from the root, the 0-arc on ties
       __syncwarp();
       int at = it.start;
       const float* row = cost + g.row * G;
-      runs_down(A, it, [&](auto ty, int b, int e) {
+      down_levels([&](auto ty, int h, bool on) {
         constexpr int TY = decltype(ty)::value;
-        for (int h = b; h < min(e, k); ++h) {
-          const int z = lz<G, TY>(at), o = lo_<G, TY>(at);
-          const float* p = row + (h + 1) * TS;
-          const float c0 = p[z], c1 = o >= 0 && o < G ? p[o] : f_inf();
-          // an infinite cost is the bottom terminal (the path stays feasible)
-          const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= ml[h] + c1);
-          if (g.act && g.s == 0) ma[h] = take0 ? 0.f : 1.f;
-          at = take0 ? z : max(min(o, G - 1), 0);
-        }
+        if (!on) return;
+        const int z = lz<G, TY>(at), o = lo_<G, TY>(at);
+        const float* p = row + (h + 1) * TS;
+        const float c0 = p[z], c1 = o >= 0 && o < G ? p[o] : f_inf();
+        // an infinite cost is the bottom terminal (the path stays feasible)
+        const bool take0 = c0 < f_inf() && (c1 == f_inf() || c0 <= ml[h] + c1);
+        if (g.s == 0) ma[h] = take0 ? 0.f : 1.f;
+        at = take0 ? z : max(min(o, G - 1), 0);
       });
     }
   }
@@ -642,11 +647,11 @@ __device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArg
   LSeg<G> g;
   g.s = lane & (G - 1);
   g.base = lane - g.s;
-  g.act = lane / G < it.nseg;
-  g.row = g.act ? lane / G : 0;
+  const bool act = lane / G < it.nseg;
+  g.row = act ? lane / G : 0;
   const LongBdd B = A.longs[A.long_order[it.first + g.row]];
   const int k = B.k;
-  const bool own = g.act && g.s == 0;
+  const bool own = act && g.s == 0;
   float* mg = gl + g.row * ST;
   float* md = df + g.row * ST;
   float* mw = al + g.row * ST;
