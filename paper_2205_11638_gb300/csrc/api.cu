@@ -102,6 +102,14 @@ dg_status enqueue_iterate(dg_arena* ar, Chain& ch, float* lam, float* M, const f
   a.omega0 = omega_of(opts);
   a.mode = mode;
   ar->avg_mode = mode;
+  if (iters > 0 && renorm <= 0) {
+    a.E = lb_out ? A.E : nullptr;
+    if (launch_small_iterate(A, a, ar->groups.data(), (int)ar->groups.size(), iters, ar->cta_smem_cap, ch)) {
+      if (lb_out) launch_lower_bound(A, lb_out, ch);
+      return check_launch("dg_iterate");
+    }
+    a.E = nullptr;
+  }
   // only the last reduction stores what later calls may read
   const int need = mode == 1 ? kNeedS : kNeedSbar;
   launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, iters > 0 ? need : kNeedS | kNeedSbar);

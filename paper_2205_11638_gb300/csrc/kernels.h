@@ -130,6 +130,18 @@ cudaError_t set_unit_smem_limit(size_t bytes);
 struct AdjArgs;
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
                  Chain& ch, bool late);
+// `iters` iterations of Alg. 1 on a small arena of unit tiles in one launch
+// (energies of the last backward sweep into a.E when not NULL); false, and
+// nothing launched, when the arena is not of that kind.
+//
+// The line: kSmallWork, the groups' estimated work (levels times a level's
+// cost, 14 W + 40).  One block's iteration costs about 2 us plus 0.6 us per
+// 1,000 of it, the chain of launches 8 us (us per iteration, one block / chain:
+// set cover 24 x 16, work 2,000 3.6 / 8.3; independent set of 400 nodes, 6,800
+// 6.1 / 8.4; tracking 3 x 40 per slot, about 20,000 12.3 / 11.2).
+constexpr int64_t kSmallWork = 10000;
+bool launch_small_iterate(const DevArena& A, const SweepArgs& a, const LaunchGroup* groups, int num_groups, int iters,
+                          size_t smem_cap, Chain& ch);
 void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, const LaunchGroup& G,
                           int wpc, size_t region, cudaStream_t st);
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,

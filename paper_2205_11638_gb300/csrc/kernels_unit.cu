@@ -13,6 +13,8 @@
 // events, the S reductions included): tracking 500 x 2,000, 50 iterations
 // 33.0 -> 22.2 ms; tracking 50 x 400 with per-slot parameters, 100 iterations
 // 10.5 -> 3.4 ms; 64 instances batched, 50 iterations 15.0 -> 11.1 ms.
+#include <algorithm>
+
 #include "kernels.h"
 #include "unit.cuh"
 
@@ -610,6 +612,105 @@ cudaError_t set_adjoint_attr(int b) {
   return e;
 }
 
+// ---- whole iterations of a small arena in one launch -----------------------
+// An arena of a few unit tiles is latency alone: a sweep and a reduction are
+// two launches of about 2 us each whatever they do.  One block instead keeps
+// lambda, M and the per-variable sums in shared memory for the whole call; a
+// block barrier stands between a sweep (a tile per warp at a time) and a
+// reduction (a variable per thread), and the arrays go back at the end.  The
+// operations and their order are the separate kernels'.
+template <int MODE>
+__global__ void __launch_bounds__(1024) k_small_iterate(DevArena A, SweepArgs a, int iters, int region_bytes) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int ns = (int)A.num_slots;
+  float* lam = reinterpret_cast<float*>(smem);
+  float* M = lam + ns;
+  float* S = M + ns;
+  float* row = reinterpret_cast<float*>(smem + ((size_t)(2 * ns + A.n) * 4 + 127) / 128 * 128 +
+                                        (size_t)warp * region_bytes);
+  constexpr int STRIDE = kStride<true, MODE>;
+  grid_wait();
+  grid_trigger();
+  for (int q = threadIdx.x; q < ns; q += blockDim.x) {
+    lam[q] = a.lam[q];
+    M[q] = a.M[q];
+  }
+  __syncthreads();
+  auto sum = [&](int i) {
+    int q[kEll], b = 0, e = 0;
+#pragma unroll
+    for (int r = 0; r < kEll; ++r) q[r] = __ldg(A.var_ell + (int64_t)r * A.n + i);
+    if (q[kEll - 1] <= -2) {
+      q[kEll - 1] = -2 - q[kEll - 1];
+      b = __ldg(A.var_ptr + i) + kEll;
+      e = __ldg(A.var_ptr + i + 1);
+    }
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < kEll; ++r)
+      if (q[r] >= 0) s += M[q[r]];
+    for (int k = b; k < e; ++k) s += M[__ldg(A.var_slots + k)];
+    return s;
+  };
+  auto reduce = [&]() {
+    for (int i = threadIdx.x; i < A.n; i += blockDim.x) {
+      const float s = sum(i);
+      S[i] = MODE == 1 ? s : __ldg(A.invdeg + i) * s;
+    }
+    __syncthreads();
+  };
+  SweepArgs w = a;
+  w.lam = lam;
+  w.M = M;
+  auto sweep = [&](auto kind, float* E) {
+    constexpr int KIND = decltype(kind)::value;
+    w.E = E;
+    for (int tile = warp; tile < A.num_tiles; tile += warps) {
+      const Tile T = A.tiles[tile];
+      const UnitShape sh = A.unit_shapes[T.unit - 1];
+      const int64_t sb = T.slot_base + lane;
+      float* x = row + lane;
+      for (int h = 0; h < T.nhops; ++h) {
+        const int64_t q = sb + h * kWarp;
+        const int v = __ldg(A.slot_var + q);
+        x[0] = lam[q];
+        x[kAvg] = v >= 0 ? S[v] : 0.0f;
+        if (MODE == 1) {
+          x[kOm] = a.omega[q];
+          x[kAl] = a.alpha[q];
+        }
+        x += STRIDE;
+      }
+      if (sh.W == 2)
+        unit_tile<KIND, MODE, 2>(A, w, T, sh, row, lane);
+      else if (sh.W == 4)
+        unit_tile<KIND, MODE, 4>(A, w, T, sh, row, lane);
+      else if (sh.W == 6)
+        unit_tile<KIND, MODE, 6>(A, w, T, sh, row, lane);
+      else
+        unit_tile<KIND, MODE, 8>(A, w, T, sh, row, lane);
+    }
+    __syncthreads();
+  };
+  reduce();
+  for (int it = 0; it < iters; ++it) {
+    sweep(TypeC<kFwd>{}, nullptr);
+    reduce();
+    sweep(TypeC<kBwd>{}, it + 1 == iters ? a.E : nullptr);
+    reduce();
+  }
+  for (int q = threadIdx.x; q < ns; q += blockDim.x) {
+    a.lam[q] = lam[q];
+    a.M[q] = M[q];
+  }
+  for (int i = threadIdx.x; i < A.n; i += blockDim.x) {
+    const float s = sum(i);
+    A.S[i] = s;
+    A.Sbar[i] = __ldg(A.invdeg + i) * s;
+  }
+}
+
 template <int KIND, int MODE>
 void launch_group(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, Chain& ch,
                   bool late) {
@@ -642,6 +743,10 @@ cudaError_t set_unit_smem_limit(size_t bytes) {
   if (e == cudaSuccess) e = set_adjoint_attr<1, 1>(b);
   if (e == cudaSuccess) e = set_adjoint_attr<0, 0>(b);
   if (e == cudaSuccess) e = set_adjoint_attr<0, 1>(b);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_small_iterate<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_small_iterate<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit_smoothed<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit_smoothed<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit_smoothed<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
@@ -667,6 +772,30 @@ void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGr
     case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, ch, late); break;
     default: launch_group<kSeed, 0>(A, a, G, wpc, region, ch, late); break;
   }
+}
+
+bool launch_small_iterate(const DevArena& A, const SweepArgs& a, const LaunchGroup* groups, int num_groups, int iters,
+                          size_t smem_cap, Chain& ch) {
+  if (A.unit_slots != A.num_slots || A.num_long > 0 || A.num_tiles < 1) return false;
+  size_t region = 0;
+  int64_t work = 0;
+  for (int g = 0; g < num_groups; ++g) {
+    region = std::max(region, (size_t)(a.mode == 1 ? groups[g].unit_bytes1 : groups[g].unit_bytes0));
+    work += groups[g].work;
+  }
+  if (work > kSmallWork) return false;
+  const size_t fixed = ((size_t)(2 * A.num_slots + A.n) * 4 + 127) / 128 * 128;
+  if (fixed + region > smem_cap) return false;
+  const int warps = (int)std::min<size_t>(std::min(32, A.num_tiles), (smem_cap - fixed) / region);
+  if (warps < std::min(8, A.num_tiles)) return false;
+  // threads beyond the tiles' warps help the reduction
+  const int threads = std::max(warps, std::min<int>(32, (A.n + 31) / 32)) * kWarp;
+  const int blocks_warps = threads / kWarp;
+  const size_t bytes = fixed + region * (size_t)blocks_warps;
+  const int use = bytes <= smem_cap ? blocks_warps : warps;
+  chain_launch(ch, a.mode == 1 ? k_small_iterate<1> : k_small_iterate<0>, 1, use * kWarp, fixed + region * use, A, a,
+               iters, (int)region);
+  return true;
 }
 
 void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, const LaunchGroup& G,
