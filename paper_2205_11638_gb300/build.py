@@ -23,7 +23,7 @@ CXX_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-pthread", f"-I{os.path.join(CUDA_HO
 
 SOURCES = ["builder.cpp", "api.cu", "kernels_sweep.cu", "kernels_unit.cu", "kernels_misc.cu", "kernels_adjoint.cu", "kernels_long.cu", "kernels_long_unit.cu",
            "kernels_params.cu", "noalloc.cu"]
-HEADERS = ["dg_internal.h", "kernels.h", "sweep.cuh", "unit.cuh"]
+HEADERS = ["dg_internal.h", "kernels.h", "sweep.cuh", "unit.cuh", "varsum.cuh"]
 
 
 def _stale(obj, deps):

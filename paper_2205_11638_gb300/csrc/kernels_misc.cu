@@ -3,7 +3,7 @@
 // re-projection onto the dual constraint of (D), the initial split of c and
 // the FP64 lower bound (Def. 2 with the unary term of the deferred
 // min-marginals).
-#include "kernels.h"
+#include "varsum.cuh"
 
 namespace dg {
 
@@ -43,15 +43,6 @@ __device__ __forceinline__ float sum_slots_warp(const DevArena& A, const float* 
     for (int j = 0; j < cnt; ++j) s += __shfl_sync(0xffffffffu, v, j);
   }
   return s;
-}
-
-// The first kEll slots of variable i; returns whether there are more.
-__device__ __forceinline__ bool ell_slots(const DevArena& A, int i, int (&q)[kEll]) {
-#pragma unroll
-  for (int r = 0; r < kEll; ++r) q[r] = __ldg(A.var_ell + (int64_t)r * A.n + i);
-  const bool more = q[kEll - 1] <= -2;
-  if (more) q[kEll - 1] = -2 - q[kEll - 1];
-  return more;
 }
 
 // S_i = sum_{j in J_i} M_ij over the variable's slots in fixed order.  Blocks
@@ -308,11 +299,6 @@ __global__ void k_gather_var(DevArena A, const float* __restrict__ v, float* out
   out[q] = var >= 0 ? v[var] : 0.f;
 }
 
-// Threads per block of the per-variable kernels, blocks over all variables and
-// over the wide ones (a warp each).
-constexpr int kVarThreads = 256;
-static int var_blocks(const DevArena& A) { return (A.n + kVarThreads - 1) / kVarThreads; }
-static int wide_blocks(const DevArena& A) { return (A.num_wide + kVarThreads / 32 - 1) / (kVarThreads / 32); }
 // The slots whose averaging term the sweeps read per slot: the mixed tiles',
 // and the long BDDs' unless all of them are unit rows.
 static int scatter_to(const DevArena& A) {

@@ -112,3 +112,34 @@ def test_smoothed_dual_vs_oracle(a):
     oE, omg = O.smoothed(lam, a)
     np.testing.assert_allclose(_np(E), oE, rtol=1e-5, atol=1e-5 * a)
     np.testing.assert_allclose(_np(A.to_csr(mg)), omg, atol=1e-4)
+
+
+@pytest.mark.parametrize("long_row", [0, 700])
+def test_transforms_at_every_list_length(long_row):
+    """Variables in 0, 1, 3, 4, 5, 31, 32, 33, 64 and 65 rows (the first four
+    slots come from columns, more than 32 are a warp's), with and without a row
+    of the long layout.  A softmax over d
+    slots and a mean are d + 2 operations of O(1) values: below 70 * 2^-24 * 10
+    = 4e-5 from FP64."""
+    deg = [0, 1, 3, 4, 5, 31, 32, 33, 64, 65]
+    n = len(deg) + 65 + long_row
+    rows = [([i, len(deg) + j], [1, 1], 0, 1) for i, d in enumerate(deg) for j in range(d)]
+    if long_row:
+        rows.append((list(range(len(deg) + 65, n)), [1] * long_row, 0, 1))
+    prob = dict(n=n, row_ptr=np.cumsum([0] + [len(r[0]) for r in rows]).astype(np.int64),
+                col=np.concatenate([r[0] for r in rows]).astype(np.int32),
+                coef=np.concatenate([r[1] for r in rows]).astype(np.int32),
+                sense=np.array([r[2] for r in rows], np.int8), rhs=np.array([r[3] for r in rows], np.int64),
+                c=np.zeros(n))
+    O = oracle.Oracle(prob)
+    A = solver.plan(prob).bind()
+    rng = np.random.default_rng(5)
+    lam, th, ah, wh, ga, gw, gt = (_f32(rng.normal(size=O.num_slots)) for _ in range(7))
+    got = A.param_transform(A.from_csr(ah), A.from_csr(wh), A.from_csr(th))
+    want = O.param_transform(ah, wh, th)
+    back = A.param_transform_backward(got[0], got[1], A.from_csr(ga), A.from_csr(gw), A.from_csr(gt))
+    want += O.param_transform_backward(want[0], want[1], ga, gw, gt)
+    lam_g = A.from_csr(lam)
+    A.nonparam_update(lam_g, A.from_csr(th))
+    for g, w in zip((*got, *back, lam_g), (*want, O.nonparam_update(lam, th))):
+        np.testing.assert_allclose(_np(A.to_csr(g)), w, atol=4e-5)
