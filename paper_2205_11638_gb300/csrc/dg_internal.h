@@ -94,8 +94,12 @@ inline size_t unit_smem_bytes(const UnitShape& s, int mode) {
 
 // ... and in the adjoint kernel: per level the staged inputs of kernels_unit.cu
 // (the gradient of lambda, the argmin word, m1 - m0, the weight, a pair per
-// variable and, in mode 1, omega).
-inline size_t unit_adjoint_bytes(int k) { return (size_t)kWarp * 4 * 7 * (size_t)k; }
+// variable and, in mode 1, omega), and the running gradients of alpha and omega
+// of the next kAdjAhead levels.
+constexpr int kAdjAhead = 8;
+inline size_t unit_adjoint_bytes(int k) {
+  return (size_t)kWarp * 4 * (7 * (size_t)k + 2 * (size_t)(k < kAdjAhead ? k : kAdjAhead));
+}
 
 inline int ring_size(int maxw) {
   int r = 2;

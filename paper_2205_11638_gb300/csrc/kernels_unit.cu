@@ -446,18 +446,26 @@ __device__ __forceinline__ void unit_adjoint_tile(const AdjArgs& a, const Tile& 
   int64_t q = T.slot_base + lane + (FWD ? (s.k - 1) * kWarp : 0);
   // the update of a level reversed (g: gradient of lambda^new with the path
   // costs' share); returns the gradient d of m1 (that of m0 is -d).  The
-  // running parameter gradients are read one level ahead.
+  // running parameter gradients come through a ring of kAdjAhead levels, every
+  // lane its own words (one level ahead in a register, each level cost the
+  // latency of DRAM).
   const bool want_a = a.g_alpha != nullptr, want_w = a.g_omega != nullptr;
-  float ga = want_a && real ? a.g_alpha[q] : 0.0f, gw = want_w && real ? a.g_omega[q] : 0.0f;
-  int left = s.k;
+  float* ring = smem + s.k * STRIDE + lane;
+  int p = 0;
   auto reverse = [&](float* y, float g) -> float {
     const int64_t at = q;
-    const float ca = ga, cw = gw;
     q += FWD ? -kWarp : kWarp;
-    if (--left > 0) {
-      if (want_a && real) ga = a.g_alpha[q];
-      if (want_w && real) gw = a.g_omega[q];
+    cp_async_wait_but<kAdjAhead - 1>();
+    float* r = ring + (p & (kAdjAhead - 1)) * 2 * kWarp;
+    const float ca = r[0], cw = r[kWarp];
+    __syncwarp();
+    if (p + kAdjAhead < s.k) {
+      const int64_t next = at + (FWD ? -kAdjAhead : kAdjAhead) * kWarp;
+      if (want_a) cp_async4(r, a.g_alpha + next);
+      if (want_w) cp_async4(r + kWarp, a.g_omega + next);
     }
+    cp_async_commit();
+    ++p;
     const float2 in = *reinterpret_cast<const float2*>(y - lane + kJIn + 2 * lane);
     const float seed = a.seed_M && real ? a.seed_M[at] : 0.0f;
     const float Mt = seed + in.x - g;
@@ -568,6 +576,12 @@ __global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int
   copy_rows<STRIDE>(m + kJDiff, a.rec_diff + T.slot_base, k, lane, pol);
   copy_rows<STRIDE>(m + kJAl, (MODE == 1 ? a.alpha : A.slot_invdeg) + T.slot_base, k, lane, pol);
   if (MODE == 1) copy_rows<STRIDE>(m + kJOm, a.omega + T.slot_base, k, lane, pol);
+  for (int j = 0; j < min(k, kAdjAhead); ++j) {  // the first levels of the ring
+    const int64_t q = T.slot_base + lane + (FWD ? k - 1 - j : j) * kWarp;
+    float* r = m + k * STRIDE + lane + j * 2 * kWarp;
+    if (a.g_alpha) cp_async4(r, a.g_alpha + q);
+    if (a.g_omega) cp_async4(r + kWarp, a.g_omega + q);
+  }
   cp_async_commit();
   cp_async_wait_one();
   __syncwarp();
