@@ -73,6 +73,7 @@ static_assert(sizeof(Tile) == 32, "Tile is 32 bytes");
 // read "largest u first".
 enum UnitType : int { kUp = 0, kDown = 1, kSwap = 2, kDrop = 3 };
 constexpr int kUnitMaxW = 8;
+constexpr int kShortK = 3;  // "short" shapes: two states and at most this many levels
 struct UnitShape {
   int32_t W;         // states per level: 2, 4, 6 or 8 (the window rounded up)
   int32_t k;         // levels
@@ -81,9 +82,11 @@ struct UnitShape {
   int32_t run_base;  // first entry of unit_runs
   int32_t nruns;     // runs of levels of one type: end level << 2 | type
   int32_t rows;      // levels whose path costs a sweep keeps: every second one of a run
-  int32_t pad;
+  int32_t types;     // short shapes: the levels' types, two bits each
 };
 static_assert(sizeof(UnitShape) == 32, "UnitShape is 32 bytes");
+
+inline bool unit_short(const UnitShape& s) { return s.W == 2 && s.k <= kShortK; }
 
 // Shared memory of one unit tile (one warp's slice) in the sweeps: the path
 // costs of `rows` levels and per level lambda, the averaging term and (mode 1)
@@ -243,6 +246,7 @@ struct LaunchGroup {
   int8_t pad[2];
   int32_t meta_bytes;     // argmin records of the recording sweeps: 64 (nmax - 2), largest tile
   int32_t unit_w;         // unit tiles: the largest W of the group (0: a group of mixed tiles)
+  int32_t unit_short;     // ... all of short shapes, by the kernels for these
   int32_t unit_bytes0;    // unit tiles: shared memory per warp, mode 0
   int32_t unit_bytes1;    // ... mode 1
 };

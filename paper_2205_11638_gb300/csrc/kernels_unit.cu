@@ -9,10 +9,12 @@
 // the sweep are recomputed by a first pass (two operations per state), which
 // is cheaper than moving 8 bytes per state through HBM.
 //
-// Measured against the node-by-node kernel of the mixed tiles (GB300, CUDA
-// events, the S reductions included): tracking 500 x 2,000, 50 iterations
-// 33.0 -> 22.2 ms; tracking 50 x 400 with per-slot parameters, 100 iterations
-// 10.5 -> 3.4 ms; 64 instances batched, 50 iterations 15.0 -> 11.1 ms.
+// Before these kernels, with the node-by-node kernel of the mixed tiles, and
+// now (GB300, wall clock, the S reductions included): tracking 500 x 2,000, 50
+// iterations 32.9 -> 18.1 ms; tracking 50 x 400 with per-slot parameters, 100
+// iterations 10.6 -> 1.8 ms; 64 instances batched, 50 iterations 14.7 -> 8.4 ms.
+// The tiles of six and eight states are 31 % of the issue slots busy, the gather
+// of the averaging terms bounds them.
 #include <algorithm>
 
 #include "kernels.h"
@@ -172,6 +174,158 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
       at = take0 ? z : o;
     });
   }
+}
+
+// ---- short tiles of two states ---------------------------------------------
+// Rows of up to kShortK variables with two states a level (pairs of an
+// independent set, linearised products, at-most-one and covering rows of a few
+// variables) are most tiles of most instances, and a level of theirs is some
+// fifteen operations: the staging, loops and run bookkeeping of k_unit were
+// four times that.  Here a tile's levels are unrolled, everything is registers,
+// and all loads are issued before the first operation, past L1, which is left
+// to the gathers (batch of 64: 175 -> 172 us an iteration).  Bound by the latency
+// of the ids, then the gathers.  Batch of 64 mixed instances: 189 -> 168 us an
+// iteration.  Rows of four variables as well made tracking slower (500 frames,
+// 361 -> 386 us), hence kShortK = 3.
+template <int TYPE>
+struct OneType {  // all levels of one type
+  template <class F>
+  static __device__ __forceinline__ void at(int, int, F&& f) {
+    f(TypeC<TYPE>{});
+  }
+};
+struct AnyType {  // two bits per level
+  template <class F>
+  static __device__ __forceinline__ void at(int types, int h, F&& f) {
+    switch (types >> (2 * h) & 3) {
+      case kUp: f(TypeC<kUp>{}); break;
+      case kDown: f(TypeC<kDown>{}); break;
+      case kSwap: f(TypeC<kSwap>{}); break;
+      default: f(TypeC<kDrop>{}); break;
+    }
+  }
+};
+
+template <int KIND, int MODE, int K, class TY>
+__device__ __forceinline__ void short_tile(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
+                                           const float (&l)[kShortK], const float (&av)[kShortK],
+                                           const float (&om)[kShortK], const float (&al)[kShortK], int lane) {
+  constexpr bool REC = KIND == kFwdRec || KIND == kBwdRec;
+  constexpr bool FWD = KIND == kFwd || KIND == kFwdRec;
+  const int64_t sb = T.slot_base + lane;
+  const bool real = lane < T.nbdd;
+  const int ty = S.types;
+  Costs<2> C[K + 1];  // the first pass' costs: SP(., T) or SP(r, .) of levels 0 .. K
+  auto update = [&](int h, float b0, float b1) -> float {
+    const float m0 = b0, m1 = l[h] + b1;
+    const float Mn = __fmul_rn(MODE == 1 ? om[h] : a.omega0, m1 - m0);
+    const float ln = unit_lambda_new<MODE>(l[h], Mn, al[h], av[h]);
+    if (real) {
+      a.lam[sb + h * kWarp] = ln;
+      a.M[sb + h * kWarp] = Mn;
+      if (REC) a.rec_diff[sb + h * kWarp] = m1 - m0;
+    }
+    return ln;
+  };
+  if (FWD) {
+    C[K] = unit_end<2>(S.accept);
+#pragma unroll
+    for (int h = K - 1; h > 0; --h)
+      TY::at(ty, h, [&](auto t) { C[h] = unit_up<2, decltype(t)::value>(C[h + 1], l[h]); });
+    Costs<2> R = unit_root<2>(S.start);
+#pragma unroll
+    for (int h = 0; h < K; ++h)
+      TY::at(ty, h, [&](auto t) {
+        constexpr int TP = decltype(t)::value;
+        float b0, b1;
+        if (REC) {
+          uint32_t rec = 0;
+          unit_minima_rec<2, TP>(R, C[h + 1], b0, b1, rec);
+          unit_up_rec<2, TP>(C[h + 1], l[h], rec);
+          R = unit_down_rec<2, TP>(R, update(h, b0, b1), rec);
+          if (real) a.rec_unit[sb + h * kWarp] = rec;
+        } else {
+          unit_minima<2, TP>(R, C[h + 1], b0, b1);
+          R = unit_down<2, TP>(R, update(h, b0, b1));
+        }
+      });
+  } else {
+    C[0] = unit_root<2>(S.start);
+#pragma unroll
+    for (int h = 0; h < K - 1; ++h)
+      TY::at(ty, h, [&](auto t) { C[h + 1] = unit_down<2, decltype(t)::value>(C[h], l[h]); });
+    Costs<2> t2 = unit_end<2>(S.accept);
+#pragma unroll
+    for (int h = K - 1; h >= 0; --h)
+      TY::at(ty, h, [&](auto t) {
+        constexpr int TP = decltype(t)::value;
+        float b0, b1;
+        if (REC) {
+          uint32_t rec = 0;
+          unit_minima_rec<2, TP>(C[h], t2, b0, b1, rec);
+          unit_down_rec<2, TP>(C[h], l[h], rec);
+          t2 = unit_up_rec<2, TP>(t2, update(h, b0, b1), rec);
+          if (real) a.rec_unit[sb + h * kWarp] = rec;
+        } else {
+          unit_minima<2, TP>(C[h], t2, b0, b1);
+          t2 = unit_up<2, TP>(t2, update(h, b0, b1));
+        }
+      });
+    if (a.E != nullptr && real) a.E[__ldg(A.slot_row + sb)] = S.start ? t2.v[1] : t2.v[0];
+  }
+}
+
+template <int KIND, int MODE, int K>
+__device__ __forceinline__ void short_types(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
+                                            const float (&l)[kShortK], const float (&av)[kShortK],
+                                            const float (&om)[kShortK], const float (&al)[kShortK], int lane) {
+  if (S.nruns == 1 && (S.types & 3) == kUp)
+    short_tile<KIND, MODE, K, OneType<kUp>>(A, a, T, S, l, av, om, al, lane);
+  else if (S.nruns == 1 && (S.types & 3) == kDown)
+    short_tile<KIND, MODE, K, OneType<kDown>>(A, a, T, S, l, av, om, al, lane);
+  else
+    short_tile<KIND, MODE, K, AnyType>(A, a, T, S, l, av, om, al, lane);
+}
+
+// One short tile (see k_unit for `late`).
+template <int KIND, int MODE>
+__device__ __forceinline__ void short_body(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
+                                           int lane, int late) {
+  const int64_t sb = T.slot_base + lane;
+  const int k = T.nhops;
+  int v[kShortK];
+#pragma unroll
+  for (int h = 0; h < kShortK; ++h) v[h] = h < k ? __ldcs(A.slot_var + sb + h * kWarp) : -1;
+  if (!late) {
+    grid_wait();
+    grid_trigger();
+  }
+  float l[kShortK], av[kShortK], om[kShortK], al[kShortK];
+  const float* src = MODE == 1 ? A.S : A.Sbar;
+#pragma unroll
+  for (int h = 0; h < kShortK; ++h) {
+    const bool on = h < k;
+    l[h] = on ? __ldcg(a.lam + sb + h * kWarp) : 0.0f;
+    av[h] = v[h] >= 0 ? src[v[h]] : 0.0f;
+    om[h] = MODE == 1 && on ? __ldcg(a.omega + sb + h * kWarp) : 0.0f;
+    al[h] = MODE == 1 && on ? __ldcg(a.alpha + sb + h * kWarp) : 0.0f;
+  }
+  switch (k) {
+    case 1: short_types<KIND, MODE, 1>(A, a, T, S, l, av, om, al, lane); break;
+    case 2: short_types<KIND, MODE, 2>(A, a, T, S, l, av, om, al, lane); break;
+    default: short_types<KIND, MODE, 3>(A, a, T, S, l, av, om, al, lane); break;
+  }
+}
+
+template <int KIND, int MODE>
+__global__ void __launch_bounds__(128) k_unit_short(DevArena A, SweepArgs a, int tile0, int tile1, int late) {
+  const int lane = threadIdx.x & 31;
+  const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (tile >= tile1) return;
+  if (late) grid_trigger();
+  const Tile T = A.tiles[tile];
+  short_body<KIND, MODE>(A, a, T, A.unit_shapes[T.unit - 1], lane, late);
+  if (late) grid_wait();
 }
 
 template <int KIND, int MODE, int WMAX>
@@ -728,16 +882,24 @@ __global__ void __launch_bounds__(1024) k_small_iterate(DevArena A, SweepArgs a,
 template <int KIND, int MODE>
 void launch_group(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, Chain& ch,
                   bool late) {
-  const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc;
+  const int nt = G.tile1 - G.tile0;
+  if constexpr (KIND == kFwd || KIND == kBwd || KIND == kFwdRec || KIND == kBwdRec) {
+    if (G.unit_short) {
+      chain_launch(ch, k_unit_short<KIND, MODE>, (nt + 3) / 4, 128, 0, A, a, G.tile0, G.tile1, late ? 1 : 0);
+      return;
+    }
+  }
+  const int grid = (nt + wpc - 1) / wpc;
   auto k = G.unit_w <= 2 ? k_unit<KIND, MODE, 2> : (G.unit_w <= 4 ? k_unit<KIND, MODE, 4> : k_unit<KIND, MODE, 8>);
   chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1, late ? 1 : 0);
 }
 
 template <int KIND, int MODE>
 cudaError_t set_attr(int b) {
-  cudaError_t e = cudaFuncSetAttribute(k_unit<KIND, MODE, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit<KIND, MODE, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit<KIND, MODE, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+  constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(k_unit<KIND, MODE, 2>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit<KIND, MODE, 4>, attr, b);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_unit<KIND, MODE, 8>, attr, b);
   return e;
 }
 

@@ -71,7 +71,22 @@ def _long_unit_rows(seed, n=700):
     return workloads.single_rows_problem(rows, n, rng.normal(size=n))
 
 
+def _short_rows(seed, copies, more=(), n=400):
+    """Every unit row of up to three variables that leaves some choice, `copies`
+    rows each, and `more` rows of six."""
+    rng = np.random.default_rng(seed)
+    kinds = [(np.array(a), sense, b) for k in (1, 2, 3) for a in np.ndindex(*(2,) * k) for sense in range(3)
+             for b in range(-k, k + 1) if workloads._free_row((None, 2 * np.array(a) - 1, sense, b))]
+    rows = []
+    for a, sense, b in kinds:
+        var = rng.integers(0, n - len(a), size=copies)
+        rows += [(v + np.arange(len(a)), 2 * a - 1, sense, b) for v in var]
+    rows += [(np.sort(rng.choice(n, size=6, replace=False)), np.ones(6, np.int64), 0, b) for b in more]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
 CASES = {
+    "independent_set": lambda: workloads.independent_set(n=500, seed=45),  # short tiles only
     "long_rows": lambda: _long_unit_rows(6),
     "assignment": lambda: workloads.assignment(L=50, R=300, cand=260, seed=44),
     "random_signs": lambda: _random_unit_rows(5),
@@ -199,3 +214,24 @@ def test_smoothed_dual_against_float64(name, scale):
         assert torch.isfinite(E).all() and torch.isfinite(marg).all()
         assert (np.abs(E.double().cpu().numpy() - oE) <= a * tol).all()
         assert (np.abs(A.to_csr(marg).double().cpu().numpy() - om) <= np.repeat(tol, np.diff(rp))).all()
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_short_tiles_of_a_large_arena_equal_the_mixed_tiles(mode):
+    """More than 8192 unit tiles, most of them short (one lane of the last of a
+    shape): these are a launch of their own between the other unit tiles' and
+    the mixed tiles'.  Plain sweeps, and recording ones through the gradients
+    (tolerance as above: 64 roundings in each of 4 sweeps)."""
+    p = _short_rows(4, 69 * 32 + 1, more=[1, 2, 3] * 50)
+    out = []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q).bind()
+        lam, M, om, al = [X.from_csr(x) for x in _vectors(p, 12)]
+        par = (om, al) if mode else (None, None)
+        g = X.backward(lam, M, *par, 2, 1, *[X.from_csr(x) for x in _vectors(p, 13)[:2]])
+        lb = X.iterate(lam, M, *par, iters=2, lb=True)
+        out.append(([X.to_csr(lam), X.to_csr(M), lb], [X.to_csr(x) for x in g]))
+    for a, b in zip(out[0][0], out[1][0]):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+    for a, b in zip(out[0][1], out[1][1]):
+        assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
