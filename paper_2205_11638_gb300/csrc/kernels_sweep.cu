@@ -1,5 +1,6 @@
 // kernels_sweep.cu -- the sweeps of Alg. 1 (generalized min-marginal
-// averaging, Sec. 3.2 of DOGE-Train) over tiles of BDDs, plus the kernels
+// averaging, Sec. 3.2 of DOGE-Train) over the mixed tiles of BDDs (unit tiles:
+// kernels_unit.cu), the launches of a whole sweep, plus the kernels
 // that evaluate min-marginals, subproblem energies and minimising
 // assignments on the same layout.
 //
