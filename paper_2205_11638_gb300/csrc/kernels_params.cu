@@ -218,12 +218,27 @@ void launch_center(const DevArena& A, const float* x, float* out, cudaStream_t s
 }
 void launch_param_transform(const DevArena& A, const float* ah, const float* wh, const float* th, float* alpha,
                             float* omega, float* theta, cudaStream_t st) {
+  // one launch, unless an output takes the place of another's input: then one by one
+  if ((alpha && (alpha == wh || alpha == th)) || (omega && (omega == ah || omega == th)) ||
+      (theta && (theta == ah || theta == wh))) {
+    if (alpha) launch_param_transform(A, ah, nullptr, nullptr, alpha, nullptr, nullptr, st);
+    if (omega) launch_param_transform(A, nullptr, wh, nullptr, nullptr, omega, nullptr, st);
+    if (theta) launch_param_transform(A, nullptr, nullptr, th, nullptr, nullptr, theta, st);
+    return;
+  }
   const int v = alpha || theta ? var_blocks(A) + wide_blocks(A) : 0;
   const unsigned g = (unsigned)v + (omega ? slot_blocks(A) : 0u);
   if (g > 0) k_param_transform<<<g, kVarThreads, 0, st>>>(A, ah, wh, th, alpha, omega, theta, var_blocks(A), v);
 }
 void launch_param_transform_bwd(const DevArena& A, const float* alpha, const float* omega, const float* ga,
                                 const float* gw, const float* gt, float* gah, float* gwh, float* gth, cudaStream_t st) {
+  if ((gah && (gah == omega || gah == gw || gah == gt)) || (gwh && (gwh == alpha || gwh == ga || gwh == gt)) ||
+      (gth && (gth == alpha || gth == omega || gth == ga || gth == gw))) {  // as above
+    if (gah) launch_param_transform_bwd(A, alpha, nullptr, ga, nullptr, nullptr, gah, nullptr, nullptr, st);
+    if (gwh) launch_param_transform_bwd(A, nullptr, omega, nullptr, gw, nullptr, nullptr, gwh, nullptr, st);
+    if (gth) launch_param_transform_bwd(A, nullptr, nullptr, nullptr, nullptr, gt, nullptr, nullptr, gth, st);
+    return;
+  }
   const int v = gah || gth ? var_blocks(A) + wide_blocks(A) : 0;
   const unsigned g = (unsigned)v + (gwh ? slot_blocks(A) : 0u);
   if (g > 0)

@@ -143,3 +143,27 @@ def test_transforms_at_every_list_length(long_row):
     A.nonparam_update(lam_g, A.from_csr(th))
     for g, w in zip((*got, *back, lam_g), (*want, O.nonparam_update(lam, th))):
         np.testing.assert_allclose(_np(A.to_csr(g)), w, atol=4e-5)
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2])
+def test_transform_outputs_in_place_of_inputs(shift):
+    """From C an output may take the place of an input: its own, or that of one
+    transformed before it.  Compared with separate buffers, bit for bit."""
+    from paper_2205_11638_gb300 import _lib
+    prob = workloads.matching_quadratic(L=40, R=40, pairs=1500, seed=7)
+    A = solver.plan(prob).bind()
+    rng = np.random.default_rng(6)
+    x = [A.from_csr(rng.normal(size=len(prob["col"]))) for _ in range(5)]
+    want = A.param_transform(*x[:3])
+    back = A.param_transform_backward(*x)
+    st = torch.cuda.current_stream().cuda_stream
+    t = [v.clone() for v in x[:3]]
+    spare = [A.zeros() for _ in range(2)]
+    # own input; omega over alpha-hat; theta over omega-hat as well
+    out = [[t[0], t[1], t[2]], [spare[0], t[0], spare[1]], [spare[0], t[0], t[1]]][shift]
+    rc = _lib.load().dg_param_transform(A._h, st, *[v.data_ptr() for v in (*t, *out)])
+    assert rc == 0 and all(torch.equal(a, b) for a, b in zip(out, want))
+    t = [v.clone() for v in x]
+    out = [[t[2], t[3], t[4]], [spare[0], t[2], spare[1]], [spare[0], t[2], t[3]]][shift]
+    rc = _lib.load().dg_param_transform_backward(A._h, st, *[v.data_ptr() for v in (*t, *out)])
+    assert rc == 0 and all(torch.equal(a, b) for a, b in zip(out, back))
