@@ -660,13 +660,16 @@ __device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArg
   const uint4* mr = rec + g.row * ST;
   const float* seed = a.seed_M ? a.seed_M + B.slot_base : nullptr;
 
-  // the update of level h reversed; returns the gradient of m1
-  auto reverse = [&](int h, float x) -> float {
+  // the update of level h reversed (on: the BDD has that level, else nothing is
+  // written and the result is not used); returns the gradient of m1
+  auto reverse = [&](int h, bool on, float gs) -> float {
+    h = min(h, k - 1);
+    const float x = mg[h] + gs;
     const float2 v = mi[h];
     const float Mt = (seed ? seed[h] : 0.0f) + v.x - x;
     const float d = (MODE == 1 ? mo[h] : a.omega0) * Mt;
     __syncwarp();
-    if (own && h < k) {
+    if (own && on) {
       mi[h] = make_float2(Mt * md[h], x * v.y);  // omega-dot, alpha-dot
       mw[h] = mw[h] * x;                         // contribution to S-dot
       md[h] = d;
@@ -727,7 +730,7 @@ __device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArg
         const uint4 w = on ? mr[h] : none;
         float gs;
         const float y = route_in(ty, x, w, gs);
-        const float d = reverse(min(h, k - 1), mg[min(h, k - 1)] + gs);
+        const float d = reverse(h, on, gs);
         x = on ? seed_in(y, w, d) : 0.0f;
       }
     });
@@ -739,7 +742,7 @@ __device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArg
         const uint4 w = on ? mr[h] : none;
         float gs;
         const float y = route_out(ty, x, w, gs);
-        const float d = reverse(min(h, k - 1), mg[min(h, k - 1)] + gs);
+        const float d = reverse(h, on, gs);
         x = on ? seed_out(ty, y, w, d) : 0.0f;
       }
     });

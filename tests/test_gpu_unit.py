@@ -235,3 +235,35 @@ def test_short_tiles_of_a_large_arena_equal_the_mixed_tiles(mode):
         assert torch.equal(a, b) and torch.isfinite(a).all()
     for a, b in zip(out[0][1], out[1][1]):
         assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
+
+
+def _packed_long_rows(num, seed, n=600):
+    """Rows "sum of k = 12", k = 40 to 60: 13 states a level held by 16 lanes, one
+    kind whatever the length, two BDDs to a warp from 1,216 of them on."""
+    rng = np.random.default_rng(seed)
+    rows = [(np.sort(rng.choice(n, size=int(k), replace=False)), np.ones(int(k), np.int64), workloads.EQ, 12)
+            for k in rng.integers(40, 61, size=num)]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_packed_segments_of_unequal_lengths(mode):
+    """Two BDDs of different lengths to a warp, a segment of lanes each: sweeps
+    bit for bit, gradients up to the rounding of sums (at most 64 roundings in
+    each of 4 sweeps, as above)."""
+    p = _packed_long_rows(1300, 14)
+    v, g = _vectors(p, 15), _vectors(p, 16)[:2]
+    out = []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q).bind()
+        assert X.plan.sizes.num_long_bdds == 1300
+        lam, M, om, al = [X.from_csr(x) for x in v]
+        par = (om, al) if mode else (None, None)
+        res = X.backward(lam, M, *par, 2, 1, *[X.from_csr(x) for x in g])
+        lb = X.iterate(lam, M, *par, iters=2, lb=True)
+        out.append(([X.to_csr(x) for x in res], [X.to_csr(lam), X.to_csr(M), lb]))
+    for a, b in zip(out[0][1], out[1][1]):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+    for a, b in zip(out[0][0], out[1][0]):
+        assert torch.isfinite(a).all()
+        assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
