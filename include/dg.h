@@ -217,7 +217,8 @@ dg_status dg_iterate(dg_arena* arena, void* stream, float* lam, float* M, const 
  * arena (with renorm != 0 it also re-projects lam onto
  * sum_j (lambda_ij + M_ij) = c_i in FP64, weights as in mode) and gives every
  * slot (i,j) the averaging term of mode (S_i / |J_i| in mode 0, S_i in mode
- * 1, which the sweep weights by alpha_ij).  dg_sweep runs one sweep of
+ * 1, which the sweep weights by alpha_ij).  Calls that only evaluate (bounds,
+ * seed, marginals) leave the averaging terms alone.  dg_sweep runs one sweep of
  * Alg. 1 (forward != 0: blocks B_1..B_u, else B_u..B_1) with that snapshot,
  * in the mode of the arena's last dg_sum_M (or S reduction of another call
  * that sweeps: dg_iterate, the checkpointed calls, dg_autotune in mode 0),
@@ -262,7 +263,7 @@ dg_status dg_lower_bound(dg_arena* arena, void* stream, const float* lam, const 
  * that cannot hand the library any scratch memory, e.g. code inside a stream
  * capture that forbids allocation or an embedder with a fixed device-memory
  * budget.  The paper has no counterpart: this is a deployment variant.  Its
- * intermediates (E^j per row, S_i and S_i/|J_i| per variable, one partial sum
+ * intermediates (E^j per row, S_i per variable, one partial sum
  * per reduction chunk, SP(., T) per node of the long BDDs) live in a static
  * device array of 4 MiB inside libdg instead of the arena's scratch area; the
  * call allocates nothing (no cudaMalloc, no allocating library routine).

@@ -39,8 +39,8 @@ struct dg_arena_s {
   size_t smem_sweep = 0, smem_adjoint = 0;
   int device = 0;
   int max_tile_rows = 0, max_tile_slots = 0, max_tile_hops = 0;
-  // mode of the averaging terms the last S reduction for a sweep wrote into
-  // the per-slot array (-1: none yet, the array holds zeros)
+  // mode of the averaging terms (per variable and per slot) the last S
+  // reduction for a sweep wrote (-1: none yet, the arrays hold zeros)
   int avg_mode = -1;
   // path costs handed from one dg_sweep to the next (DG_SWEEP_COSTS_*): every
   // API call advances `epoch`; the sweep that wrote the costs records its
@@ -110,9 +110,8 @@ dg_status enqueue_iterate(dg_arena* ar, Chain& ch, float* lam, float* M, const f
     }
     a.E = nullptr;
   }
-  // only the last reduction stores what later calls may read
-  const int need = mode == 1 ? kNeedS : kNeedSbar;
-  launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, iters > 0 ? need : kNeedS | kNeedSbar);
+  // only the last reduction stores S, which later calls may read
+  launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, iters == 0);
   // every sweep hands its path costs to the next one (the S reductions
   // between them leave lambda alone), except into the first sweep, whose
   // lambda comes from the caller, and across a re-projection
@@ -123,14 +122,14 @@ dg_status enqueue_iterate(dg_arena* ar, Chain& ch, float* lam, float* M, const f
     a.cost_out = A.nodecost;
     a.cost_in = handed ? A.nodecost : nullptr;
     launch_sweep(kFwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), ch);
-    launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, need);
+    launch_reduce_S(A, M, lam, alpha, mode, false, ch, Scatter::kSweep, false);
     if (lb_out && it == iters - 1) a.E = A.E;
     handed = it + 1 < iters && !rn;
     a.cost_out = handed ? A.nodecost : nullptr;
     a.cost_in = A.nodecost;
     launch_sweep(kBwd, A, a, threads, ar->groups.data(), (int)ar->groups.size(), ch);
     launch_reduce_S(A, M, lam, alpha, mode, rn, ch, it + 1 < iters ? Scatter::kSweep : Scatter::kNone,
-                    it + 1 < iters ? need : kNeedS | kNeedSbar);
+                    it + 1 == iters);
   }
   if (lb_out) {
     if (iters == 0) {
@@ -403,7 +402,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.nodecost = (float*)(b + P.off.nodecost);
   A.slot_invdeg = (float*)(b + P.off.slot_invdeg);
   A.S = (float*)(b + P.off.S);
-  A.Sbar = (float*)(b + P.off.Sbar);
+  A.var_avg = (float*)(b + P.off.var_avg);
   A.slot_avg = (float*)(b + P.off.slot_avg);
   A.E = (float*)(b + P.off.E);
   A.lb_part = (double*)(b + P.off.lb_part);

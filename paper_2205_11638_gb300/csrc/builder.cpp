@@ -1014,7 +1014,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
   P.off.long_order = put(P.long_order.size() * 4);
   P.off.long_items = put(P.long_items.size() * sizeof(LongItem));
   P.off.S = put((size_t)n * 4);
-  P.off.Sbar = put((size_t)n * 4);
+  P.off.var_avg = put((size_t)n * 4);
   P.off.slot_avg = put((size_t)num_slots * 4);
   P.off.E = put((size_t)m * 4);
   P.off.lb_part = put((size_t)num_chunks * 8);

@@ -203,10 +203,13 @@ struct DevArena {
   // per slot: 1/|J_i| of its variable (0 for padding), filled when the arena
   // is bound; the adjoint's alpha in mode 0
   float* slot_invdeg;
-  float* S;                 // scratch: per-variable sum of M (snapshot)
-  float* Sbar;              // scratch: S_i / |J_i| (the mode-0 averaging term)
-  float* slot_avg;          // scratch per slot: the averaging term of its variable (Sbar_i in mode 0,
-                            // S_i in mode 1) as the last S reduction before a sweep left it; 0 for padding
+  float* S;                 // scratch: per-variable sum of M (the last S reduction's)
+  // scratch per variable and per slot: the averaging term of the variable
+  // (S_i / |J_i| in mode 0, S_i in mode 1) as the last S reduction before a
+  // sweep left it.  The unit rows gather var_avg, the others read slot_avg (0
+  // for padding); a reduction for a bound or a seed changes neither
+  float* var_avg;
+  float* slot_avg;
   float* E;                 // scratch: E^j per original row
   double* lb_part;          // scratch: one partial sum per lb chunk
   int32_t n;
@@ -306,7 +309,7 @@ struct Plan {
   struct Off {
     size_t tiles, unit_shapes, unit_runs, desc, lohi8, slot_var, slot_row, var_ptr, var_slots, var_ell, wide_vars, c, invdeg, inst_row_ptr,
         inst_var_ptr,
-        lb_chunks, inst_chunk_ptr, inst_unc, longs, long_code, long_lvl, long_in_ptr, long_in, long_order, long_items, S, Sbar, slot_avg, E, lb_part,
+        lb_chunks, inst_chunk_ptr, inst_unc, longs, long_code, long_lvl, long_in_ptr, long_in, long_order, long_items, S, var_avg, slot_avg, E, lb_part,
         long_d, long_t, nodecost, slot_invdeg, total;
   } off{};
   size_t smem_sweep = 0;   // dynamic smem of the sweep kernels

@@ -155,13 +155,15 @@ void launch_sweep(int kind, const DevArena& A, const SweepArgs& a, int threads, 
 
 // S_i = sum_{k in J_i} M_ik in fixed slot order; with renorm, also
 // lambda_ij += alpha_ij * (c_i - sum_k (lambda_ik + M_ik)) computed in FP64.
-// Before a sweep also the mode's averaging term into A.slot_avg for the slots
-// the sweep reads it from: those of the mixed tiles and the long BDDs before
-// a sweep (the unit tiles gather S or Sbar themselves).
+// Before a sweep (kSweep) also the mode's averaging term, into A.var_avg and,
+// for the mixed tiles and the long BDDs that are no unit rows, A.slot_avg: the
+// snapshot sweeps read, which a reduction for a bound or a seed (kNone) leaves
+// alone.  store_S: whether S itself is read afterwards (always stored by a
+// re-projection).
 enum class Scatter { kNone, kSweep };
-constexpr int kNeedS = 1, kNeedSbar = 2;  // which of S and Sbar the reduction stores
+constexpr int kNeedS = 1, kNeedAvg = 2;
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
-                     Chain& ch, Scatter to, int need = kNeedS | kNeedSbar);
+                     Chain& ch, Scatter to, bool store_S = true);
 void launch_init(const DevArena& A, float* lam, float* M, cudaStream_t st);
 // per-instance FP64 lower bound from A.E and A.S
 void launch_lower_bound(const DevArena& A, double* lb_out, Chain& ch);

@@ -586,7 +586,7 @@ __device__ __forceinline__ void long_unit_item(const DevArena& A, const SweepArg
   if (UPDATE) {
     cp_async_wait_one();
     __syncwarp();
-    const float* src = MODE == 1 ? A.S : A.Sbar;
+    const float* src = A.var_avg;
     for (int r = 0; r < it.nseg; ++r) {
       const int k = A.longs[A.long_order[it.first + r]].k;
 #pragma unroll 4

@@ -47,11 +47,11 @@ __device__ __forceinline__ float sum_slots_warp(const DevArena& A, const float* 
 
 // S_i = sum_{j in J_i} M_ij over the variable's slots in fixed order.  Blocks
 // below nblk take a variable per thread, the others a wide variable (more than
-// kWide slots) per warp.  `need`: which of S and Sbar to store.  With SCATTER
-// every slot in [from, to) of the variable also receives the averaging term a
-// sweep adds (Sbar_i = S_i / |J_i| in mode 0, S_i in mode 1, which it
-// multiplies by alpha_ij); the unit rows' sweeps gather S or Sbar instead,
-// which halves the reduction's random accesses.
+// kWide slots) per warp.  `need`: whether to store S (kNeedS) and, before a
+// sweep (kNeedAvg), the averaging term it adds (S_i / |J_i| in mode 0, S_i in
+// mode 1, which it multiplies by alpha_ij).  With SCATTER every slot in
+// [from, to) of the variable also receives that term; the unit rows' sweeps
+// gather it per variable instead, which halves the reduction's random accesses.
 template <bool SCATTER>
 __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* M, int mode, int need, int from, int to,
                                                    int nblk) {
@@ -79,13 +79,12 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* M, in
   grid_trigger();
   if (!mine) return;
   const float s = wide ? sum_slots_warp(A, M, b, e, lane) : sum_slots(A, M, q, b, e);
-  const float sbar = __ldg(A.invdeg + i) * s;
+  const float t = mode == 1 ? s : __ldg(A.invdeg + i) * s;
   if (!wide || lane == 0) {
     if (need & kNeedS) A.S[i] = s;
-    if (need & kNeedSbar) A.Sbar[i] = sbar;
+    if (need & kNeedAvg) A.var_avg[i] = t;
   }
   if (SCATTER) {
-    const float t = mode == 1 ? s : sbar;
     if (!wide) {
 #pragma unroll
       for (int r = 0; r < kEll; ++r)
@@ -103,7 +102,8 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* M, in
 // r_i = c_i - sum_j (lambda_ij + M_ij) is spread with the averaging weights.
 template <bool SCATTER>
 __global__ void __launch_bounds__(256) k_reduce_renorm(DevArena A, const float* __restrict__ M, float* lam,
-                                                        const float* __restrict__ alpha, int mode, int from, int to) {
+                                                        const float* __restrict__ alpha, int mode, int need, int from,
+                                                        int to) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= A.n) return;
   const int b = __ldg(A.var_ptr + i), e = __ldg(A.var_ptr + i + 1);
@@ -115,13 +115,12 @@ __global__ void __launch_bounds__(256) k_reduce_renorm(DevArena A, const float* 
     s += mk;
     tot += (double)lam[q] + (double)mk;
   }
-  const float sbar = __ldg(A.invdeg + i) * s;
+  const float inv = __ldg(A.invdeg + i);
+  const float t = mode == 1 ? s : inv * s;
   A.S[i] = s;
-  A.Sbar[i] = sbar;
+  if (need & kNeedAvg) A.var_avg[i] = t;
   if (e > b) {
     const double r = A.c[i] - tot;
-    const float inv = __ldg(A.invdeg + i);
-    const float t = mode == 1 ? s : sbar;
     for (int k = b; k < e; ++k) {
       const int q = __ldg(A.var_slots + k);
       const double w = mode == 1 ? (double)alpha[q] : (double)inv;
@@ -320,15 +319,16 @@ void launch_gather_var(const DevArena& A, const float* v, float* out_slot, cudaS
 }
 
 void launch_reduce_S(const DevArena& A, const float* M, float* lam, const float* alpha, int mode, bool renorm,
-                     Chain& ch, Scatter to, int need) {
+                     Chain& ch, Scatter to, bool store_S) {
   const int G = var_blocks(A);
   if (G == 0) return;
   const int from = A.unit_slots, end = scatter_to(A);
   const bool scatter = to == Scatter::kSweep && from < end;
+  const int need = (store_S ? kNeedS : 0) | (to == Scatter::kSweep ? kNeedAvg : 0);
   if (renorm) {
     ch.linked = false;
-    scatter ? k_reduce_renorm<true><<<G, kVarThreads, 0, ch.ss.main>>>(A, M, lam, alpha, mode, from, end)
-            : k_reduce_renorm<false><<<G, kVarThreads, 0, ch.ss.main>>>(A, M, lam, alpha, mode, from, end);
+    scatter ? k_reduce_renorm<true><<<G, kVarThreads, 0, ch.ss.main>>>(A, M, lam, alpha, mode, need, from, end)
+            : k_reduce_renorm<false><<<G, kVarThreads, 0, ch.ss.main>>>(A, M, lam, alpha, mode, need, from, end);
   } else {
     chain_launch(ch, scatter ? k_reduce_S<true> : k_reduce_S<false>, G + wide_blocks(A), kVarThreads, 0, A, M, mode,
                  need, from, end, G);

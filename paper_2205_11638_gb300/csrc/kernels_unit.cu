@@ -301,7 +301,7 @@ __device__ __forceinline__ void short_body(const DevArena& A, const SweepArgs& a
     grid_trigger();
   }
   float l[kShortK], av[kShortK], om[kShortK], al[kShortK];
-  const float* src = MODE == 1 ? A.S : A.Sbar;
+  const float* src = A.var_avg;
 #pragma unroll
   for (int h = 0; h < kShortK; ++h) {
     const bool on = h < k;
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
     __syncwarp();
     // the averaging terms (S_i in mode 1, S_i / |J_i| in mode 0) replace the
     // ids; they are not needed before the second pass
-    const float* src = MODE == 1 ? A.S : A.Sbar;
+    const float* src = A.var_avg;
     float* q = m + kAvg + lane;
 #pragma unroll 2
     for (int h = 0; h < k; ++h) {
@@ -861,21 +861,19 @@ __global__ void __launch_bounds__(1024) k_small_iterate(DevArena A, SweepArgs a,
     }
     __syncthreads();
   };
-  reduce();
   for (int it = 0; it < iters; ++it) {
+    reduce();
     sweep(TypeC<kFwd>{}, nullptr);
     reduce();
     sweep(TypeC<kBwd>{}, it + 1 == iters ? a.E : nullptr);
-    reduce();
   }
   for (int q = threadIdx.x; q < ns; q += blockDim.x) {
     a.lam[q] = lam[q];
     a.M[q] = M[q];
   }
   for (int i = threadIdx.x; i < A.n; i += blockDim.x) {
-    const float s = sum(i);
-    A.S[i] = s;
-    A.Sbar[i] = __ldg(A.invdeg + i) * s;
+    A.var_avg[i] = S[i];  // the last sweep's
+    A.S[i] = sum(i);
   }
 }
 

@@ -5,7 +5,7 @@
 // code running inside a CUDA graph capture that forbids cudaMalloc, embedders
 // whose allocator is owned by another runtime, or a serving loop with a
 // fixed, pre-planned memory budget.  dg_lower_bound writes its intermediates
-// (E^j per row, S_i and S_i / |J_i| per variable, one FP64 partial sum per
+// (E^j per row, S_i per variable, one FP64 partial sum per
 // reduction chunk, the path costs of long BDDs) into the scratch area of the
 // caller's arena buffer; this
 // variant keeps them in one file-scope __device__ array instead, so the
@@ -14,8 +14,8 @@
 //
 // Limits and sharing:
 //  * the array holds kNoallocScratchBytes (4 MiB); arenas whose intermediates
-//    need more (4 m + 8 n + 8 chunks + 4 per node of the long BDDs bytes) are
-//    rejected with DG_EINVAL;
+//    need more (4 m + 8 n + 8 chunks + 4 per node of the long BDDs bytes; of
+//    the 8 n half is in use) are rejected with DG_EINVAL;
 //  * every GPU that loads libdg holds the array until the process exits;
 //  * all calls share it: two calls whose kernels overlap on the GPU (on
 //    different streams, or from different host threads) race on it.  Calls
@@ -82,8 +82,7 @@ dg_status lower_bound_noalloc(const DevArena& arena, const LaunchGroup* groups, 
   DevArena A = arena;  // same structure, intermediates redirected
   A.E = reinterpret_cast<float*>(p);
   A.S = reinterpret_cast<float*>(p + bE);
-  A.Sbar = reinterpret_cast<float*>(p + bE + bS);
-  A.slot_avg = nullptr;  // the bound's S reduction leaves the per-slot terms alone
+  A.var_avg = A.slot_avg = nullptr;  // the bound's S reduction leaves the sweeps' averaging terms alone
   A.lb_part = reinterpret_cast<double*>(p + bE + 2 * bS);
   A.long_t = reinterpret_cast<float*>(p + bE + 2 * bS + bP);  // SP(., T) of the long BDDs' nodes
   A.long_d = nullptr;                                         // not read by the energy pass
