@@ -423,6 +423,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   for (int mode = 0; mode < 2; ++mode) A.long_unit_smem[mode] = P.long_unit_smem[mode];
   A.long_unit_adj_smem = P.long_unit_adj_smem;
   A.long_wide_smem = P.long_wide_smem;
+  A.chained = P.chained ? 1 : 0;
   {
     // lanes per narrow long BDD: the widest level's power of two (or the
     // option's, if larger); by default doubled (fewer BDDs per warp) while

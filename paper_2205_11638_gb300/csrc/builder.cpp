@@ -710,12 +710,26 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       const Tile& tl = P.tiles[t];
       return !tl.unit ? 2 : (short_kernels && unit_short(P.unit_shapes[tl.unit - 1]) ? 1 : 0);
     };
+    // ... and an arena of unit tiles alone is one launch (then chained, see
+    // Plan::chained) while its tiles, at the largest one's footprint, fill the
+    // chip at most kOneLaunchFills times and that footprint leaves at least
+    // seven warps per SM.  us per iteration (plain; per slot; recorded and
+    // reversed), one launch / several forked: tracking with 50 frames of 400
+    // detections 17; 18; 53 / 29; 29; 75, 25 frames of 2,000, 2.8 fills 33; 34;
+    // 90 / 38; 40; 98, 50 frames, 5.2 fills 49; 54; 152 / 51; 59; 153, 80 frames,
+    // 10 fills 70; 85; 253 / 70; 77; 224.
+    constexpr size_t kOneLaunchFills = 6, kOneLaunchSmem = 32 * 1024;
+    const size_t largest = T > 0 ? group_smem(0) : 0;
+    int others = 0;  // tiles that are not the short kernels'
+    for (int t = 0; t < T; ++t) others += group_kind(t) == 0;
+    const bool one_launch = T > 0 && nunit == T && long_rows.empty() && largest <= kOneLaunchSmem &&
+                            (size_t)others <= kOneLaunchFills * kSms * std::min<size_t>(64, kSmSmem / largest);
     for (int t = 0; t <= T; ++t) {
       const size_t r = t < T ? group_smem(t) : 0;
       const bool full = gmax > 0 && (size_t)(t - t0) >= kSms * std::min<size_t>(64, kSmSmem / gmax);
       // (short unit tiles need no shared memory: one group whatever their size)
       const int kind = t < T ? group_kind(t) : 3, kind0 = t > t0 ? group_kind(t0) : kind;
-      const bool cut = kind != kind0 || (kind != 1 && full && (double)r < kGroupRatio * (double)gmax);
+      const bool cut = kind != kind0 || (kind != 1 && full && !one_launch && (double)r < kGroupRatio * (double)gmax);
       if (t == T || (t > t0 && cut)) {
         if (t > t0) {
           LaunchGroup g{};
@@ -922,6 +936,10 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     // the longest items first
     std::stable_sort(P.long_items.begin(), P.long_items.end(),
                      [](const LongItem& x, const LongItem& y) { return x.kmax > y.kmax; });
+    constexpr int kChainTiles = 16384;
+    P.chained = P.num_long_unit == (int32_t)P.longs.size() &&
+                (T == 0 || (nunit == T && P.longs.empty() &&
+                            (P.groups.size() == 1 || (P.groups.size() == 2 && P.groups[1].unit_short && T <= kChainTiles))));
     P.num_long_narrow = (int32_t)P.long_order.size();
     P.long_lanes = opts ? opts->long_lanes : 0;
     size_t wide = 0;
@@ -1350,6 +1368,12 @@ dg_status validate_plan(const Plan& P) {
     t0 = g.tile1;
   }
   if (t0 != T) return bad("launch groups do not cover the tiles");
+  // a chain launches the kernels of the unit rows alone
+  if (P.chained) {
+    if (P.num_long_unit != (int32_t)P.longs.size()) return bad("chained launches with other long BDDs");
+    for (const LaunchGroup& g : P.groups)
+      if (g.unit_w == 0) return bad("chained launches with mixed tiles");
+  }
   // bound chunks: per instance its rows, then its variables, in order
   const int ni = P.sizes.num_inst;
   for (int k = 0; k < ni; ++k) {

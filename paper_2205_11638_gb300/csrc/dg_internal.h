@@ -231,6 +231,7 @@ struct DevArena {
   int32_t long_unit_smem[2];  // shared memory of the largest work item, mode 0 and 1
   int32_t long_unit_adj_smem;
   int32_t long_lanes;       // lanes per narrow BDD in the plain sweeps (a power of two, set at bind)
+  int32_t chained;          // a sweep's launches form one chain (see Plan::chained)
 };
 
 // Tiles that one kernel launch sweeps: consecutive tiles whose shared-memory
@@ -274,6 +275,16 @@ struct Plan {
   int32_t unit_slots = 0, unit_nodes = 0;
   std::vector<LaunchGroup> groups;
   std::vector<AdjGroup> adj_groups;
+  // Whether a sweep's launches form one chain on the caller's stream instead of
+  // forking onto the arena's streams.  A small arena's time is launch latency,
+  // which the chain hides; but its kernels run one after another, so that only
+  // arenas of one launch group take it (or of long unit BDDs alone), or of two
+  // when the second is of short tiles and small (kChainTiles): these need no
+  // shared memory and little time.  us per iteration and per iteration recorded
+  // and reversed, chained / forked: batch of 8, 12,300 tiles, two groups 42 / 51
+  // and 114 / 115; tracking with 80 frames of 2,000, 15,200 tiles, four groups
+  // 99 / 71 and 279 / 223.
+  bool chained = false;
   std::vector<uint16_t> desc;
   std::vector<uint16_t> lohi8;
   std::vector<int32_t> slot_var, slot_row;

@@ -106,22 +106,8 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 
-// Whether a sweep's launches form one chain on the caller's stream instead of
-// forking onto the arena's streams: arenas of unit tiles only with one launch
-// group or up to kChainTiles tiles, and arenas of long unit BDDs only.  A small
-// arena's time is launch latency, which the chain hides (20 iterations of
-// tracking, us per iteration chained / forked: 50 frames, 9,500 tiles 52 / 57;
-// 4 batched instances, 5,000 tiles 25 / 36); a large one's launch groups share
-// the SMs better side by side, large shared-memory tiles next to narrow ones,
-// than one after another (100 frames, 19,000 tiles 88 / 82; 500 frames, 96,000
-// tiles 438 / 370).
 // Kinds of long BDDs an arena has (unit rows, others).
 inline int long_launches(const DevArena& A) { return (A.num_long_items > 0) + (A.num_long > A.num_long_unit); }
-constexpr int kChainTiles = 16384;
-inline bool chained_sweeps(const DevArena& A, int num_groups) {
-  if (num_groups == 0) return A.num_long == A.num_long_unit;
-  return A.unit_slots == A.num_slots && (num_groups == 1 || A.num_tiles <= kChainTiles);
-}
 
 cudaError_t set_sweep_smem_limit(size_t bytes);
 cudaError_t set_unit_smem_limit(size_t bytes);
@@ -129,7 +115,7 @@ cudaError_t set_unit_smem_limit(size_t bytes);
 // `region` bytes to a CTA.
 struct AdjArgs;
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
-                 Chain& ch, bool late);
+                 Chain& ch);
 // `iters` iterations of Alg. 1 on a small arena of unit tiles in one launch
 // (energies of the last backward sweep into a.E when not NULL); false, and
 // nothing launched, when the arena is not of that kind.
@@ -145,7 +131,7 @@ bool launch_small_iterate(const DevArena& A, const SweepArgs& a, const LaunchGro
 void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, const LaunchGroup& G,
                           int wpc, size_t region, cudaStream_t st);
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
-                         Chain& ch, bool late);
+                         Chain& ch);
 // Dynamic shared memory one CTA may use; launchers put fewer warps in a CTA
 // when their tiles need more.
 void set_cta_smem_cap(size_t bytes);

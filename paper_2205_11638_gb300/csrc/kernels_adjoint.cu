@@ -247,7 +247,7 @@ cudaError_t set_adjoint_smem_limit(size_t bytes) {
 template <int FWD, int MODE>
 static void launch_adj(const DevArena& A, const AdjArgs& a, const AdjGroup* groups, int num_groups, size_t cap,
                        Chain& ch) {
-  const bool chained = chained_sweeps(A, num_groups);
+  const bool chained = A.chained != 0;
   const StreamSet& ss = ch.ss;
   const bool fork = !chained && num_groups + long_launches(A) > 1 && ss.ready;
   if (fork) ss.begin();
@@ -268,11 +268,11 @@ static void launch_adj(const DevArena& A, const AdjArgs& a, const AdjGroup* grou
     const int wpc = best_warps_per_cta(region, 4, cap);
     if (G.unit_w > 0) {
       if (chained) {
-        launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, ch, g > 0);
+        launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, ch);
       } else {
         Chain own;
         own.ss.main = fork ? ss.of(G.stream) : ss.main;
-        launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, own, false);
+        launch_unit_adjoint(FWD != 0, A, a, G, wpc, region, own);
       }
       continue;
     }

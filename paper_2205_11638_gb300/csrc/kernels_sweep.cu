@@ -420,7 +420,7 @@ void StreamSet::end() const {
 template <int KIND, int MODE>
 static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, const LaunchGroup* groups,
                           int num_groups, Chain& ch) {
-  const bool chained = chained_sweeps(A, num_groups);
+  const bool chained = A.chained != 0;
   const StreamSet& ss = ch.ss;
   const bool fork = !chained && num_groups + long_launches(A) > 1 && ss.ready;
   if (fork) ss.begin();
@@ -455,11 +455,11 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
       wpc = best_warps_per_cta(region, wpc, g_cta_smem_cap);
     if (unit) {
       if (chained) {
-        launch_unit(KIND, A, a, G, wpc, region, ch, g > 0);
+        launch_unit(KIND, A, a, G, wpc, region, ch);
       } else {
         Chain own;
         own.ss.main = fork ? ss.of(G.stream) : ss.main;
-        launch_unit(KIND, A, a, G, wpc, region, own, false);
+        launch_unit(KIND, A, a, G, wpc, region, own);
       }
       continue;
     }

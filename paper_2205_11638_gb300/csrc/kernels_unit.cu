@@ -287,19 +287,17 @@ __device__ __forceinline__ void short_types(const DevArena& A, const SweepArgs& 
     short_tile<KIND, MODE, K, AnyType>(A, a, T, S, l, av, om, al, lane);
 }
 
-// One short tile (see k_unit for `late`).
+// One short tile.
 template <int KIND, int MODE>
 __device__ __forceinline__ void short_body(const DevArena& A, const SweepArgs& a, const Tile& T, const UnitShape& S,
-                                           int lane, int late) {
+                                           int lane) {
   const int64_t sb = T.slot_base + lane;
   const int k = T.nhops;
   int v[kShortK];
 #pragma unroll
   for (int h = 0; h < kShortK; ++h) v[h] = h < k ? __ldcs(A.slot_var + sb + h * kWarp) : -1;
-  if (!late) {
-    grid_wait();
-    grid_trigger();
-  }
+  grid_wait();
+  grid_trigger();
   float l[kShortK], av[kShortK], om[kShortK], al[kShortK];
   const float* src = A.var_avg;
 #pragma unroll
@@ -318,19 +316,16 @@ __device__ __forceinline__ void short_body(const DevArena& A, const SweepArgs& a
 }
 
 template <int KIND, int MODE>
-__global__ void __launch_bounds__(128) k_unit_short(DevArena A, SweepArgs a, int tile0, int tile1, int late) {
+__global__ void __launch_bounds__(128) k_unit_short(DevArena A, SweepArgs a, int tile0, int tile1) {
   const int lane = threadIdx.x & 31;
   const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (tile >= tile1) return;
-  if (late) grid_trigger();
   const Tile T = A.tiles[tile];
-  short_body<KIND, MODE>(A, a, T, A.unit_shapes[T.unit - 1], lane, late);
-  if (late) grid_wait();
+  short_body<KIND, MODE>(A, a, T, A.unit_shapes[T.unit - 1], lane);
 }
 
 template <int KIND, int MODE, int WMAX>
-__global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int region_bytes, int tile0, int tile1,
-                                              int late) {
+__global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int region_bytes, int tile0, int tile1) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int tile = tile0 + blockIdx.x * (blockDim.x >> 5) + warp;
@@ -341,10 +336,6 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
   const int k = T.nhops;
   float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
   const uint64_t pol = l2_evict_first();
-  // A late group of a sweep starts when the group before it has waited for the
-  // kernel before the sweep (its trigger comes after), so only at its end does
-  // it wait: for that group.
-  if (late) grid_trigger();
   // the variable ids come first, into the words of the averaging terms, so
   // that the gather can follow as soon as they are there: two memory latencies
   // per tile whatever its length (ids loaded into registers a few levels at a
@@ -354,10 +345,8 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
     cp_async_commit();
   }
   const UnitShape S = A.unit_shapes[T.unit - 1];
-  if (!late) {
-    grid_wait();
-    grid_trigger();
-  }
+  grid_wait();
+  grid_trigger();
   copy_rows<STRIDE>(m, a.lam + T.slot_base, k, lane, pol);
   if (UPDATE && MODE == 1) {
     copy_rows<STRIDE>(m + kOm, a.omega + T.slot_base, k, lane, pol);
@@ -391,7 +380,6 @@ __global__ void __launch_bounds__(128) k_unit(DevArena A, SweepArgs a, int regio
     unit_tile<KIND, MODE, 6>(A, a, T, S, m, lane);
   else if (WMAX >= 8)
     unit_tile<KIND, MODE, 8>(A, a, T, S, m, lane);
-  if (late) grid_wait();
 }
 
 // ---- smoothed subproblems --------------------------------------------------
@@ -706,8 +694,7 @@ __device__ __forceinline__ void unit_adjoint_tile(const AdjArgs& a, const Tile& 
 }
 
 template <int FWD, int MODE, int WMAX>
-__global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int region_bytes, int tile0, int tile1,
-                                                      int late) {
+__global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int region_bytes, int tile0, int tile1) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int STRIDE = kWarp * (MODE == 1 ? 7 : 6);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -717,14 +704,11 @@ __global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int
   const int k = T.nhops;
   float* m = reinterpret_cast<float*>(smem + (size_t)warp * region_bytes);
   const uint64_t pol = l2_evict_first();
-  if (late) grid_trigger();  // see k_unit
   copy_rows<STRIDE>(m + kJIn, A.slot_var + T.slot_base, k, lane, pol);
   cp_async_commit();
   const UnitShape S = A.unit_shapes[T.unit - 1];
-  if (!late) {
-    grid_wait();
-    grid_trigger();
-  }
+  grid_wait();
+  grid_trigger();
   copy_rows<STRIDE>(m, a.g_lam + T.slot_base, k, lane, pol);
   copy_rows<STRIDE>(m + kJRec, a.rec_unit + T.slot_base, k, lane, pol);
   copy_rows<STRIDE>(m + kJDiff, a.rec_diff + T.slot_base, k, lane, pol);
@@ -758,16 +742,14 @@ __global__ void __launch_bounds__(128) k_unit_adjoint(DevArena A, AdjArgs a, int
     unit_adjoint_tile<FWD, MODE, 6>(a, T, s, m, lane);
   else if (WMAX >= 8)
     unit_adjoint_tile<FWD, MODE, 8>(a, T, s, m, lane);
-  if (late) grid_wait();
 }
 
 template <int FWD, int MODE>
-void launch_adjoint_group(const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region, Chain& ch,
-                          bool late) {
+void launch_adjoint_group(const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region, Chain& ch) {
   const int nt = G.tile1 - G.tile0, grid = (nt + wpc - 1) / wpc;
   auto k = G.unit_w <= 2 ? k_unit_adjoint<FWD, MODE, 2>
                          : (G.unit_w <= 4 ? k_unit_adjoint<FWD, MODE, 4> : k_unit_adjoint<FWD, MODE, 8>);
-  chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1, late ? 1 : 0);
+  chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1);
 }
 
 template <int FWD, int MODE>
@@ -878,18 +860,17 @@ __global__ void __launch_bounds__(1024) k_small_iterate(DevArena A, SweepArgs a,
 }
 
 template <int KIND, int MODE>
-void launch_group(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, Chain& ch,
-                  bool late) {
+void launch_group(const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region, Chain& ch) {
   const int nt = G.tile1 - G.tile0;
   if constexpr (KIND == kFwd || KIND == kBwd || KIND == kFwdRec || KIND == kBwdRec) {
     if (G.unit_short) {
-      chain_launch(ch, k_unit_short<KIND, MODE>, (nt + 3) / 4, 128, 0, A, a, G.tile0, G.tile1, late ? 1 : 0);
+      chain_launch(ch, k_unit_short<KIND, MODE>, (nt + 3) / 4, 128, 0, A, a, G.tile0, G.tile1);
       return;
     }
   }
   const int grid = (nt + wpc - 1) / wpc;
   auto k = G.unit_w <= 2 ? k_unit<KIND, MODE, 2> : (G.unit_w <= 4 ? k_unit<KIND, MODE, 4> : k_unit<KIND, MODE, 8>);
-  chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1, late ? 1 : 0);
+  chain_launch(ch, k, grid, wpc * kWarp, region * wpc, A, a, (int)region, G.tile0, G.tile1);
 }
 
 template <int KIND, int MODE>
@@ -931,20 +912,20 @@ cudaError_t set_unit_smem_limit(size_t bytes) {
 }
 
 void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGroup& G, int wpc, size_t region,
-                 Chain& ch, bool late) {
+                 Chain& ch) {
   const bool m1 = a.mode == 1;
   switch (kind) {
-    case kFwd: m1 ? launch_group<kFwd, 1>(A, a, G, wpc, region, ch, late) : launch_group<kFwd, 0>(A, a, G, wpc, region, ch, late); break;
-    case kBwd: m1 ? launch_group<kBwd, 1>(A, a, G, wpc, region, ch, late) : launch_group<kBwd, 0>(A, a, G, wpc, region, ch, late); break;
+    case kFwd: m1 ? launch_group<kFwd, 1>(A, a, G, wpc, region, ch) : launch_group<kFwd, 0>(A, a, G, wpc, region, ch); break;
+    case kBwd: m1 ? launch_group<kBwd, 1>(A, a, G, wpc, region, ch) : launch_group<kBwd, 0>(A, a, G, wpc, region, ch); break;
     case kFwdRec:
-      m1 ? launch_group<kFwdRec, 1>(A, a, G, wpc, region, ch, late) : launch_group<kFwdRec, 0>(A, a, G, wpc, region, ch, late);
+      m1 ? launch_group<kFwdRec, 1>(A, a, G, wpc, region, ch) : launch_group<kFwdRec, 0>(A, a, G, wpc, region, ch);
       break;
     case kBwdRec:
-      m1 ? launch_group<kBwdRec, 1>(A, a, G, wpc, region, ch, late) : launch_group<kBwdRec, 0>(A, a, G, wpc, region, ch, late);
+      m1 ? launch_group<kBwdRec, 1>(A, a, G, wpc, region, ch) : launch_group<kBwdRec, 0>(A, a, G, wpc, region, ch);
       break;
-    case kMinMarg: launch_group<kMinMarg, 0>(A, a, G, wpc, region, ch, late); break;
-    case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, ch, late); break;
-    default: launch_group<kSeed, 0>(A, a, G, wpc, region, ch, late); break;
+    case kMinMarg: launch_group<kMinMarg, 0>(A, a, G, wpc, region, ch); break;
+    case kEnergy: launch_group<kEnergy, 0>(A, a, G, wpc, region, ch); break;
+    default: launch_group<kSeed, 0>(A, a, G, wpc, region, ch); break;
   }
 }
 
@@ -980,13 +961,13 @@ void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float*
 }
 
 void launch_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, const AdjGroup& G, int wpc, size_t region,
-                         Chain& ch, bool late) {
+                         Chain& ch) {
   if (forward)
-    a.mode == 1 ? launch_adjoint_group<1, 1>(A, a, G, wpc, region, ch, late)
-                : launch_adjoint_group<1, 0>(A, a, G, wpc, region, ch, late);
+    a.mode == 1 ? launch_adjoint_group<1, 1>(A, a, G, wpc, region, ch)
+                : launch_adjoint_group<1, 0>(A, a, G, wpc, region, ch);
   else
-    a.mode == 1 ? launch_adjoint_group<0, 1>(A, a, G, wpc, region, ch, late)
-                : launch_adjoint_group<0, 0>(A, a, G, wpc, region, ch, late);
+    a.mode == 1 ? launch_adjoint_group<0, 1>(A, a, G, wpc, region, ch)
+                : launch_adjoint_group<0, 0>(A, a, G, wpc, region, ch);
 }
 
 }  // namespace dg

@@ -267,3 +267,67 @@ def test_packed_segments_of_unequal_lengths(mode):
     for a, b in zip(out[0][0], out[1][0]):
         assert torch.isfinite(a).all()
         assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
+
+
+def _two_footprints(seed, n=3000):
+    """Unit rows alone in tiles of two footprints: 10,000 covering rows of 126
+    variables, which fill the chip by themselves, and 2,000 of four."""
+    rng = np.random.default_rng(seed)
+    rows = [(rng.integers(0, n - 126) + np.arange(126), np.ones(126, np.int64), workloads.GE, 1) for _ in range(10000)]
+    rows += [(rng.integers(0, n - 4) + np.arange(4), np.ones(4, np.int64), workloads.LE, 1) for _ in range(2000)]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+def _mostly_short(seed, n=20000):
+    """Unit rows alone, most of them of two and three variables: 8,320 tiles of
+    these and 60 of six."""
+    rng = np.random.default_rng(seed)
+    rows = []
+    for a, sense, b in (([1, 1], workloads.LE, 1), ([1, 1], workloads.GE, 1), ([1, 1, 1], workloads.LE, 1),
+                        ([-1, -1, 1], workloads.LE, 0)):
+        rows += [(v + np.arange(len(a)), np.array(a), sense, b) for v in rng.integers(0, n - 3, size=2080 * 32)]
+    rows += [(v + np.arange(6), np.ones(6, np.int64), 0, 1) for v in rng.integers(0, n - 6, size=60 * 32)]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+# instance, launch groups: one launch for tiles of many shapes; two, the second
+# of short tiles, one after the other; two on streams of their own
+LAUNCHES = {
+    "one": (lambda: workloads.tracking(frames=50, dets=400, seed=46), 1),
+    "short_second": (lambda: _mostly_short(7), 2),
+    "forked": (lambda: _two_footprints(8), 2),
+}
+
+
+@pytest.mark.parametrize("name", sorted(LAUNCHES))
+@pytest.mark.parametrize("mode", [0, 1])
+def test_launches_of_a_unit_arena(name, mode):
+    """Every call's launches, chained or forked, against the doubled problem's:
+    sweeps over many iterations, marginals, energies and minimisers bit for bit,
+    gradients up to the rounding of sums (tolerance as above, 4 sweeps)."""
+    make, groups = LAUNCHES[name]
+    p = make()
+    exact, grads = [], []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q).bind()
+        if q is p:
+            assert X.plan.sizes.num_launch_groups == groups
+            X.plan.validate()
+        lam, M, om, al = [X.from_csr(x) for x in _vectors(p, 17)]
+        par = (om, al) if mode else (None, None)
+        grads.append([X.to_csr(x) for x in X.backward(lam, M, *par, 2, 2, *[X.from_csr(x) for x in _vectors(p, 18)[:2]])])
+        l2, M2 = lam.clone(), M.clone()
+        X.iterate_checkpointed(l2, M2, *par, iters=3, ckpt_every=3)
+        m0, m1 = X.min_marginals(lam)
+        lb0, E = X.lower_bound(lam, M, energies=True)
+        gl, gM = X.lb_seed(lam, M)
+        g = X.graph(lam, M, *par, iters=2)
+        torch.cuda.synchronize()
+        lb = X.iterate(lam, M, *par, iters=50, lb=True)
+        g.replay()
+        exact.append([X.to_csr(x) for x in (l2, M2, m0, m1, gl, gM, lam, M)] + [lb0, E, lb])
+    for a, b in zip(*exact):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+    for a, b in zip(*grads):
+        assert torch.isfinite(a).all()
+        assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
