@@ -840,6 +840,7 @@ __global__ void __launch_bounds__(1024) k_small_iterate(DevArena A, SweepArgs a,
         unit_tile<KIND, MODE, 6>(A, w, T, sh, row, lane);
       else
         unit_tile<KIND, MODE, 8>(A, w, T, sh, row, lane);
+      __syncwarp();  // the next tile of another shape places its inputs over other lanes' path costs
     }
     __syncthreads();
   };

@@ -331,3 +331,32 @@ def test_launches_of_a_unit_arena(name, mode):
     for a, b in zip(*grads):
         assert torch.isfinite(a).all()
         assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
+
+
+def _many_small_shapes(seed, n=60):
+    """Clauses of every sign pattern of two to four variables and of eight of
+    five, one to four rows each: a tile per pattern, 36 in all, more than a block
+    has warps and few enough for the kernel that runs whole iterations of a small
+    arena."""
+    rng = np.random.default_rng(seed)
+    signs = [2 * np.array(a) - 1 for k in (2, 3, 4) for a in np.ndindex(*(2,) * k)]
+    signs += [2 * np.array(a) - 1 for a in list(np.ndindex(*(2,) * 5))[seed % 4::4]]
+    rows = [(np.sort(rng.choice(n, size=len(a), replace=False)), a, workloads.GE, 1 - int((a < 0).sum()))
+            for a in signs for _ in range(int(rng.integers(1, 5)))]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("seed", [21, 22, 23])
+def test_small_arena_of_many_shapes(seed, mode):
+    p = _many_small_shapes(seed)
+    out = []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q).bind()
+        lam, M, om, al = [X.from_csr(x) for x in _vectors(p, 19)]
+        lb = X.iterate(lam, M, om if mode else None, al if mode else None, iters=100, lb=True)
+        out.append((X.to_csr(lam), X.to_csr(M), lb))
+        if q is p:
+            assert X.plan.sizes.num_tiles > 32
+    for a, b in zip(*out):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
