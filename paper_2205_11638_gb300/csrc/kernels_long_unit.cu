@@ -255,6 +255,7 @@ __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs
       auto step = [&](int h, bool on) {
         const In nxt = input(h + 1);
         const float tz1 = pz[(h + 2) * TS], to1 = po[(h + 2) * TS];
+        __syncwarp();  // every lane has read a level before any replaces its inputs
         const float n = from_neighbour<G, TY>(R, g, f_inf());
         const float x0 = R + tz, x1 = ov ? R + to : f_inf();
         const float b0 = seg_min<G>(x0), b1 = seg_min<G>(x1);
@@ -304,6 +305,7 @@ __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs
       constexpr int TY = decltype(ty)::value;
       const In nxt = input(h - 1);
       const float r1 = mt[max(h - 1, 0) * TS];
+      __syncwarp();  // as above
       float tz, to;
       children<G, TY>(t, g, tz, to);
       const float x0 = r + tz, x1 = r + to;
