@@ -422,6 +422,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.num_long_items = (int32_t)P.long_items.size();
   for (int mode = 0; mode < 2; ++mode) A.long_unit_smem[mode] = P.long_unit_smem[mode];
   A.long_unit_adj_smem = P.long_unit_adj_smem;
+  A.long_wide_block = P.long_wide_block ? 1 : 0;
   A.long_wide_smem = P.long_wide_smem;
   A.chained = P.chained ? 1 : 0;
   {

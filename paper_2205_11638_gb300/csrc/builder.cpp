@@ -698,7 +698,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
         opts && opts->group_ratio_pct > 0 && opts->group_ratio_pct <= 100 ? opts->group_ratio_pct / 100.0 : 0.85;
     // ... or any smaller one while the group's tiles do not fill the chip (its
     // smaller tiles then cost it no occupancy and save a launch)
-    constexpr size_t kSms = 152, kSmSmem = 224 * 1024;
+    constexpr size_t kSmSmem = 224 * 1024;
     int32_t t0 = 0;
     size_t gmax = 0;
     auto group_smem = [&](int t) {
@@ -910,7 +910,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       // warps per SM (a warp's levels are a chain of dependent steps, which
       // other warps hide), and as fit shared memory
       int nseg = G <= kUnitMaxW ? kWarp : kWarp / G;
-      while (nseg > 1 && ((int64_t)(e - i) < 4LL * 152 * nseg || long_unit_bytes(nseg, G, kmax, 1) > 64 * 1024 ||
+      while (nseg > 1 && ((int64_t)(e - i) < 4LL * kSms * nseg || long_unit_bytes(nseg, G, kmax, 1) > 64 * 1024 ||
                           long_unit_adjoint_bytes(nseg, kmax) > 64 * 1024))
         nseg /= 2;
       const int32_t run_base = (int32_t)P.unit_runs.size();
@@ -943,12 +943,29 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     P.num_long_narrow = (int32_t)P.long_order.size();
     P.long_lanes = opts ? opts->long_lanes : 0;
     size_t wide = 0;
+    int64_t wide_nodes = 0;
     for (size_t b = 0; b < P.longs.size(); ++b)
       if (P.longs[b].maxw > kWarp) {
         P.long_order.push_back((int32_t)b);
         wide = std::max(wide, (size_t)(P.longs[b].nn + 2) * 8);
+        wide_nodes += P.longs[b].nn;
       }
-    P.long_wide_smem = wide <= 200 * 1024 ? (int32_t)wide : 0;
+    // Team of a wide one: a block is faster on its own, warps fill the chip
+    // better once there are many BDDs, the later the more nodes these have.
+    // Path costs in shared memory while the blocks this leaves room for (at most
+    // eight an SM, by their threads) are all of them.  us per iteration and per
+    // iteration recorded and reversed, shared memory / scratch / warps:
+    //   1,850 nodes a BDD: 608 BDDs 89, 372 / 97, 376 / 132, 492
+    //                    1,520 BDDs 174, 811 / 184, 814 / 136, 678
+    //   16,900 nodes:      152 BDDs 217, 1180 / 252, 1226 / 670, 3491
+    //                      608 BDDs 1360, 3232 / 425, 1859 / 1236, 5092
+    //                    3,648 BDDs - / 1469, 7278 / 1425, 6102
+    //   71,000 nodes:    3,648 BDDs - / 4007, 21386 / 5965, 23425
+    //                    4,864 BDDs - / 5303, 30087 / 6310, 25236
+    const int64_t nwide = (int64_t)P.longs.size() - P.num_long_narrow;
+    const int64_t fit = wide <= 200 * 1024 ? std::min<int64_t>(8, (int64_t)(227 * 1024 / (wide + 1024))) : 0;
+    P.long_wide_smem = nwide <= kSms * fit ? (int32_t)wide : 0;
+    P.long_wide_block = nwide <= kSms * std::min<int64_t>(24, 6 + (nwide ? wide_nodes / nwide : 0) / 1700);
   }
   const int64_t num_slots = slot_base;
   if (num_slots >= (int64_t)INT32_MAX || node_base >= (int64_t)INT32_MAX)

@@ -27,6 +27,7 @@ constexpr uint32_t kBotCode = 1u;
 constexpr int kMaxNodesPerBdd = 254;
 constexpr int kWarp = 32;
 constexpr int kMaxWidth = 128;  // nodes of one BDD level (child ranks are 8-bit)
+constexpr int kSms = 152;      // SMs the layout is chosen for (a plan is made without a device)
 constexpr int kStreams = 4;    // streams one sweep's launch groups run on
 // The first kEll slots of every variable are also stored column by column
 // (var_ell[r * n + i], ELLPACK layout) so that the S reduction reads them
@@ -227,7 +228,8 @@ struct DevArena {
   int32_t num_long_narrow;  // narrow long BDDs (the head of long_order)
   int32_t num_long_unit;    // ... of them, the unit ones (its very head)
   int32_t num_long_items;
-  int32_t long_wide_smem;   // shared memory of the largest wide long BDD's path costs (0: one does not fit)
+  int32_t long_wide_block;  // whether the wide long BDDs are swept by a block each, or a warp
+  int32_t long_wide_smem;   // shared memory of the largest wide long BDD's path costs (0: they stay in long_d, long_t)
   int32_t long_unit_smem[2];  // shared memory of the largest work item, mode 0 and 1
   int32_t long_unit_adj_smem;
   int32_t long_lanes;       // lanes per narrow BDD in the plain sweeps (a power of two, set at bind)
@@ -312,6 +314,7 @@ struct Plan {
   int32_t num_long_narrow = 0, num_long_unit = 0;
   std::vector<LongItem> long_items;
   int32_t long_unit_smem[2] = {0, 0}, long_unit_adj_smem = 0, long_wide_smem = 0;
+  bool long_wide_block = false;
   int32_t long_lanes = 0;           // dg_options::long_lanes (0: chosen at bind)
   std::vector<int64_t> long_rank_ptr;  // per long BDD, first entry of long_lo / long_hi
   std::vector<int32_t> long_lo, long_hi;  // child ranks as in lo8 / hi8 (-2 bottom, -1 top)

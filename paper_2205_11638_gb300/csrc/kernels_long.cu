@@ -6,8 +6,9 @@
 // recursions over one BDD visit its levels one after another.
 //
 // Execution model: one team of threads per BDD, a warp for BDDs of at most 32
-// nodes a level and a block of 256 threads for wider ones (a level of 169 nodes
-// took a warp six rounds of dependent loads); the nodes of a level are spread
+// nodes a level and for many wider ones, a block of 256 threads for few wider
+// ones (a level of 169 nodes takes a warp six rounds of dependent loads; the
+// line is drawn where Plan::long_wide_block is set); the nodes of a level are spread
 // over the team (node f + id, f + id + size, ...), the levels are walked in
 // turn with a barrier of the team between them.  The min-marginals of a level (App. B:
 // m^beta = min over the level's nodes of SP(r, v) + SP(s^beta(v), T), plus
@@ -647,17 +648,16 @@ __device__ __forceinline__ void long_sweep(const DevArena& A, const SweepArgs& a
   if ((BWD || KIND == kEnergy) && a.E != nullptr && tm.id == 0) a.E[c.B.row] = c.t[2];  // E^j = SP(r, T)
 }
 
+// The BDDs long_order[first .. last), a warp each.
 template <int KIND, int MODE>
-__global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a) {
-  // BDDs of at most 32 nodes a level that are no unit rows (their plain sweeps
-  // run in k_long_narrow)
+__global__ void __launch_bounds__(128) k_long_sweep(DevArena A, SweepArgs a, int first, int last) {
   WarpTeam tm{(int)threadIdx.x & 31};
-  const int b = A.num_long_unit + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= A.num_long_narrow) return;  // whole warp leaves
+  const int b = first + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= last) return;  // whole warp leaves
   long_sweep<KIND, MODE>(A, a, long_ctx(A, A.long_order[b]), tm);
 }
 
-// The wide long BDDs, a block each.  Their path costs stay in shared memory
+// The wide long BDDs, a block each (see Plan::long_wide_block).  Their path costs stay in shared memory
 // when they fit (smem): read from the arena's scratch when the sweep before
 // left them, written back at the end for the sweep after.
 template <int KIND, int MODE>
@@ -907,10 +907,10 @@ __device__ __forceinline__ void long_adjoint(const DevArena& A, const AdjArgs& a
 }
 
 template <int FWD, int MODE>
-__global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a) {
+__global__ void __launch_bounds__(128) k_long_adjoint(DevArena A, AdjArgs a, int first, int last) {
   WarpTeam tm{(int)threadIdx.x & 31};
-  const int b = A.num_long_unit + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= A.num_long_narrow) return;
+  const int b = first + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= last) return;
   long_adjoint<FWD, MODE>(A, a, long_ctx(A, A.long_order[b]), tm);
 }
 
@@ -925,53 +925,44 @@ namespace {
 
 constexpr int kLongWarps = 4;  // BDDs (warps) per CTA
 
-int long_grid(const DevArena& A) { return (A.num_long + kLongWarps - 1) / kLongWarps; }
-// ... of the narrow ones that are no unit rows (kernels_long_unit.cu)
-int long_grid_narrow(const DevArena& A) { return (A.num_long_narrow - A.num_long_unit + kLongWarps - 1) / kLongWarps; }
+int long_grid(int n) { return (n + kLongWarps - 1) / kLongWarps; }
+
+// Where the BDDs that are swept by a warp each end in long_order (the wide
+// ones after that by a block each).
+int warps_end(const DevArena& A) { return A.long_wide_block ? A.num_long_narrow : A.num_long; }
 
 template <int KIND, int MODE>
-void launch_wide(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  const int g = A.num_long - A.num_long_narrow;
+void launch_warps(const DevArena& A, const SweepArgs& a, int first, int last, cudaStream_t st) {
+  if (last > first)
+    k_long_sweep<KIND, MODE><<<long_grid(last - first), kLongWarps * kWarp, 0, st>>>(A, a, first, last);
+}
+
+template <int KIND, int MODE>
+void launch_long_mode(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
+  int first = A.num_long_unit;  // the unit ones: kernels_long_unit.cu
+  if constexpr (KIND == kFwd || KIND == kBwd) {
+    if (A.num_long_narrow > first) {
+      const int warps = (A.num_long_narrow - first + kWarp / A.long_lanes - 1) / (kWarp / A.long_lanes);
+      k_long_narrow<KIND, MODE><<<long_grid(warps), kLongWarps * kWarp, 0, st>>>(A, a);
+    }
+    first = A.num_long_narrow;
+  }
+  launch_warps<KIND, MODE>(A, a, first, warps_end(A), st);
+  const int g = A.num_long - warps_end(A);
   if (g > 0) k_long_wide<KIND, MODE><<<g, BlockTeam::kSize, A.long_wide_smem, st>>>(A, a, A.long_wide_smem);
 }
 
 template <int KIND>
 void launch_long_kind(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (A.num_long_narrow > A.num_long_unit) {
-    if constexpr (KIND == kFwd || KIND == kBwd) {
-      const int per = kWarp / A.long_lanes;
-      const int warps = (A.num_long_narrow - A.num_long_unit + per - 1) / per;
-      const int ng = (warps + kLongWarps - 1) / kLongWarps;
-      if (a.mode == 1)
-        k_long_narrow<KIND, 1><<<ng, kLongWarps * kWarp, 0, st>>>(A, a);
-      else
-        k_long_narrow<KIND, 0><<<ng, kLongWarps * kWarp, 0, st>>>(A, a);
-    } else if (a.mode == 1) {
-      k_long_sweep<KIND, 1><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
-    } else {
-      k_long_sweep<KIND, 0><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
-    }
-  }
-  a.mode == 1 ? launch_wide<KIND, 1>(A, a, st) : launch_wide<KIND, 0>(A, a, st);
+  a.mode == 1 ? launch_long_mode<KIND, 1>(A, a, st) : launch_long_mode<KIND, 0>(A, a, st);
 }
 
-// kMinMarg, kEnergy, kSeed: no omega, no alpha
-template <int KIND>
-void launch_long_plain(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (A.num_long_narrow > A.num_long_unit)
-    k_long_sweep<KIND, 0><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
-  launch_wide<KIND, 0>(A, a, st);
-}
-
-template <int FWD>
-void launch_adjoint_kind(const DevArena& A, const AdjArgs& a, cudaStream_t st) {
-  const int g = A.num_long_narrow - A.num_long_unit, gw = A.num_long - A.num_long_narrow;
-  if (g > 0)
-    a.mode == 1 ? k_long_adjoint<FWD, 1><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a)
-                : k_long_adjoint<FWD, 0><<<long_grid_narrow(A), kLongWarps * kWarp, 0, st>>>(A, a);
-  if (gw > 0)
-    a.mode == 1 ? k_long_wide_adjoint<FWD, 1><<<gw, BlockTeam::kSize, 0, st>>>(A, a)
-                : k_long_wide_adjoint<FWD, 0><<<gw, BlockTeam::kSize, 0, st>>>(A, a);
+template <int FWD, int MODE>
+void launch_adjoint_mode(const DevArena& A, const AdjArgs& a, cudaStream_t st) {
+  const int first = A.num_long_unit, last = warps_end(A), g = A.num_long - last;
+  if (last > first)
+    k_long_adjoint<FWD, MODE><<<long_grid(last - first), kLongWarps * kWarp, 0, st>>>(A, a, first, last);
+  if (g > 0) k_long_wide_adjoint<FWD, MODE><<<g, BlockTeam::kSize, 0, st>>>(A, a);
 }
 
 }  // namespace
@@ -983,9 +974,10 @@ void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStre
     case kBwd: launch_long_kind<kBwd>(A, a, st); break;
     case kFwdRec: launch_long_kind<kFwdRec>(A, a, st); break;
     case kBwdRec: launch_long_kind<kBwdRec>(A, a, st); break;
-    case kMinMarg: launch_long_plain<kMinMarg>(A, a, st); break;
-    case kEnergy: launch_long_plain<kEnergy>(A, a, st); break;
-    default: launch_long_plain<kSeed>(A, a, st); break;
+    // (no omega, no alpha)
+    case kMinMarg: launch_long_mode<kMinMarg, 0>(A, a, st); break;
+    case kEnergy: launch_long_mode<kEnergy, 0>(A, a, st); break;
+    default: launch_long_mode<kSeed, 0>(A, a, st); break;
   }
 }
 
@@ -1008,11 +1000,14 @@ cudaError_t set_long_smem_limit(size_t bytes) {
 
 void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, cudaStream_t st) {
   if (A.num_long == 0) return;
-  k_long_smoothed<<<long_grid(A), kLongWarps * kWarp, 0, st>>>(A, lam, a_s, E_a, marg);
+  k_long_smoothed<<<long_grid(A.num_long), kLongWarps * kWarp, 0, st>>>(A, lam, a_s, E_a, marg);
 }
 
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st) {
-  forward ? launch_adjoint_kind<1>(A, a, st) : launch_adjoint_kind<0>(A, a, st);
+  if (forward)
+    a.mode == 1 ? launch_adjoint_mode<1, 1>(A, a, st) : launch_adjoint_mode<1, 0>(A, a, st);
+  else
+    a.mode == 1 ? launch_adjoint_mode<0, 1>(A, a, st) : launch_adjoint_mode<0, 0>(A, a, st);
 }
 
 }  // namespace dg

@@ -189,3 +189,55 @@ def test_long_adjoint_checkpoint_interval_bit_identical():
     for o in outs[1:]:
         for x, y in zip(o, outs[0]):
             assert torch.equal(x, y)
+
+
+def _wide_rows(num, terms, top, rhs, seed, group=20):
+    """`num` knapsack rows of `terms` variables, `group` of them over variables of
+    their own, so that the first rows are a problem by themselves."""
+    rng = np.random.default_rng(seed)
+    n0 = terms + terms // 2
+    rows = []
+    for j in range(num):
+        first = j // group * n0
+        rows.append((first + np.sort(rng.choice(n0, size=terms, replace=False)), rng.integers(1, top, size=terms),
+                     workloads.LE, rhs))
+    n = -(-num // group) * n0
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n)), n0
+
+
+@pytest.mark.parametrize("per_slot", [False, True])
+@pytest.mark.parametrize("num,terms,top,rhs", [(1300, 30, 31, 200), (160, 100, 40, 200)])
+def test_wide_bdds_by_any_team(num, terms, top, rhs, per_slot):
+    """Wide BDDs swept by a warp each (1,300 of them) or by a block with the path
+    costs in the arena's scratch (160 larger ones), against the first 20 alone
+    (blocks, path costs in shared memory): the same additions and exact minima,
+    so everything but the gradients is equal bit for bit; these differ by the
+    rounding of sums over a level and the levels (at most 100 levels and 400
+    nodes, 2 iterations of 2 sweeps, 2^-24 each)."""
+    prob, n0 = _wide_rows(num, terms, top, rhs, seed=31)
+    nnz = 20 * terms
+    head = dict(n=n0, row_ptr=prob["row_ptr"][:21], col=prob["col"][:nnz], coef=prob["coef"][:nnz],
+                sense=prob["sense"][:20], rhs=prob["rhs"][:20], c=prob["c"][:n0])
+    rng = np.random.default_rng(32)
+    all_nnz = len(prob["col"])
+    v = [rng.normal(size=all_nnz), 0.1 * rng.normal(size=all_nnz), rng.uniform(0.2, 0.8, size=all_nnz),
+         rng.uniform(0.01, 0.2, size=all_nnz), rng.normal(size=all_nnz), rng.normal(size=all_nnz)]
+    out, grads = [], []
+    for p, k in ((prob, all_nnz), (head, nnz)):
+        A = solver.plan(p).bind()
+        lam, M, om, al, gl, gM = [A.from_csr(x[:k]) for x in v]
+        par = (om, al) if per_slot else (None, None)
+        grads.append([A.to_csr(x)[:nnz] for x in A.backward(lam, M, *par, 2, 1, gl, gM)])
+        l2, M2 = lam.clone(), M.clone()
+        A.iterate_checkpointed(l2, M2, *par, iters=2, ckpt_every=2)
+        m0, m1 = A.min_marginals(lam)
+        _, E = A.lower_bound(lam, M, energies=True)
+        seed, _ = A.lb_seed(lam, M)
+        A.iterate(lam, M, *par, iters=2)
+        assert torch.equal(lam, l2) and torch.equal(M, M2)
+        out.append([A.to_csr(x)[:nnz] for x in (lam, M, m0, m1, seed)] + [E[:20]])
+    for a, b in zip(*out):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+    for a, b in zip(*grads):
+        assert torch.isfinite(a).all()
+        assert (a - b).abs().max() <= (400 + 100) * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
