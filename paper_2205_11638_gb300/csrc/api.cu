@@ -420,6 +420,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.num_long_unit = P.num_long_unit;
   A.long_items = (const LongItem*)(b + P.off.long_items);
   A.num_long_items = (int32_t)P.long_items.size();
+  A.long_plain = P.long_plain;
   for (int mode = 0; mode < 2; ++mode) A.long_unit_smem[mode] = P.long_unit_smem[mode];
   A.long_unit_adj_smem = P.long_unit_adj_smem;
   A.long_wide_block = P.long_wide_block ? 1 : 0;
@@ -430,13 +431,13 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
     // option's, if larger); by default doubled (fewer BDDs per warp) while
     // that leaves fewer than four warps per SM
     int G = 1, maxw = 1, sms = 1;
-    for (int32_t i = P.num_long_unit; i < P.num_long_narrow; ++i) maxw = std::max(maxw, P.longs[P.long_order[i]].maxw);
+    for (int32_t i = P.long_plain; i < P.num_long_narrow; ++i) maxw = std::max(maxw, P.longs[P.long_order[i]].maxw);
     while (G < maxw) G <<= 1;
     if (P.long_lanes > 0) {
       G = std::max(G, (int)P.long_lanes);
     } else {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ar->device);
-      const int64_t packed = P.num_long_narrow - P.num_long_unit;
+      const int64_t packed = P.num_long_narrow - P.long_plain;
       while (G < kWarp && (packed + kWarp / G - 1) / (kWarp / G) < 4LL * sms) G <<= 1;
     }
     A.long_lanes = G;

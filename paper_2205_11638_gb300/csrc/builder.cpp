@@ -937,7 +937,26 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     std::stable_sort(P.long_items.begin(), P.long_items.end(),
                      [](const LongItem& x, const LongItem& y) { return x.kmax > y.kmax; });
     constexpr int kChainTiles = 16384;
-    P.chained = P.num_long_unit == (int32_t)P.longs.size() &&
+    // Plain sweeps of the unit ones.  Their kernels walk every level twice, with
+    // the path costs in shared memory, which leaves few warps to an SM when the
+    // rows are long and wide; the general kernel takes the costs of the sweep
+    // before and needs none.  A sweep's time: levels times a step over the warps
+    // an SM holds, against the larger of one row's chain and the SM's rate (ns a
+    // level).  us per iteration, unit / general: 13 states, 700 variables, 3,500
+    // rows 995 / 1112, 5,000 rows 1478 / 1187; 31 states, 1,000 variables, 1,200
+    // rows 1156 / 1472, 2,000 rows 2022 / 1584; 6 states, 1,300 variables, 6,000
+    // rows 1941 / 2028; 2 states, 1,300 variables, 20,000 rows 2310 / 4797.
+    {
+      const double warps = std::min(32, 227 * 1024 / (std::max(P.long_unit_smem[0], 1) + 1024));
+      double unit = 0, rate = 0, chain = 0;
+      for (const LongItem& it : P.long_items) {
+        unit += it.kmax * (it.G <= kUnitMaxW ? 75.0 : (it.G == 16 ? 130.0 : 77.0)) / (warps * kSms);
+        rate += (double)it.nseg * it.kmax * (it.G <= kUnitMaxW ? 15.0 : (it.G == 16 ? 24.0 : 45.0)) / kSms;
+        chain = std::max(chain, 800.0 * it.kmax);
+      }
+      P.long_plain = unit > std::max(rate, chain) ? 0 : P.num_long_unit;
+    }
+    P.chained = P.long_plain == (int32_t)P.longs.size() &&
                 (T == 0 || (nunit == T && P.longs.empty() &&
                             (P.groups.size() == 1 || (P.groups.size() == 2 && P.groups[1].unit_short && T <= kChainTiles))));
     P.num_long_narrow = (int32_t)P.long_order.size();
@@ -1326,6 +1345,7 @@ dg_status validate_plan(const Plan& P) {
     }
     for (char c : in_item)
       if (!c) return bad("long unit BDD in no item");
+    if (P.long_plain != 0 && P.long_plain != P.num_long_unit) return bad("long BDDs of the plain sweeps malformed");
     std::vector<char> listed(P.longs.size(), 0);
     for (size_t i = 0; i < P.long_order.size(); ++i) {
       const int32_t b = P.long_order[i];
@@ -1387,7 +1407,7 @@ dg_status validate_plan(const Plan& P) {
   if (t0 != T) return bad("launch groups do not cover the tiles");
   // a chain launches the kernels of the unit rows alone
   if (P.chained) {
-    if (P.num_long_unit != (int32_t)P.longs.size()) return bad("chained launches with other long BDDs");
+    if (P.long_plain != (int32_t)P.longs.size()) return bad("chained launches with other long BDDs");
     for (const LaunchGroup& g : P.groups)
       if (g.unit_w == 0) return bad("chained launches with mixed tiles");
   }

@@ -228,6 +228,7 @@ struct DevArena {
   int32_t num_long_narrow;  // narrow long BDDs (the head of long_order)
   int32_t num_long_unit;    // ... of them, the unit ones (its very head)
   int32_t num_long_items;
+  int32_t long_plain;       // long_order[long_plain ..): plain sweeps by kernels_long.cu (num_long_unit, or 0: all)
   int32_t long_wide_block;  // whether the wide long BDDs are swept by a block each, or a warp
   int32_t long_wide_smem;   // shared memory of the largest wide long BDD's path costs (0: they stay in long_d, long_t)
   int32_t long_unit_smem[2];  // shared memory of the largest work item, mode 0 and 1
@@ -315,6 +316,7 @@ struct Plan {
   std::vector<LongItem> long_items;
   int32_t long_unit_smem[2] = {0, 0}, long_unit_adj_smem = 0, long_wide_smem = 0;
   bool long_wide_block = false;
+  int32_t long_plain = 0;  // see DevArena
   int32_t long_lanes = 0;           // dg_options::long_lanes (0: chosen at bind)
   std::vector<int64_t> long_rank_ptr;  // per long BDD, first entry of long_lo / long_hi
   std::vector<int32_t> long_lo, long_hi;  // child ranks as in lo8 / hi8 (-2 bottom, -1 top)

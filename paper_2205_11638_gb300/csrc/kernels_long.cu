@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(128) k_long_narrow(DevArena A, SweepArgs a) {
   constexpr bool FWD = KIND == kFwd;
   const int lane = threadIdx.x & 31;
   const int G = A.long_lanes;
-  const int first = A.num_long_unit + (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (kWarp / G);
+  const int first = A.long_plain + (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (kWarp / G);
   if (first >= A.num_long_narrow) return;  // whole warp leaves
   Seg g;
   g.s = lane & (G - 1);
@@ -941,6 +941,7 @@ template <int KIND, int MODE>
 void launch_long_mode(const DevArena& A, const SweepArgs& a, cudaStream_t st) {
   int first = A.num_long_unit;  // the unit ones: kernels_long_unit.cu
   if constexpr (KIND == kFwd || KIND == kBwd) {
+    first = A.long_plain;
     if (A.num_long_narrow > first) {
       const int warps = (A.num_long_narrow - first + kWarp / A.long_lanes - 1) / (kWarp / A.long_lanes);
       k_long_narrow<KIND, MODE><<<long_grid(warps), kLongWarps * kWarp, 0, st>>>(A, a);
@@ -968,7 +969,7 @@ void launch_adjoint_mode(const DevArena& A, const AdjArgs& a, cudaStream_t st) {
 }  // namespace
 
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st) {
-  if (A.num_long == A.num_long_unit) return;
+  if (A.num_long == (kind == kFwd || kind == kBwd ? A.long_plain : A.num_long_unit)) return;
   switch (kind) {
     case kFwd: launch_long_kind<kFwd>(A, a, st); break;
     case kBwd: launch_long_kind<kBwd>(A, a, st); break;

@@ -299,9 +299,9 @@ __global__ void k_gather_var(DevArena A, const float* __restrict__ v, float* out
 }
 
 // The slots whose averaging term the sweeps read per slot: the mixed tiles',
-// and the long BDDs' unless all of them are unit rows.
+// and the long BDDs' unless all of them sweep as unit rows.
 static int scatter_to(const DevArena& A) {
-  return A.num_long == A.num_long_unit ? A.long_slot_base : (int)A.num_slots;
+  return A.num_long == A.long_plain ? A.long_slot_base : (int)A.num_slots;
 }
 
 void launch_slot_inputs(const DevArena& A, const float* x, const float* sd_in, float* out_var, const float* S_var,

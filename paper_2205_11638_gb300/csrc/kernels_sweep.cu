@@ -428,7 +428,7 @@ static void launch_groups(const DevArena& A, const SweepArgs& a, int threads, co
     // the long BDDs first: their launch is a few warps walking long chains
     ch.linked = false;
     launch_long_sweep(KIND, A, a, fork ? ss.of(A.long_stream) : ss.main);
-    if (A.num_long_items > 0) {
+    if (A.num_long_items > 0 && !((KIND == kFwd || KIND == kBwd) && A.long_plain == 0)) {
       // side by side with the other long BDDs' walks
       Chain own;
       own.ss.main = fork ? ss.of(A.long_stream + (A.num_long > A.num_long_unit ? 1 : 0)) : ss.main;

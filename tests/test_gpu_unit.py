@@ -346,6 +346,43 @@ def _many_small_shapes(seed, n=60):
     return workloads.single_rows_problem(rows, n, rng.normal(size=n))
 
 
+def _many_long_wide_rows(seed, num=1700, n=3000):
+    """Rows "sum of k = 30", k = 990 to 1000: 31 states a level, so long and so
+    many that their plain sweeps run in the general kernels (the other calls do
+    not), and a few of another kind and short ones next to them."""
+    rng = np.random.default_rng(seed)
+    kinds = [(int(k), workloads.EQ, 30) for k in rng.integers(990, 1001, size=num)]
+    kinds += [(300, workloads.LE, 1)] * 8 + [(3, workloads.GE, 1)] * 40
+    rows = [(f + np.arange(k), np.ones(k, np.int64), s, b) for (k, s, b), f in
+            zip(kinds, rng.integers(0, n - 1000, size=len(kinds)))]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_long_unit_rows_swept_by_the_general_kernels(mode):
+    """Plain sweeps against recording ones and against the doubled problem, bit
+    for bit, with bounds and sweeps by hand in between."""
+    p = _many_long_wide_rows(24)
+    out = []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q).bind()
+        X.plan.validate()
+        lam, M, om, al = [X.from_csr(x) for x in _vectors(p, 20)]
+        par = (om, al) if mode else (None, None)
+        l2, M2 = lam.clone(), M.clone()
+        X.iterate_checkpointed(l2, M2, *par, iters=2, ckpt_every=1)
+        lb = X.iterate(lam, M, *par, iters=2, lb=True)
+        assert torch.equal(lam, l2) and torch.equal(M, M2)
+        X.sum_M(M, alpha=par[1])
+        X.sweep(lam, M, forward=True, omega=par[0], alpha=par[1], costs_out=True)
+        X.sum_M(M, alpha=par[1])
+        X.sweep(lam, M, forward=False, omega=par[0], alpha=par[1], costs_in=True, energy=True)
+        lb2 = X.lower_bound(lam, M)
+        out.append((X.to_csr(lam), X.to_csr(M), lb, lb2))
+    for a, b in zip(*out):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("seed", [21, 22, 23])
 def test_small_arena_of_many_shapes(seed, mode):
