@@ -397,7 +397,8 @@ dg_status dg_autotune(dg_arena* arena, void* stream, float* lam, float* M, int32
  * DG_ECUDA if the stream reports an error. */
 dg_status dg_wait(void* stream, int32_t timeout_ms);
 
-/* Number of kernel launches one dg_iterate call with these arguments issues. */
+/* Number of kernel launches one dg_iterate call with these arguments issues
+ * (a few tiles of +-1 rows iterate in a single one). */
 int32_t dg_iterate_launches(const dg_arena* arena, int32_t iters, int32_t want_lb, const dg_options* opts);
 
 #ifdef __cplusplus

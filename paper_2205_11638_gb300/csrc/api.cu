@@ -608,11 +608,15 @@ dg_status dg_wait(void* stream, int32_t timeout_ms) {
 }
 
 int32_t dg_iterate_launches(const dg_arena* ar, int32_t iters, int32_t want_lb, const dg_options* opts) {
-  (void)opts;
-  const int32_t g = ar ? (int32_t)ar->groups.size() + (ar->dev.num_long > 0 ? 1 : 0) : 1;
-  int32_t l = 1 + iters * (2 * g + 2);
-  if (want_lb) l += 2 + (iters == 0 ? g : 0);
-  return l;
+  if (!ar) return 1 + 4 * iters + (want_lb ? 2 + (iters == 0) : 0);  // of one launch group
+  const DevArena& A = ar->dev;
+  const int32_t lb = want_lb ? (A.num_lb_chunks > 0) + 1 : 0;
+  if (iters > 0 && !(opts && opts->renorm_every > 0) &&
+      small_arena(A, ar->groups.data(), (int)ar->groups.size(), ar->cta_smem_cap))
+    return 1 + lb;
+  const int32_t g = (int32_t)ar->groups.size(), s = A.n > 0;  // a reduction
+  return s + iters * 2 * (g + long_sweep_kernels(A, true) + s) + lb +
+         (want_lb && iters == 0 ? g + long_sweep_kernels(A, false) : 0);
 }
 
 dg_status dg_sum_M(dg_arena* ar, void* stream, const float* M, float* lam, const float* alpha, int32_t mode,

@@ -126,6 +126,7 @@ void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGr
 // set cover 24 x 16, work 2,000 3.6 / 8.3; independent set of 400 nodes, 6,800
 // 6.1 / 8.4; tracking 3 x 40 per slot, about 20,000 12.3 / 11.2).
 constexpr int64_t kSmallWork = 10000;
+bool small_arena(const DevArena& A, const LaunchGroup* groups, int num_groups, size_t smem_cap);
 bool launch_small_iterate(const DevArena& A, const SweepArgs& a, const LaunchGroup* groups, int num_groups, int iters,
                           size_t smem_cap, Chain& ch);
 void launch_unit_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, const LaunchGroup& G,
@@ -221,6 +222,8 @@ cudaError_t set_long_unit_smem_limit(size_t bytes);
 void launch_long_unit(int kind, const DevArena& A, const SweepArgs& a, Chain& ch);
 void launch_long_unit_adjoint(bool forward, const DevArena& A, const AdjArgs& a, Chain& ch);
 void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStream_t st);
+// Kernels of one sweep over the long BDDs (those of the unit rows included).
+int long_sweep_kernels(const DevArena& A, bool plain);
 void launch_long_smoothed(const DevArena& A, const float* lam, float a_s, float* E_a, float* marg, cudaStream_t st);
 void launch_long_adjoint(bool forward, const DevArena& A, const AdjArgs& a, cudaStream_t st);
 

@@ -982,6 +982,15 @@ void launch_long_sweep(int kind, const DevArena& A, const SweepArgs& a, cudaStre
   }
 }
 
+int long_sweep_kernels(const DevArena& A, bool plain) {
+  const int first = plain ? A.long_plain : A.num_long_unit;
+  const int narrow = A.num_long_narrow > first, wide = A.num_long > A.num_long_narrow;
+  // (a warp each, the narrow and the wide ones are one launch unless the narrow
+  // ones pack several to a warp)
+  const int general = plain || A.long_wide_block ? narrow + wide : (narrow || wide);
+  return general + (A.num_long_items > 0 && !(plain && A.long_plain == 0));
+}
+
 cudaError_t set_long_smem_limit(size_t bytes) {
   const int b = (int)bytes;
   constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;

@@ -930,20 +930,34 @@ void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGr
   }
 }
 
+namespace {
+// lambda, M and the per-variable sums, and a warp's slice, in shared memory
+size_t small_fixed(const DevArena& A) { return ((size_t)(2 * A.num_slots + A.n) * 4 + 127) / 128 * 128; }
+size_t small_region(const LaunchGroup* groups, int num_groups, int mode) {
+  size_t region = 0;
+  for (int g = 0; g < num_groups; ++g)
+    region = std::max(region, (size_t)(mode == 1 ? groups[g].unit_bytes1 : groups[g].unit_bytes0));
+  return region;
+}
+int small_warps(const DevArena& A, size_t region, size_t smem_cap) {
+  return (int)std::min<size_t>(std::min(32, A.num_tiles), (smem_cap - small_fixed(A)) / region);
+}
+}  // namespace
+
+bool small_arena(const DevArena& A, const LaunchGroup* groups, int num_groups, size_t smem_cap) {
+  if (A.unit_slots != A.num_slots || A.num_long > 0 || A.num_tiles < 1) return false;
+  int64_t work = 0;
+  for (int g = 0; g < num_groups; ++g) work += groups[g].work;
+  if (work > kSmallWork) return false;
+  const size_t region = small_region(groups, num_groups, 1);  // whatever the mode: the larger
+  return small_fixed(A) + region <= smem_cap && small_warps(A, region, smem_cap) >= std::min(8, A.num_tiles);
+}
+
 bool launch_small_iterate(const DevArena& A, const SweepArgs& a, const LaunchGroup* groups, int num_groups, int iters,
                           size_t smem_cap, Chain& ch) {
-  if (A.unit_slots != A.num_slots || A.num_long > 0 || A.num_tiles < 1) return false;
-  size_t region = 0;
-  int64_t work = 0;
-  for (int g = 0; g < num_groups; ++g) {
-    region = std::max(region, (size_t)(a.mode == 1 ? groups[g].unit_bytes1 : groups[g].unit_bytes0));
-    work += groups[g].work;
-  }
-  if (work > kSmallWork) return false;
-  const size_t fixed = ((size_t)(2 * A.num_slots + A.n) * 4 + 127) / 128 * 128;
-  if (fixed + region > smem_cap) return false;
-  const int warps = (int)std::min<size_t>(std::min(32, A.num_tiles), (smem_cap - fixed) / region);
-  if (warps < std::min(8, A.num_tiles)) return false;
+  if (!small_arena(A, groups, num_groups, smem_cap)) return false;
+  const size_t region = small_region(groups, num_groups, a.mode), fixed = small_fixed(A);
+  const int warps = small_warps(A, region, smem_cap);
   // threads beyond the tiles' warps help the reduction
   const int threads = std::max(warps, std::min<int>(32, (A.n + 31) / 32)) * kWarp;
   const int blocks_warps = threads / kWarp;
