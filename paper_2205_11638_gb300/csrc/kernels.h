@@ -121,10 +121,12 @@ void launch_unit(int kind, const DevArena& A, const SweepArgs& a, const LaunchGr
 // nothing launched, when the arena is not of that kind.
 //
 // The line: kSmallWork, the groups' estimated work (levels times a level's
-// cost, 14 W + 40).  One block's iteration costs about 2 us plus 0.6 us per
-// 1,000 of it, the chain of launches 8 us (us per iteration, one block / chain:
-// set cover 24 x 16, work 2,000 3.6 / 8.3; independent set of 400 nodes, 6,800
-// 6.1 / 8.4; tracking 3 x 40 per slot, about 20,000 12.3 / 11.2).
+// cost, 14 W + 40) plus 1.2 per variable.  One block's iteration costs about
+// 2 us plus 0.6 us per 1,000 of it, the chain of launches 7 us whatever the
+// variables (us per iteration, one block / chain: set cover 24 x 16, work 2,000
+// 3.6 / 8.3; independent set of 400 nodes, 7,300 5.9 / 7.4; tracking 3 x 40 per
+// slot, about 20,000 12.3 / 11.2; 20 rows over 2,000 variables 3.1 / 7.1, over
+// 8,000 7.4 / 7.2, over 32,000 31.5 / 7.2).
 constexpr int64_t kSmallWork = 10000;
 bool small_arena(const DevArena& A, const LaunchGroup* groups, int num_groups, size_t smem_cap);
 bool launch_small_iterate(const DevArena& A, const SweepArgs& a, const LaunchGroup* groups, int num_groups, int iters,

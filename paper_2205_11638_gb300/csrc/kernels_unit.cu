@@ -946,7 +946,7 @@ int small_warps(const DevArena& A, size_t region, size_t smem_cap) {
 
 bool small_arena(const DevArena& A, const LaunchGroup* groups, int num_groups, size_t smem_cap) {
   if (A.unit_slots != A.num_slots || A.num_long > 0 || A.num_tiles < 1) return false;
-  int64_t work = 0;
+  int64_t work = (int64_t)A.n + A.n / 5;
   for (int g = 0; g < num_groups; ++g) work += groups[g].work;
   if (work > kSmallWork) return false;
   const size_t region = small_region(groups, num_groups, 1);  // whatever the mode: the larger

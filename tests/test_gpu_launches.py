@@ -75,3 +75,13 @@ def test_launch_count(name, mode):
                                           _ptr(al), mode, iters, _ptr(lb) if want else None, ctypes.byref(o)) == 0
                 told = lib.dg_iterate_launches(A._h, iters, int(want), ctypes.byref(o))
                 assert told == _kernels(stream, call), (renorm, iters, want)
+
+
+@pytest.mark.parametrize("n,launches", [(100, 1), (4000, 1), (8300, 9), (32000, 9)])
+def test_one_launch_while_the_variables_are_few(n, launches):
+    """A few rows over many variables: one block would spend its time summing
+    over variables, so that from some 8,000 on the launches are separate."""
+    rng = np.random.default_rng(n)
+    rows = [(np.sort(rng.choice(n, size=3, replace=False)), np.ones(3, np.int64), workloads.GE, 1) for _ in range(20)]
+    A = solver.plan(workloads.single_rows_problem(rows, n, rng.normal(size=n))).bind()
+    assert A.iterate_launches(2) == launches
