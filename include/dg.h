@@ -78,7 +78,9 @@ typedef struct dg_options {
   int32_t tile_nodes;    /* reserved (tiles hold 32 BDDs, one per lane) */
   int32_t tile_slots;    /* reserved */
   int32_t block_threads; /* threads per CTA of the sweep kernels: 32, 64, 96 or
-                            128 (one tile per warp; default 128) */
+                            128 (one tile per warp; default 128).  Not used by
+                            the kernels of short tiles of +-1 rows and of whole
+                            iterations of a small arena */
   int32_t renorm_every;  /* FP64 re-projection of lambda onto sum_j(lambda+M)=c
                             every k iterations (0 = never) */
   float omega;           /* damping of mode 0 (default 0.5 when 0) */
@@ -90,13 +92,16 @@ typedef struct dg_options {
                             into tiles (default 16384) */
   int32_t group_ratio_pct; /* a launch group keeps tiles whose shared-memory
                               footprint is at least this percent of its largest
-                              (default 85) */
+                              (default 85), and smaller ones while its tiles do
+                              not fill the chip */
   int32_t long_lanes;    /* lanes given to each long BDD whose levels have at
                             most 32 nodes in the plain sweeps: 1, 2, 4, 8, 16
                             or 32, raised to the widest such level's power of
                             two (default: chosen by dg_bind, at least four
-                            warps per SM); any other value fails dg_plan with
-                            DG_EINVAL */
+                            warps per SM).  Long rows of +1 and -1: 32 over
+                            this many BDDs to a warp in every sweep, fewer where
+                            shared memory asks for it.  Any other value fails
+                            dg_plan with DG_EINVAL */
   int32_t reserved[4];
 } dg_options;
 

@@ -909,9 +909,11 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       // BDDs per warp: as many as lanes allow while that leaves at least four
       // warps per SM (a warp's levels are a chain of dependent steps, which
       // other warps hide), and as fit shared memory
-      int nseg = G <= kUnitMaxW ? kWarp : kWarp / G;
-      while (nseg > 1 && ((int64_t)(e - i) < 4LL * kSms * nseg || long_unit_bytes(nseg, G, kmax, 1) > 64 * 1024 ||
-                          long_unit_adjoint_bytes(nseg, kmax) > 64 * 1024))
+      // (or as many as dg_options::long_lanes asks for)
+      const int lanes = opts ? opts->long_lanes : 0;
+      int nseg = std::min(G <= kUnitMaxW ? kWarp : kWarp / G, lanes > 0 ? kWarp / lanes : kWarp);
+      while (nseg > 1 && ((lanes == 0 && (int64_t)(e - i) < 4LL * kSms * nseg) ||
+                          long_unit_bytes(nseg, G, kmax, 1) > 64 * 1024 || long_unit_adjoint_bytes(nseg, kmax) > 64 * 1024))
         nseg /= 2;
       const int32_t run_base = (int32_t)P.unit_runs.size();
       for (int h = 0; h < U.s.k; ++h)

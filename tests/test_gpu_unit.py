@@ -397,3 +397,43 @@ def test_small_arena_of_many_shapes(seed, mode):
             assert X.plan.sizes.num_tiles > 32
     for a, b in zip(*out):
         assert torch.equal(a, b) and torch.isfinite(a).all()
+
+
+def _lanes_rows(seed, n=400):
+    """Long rows of several lengths of four kinds: two, six, 13 and 31 states."""
+    rng = np.random.default_rng(seed)
+    rows = []
+    for b, lo, hi, num in ((1, 128, 170, 70), (5, 60, 80, 45), (12, 40, 60, 45), (30, 61, 75, 9)):
+        rows += [(np.sort(rng.choice(n, size=int(k), replace=False)), np.ones(int(k), np.int64), workloads.EQ, b)
+                 for k in rng.integers(lo, hi, size=num)]
+    return workloads.single_rows_problem(rows, n, rng.normal(size=n))
+
+
+@pytest.mark.parametrize("lanes", [1, 2, 8, 32])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_long_unit_rows_at_any_packing(lanes, mode):
+    """32 / lanes BDDs of unequal lengths to a warp (at most one per G lanes
+    above eight states): all calls bit for bit, gradients up to the rounding of
+    sums (tolerance as above, 4 sweeps)."""
+    p = _lanes_rows(25)
+    exact, grads = [], []
+    for q in (p, _doubled(p)):
+        X = solver.plan(q, long_lanes=lanes).bind()
+        X.plan.validate()
+        assert X.plan.sizes.num_tiles == 0
+        lam, M, om, al = [X.from_csr(x) for x in _vectors(p, 26)]
+        par = (om, al) if mode else (None, None)
+        grads.append([X.to_csr(x) for x in X.backward(lam, M, *par, 2, 1, *[X.from_csr(x) for x in _vectors(p, 27)[:2]])])
+        l2, M2 = lam.clone(), M.clone()
+        X.iterate_checkpointed(l2, M2, *par, iters=3, ckpt_every=3)
+        m0, m1 = X.min_marginals(lam)
+        lb0, E = X.lower_bound(lam, M, energies=True)
+        gl, gM = X.lb_seed(lam, M)
+        lb = X.iterate(lam, M, *par, iters=3, lb=True)
+        assert torch.equal(lam, l2) and torch.equal(M, M2)
+        exact.append([X.to_csr(x) for x in (lam, M, m0, m1, gl, gM)] + [lb0, E, lb])
+    for a, b in zip(*exact):
+        assert torch.equal(a, b) and torch.isfinite(a).all()
+    for a, b in zip(*grads):
+        assert torch.isfinite(a).all()
+        assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
