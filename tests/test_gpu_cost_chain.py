@@ -195,3 +195,26 @@ def test_graph_replay_counts_as_a_call_on_the_arena():
     A.sweep(lam, M, forward=False)
     torch.cuda.synchronize()
     assert torch.isfinite(lam).all()
+
+
+@pytest.mark.parametrize("name", ["matching", "tracking_40x400"])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_handed_on_costs_bit_identical_on_general_rows(name, mode):
+    """The same with coefficients and right-hand sides doubled: rows of +1 and -1
+    recompute the costs whether they are handed on or not, these read them."""
+    prob = CASES[name]()
+    prob = dict(prob, coef=(2 * prob["coef"]).astype(np.int32), rhs=(2 * prob["rhs"]).astype(np.int32))
+    A = solver.plan(prob).bind()
+    om, al = _mode1(prob, A) if mode else (None, None)
+    lam0, M0 = A.init_lambda()
+    outs = []
+    for how in ("iterate", "handoff", "recompute"):
+        lam, M = lam0.clone(), M0.clone()
+        if how == "iterate":
+            A.iterate(lam, M, om, al, iters=6)
+        else:
+            _manual(A, lam, M, 6, om, al, handoff=how == "handoff")
+        assert torch.isfinite(lam).all() and torch.isfinite(M).all()
+        outs.append((lam, M))
+    for lam, M in outs[1:]:
+        assert torch.equal(lam, outs[0][0]) and torch.equal(M, outs[0][1])

@@ -241,3 +241,29 @@ def test_wide_bdds_by_any_team(num, terms, top, rhs, per_slot):
     for a, b in zip(*grads):
         assert torch.isfinite(a).all()
         assert (a - b).abs().max() <= (400 + 100) * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
+
+
+@pytest.mark.parametrize("per_slot", [False, True])
+@pytest.mark.parametrize("lanes", [0, 2, 8])
+def test_general_narrow_rows_plain_sweeps_equal_recording_sweeps(lanes, per_slot):
+    """The assignment rows with coefficients and right-hand sides doubled: the
+    same BDDs, but no unit rows, so that the plain sweeps run in k_long_narrow
+    (one BDD of two states a level to a warp, 16, or 4, of different lengths)
+    and the recording ones in the general level loop: bit for bit, and the same
+    as the unit rows' kernels."""
+    prob = workloads.assignment(L=120, R=300, cand=280, seed=22)
+    twice = dict(prob, coef=(2 * prob["coef"]).astype(np.int32), rhs=(2 * prob["rhs"]).astype(np.int32))
+    rng = np.random.default_rng(5)
+    al_c, om_c = _softmax_alpha(prob["col"], prob["n"], rng), rng.uniform(0.2, 0.8, size=len(prob["col"]))
+    out = []
+    for p in (twice, prob):
+        A = solver.plan(p, long_lanes=lanes).bind()
+        om, al = (A.from_csr(om_c), A.from_csr(al_c)) if per_slot else (None, None)
+        lam0, M0 = A.init_lambda()
+        l1, m1, l2, m2 = lam0.clone(), M0.clone(), lam0.clone(), M0.clone()
+        lb1 = A.iterate(l1, m1, om, al, iters=6, lb=True)
+        _, lb2 = A.iterate_checkpointed(l2, m2, om, al, iters=6, ckpt_every=6, lb=True)
+        assert torch.equal(l1, l2) and torch.equal(m1, m2) and torch.equal(lb1, lb2)
+        out.append((A.to_csr(l1), A.to_csr(m1), lb1))
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
