@@ -89,7 +89,8 @@ typedef struct dg_options {
                             image (0 = none); exceeding it fails with
                             DG_ENOMEM before the image is allocated */
   int32_t chunk_rows;    /* rows per locality chunk before BDDs are sorted
-                            into tiles (default 16384) */
+                            into tiles (default 16384, which is also the least
+                            for rows of +1 and -1) */
   int32_t group_ratio_pct; /* a launch group keeps tiles whose shared-memory
                               footprint is at least this percent of its largest
                               (default 85), and smaller ones while its tiles do

@@ -479,16 +479,18 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
 
   // ---- 2. tiles: 32 BDDs per tile, one per lane ---------------------------
   // Rows are cut into chunks of consecutive rows (so that a tile's variables,
-  // and the S values its lanes gather, stay close together).  Inside a chunk
-  // the unit rows of one shape fill tiles of their own (row order), the other
-  // rows are sorted by hop count and node count, longest first, and every 32
-  // consecutive ones form a tile.  Inside a tile everything is interleaved by
+  // and the S values its lanes gather, stay close together).  The unit rows of
+  // one shape fill tiles of their own, in row order whatever the chunk; theirs
+  // is kUnitChunk rows at least, since every chunk leaves a tile per shape partly
+  // filled.  The other rows are sorted by hop count and node count inside a
+  // chunk, longest first, and every 32 consecutive ones form a tile.  Inside a tile everything is interleaved by
   // lane: slot (h, b) is slot_base + 32 h + b and node number n of lane b is
   // element 32 n + b of the per-tile arrays.  Node numbers 0 and 1 stand for
   // the top and bottom terminals, the BDD's own nodes are numbered 2, 3, ...
   // level by level; child codes are node numbers (8 bits).
   // Rows of the long BDDs take no tile (they are laid out after the tiles).
-  const int64_t kChunkRows = opts && opts->chunk_rows > 0 ? opts->chunk_rows : 16384;
+  constexpr int64_t kUnitChunk = 16384;
+  const int64_t kChunkRows = opts && opts->chunk_rows > 0 ? opts->chunk_rows : kUnitChunk;
   struct TileSrc {
     int64_t first;  // its rows: order[first .. first + count)
     int count, unit;
@@ -505,10 +507,10 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     std::vector<std::pair<int32_t, int64_t>> by_shape;
     std::vector<int64_t> mixed;
     std::vector<TileSrc> part;
-    for (int64_t c0 = 0; c0 < m; c0 += kChunkRows) {
-      const int64_t c1 = std::min(m, c0 + kChunkRows);
+    const int64_t step = std::max(kChunkRows, kUnitChunk);
+    for (int64_t c0 = 0; c0 < m; c0 += step) {
+      const int64_t c1 = std::min(m, c0 + step);
       by_shape.clear();
-      mixed.clear();
       part.clear();
       for (int64_t j = c0; j < c1; ++j) {
         if (P.long_of_row[j] >= 0) continue;
@@ -539,17 +541,18 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
         for (int64_t y = t.first; y < t.first + t.count; ++y)
           (own ? order : mixed).push_back(by_shape[y].second);
       }
-      std::stable_sort(mixed.begin(), mixed.end(), [&](int64_t x, int64_t y) {
-        const int64_t kx = R->row_ptr[x + 1] - R->row_ptr[x], ky = R->row_ptr[y + 1] - R->row_ptr[y];
-        if (kx != ky) return kx > ky;
-        const int64_t nx = P.node_ptr[x + 1] - P.node_ptr[x], ny = P.node_ptr[y + 1] - P.node_ptr[y];
-        return nx != ny ? nx > ny : x < y;
-      });
-      for (size_t x = 0; x < mixed.size(); x += kWarp) {
-        const size_t e = std::min(mixed.size(), x + kWarp);
-        src.push_back({(int64_t)order.size(), (int)(e - x), -1});
-        order.insert(order.end(), mixed.begin() + x, mixed.begin() + e);
-      }
+    }
+    std::sort(mixed.begin(), mixed.end(), [&](int64_t x, int64_t y) {
+      if (x / kChunkRows != y / kChunkRows) return x < y;
+      const int64_t kx = R->row_ptr[x + 1] - R->row_ptr[x], ky = R->row_ptr[y + 1] - R->row_ptr[y];
+      if (kx != ky) return kx > ky;
+      const int64_t nx = P.node_ptr[x + 1] - P.node_ptr[x], ny = P.node_ptr[y + 1] - P.node_ptr[y];
+      return nx != ny ? nx > ny : x < y;
+    });
+    for (size_t x = 0; x < mixed.size(); x += kWarp) {
+      const size_t e = std::min(mixed.size(), x + kWarp);
+      src.push_back({(int64_t)order.size(), (int)(e - x), -1});
+      order.insert(order.end(), mixed.begin() + x, mixed.begin() + e);
     }
   }
   int max_hops = 0, max_width = 0;

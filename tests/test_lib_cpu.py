@@ -280,3 +280,27 @@ def test_plan_is_deterministic():
     for j in (0, 7, len(rows["row_ptr"]) - 2):
         for a, b in zip(P1.bdd(j), P2.bdd(j)):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("chunk", [1, 8, 64, 512, 16384, 32768])
+@pytest.mark.parametrize("double", [False, True])
+def test_small_locality_chunks_do_not_inflate_the_arena(chunk, double):
+    """chunk_rows orders rows, it does not cut tiles short: whatever its value,
+    padding adds at most one tile of the longest rows per shape (rows of +1 and
+    -1, 64 shapes at most left partly filled per 16,384 rows), or the difference of
+    the lengths sorted next to each other (the others: at most twice the longest
+    over the mean)."""
+    rows = workloads.tracking(frames=20, dets=300)
+    if double:
+        rows = dict(rows, coef=(2 * rows["coef"]).astype(np.int32), rhs=(2 * rows["rhs"]).astype(np.int32))
+    P = solver.plan(rows, chunk_rows=chunk)
+    P.validate()
+    k = np.diff(rows["row_ptr"])
+    real, m = int(P.sizes.num_lambda), len(k)
+    if double:
+        assert P.sizes.num_tiles == -(-m // 32)
+        assert P.sizes.num_slots <= real * 2 * k.max() / k.mean()
+    else:
+        chunks = -(-m // max(chunk, 16384))
+        assert P.sizes.num_slots <= 1.25 * real + chunks * 64 * 32 * k.max()
+        assert P.sizes.num_tiles <= 1.25 * m / 32 + chunks * 64
