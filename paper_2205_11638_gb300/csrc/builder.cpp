@@ -702,8 +702,11 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     // ... or any smaller one while the group's tiles do not fill the chip (its
     // smaller tiles then cost it no occupancy and save a launch)
     constexpr size_t kSmSmem = 224 * 1024;
+    // ... but no tile that would keep the group's recording sweeps from fitting a
+    // CTA: these take the largest footprint and the largest records together
+    constexpr size_t kCtaSmem = 227 * 1024;
     int32_t t0 = 0;
-    size_t gmax = 0;
+    size_t gmax = 0, rec_max = 0, meta_max = 0;
     auto group_smem = [&](int t) {
       const Tile& tl = P.tiles[t];
       return tl.unit ? unit_smem_bytes(P.unit_shapes[tl.unit - 1], 1)
@@ -732,7 +735,14 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       const bool full = gmax > 0 && (size_t)(t - t0) >= kSms * std::min<size_t>(64, kSmSmem / gmax);
       // (short unit tiles need no shared memory: one group whatever their size)
       const int kind = t < T ? group_kind(t) : 3, kind0 = t > t0 ? group_kind(t0) : kind;
-      const bool cut = kind != kind0 || (kind != 1 && full && !one_launch && (double)r < kGroupRatio * (double)gmax);
+      size_t rec = 0, meta = 0;
+      if (kind == 2) {
+        const Tile& tl = P.tiles[t];
+        rec = std::max(r, sweep_smem_bytes_bwd(tl.nmax, tl.nhops, 1));
+        meta = (size_t)(tl.nmax - 2) * kWarp * 2;
+      }
+      const bool cut = kind != kind0 || (kind != 1 && full && !one_launch && (double)r < kGroupRatio * (double)gmax) ||
+                       (std::max(rec, rec_max) + std::max(meta, meta_max) > kCtaSmem && rec + meta <= kCtaSmem);
       if (t == T || (t > t0 && cut)) {
         if (t > t0) {
           LaunchGroup g{};
@@ -741,9 +751,11 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
           P.groups.push_back(g);
         }
         t0 = t;
-        gmax = 0;
+        gmax = rec_max = meta_max = 0;
       }
       gmax = std::max(gmax, r);
+      rec_max = std::max(rec_max, rec);
+      meta_max = std::max(meta_max, meta);
     }
     for (LaunchGroup& g : P.groups)
       for (int t = g.tile0; t < g.tile1; ++t) {

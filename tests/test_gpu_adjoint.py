@@ -346,3 +346,22 @@ def test_forward_and_adjoint_replay_from_a_cuda_graph():
     torch.cuda.synchronize()
     for a, b in zip(eager, outs):
         assert torch.equal(a, b)
+
+
+def test_tiles_of_many_levels_next_to_tiles_of_many_nodes():
+    """Rows of 241 levels of one node and rows of 54 levels and 254 nodes, each
+    recordable by itself: their launch groups have to be too (the largest
+    footprint and the largest records of a group's tiles count together).  Equal
+    to plain iterations bit for bit."""
+    rows = [(np.arange(241), 2 * np.ones(241, np.int64), workloads.LE, 2 * 241)] * 32
+    rows += [(j + np.arange(54), 2 * np.ones(54, np.int64), workloads.LE, 8) for j in range(32)]
+    A = solver.plan(workloads.single_rows_problem(rows, 241, np.linspace(-1, 1, 241))).bind()
+    lam, M = A.init_lambda()
+    l2, M2 = lam.clone(), M.clone()
+    one = torch.full_like(lam, 0.5) * A.real
+    for par in ((None, None), (one, one / 64)):
+        A.iterate(lam, M, *par, iters=2)
+        w, _ = A.iterate_checkpointed(l2, M2, *par, iters=2, ckpt_every=2)
+        assert torch.equal(lam, l2) and torch.equal(M, M2)
+        for g in A.backward_checkpointed(*par, 2, 2, one, one, w):
+            assert torch.isfinite(g).all()
