@@ -1312,6 +1312,13 @@ dg_status validate_plan(const Plan& P) {
       return bad("long BDD order malformed");
     if (P.long_lanes < 0 || P.long_lanes > kWarp || (P.long_lanes & (P.long_lanes - 1)) != 0)
       return bad("lanes per narrow long BDD not a power of two up to 32");
+    std::vector<char> listed(P.longs.size(), 0);
+    for (size_t i = 0; i < P.long_order.size(); ++i) {
+      const int32_t b = P.long_order[i];
+      if (b < 0 || b >= (int32_t)P.longs.size() || listed[b]++) return bad("long BDD order not a permutation");
+      if ((P.longs[b].maxw <= kWarp) != ((int32_t)i < P.num_long_narrow))
+        return bad("long BDD order: narrow and wide BDDs mixed");
+    }
     // the unit ones: every item's BDDs have its shape, state for node
     if (P.num_long_unit < 0 || P.num_long_unit > P.num_long_narrow) return bad("long unit BDDs not narrow");
     std::vector<char> in_item(P.num_long_unit, 0);
@@ -1363,13 +1370,6 @@ dg_status validate_plan(const Plan& P) {
     for (char c : in_item)
       if (!c) return bad("long unit BDD in no item");
     if (P.long_plain != 0 && P.long_plain != P.num_long_unit) return bad("long BDDs of the plain sweeps malformed");
-    std::vector<char> listed(P.longs.size(), 0);
-    for (size_t i = 0; i < P.long_order.size(); ++i) {
-      const int32_t b = P.long_order[i];
-      if (b < 0 || b >= (int32_t)P.longs.size() || listed[b]++) return bad("long BDD order not a permutation");
-      if ((P.longs[b].maxw <= kWarp) != ((int32_t)i < P.num_long_narrow))
-        return bad("long BDD order: narrow and wide BDDs mixed");
-    }
   }
   if (real_slots != NL || real_nodes != P.sizes.num_nodes) return bad("slot or node count mismatch");
   // variables: CSR and ELL columns point back at their own slots, rows ascending

@@ -304,3 +304,21 @@ def test_small_locality_chunks_do_not_inflate_the_arena(chunk, double):
         chunks = -(-m // max(chunk, 16384))
         assert P.sizes.num_slots <= 1.25 * real + chunks * 64 * 32 * k.max()
         assert P.sizes.num_tiles <= 1.25 * m / 32 + chunks * 64
+
+
+def test_validator_catches_each_corruption_of_long_rows(tmp_path):
+    """As above on a plan with long rows: every number the kernels of the long
+    rows index with is checked before the validator itself uses it."""
+    from paper_2205_11638_gb300 import build as B
+    csrc = os.path.join(ROOT, "paper_2205_11638_gb300", "csrc")
+    exe = tmp_path / "validate_long_harness"
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-pthread", f"-I{os.path.join(B.CUDA_HOME, 'include')}",
+                           f"-I{os.path.join(ROOT, 'include')}", f"-I{csrc}",
+                           os.path.join(ROOT, "tests", "validate_long_harness.cpp"),
+                           os.path.join(csrc, "builder.cpp"), "-o", str(exe)])
+    out = subprocess.check_output([str(exe)], text=True).strip().splitlines()
+    res = {ln.split("|")[0]: (int(ln.split("|")[1]), ln.split("|", 2)[2]) for ln in out}
+    assert res.pop("intact") == (0, "")
+    assert len(res) == 11
+    for name, (st, msg) in res.items():
+        assert st == _lib.DG_EINVAL and msg.startswith("dg_plan_validate:"), (name, st, msg)
