@@ -292,7 +292,7 @@ dg_status dg_lb_seed(dg_arena* arena, void* stream, const float* lam, const floa
 /* --- adjoint (Alg. 2) ----------------------------------------------------- */
 
 /* Device workspace dg_backward needs for `iters` iterations with a
- * checkpoint every `ckpt_every` iterations. */
+ * checkpoint every `ckpt_every` iterations (at any alignment). */
 size_t dg_backward_workspace_bytes(const dg_arena* arena, int32_t iters, int32_t ckpt_every);
 
 /* Backpropagation through `iters` iterations of dg_iterate started from

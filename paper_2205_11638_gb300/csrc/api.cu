@@ -837,6 +837,7 @@ void dg_graph_destroy(dg_graph_t* g) {
 
 namespace {
 
+constexpr size_t kWorkspaceAlign = 256;
 struct BwdLayout {
   size_t ck_lam, ck_M, rec_meta, rec_amin, rec_unit, rec_diff, seg_S, w_lam, w_M, sdot, sd_a, sd_b, var_in, slot_in, rec_lmeta,
       rec_lamin, rec_lunit, long_a1, long_a2, total;
@@ -890,8 +891,13 @@ BwdLayout backward_layout(const dg_arena* ar, int iters, int ckpt_every) {
   L.rec_lunit = put((size_t)2 * L.k * L.lunit_stride);
   L.long_a1 = put(lcost * 4);
   L.long_a2 = put(lcost * 4);
-  L.total = o;
+  L.total = o + kWorkspaceAlign - 1;  // wherever the caller's buffer starts
   return L;
+}
+// Where the layout's offsets count from: the recording sweeps and the adjoint
+// move whole 16-byte pieces of it.
+char* workspace_base(void* workspace) {
+  return (char*)(((uintptr_t)workspace + kWorkspaceAlign - 1) / kWorkspaceAlign * kWorkspaceAlign);
 }
 
 // Runs `k` iterations from (lam, M) as recording sweeps: before sweep sw the
@@ -997,7 +1003,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
     if (e != cudaSuccess) return cuda_fail(e, "dg_backward");
     return DG_OK;
   }
-  char* w = (char*)workspace;
+  char* w = workspace_base(workspace);
   float* ck_lam = (float*)(w + L.ck_lam);
   float* ck_M = (float*)(w + L.ck_M);
   char* rec_meta = w + L.rec_meta;
@@ -1172,7 +1178,7 @@ dg_status dg_iterate_checkpointed(dg_arena* ar, void* stream, float* lam, float*
     return fail(DG_EINVAL, "dg_iterate_checkpointed: workspace smaller than dg_backward_workspace_bytes()");
   cudaStream_t st = (cudaStream_t)stream;
   const size_t bNS = (size_t)ar->sizes.num_slots * 4;
-  char* w = (char*)workspace;
+  char* w = workspace_base(workspace);
   Chain ch = chain_for(ar, st);
   for (int c = 0; c < L.nseg; ++c) {
     ch.linked = false;

@@ -365,3 +365,28 @@ def test_tiles_of_many_levels_next_to_tiles_of_many_nodes():
         assert torch.equal(lam, l2) and torch.equal(M, M2)
         for g in A.backward_checkpointed(*par, 2, 2, one, one, w):
             assert torch.isfinite(g).all()
+
+
+@pytest.mark.parametrize("name", ["long_rows_only", "tiles"])
+def test_workspace_at_any_alignment(name):
+    """The workspace is a byte buffer: wherever it starts, the same gradients."""
+    if name == "tiles":
+        prob = workloads.tracking(frames=5, dets=60, seed=4)
+    else:
+        prob = workloads.assignment(L=12, R=300, cand=260, seed=5)
+    A = solver.plan(prob).bind()
+    lam0, M0 = A.init_lambda()
+    g = torch.randn(A.num_slots, device=A.device, generator=torch.Generator(A.device).manual_seed(1)) * A.real
+    need = A.backward_workspace_bytes(4, 2)
+    want = None
+    for offset in (0, 1, 4, 8, 40):
+        buf = torch.empty(need + 64, dtype=torch.uint8, device=A.device)[offset:offset + need]
+        lam, M = lam0.clone(), M0.clone()
+        A.iterate_checkpointed(lam, M, None, None, 4, 2, workspace=buf)
+        got = [*A.backward_checkpointed(None, None, 4, 2, g, g, buf), lam, M]
+        outs = [A.zeros() for _ in range(4)]
+        A.backward_into(lam0, M0, None, None, 4, 2, g, g, outs, workspace=buf)
+        got += outs
+        want = want or got
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
