@@ -423,6 +423,7 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   A.long_plain = P.long_plain;
   for (int mode = 0; mode < 2; ++mode) A.long_unit_smem[mode] = P.long_unit_smem[mode];
   A.long_unit_adj_smem = P.long_unit_adj_smem;
+  for (const LongItem& it : P.long_items) A.long_rec_words = std::max(A.long_rec_words, it.G <= kUnitMaxW ? 1 : 4);
   A.long_wide_block = P.long_wide_block ? 1 : 0;
   A.long_wide_smem = P.long_wide_smem;
   A.chained = P.chained ? 1 : 0;
@@ -880,14 +881,15 @@ BwdLayout backward_layout(const dg_arena* ar, int iters, int ckpt_every) {
   L.var_in = put(n * 8);
   L.slot_in = put(US < NS ? NS * 8 : 0);
   // long BDDs: node and slot records of every sweep of one segment, and the
-  // per-node gradients of the adjoint
-  const size_t lcost = (size_t)ar->dev.long_cost_size, lslots = NS - (size_t)ar->dev.long_slot_base;
+  // per-node gradients of the adjoint (none of these for the unit ones)
+  const bool general = ar->dev.num_long > ar->dev.num_long_unit;
+  const size_t lcost = general ? (size_t)ar->dev.long_cost_size : 0, lslots = NS - (size_t)ar->dev.long_slot_base;
   L.lmeta_stride = lcost * 4;
-  L.lamin_stride = lslots * 8;
+  L.lamin_stride = general ? lslots * 8 : 0;
   L.rec_lmeta = put((size_t)2 * L.k * L.lmeta_stride);
   L.rec_lamin = put((size_t)2 * L.k * L.lamin_stride);
-  // ... of the long unit BDDs four words per long slot (none without them)
-  L.lunit_stride = ar->dev.num_long_unit > 0 ? lslots * 16 : 0;
+  // ... of the long unit BDDs a word or four per long slot
+  L.lunit_stride = lslots * 4 * (size_t)ar->dev.long_rec_words;
   L.rec_lunit = put((size_t)2 * L.k * L.lunit_stride);
   L.long_a1 = put(lcost * 4);
   L.long_a2 = put(lcost * 4);
@@ -930,7 +932,7 @@ dg_status enqueue_recorded_segment(dg_arena* ar, Chain& ch, float* lam, float* M
     ra.rec_diff = (float*)(w + L.rec_diff) + (size_t)sw * NS;
     ra.rec_lmeta = (int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
     ra.rec_lamin = (int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
-    ra.rec_lunit = (uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
+    ra.rec_lunit = (uint32_t*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
     // each recording sweep hands its path costs (and records) to the next
     ra.cost_out = A.nodecost;
     if (sw > 0) {
@@ -1095,8 +1097,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       ra.rec_diff = rec_diff + (size_t)sw * NS;
       ra.rec_lmeta = (int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
       ra.rec_lamin = (int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
-      ra.rec_lunit = (uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
-    ra.rec_lunit = (uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
+      ra.rec_lunit = (uint32_t*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
       ra.cost_out = A.nodecost;  // handed on from recording sweep to recording sweep
       if (sw > 0) {
         ra.cost_in = A.nodecost;
@@ -1120,7 +1121,7 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
       aa.rec_diff = rec_diff + (size_t)sw * NS;
       aa.rec_lmeta = (const int32_t*)(w + L.rec_lmeta + (size_t)sw * L.lmeta_stride);
       aa.rec_lamin = (const int2*)(w + L.rec_lamin + (size_t)sw * L.lamin_stride);
-      aa.rec_lunit = (const uint4*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
+      aa.rec_lunit = (const uint32_t*)(w + L.rec_lunit + (size_t)sw * L.lunit_stride);
       aa.S_in = seg_S + (size_t)sw * n;
       aa.seed_M = gsw == last_sweep ? g_M_T : nullptr;
       aa.sdot_next = gsw == last_sweep ? nullptr : sd_next;

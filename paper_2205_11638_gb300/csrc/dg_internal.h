@@ -233,6 +233,7 @@ struct DevArena {
   int32_t long_wide_smem;   // shared memory of the largest wide long BDD's path costs (0: they stay in long_d, long_t)
   int32_t long_unit_smem[2];  // shared memory of the largest work item, mode 0 and 1
   int32_t long_unit_adj_smem;
+  int32_t long_rec_words;   // words per slot of the long unit BDDs' records: 4, 1 when lanes hold all of them, 0 for none
   int32_t long_lanes;       // lanes per narrow BDD in the plain sweeps (a power of two, set at bind)
   int32_t chained;          // a sweep's launches form one chain (see Plan::chained)
 };

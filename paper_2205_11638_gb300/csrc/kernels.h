@@ -47,9 +47,11 @@ struct SweepArgs {
   // hi-choice, per long slot (from long_slot_base) the argmin nodes of m0, m1
   int32_t* rec_lmeta;
   int2* rec_lamin;
-  // ... and for the long unit BDDs per long slot (from long_slot_base) the
-  // out-arc bits of the level, the in-arc bits of the next, and argmin states
-  uint4* rec_lunit;
+  // ... and for the long unit BDDs per long slot (from long_slot_base)
+  // long_rec_words words: the unit tiles' word where a lane holds a level, else
+  // the out-arc bits of the level, the in-arc bits of the next, and the argmin
+  // states
+  uint32_t* rec_lunit;
 };
 
 // The caller's stream plus kStreams - 1 auxiliary streams of an arena: the
@@ -186,7 +188,7 @@ struct AdjArgs {
   // SP(., T) and SP(r, .)
   const int32_t* rec_lmeta;
   const int2* rec_lamin;
-  const uint4* rec_lunit;
+  const uint32_t* rec_lunit;
   float* long_a1;
   float* long_a2;
 };

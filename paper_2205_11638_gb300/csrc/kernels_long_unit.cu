@@ -236,7 +236,7 @@ __device__ __forceinline__ void walk_segments(const DevArena& A, const SweepArgs
     const uint32_t b0 = seg_bits<G>(x0 == m0, g.base), b1 = seg_bits<G>(x1 == m1, g.base);
     const int v0 = b0 ? 31 - __clz((int)b0) : 0, v1 = b1 ? 31 - __clz((int)b1) : 0;
     if (g.s == 0 && on)
-      a.rec_lunit[(int64_t)B.slot_base + h - A.long_slot_base] =
+      reinterpret_cast<uint4*>(a.rec_lunit)[(int64_t)B.slot_base + h - A.long_slot_base] =
           make_uint4(tb, rb, (uint32_t)v0 | (uint32_t)v1 << 8 | ex << 16, 0u);
   };
 
@@ -456,7 +456,8 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
       if (u == it.start) e = t.v[u];
     a.E[B.row] = e;
   };
-  uint4* rec_out = REC ? a.rec_lunit + (B.slot_base - A.long_slot_base) : nullptr;
+  const int words = A.long_rec_words;
+  uint32_t* rec_out = REC ? a.rec_lunit + (int64_t)(B.slot_base - A.long_slot_base) * words : nullptr;
 
   if (FWD || KIND == kMinMarg) {
     first_up();
@@ -476,7 +477,7 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
           unit_minima_rec<W, TY>(R, t1, b0, b1, rec);
           unit_up_rec<W, TY>(t1, in.l, rec);
           R = unit_down_rec<W, TY>(R, update(h, in, b0, b1), rec);
-          rec_out[h].x = rec;
+          rec_out[h * words] = rec;
         } else {
           unit_minima<W, TY>(R, t1, b0, b1);
           float ln = in.l;
@@ -521,7 +522,7 @@ __device__ __forceinline__ void walk_lanes(const DevArena& A, const SweepArgs& a
           unit_minima_rec<W, TY>(r, t, b0, b1, rec);
           unit_down_rec<W, TY>(r, in.l, rec);
           t = unit_up_rec<W, TY>(t, update(h, in, b0, b1), rec);
-          rec_out[h].x = rec;
+          rec_out[h * words] = rec;
         } else {
           unit_minima<W, TY>(r, t, b0, b1);
           t = unit_up<W, TY>(t, update(h, in, b0, b1));
@@ -781,7 +782,7 @@ __device__ __forceinline__ void adjoint_segments(const DevArena& A, const AdjArg
 // ... in the registers of the BDD's lane (lanes and levels as in walk_lanes).
 template <int FWD, int MODE, int W>
 __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& a, const LongItem& it,
-                                              const uint4* rec, float2* in, float* gl, float* df, float* al,
+                                              const uint32_t* rec, float2* in, float* gl, float* df, float* al,
                                               const float* om, int lane) {
   const int ST = long_unit_stride(it.kmax), row = lane % it.nseg;
   const LongBdd B = A.longs[A.long_order[it.first + row]];
@@ -791,7 +792,7 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
   float* mw = al + row * ST;
   const float* mo = om + row * ST;
   float2* mi = in + row * ST;
-  const uint4* mr = rec + row * ST;
+  const uint32_t* mr = rec + row * ST;
   const float* seed = a.seed_M ? a.seed_M + B.slot_base : nullptr;
   auto down_levels = [&](auto&& step) {
     runs_down(A, it, [&](auto ty, int b, int e) {
@@ -816,7 +817,7 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
   };
   auto input = [&](int h) {
     const int x = min(max(h, 0), last);
-    return In{mr[x].x, mg[x], md[x], mw[x], MODE == 1 ? mo[x] : a.omega0, seed ? seed[x] : 0.0f, mi[x]};
+    return In{mr[x], mg[x], md[x], mw[x], MODE == 1 ? mo[x] : a.omega0, seed ? seed[x] : 0.0f, mi[x]};
   };
   auto reverse = [&](int h, const In& x, float g) -> float {
     const float Mt = x.seed + x.v.x - g;
@@ -850,12 +851,12 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
     __syncwarp();
     // SP(., T) under lambda^old: its gradient flows top-down
     clear(x);
-    uint32_t rc = mr[0].x;
+    uint32_t rc = mr[0];
     float d = md[0], g0 = mg[0];
     down_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
       const int n = min(h + 1, last);
-      const uint32_t rc1 = mr[n].x;
+      const uint32_t rc1 = mr[n];
       const float d1 = md[n], g1 = mg[n];
       __syncwarp();
       if (on) {
@@ -891,12 +892,12 @@ __device__ __forceinline__ void adjoint_lanes(const DevArena& A, const AdjArgs& 
     __syncwarp();
     // SP(r, .) under lambda^old: its gradient flows bottom-up
     clear(x);
-    uint32_t rc = mr[last].x;
+    uint32_t rc = mr[last];
     float d = md[last], g0 = mg[last];
     up_levels([&](auto ty, int h, bool on) {
       constexpr int TY = decltype(ty)::value;
       const int n = max(h - 1, 0);
-      const uint32_t rc1 = mr[n].x;
+      const uint32_t rc1 = mr[n];
       const float d1 = md[n], g1 = mg[n];
       __syncwarp();
       if (on) {
@@ -940,8 +941,15 @@ __device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const 
     copy_row(df + r * ST, a.rec_diff + B.slot_base, B.k, lane, pol);
     copy_row(al + r * ST, (MODE == 1 ? a.alpha : A.slot_invdeg) + B.slot_base, B.k, lane, pol);
     if (MODE == 1) copy_row(om + r * ST, a.omega + B.slot_base, B.k, lane, pol);
-    const uint4* src = a.rec_lunit + (B.slot_base - A.long_slot_base);
-    for (int h = lane; h < B.k; h += kWarp) cp_async16(rec + r * ST + h, src + h, pol);
+    // (a lane's BDD: the first word of a slot, side by side)
+    const int words = A.long_rec_words;
+    const uint32_t* src = a.rec_lunit + (int64_t)(B.slot_base - A.long_slot_base) * words;
+    if (G > kUnitMaxW)
+      for (int h = lane; h < B.k; h += kWarp) cp_async16(rec + r * ST + h, src + 4 * h, pol);
+    else if (words == 1)
+      copy_row(reinterpret_cast<float*>(rec) + r * ST, src, B.k, lane, pol);
+    else
+      for (int h = lane; h < B.k; h += kWarp) cp_async4(reinterpret_cast<uint32_t*>(rec) + r * ST + h, src + 4 * h);
   }
   cp_async_commit();
   cp_async_wait_one();
@@ -956,7 +964,7 @@ __device__ __forceinline__ void long_unit_adjoint_item(const DevArena& A, const 
   __syncwarp();
 
   if constexpr (G <= kUnitMaxW)
-    adjoint_lanes<FWD, MODE, G>(A, a, it, rec, in, gl, df, al, om, lane);
+    adjoint_lanes<FWD, MODE, G>(A, a, it, reinterpret_cast<const uint32_t*>(rec), in, gl, df, al, om, lane);
   else
     adjoint_segments<FWD, MODE, G>(A, a, it, rec, in, gl, df, al, om, lane);
   __syncwarp();

@@ -437,3 +437,12 @@ def test_long_unit_rows_at_any_packing(lanes, mode):
     for a, b in zip(*grads):
         assert torch.isfinite(a).all()
         assert (a - b).abs().max() <= 64 * 4 * 2.0 ** -24 * b.abs().max().clamp(min=1e-30)
+
+
+def test_workspace_of_long_unit_rows():
+    """Their records (a word a level where a lane holds it) replace those of the
+    general kernels (16 bytes for two states): no more memory for a training step
+    than the doubled problem takes, and 5 % for partly filled tiles."""
+    p = workloads.assignment(L=30, R=300, cand=260, seed=44)
+    a, b = [solver.plan(q).bind().backward_workspace_bytes(10, 10) for q in (p, _doubled(p))]
+    assert a <= 1.05 * b
