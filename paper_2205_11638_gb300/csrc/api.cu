@@ -1074,7 +1074,10 @@ dg_status backward_impl(dg_arena* ar, void* stream, const float* lam0, const flo
   aa.slot_in = slot_in;
   aa.var_in = var_in;
   // padding slots belong to no variable: their inputs stay 0
-  if (e == cudaSuccess && (size_t)A.unit_slots < NS) e = cudaMemsetAsync(slot_in, 0, NS * 8, st);
+  if (e == cudaSuccess && (size_t)A.unit_slots < NS) {
+    ch.linked = false;
+    e = cudaMemsetAsync(slot_in, 0, NS * 8, st);
+  }
   aa.long_a1 = (float*)(w + L.long_a1);
   aa.long_a2 = (float*)(w + L.long_a2);
   const int last_sweep = 2 * iters - 1;
