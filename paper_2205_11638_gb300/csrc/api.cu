@@ -231,7 +231,7 @@ dg_status dg_launch_group(const dg_plan_t* plan, int32_t g, int32_t* tile0, int3
   const LaunchGroup& G = plan->p.groups[g];
   if (tile0) *tile0 = G.tile0;
   if (tile1) *tile1 = G.tile1;
-  if (region_bytes) *region_bytes = G.region_bytes0;
+  if (region_bytes) *region_bytes = G.unit_short ? 0 : (G.unit_w ? G.unit_bytes0 : G.region_bytes0);
   if (stream) *stream = G.stream;
   return DG_OK;
 }

@@ -322,3 +322,15 @@ def test_validator_catches_each_corruption_of_long_rows(tmp_path):
     assert len(res) == 11
     for name, (st, msg) in res.items():
         assert st == _lib.DG_EINVAL and msg.startswith("dg_plan_validate:"), (name, st, msg)
+
+
+def test_launch_group_reports_the_memory_its_kernels_use():
+    """Per level two words and, for every second level but the last, the path
+    costs of two states; nothing for rows of up to three levels; the general
+    kernels' staging once the rows are doubled."""
+    def amo(k, twice=1):
+        rows = [(np.arange(k), twice * np.ones(k, np.int64), workloads.LE, twice)] * 32
+        return workloads.single_rows_problem(rows, k, np.ones(k))
+    assert [g[2] for g in solver.plan(amo(6)).launch_groups()] == [32 * 4 * (2 * 6 + 2 * 2)]
+    assert [g[2] for g in solver.plan(amo(3)).launch_groups()] == [0]
+    assert solver.plan(amo(6, 2)).launch_groups()[0][2] > 32 * 4 * (2 * 6 + 2 * 2)
