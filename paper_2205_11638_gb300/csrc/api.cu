@@ -464,16 +464,32 @@ dg_status dg_bind(const dg_plan_t* plan, void* arena_dev, size_t arena_bytes, vo
   S.num_arcs = 2 * P.sizes.num_nodes;
   const double Nv = (double)P.sizes.num_nodes, Nl = (double)P.sizes.num_lambda, n = (double)P.sizes.n;
   S.bytes_per_iter = 32.0 * Nv + 48.0 * Nl + 16.0 * n;
-  const double NVp = (double)P.sizes.num_nodes_padded, ns = (double)P.sizes.num_slots;
-  // per sweep (the path costs handed on, as inside dg_iterate): children
-  // 2 B and the costs read and written 8 B per node; descriptor, lambda read
-  // and write, M write, averaging term 18 B per slot; alpha 4 B per lambda
-  // (mode 1).  Per S reduction: M read and averaging term written 8 B per
-  // lambda, ELL columns 16 B and S, S/|J_i| 8 B per variable.
-  // long BDDs per sweep: children 8 B, in-arcs ~8 B and the path costs 8 B
-  // per node
-  S.actual_bytes_per_iter = 2.0 * (10.0 * NVp + 18.0 * ns + 4.0 * Nl) + 2.0 * (24.0 * n + 8.0 * Nl) +
-                            2.0 * 24.0 * (double)P.sizes.num_long_nodes;
+  // a plain iteration inside dg_iterate, mode 0.  Per sweep: unit tiles a
+  // variable id and lambda read per slot, the averaging term read and lambda
+  // and M written per pair; mixed tiles the child codes 2 B and the handed-on
+  // path costs, read and written, 8 B per node, and descriptor, lambda read and
+  // written, M and the averaging term 18 B per slot; long BDDs as the unit tiles
+  // per level, or (other rows, and unit rows swept with these) children 8 B,
+  // in-arcs ~8 B and path costs 8 B per node and 16 B per level.  Per S
+  // reduction: M 4 B per pair, the averaging term written 4 B per pair that
+  // reads it per slot, ELL columns 16 B and the term 4 B per variable.
+  double unit_pairs = 0, long_levels = 0, general_levels = 0, general_nodes = 0;
+  for (const Tile& t : P.tiles)
+    if (t.unit) unit_pairs += (double)t.nhops * t.nbdd;
+  for (int32_t i = 0; i < (int32_t)P.longs.size(); ++i) {
+    const LongBdd& L = P.longs[P.long_order[i]];
+    long_levels += L.k;
+    if (i < P.long_plain) continue;
+    general_levels += L.k;
+    general_nodes += L.nn;
+  }
+  const double mixed_pairs = Nl - unit_pairs - long_levels;
+  const double mixed_nodes = (double)P.sizes.num_nodes_padded - P.unit_nodes;
+  const double sweep = 8.0 * P.unit_slots + 12.0 * unit_pairs + 10.0 * mixed_nodes +
+                       18.0 * (P.long_slot_base - P.unit_slots) + 20.0 * (long_levels - general_levels) +
+                       24.0 * general_nodes + 16.0 * general_levels;
+  const double scattered = mixed_pairs + (P.long_plain < (int32_t)P.longs.size() ? long_levels : 0.0);
+  S.actual_bytes_per_iter = 2.0 * (sweep + 4.0 * Nl + 4.0 * scattered + 20.0 * n);
   for (int i = 0; i < 64; ++i) S.hop_histogram[i] = P.hop_histogram[i];
   *out = ar;
   return DG_OK;

@@ -85,3 +85,18 @@ def test_one_launch_while_the_variables_are_few(n, launches):
     rows = [(np.sort(rng.choice(n, size=3, replace=False)), np.ones(3, np.int64), workloads.GE, 1) for _ in range(20)]
     A = solver.plan(workloads.single_rows_problem(rows, n, rng.normal(size=n))).bind()
     assert A.iterate_launches(2) == launches
+
+
+def test_bytes_of_an_iteration():
+    """Rows of +1 and -1 move 20 bytes a pair and sweep and no node data, 4 bytes
+    a pair and 20 a variable in a reduction (partly filled tiles add their ids
+    and lambda, at most 8 bytes a slot); the doubled rows at least the child codes
+    and path costs of their nodes on top."""
+    p = workloads.tracking(frames=30, dets=400, seed=9)
+    A, B = solver.plan(p).bind(), solver.plan(_doubled(p)).bind()
+    pairs, n = len(p["col"]), p["n"]
+    least = 2 * (20 * pairs + 4 * pairs + 20 * n)
+    assert least <= A.stats.actual_bytes_per_iter <= least + 2 * 8 * (A.num_slots - pairs)
+    assert B.stats.actual_bytes_per_iter >= 2 * (10 * int(B.plan.sizes.num_nodes) + 16 * pairs) + 2 * 8 * pairs
+    L = solver.plan(workloads.assignment(L=20, R=300, cand=260, seed=44)).bind()
+    assert L.stats.actual_bytes_per_iter < 2 * (28 * L.num_slots + 20 * L.n)
