@@ -591,20 +591,32 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     return src[t].unit >= 0 ? unit_smem_bytes(units[src[t].unit].s, 1)
                             : sweep_smem_bytes(tile_nmax[t], tile_nh[t], 1, ring_size(tile_maxw[t]));
   };
+  int nunit = 0, nshort = 0;
+  size_t largest = 1;  // footprint
+  for (int t = 0; t < T; ++t) {
+    nunit += src[t].unit >= 0;
+    nshort += src[t].unit >= 0 && unit_short(units[src[t].unit].s);
+    largest = std::max(largest, tile_smem(t));
+  }
+  // An arena of unit tiles alone is one launch (then chained, see Plan::chained)
+  // while its tiles, at the largest one's footprint, fill the chip at most
+  // kOneLaunchFills times and that footprint leaves at least seven warps per SM.
+  // us per iteration (plain; per slot; recorded and reversed), one launch /
+  // several forked: tracking with 50 frames of 400 detections 17; 18; 53 / 29;
+  // 29; 75, 25 frames of 2,000, 2.8 fills 33; 34; 90 / 38; 40; 98, 50 frames, 5.2
+  // fills 49; 54; 152 / 51; 59; 153, 80 frames, 10 fills 70; 85; 253 / 70; 77; 224.
+  constexpr size_t kSmSmem = 224 * 1024, kOneLaunchFills = 6, kOneLaunchSmem = 32 * 1024;
+  const bool one_launch = nunit == T && long_rows.empty() && largest <= kOneLaunchSmem &&
+                          (size_t)T <= kOneLaunchFills * kSms * std::min<size_t>(64, kSmSmem / largest);
   // The kernels for short unit tiles take them where they are most of the unit
   // tiles.  As one more launch group they cost a few microseconds a sweep (the
   // launch, or the fork and join of a stream), so only where they are all, or
-  // next to many others.  Measured (GB300) without and with them: independent
-  // set of 10,000 (all short) 9.9 -> 9.35 us an iteration; batches of 64 and 8
-  // mixed instances 189 -> 168 and 49.6 -> 48.6, of 4 (5,000 tiles) 25 -> 36;
-  // matching, 1,900 tiles, training pass 1.53 -> 1.75 ms.
+  // next to many others, and where that is not one launch more.  us an iteration
+  // without and with them: batch of 64 mixed instances, replayed from a graph,
+  // 159 / 144; of 8, 12,300 tiles, one launch without, 37 / 43; of 4 19 / 33;
+  // matching 16 / 20.
   constexpr int kShortTiles = 8192;
-  int nunit = 0, nshort = 0;
-  for (const auto& x : src) {
-    nunit += x.unit >= 0;
-    nshort += x.unit >= 0 && unit_short(units[x.unit].s);
-  }
-  const bool short_kernels = nshort == nunit || (2 * nshort >= nunit && nunit >= kShortTiles);
+  const bool short_kernels = nshort == nunit || (2 * nshort >= nunit && nunit >= kShortTiles && !one_launch);
   // (kind 0: unit tiles, 1: short unit tiles, 2: mixed tiles)
   auto tile_kind = [&](int t) {
     return src[t].unit < 0 ? 2 : (short_kernels && unit_short(units[src[t].unit].s) ? 1 : 0);
@@ -701,7 +713,6 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
         opts && opts->group_ratio_pct > 0 && opts->group_ratio_pct <= 100 ? opts->group_ratio_pct / 100.0 : 0.85;
     // ... or any smaller one while the group's tiles do not fill the chip (its
     // smaller tiles then cost it no occupancy and save a launch)
-    constexpr size_t kSmSmem = 224 * 1024;
     // ... but no tile that would keep the group's recording sweeps from fitting a
     // CTA: these take the largest footprint and the largest records together
     constexpr size_t kCtaSmem = 227 * 1024;
@@ -716,20 +727,6 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       const Tile& tl = P.tiles[t];
       return !tl.unit ? 2 : (short_kernels && unit_short(P.unit_shapes[tl.unit - 1]) ? 1 : 0);
     };
-    // ... and an arena of unit tiles alone is one launch (then chained, see
-    // Plan::chained) while its tiles, at the largest one's footprint, fill the
-    // chip at most kOneLaunchFills times and that footprint leaves at least
-    // seven warps per SM.  us per iteration (plain; per slot; recorded and
-    // reversed), one launch / several forked: tracking with 50 frames of 400
-    // detections 17; 18; 53 / 29; 29; 75, 25 frames of 2,000, 2.8 fills 33; 34;
-    // 90 / 38; 40; 98, 50 frames, 5.2 fills 49; 54; 152 / 51; 59; 153, 80 frames,
-    // 10 fills 70; 85; 253 / 70; 77; 224.
-    constexpr size_t kOneLaunchFills = 6, kOneLaunchSmem = 32 * 1024;
-    const size_t largest = T > 0 ? group_smem(0) : 0;
-    int others = 0;  // tiles that are not the short kernels'
-    for (int t = 0; t < T; ++t) others += group_kind(t) == 0;
-    const bool one_launch = T > 0 && nunit == T && long_rows.empty() && largest <= kOneLaunchSmem &&
-                            (size_t)others <= kOneLaunchFills * kSms * std::min<size_t>(64, kSmSmem / largest);
     for (int t = 0; t <= T; ++t) {
       const size_t r = t < T ? group_smem(t) : 0;
       const bool full = gmax > 0 && (size_t)(t - t0) >= kSms * std::min<size_t>(64, kSmSmem / gmax);
@@ -953,7 +950,6 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
     // the longest items first
     std::stable_sort(P.long_items.begin(), P.long_items.end(),
                      [](const LongItem& x, const LongItem& y) { return x.kmax > y.kmax; });
-    constexpr int kChainTiles = 16384;
     // Plain sweeps of the unit ones.  Their kernels walk every level twice, with
     // the path costs in shared memory, which leaves few warps to an SM when the
     // rows are long and wide; the general kernel takes the costs of the sweep
@@ -974,8 +970,7 @@ dg_status build_plan(const dg_rows* R, const dg_options* opts, Plan& P) {
       P.long_plain = unit > std::max(rate, chain) ? 0 : P.num_long_unit;
     }
     P.chained = P.long_plain == (int32_t)P.longs.size() &&
-                (T == 0 || (nunit == T && P.longs.empty() &&
-                            (P.groups.size() == 1 || (P.groups.size() == 2 && P.groups[1].unit_short && T <= kChainTiles))));
+                (T == 0 || (nunit == T && P.longs.empty() && P.groups.size() == 1));
     P.num_long_narrow = (int32_t)P.long_order.size();
     P.long_lanes = opts ? opts->long_lanes : 0;
     size_t wide = 0;

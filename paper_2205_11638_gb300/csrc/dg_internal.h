@@ -282,12 +282,9 @@ struct Plan {
   // Whether a sweep's launches form one chain on the caller's stream instead of
   // forking onto the arena's streams.  A small arena's time is launch latency,
   // which the chain hides; but its kernels run one after another, so that only
-  // arenas of one launch group take it (or of long unit BDDs alone), or of two
-  // when the second is of short tiles and small (kChainTiles): these need no
-  // shared memory and little time.  us per iteration and per iteration recorded
-  // and reversed, chained / forked: batch of 8, 12,300 tiles, two groups 42 / 51
-  // and 114 / 115; tracking with 80 frames of 2,000, 15,200 tiles, four groups
-  // 99 / 71 and 279 / 223.
+  // arenas of one launch group take it, or of long unit BDDs alone.  us per
+  // iteration and per iteration recorded and reversed, chained / forked: tracking
+  // with 80 frames of 2,000, 15,200 tiles, four groups 99 / 71 and 279 / 223.
   bool chained = false;
   std::vector<uint16_t> desc;
   std::vector<uint16_t> lohi8;

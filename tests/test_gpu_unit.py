@@ -290,11 +290,11 @@ def _mostly_short(seed, n=20000):
     return workloads.single_rows_problem(rows, n, rng.normal(size=n))
 
 
-# instance, launch groups: one launch for tiles of many shapes; two, the second
-# of short tiles, one after the other; two on streams of their own
+# instance, launch groups: one launch for tiles of many shapes, and where most
+# are short; two on streams of their own
 LAUNCHES = {
     "one": (lambda: workloads.tracking(frames=50, dets=400, seed=46), 1),
-    "short_second": (lambda: _mostly_short(7), 2),
+    "mostly_short": (lambda: _mostly_short(7), 1),
     "forked": (lambda: _two_footprints(8), 2),
 }
 
