@@ -82,7 +82,7 @@ def _profile_traffic(kernel_key: str, src_sha: str):
 
 def _kernel_source_sha():
     h = hashlib.sha256()
-    for f in ("kernels_sweep.cu", "sweep.cuh"):
+    for f in ("kernels_sweep.cu", "kernels_unit.cu", "sweep.cuh", "unit.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2205_11638_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -415,10 +415,10 @@ def _independent_set_measurement(solver, torch, iters=200, reps=5):
 def _long_rows_measurement(solver, torch, iters=50, reps=3):
     """Sparse assignment with long rows (2,000 x 2,000, 300 candidates per
     left node: 4,000 rows of about 300 variables, every BDD beyond a tile
-    lane, every level two nodes wide): the plain sweeps of narrow long BDDs,
-    several to a warp.  Arc updates per second over a CUDA-graph replay of
-    50 iterations, and the roofline of the long-BDD sweep kernel from its
-    own CUDA-event time."""
+    lane, every level two nodes wide): the plain sweeps of long rows of +1,
+    a BDD's level in one lane's registers.  Arc updates per second over a
+    CUDA-graph replay of 50 iterations, and the roofline of that sweep kernel
+    from its own CUDA-event time (16 B per pair and 4 B per variable)."""
     prob = workloads.assignment()
     A = solver.plan(prob).bind()
     st = A.stats
@@ -455,14 +455,14 @@ def _long_rows_measurement(solver, torch, iters=50, reps=3):
     t = statistics.median(ms)
     sweep_ms = statistics.mean(sw)
     Nv, Nl = st.sizes.num_nodes, st.sizes.num_lambda
-    sweep_bytes = 16.0 * Nv + 16.0 * Nl
+    sweep_bytes = 16.0 * Nl + 4.0 * float(st.sizes.n)
     peak, peak_src = _peaks()
     achieved = sweep_bytes / (sweep_ms * 1e-3) / 1e9
     return {"workload": "assignment_2000x300", "n_vars": int(st.sizes.n), "constraints": int(st.sizes.m),
             "N_lambda": int(Nl), "N_v": int(Nv), "long_bdds": int(st.sizes.num_long_bdds),
             "long_nodes": int(st.sizes.num_long_nodes), "iterations": iters,
             "value": 4 * Nv * iters / (t * 1e-3), "unit": UNIT, "ms_per_iteration": t / iters,
-            "roofline": {"bound": "hbm", "kernel": "k_long_narrow (forward and backward; long BDDs of narrow levels, several to a warp)",
+            "roofline": {"bound": "hbm", "kernel": "k_long_unit (forward and backward; long rows of +1, a BDD to a lane)",
                          "algorithmic_bytes_per_launch": sweep_bytes, "avg_launch_ms": sweep_ms,
                          "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "peak_source": peak_src},
@@ -788,21 +788,32 @@ def run_ours(args):
     ms_per_step = total_ms / args.steps
 
     # roofline of the dominant kernel (the sweep; forward and backward have
-    # the same algorithmic bytes): 16 B per node + 16 B per slot per sweep
-    sweep_bytes = 16.0 * Nv + 16.0 * Nl
+    # the same algorithmic bytes).  Rows of +1 and -1 need no node data: per pair
+    # lambda read and written, M written and a variable id 16 B, the averaging
+    # term 4 B per variable; others 16 B per node + 16 B per slot
+    unit_rows = bool((np.abs(prob["coef"]) == 1).all())
+    node_bytes = 16.0 * Nv + 16.0 * Nl
+    sweep_bytes = 16.0 * Nl + 4.0 * n if unit_rows else node_bytes
     sweep_ms = statistics.mean(t_fwd + t_bwd)
     peak, peak_src = _peaks()
     achieved = sweep_bytes / (sweep_ms * 1e-3) / 1e9
     src_sha = _kernel_source_sha()
     traffic = _profile_traffic(f"sweep_{args.workload}", src_sha)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": traffic, "peak_source": peak_src, "kernel": "k_sweep (forward and backward)",
+            "traffic": traffic, "peak_source": peak_src,
+            "kernel": "k_unit (forward and backward; rows of +1 and -1)" if unit_rows else "k_sweep (forward and backward)",
             "algorithmic_bytes_per_launch": sweep_bytes, "avg_launch_ms": sweep_ms,
+            # the byte count of sweeps that read every BDD node, for comparison with
+            # figures taken that way: no kernel moves these bytes for rows of +-1
+            "node_data_bytes_per_launch": node_bytes,
+            "node_data_frac": node_bytes / (sweep_ms * 1e-3) / 1e9 / peak,
+            "iteration_bytes_moved": st.actual_bytes_per_iter,
+            "iteration_moved_frac": st.actual_bytes_per_iter / (ms_per_step * 1e-3) / 1e9 / peak,
             "iteration_algorithmic_bytes": st.bytes_per_iter,
             "iteration_frac": st.bytes_per_iter / (ms_per_step * 1e-3) / 1e9 / peak,
             "dram_traffic_frac": (traffic / (sweep_ms * 1e-3) / 1e9 / peak) if traffic else None,
             "kernel_source_sha": src_sha}
-    shares = {"k_sweep_fwd": sum(t_fwd), "k_reduce_S": sum(t_red) + 0.0, "k_sweep_bwd": sum(t_bwd),
+    shares = {"sweep_fwd": sum(t_fwd), "k_reduce_S": sum(t_red) + 0.0, "sweep_bwd": sum(t_bwd),
               "k_reduce_S+k_lb": sum(t_tail)}
     tot = sum(shares.values())
     shares = {k: v / tot for k, v in shares.items()}
