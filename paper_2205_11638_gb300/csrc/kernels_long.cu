@@ -23,11 +23,13 @@
 // are handed on) skips its first pass: they are already in place.
 //
 // The plain forward and backward sweeps of the long BDDs whose levels have
-// at most 32 nodes (long cardinality and assignment rows) run in
-// k_long_narrow instead: several such BDDs to a warp, G lanes each, the
-// costs of the sweep direction in registers (see narrow_down / narrow_up).
-// The recording sweeps, energies, seeds, min-marginals, smoothed
-// subproblems and adjoints keep one warp per BDD.
+// at most 32 nodes run in k_long_narrow instead: several such BDDs to a warp, G
+// lanes each, the costs of the sweep direction in registers (see narrow_down /
+// narrow_up).  Their recording sweeps, energies, seeds, min-marginals and
+// adjoints keep one warp per BDD.  Rows of +1 and -1 among them (long cardinality
+// and assignment rows) have kernels of their own (kernels_long_unit.cu) for all
+// but the smoothed subproblems, and for plain sweeps where Plan::long_plain says
+// so.
 //
 // The arithmetic is the lane kernels': the same FP32 operations per arc;
 // minima are exact, so values do not depend on the order of the reduction;

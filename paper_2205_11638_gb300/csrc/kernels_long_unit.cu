@@ -16,7 +16,9 @@
 // recomputed into shared memory by a first walk, and each step's words are
 // read one step ahead.  New lambda and M replace the staged inputs and leave
 // in one coalesced pass.  The loops over explicit children and in-arcs in
-// global memory (kernels_long.cu) take half a microsecond a level.
+// global memory (kernels_long.cu) take half a microsecond a level, but need no
+// shared memory: long, wide and many rows make their plain sweeps there (see
+// where Plan::long_plain is set).
 //
 // Same FP32 operations, tie rules and records as there: results are equal bit
 // for bit, gradients up to the rounding of sums.

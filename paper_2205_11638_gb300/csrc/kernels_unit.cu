@@ -11,10 +11,12 @@
 //
 // Before these kernels, with the node-by-node kernel of the mixed tiles, and
 // now (GB300, wall clock, the S reductions included): tracking 500 x 2,000, 50
-// iterations 32.9 -> 18.1 ms; tracking 50 x 400 with per-slot parameters, 100
-// iterations 10.6 -> 1.8 ms; 64 instances batched, 50 iterations 14.7 -> 8.4 ms.
-// The tiles of six and eight states are 31 % of the issue slots busy, the gather
-// of the averaging terms bounds them.
+// iterations 33.0 -> 17.9 ms; tracking 50 x 400 with per-slot parameters, 100
+// iterations 10.5 -> 1.6 ms; 64 instances batched, 50 iterations 15.3 -> 8.4 ms.
+// No unit is saturated: the launches of six and eight states issue in 21 to 30 %
+// of the slots at 17 to 44 % of the warps, DRAM at 11 to 15 % and L1 at 22 to
+// 31 % of their rates; the tiles wait for their ids, then for the gather of the
+// averaging terms, with as few warps as shared memory leaves.
 #include <algorithm>
 
 #include "kernels.h"
@@ -65,7 +67,6 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
       if (u == s.start) e = t.v[u];
     a.E[__ldg(A.slot_row + sb)] = e;
   };
-  // the update of a level from its minima; returns lambda^new
   // where the sweep leaves the level at hand
   const int64_t first = sb + (BWD ? s.k * kWarp : 0);
   float* g0 = (KIND == kMinMarg ? a.out2 : a.lam) + first;
@@ -80,6 +81,7 @@ __device__ __forceinline__ void unit_tile(const DevArena& A, const SweepArgs& a,
       gr += by;
     }
   };
+  // the update of a level from its minima; returns lambda^new
   auto update = [&](const float* x, float b0, float b1) -> float {
     const float l = x[0];
     const float m0 = b0, m1 = l + b1;
