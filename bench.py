@@ -844,7 +844,7 @@ def run_ours(args):
     # with one segment (the forward records every sweep: the argmin records
     # of all 2T sweeps stay in HBM and nothing is recomputed).  The headline
     # is the one-segment run when its workspace takes at most half of the
-    # free device memory (46.6 GB of the GB300's 280 GB for 100 iterations of
+    # free device memory (35.5 GB of the GB300's 280 GB for 100 iterations of
     # the tracking instance), else the checkpointed one; both are reported.
     adjoint = None
     if not args.no_adjoint:
