@@ -75,12 +75,11 @@ __global__ void __launch_bounds__(256) k_reduce_S(DevArena A, const float* M, in
       mine = e - b <= kWide - kEll;  // else a wide variable
     }
   }
-  const float inv = mode != 1 && mine ? __ldg(A.invdeg + i) : 1.0f;
   grid_wait();
   grid_trigger();
   if (!mine) return;
   const float s = wide ? sum_slots_warp(A, M, b, e, lane) : sum_slots(A, M, q, b, e);
-  const float t = inv * s;
+  const float t = mode == 1 ? s : __ldg(A.invdeg + i) * s;
   if (!wide || lane == 0) {
     if (need & kNeedS) A.S[i] = s;
     if (need & kNeedAvg) A.var_avg[i] = t;
